@@ -16,8 +16,12 @@
 //      inverted 32 x 32 diagonal blocks, then off-diagonal blocks -A^{-1} B D^{-1} level by level).
 //      Columns go from selection order to ascending I as they are written.
 //   4. W_p = U[I, :] V^T (Eq. 1).
-// FP64 runs on the CUDA cores (tensor-core FP64 is no faster on this part); every kernel here is
-// bound by FP64 issue rate or by streaming Z, and none waits on another CTA.
+// Products of 2^20 multiply-adds and more run on the tensor cores by exact slices (gemm_f64_tc.cu);
+// small ones, the panels of the Cholesky factorisation and the greedy steps run on the CUDA cores,
+// bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured on the two
+// parts that this replaced (all products on the CUDA cores; Cholesky by rank-1 updates):
+// 4096 x 4096, r = 2048: products 90.4 ms, Cholesky 37.8 ms of 310 ms; now 190 ms in all;
+// the M solves at m = n = 2048, r = 1024: 142.1 -> 21.3 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -29,29 +33,7 @@
 
 namespace {
 
-// ---- generic float64 GEMM --------------------------------------------------------------------
-// C[crow(i), ccol(j)] = beta C + alpha sum_k A(i, k) B(k, j), with
-//   A(i, k) = A[arow(i) * sa_i + k * sa_k],  arow(i) = aidx ? aidx[i] : i
-//   B(k, j) = B[k * sb_k + j * sb_j]
-//   C at C[i * ldc + (cidx ? cidx[j] : j)]
-// and a batch index z (blockIdx.z) offsetting A, B and C by za, zb, zc elements. `tri`: 1 = B is
-// lower triangular (B(k, j) = 0 for k < j), 2 = B is upper triangular (B(k, j) = 0 for k > j);
-// the k loop then skips the zero blocks.
-struct GemmF64 {
-  int M, N, K;
-  const double* A;
-  const int32_t* aidx;
-  int64_t sa_i, sa_k;
-  const double* B;
-  int64_t sb_k, sb_j;
-  double* C;
-  const int32_t* cidx;
-  int64_t ldc;
-  double alpha, beta;
-  int tri;
-  int64_t za, zb, zc;
-};
-
+// ---- float64 GEMM on the CUDA cores (GemmF64 in pifa_internal.h): small products ------------
 constexpr int GT = 64, GK = 16;  // output tile 64 x 64, k step 16; 256 threads, 4 x 4 outputs each
 
 __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
@@ -62,9 +44,11 @@ __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
   const double* A = p.A + blockIdx.z * p.za;
   const double* B = p.B + blockIdx.z * p.zb;
   double* C = p.C + blockIdx.z * p.zc;
+  if (p.lower && j0 > i0 + GT - 1) return;
   int kbeg = 0, kend = p.K;
-  if (p.tri == 1) kbeg = (j0 / GK) * GK;
-  if (p.tri == 2) kend = min(p.K, j0 + GT);
+  if (p.tri & 1) kbeg = (j0 / GK) * GK;
+  if (p.tri & 4) kbeg = max(kbeg, (i0 / GK) * GK);
+  if (p.tri & 2) kend = min(p.K, j0 + GT);
   double acc[4][4] = {};
   for (int k0 = kbeg; k0 < kend; k0 += GK) {
     for (int e = threadIdx.x; e < GT * GK; e += 256) {
@@ -120,25 +104,126 @@ int run_gemm_f64(const GemmF64& p, int batch, cudaStream_t s) {
   return e == cudaSuccess ? PIFA_OK : pifa_fail_cuda("compress: gemm launch", e);
 }
 
-// ---- Cholesky of G (r x r, lower triangle used), one column per launch -----------------------
-// Step j: L[i][j] = G[i][j] / sqrt(G[j][j]) for i >= j, and the trailing lower triangle
-// G[i][l] -= G[i][j] G[l][j] / G[j][j] for j < l <= i. Column j of G is only read in step j, so
-// the two parts need no ordering between threads. A non-positive pivot flags `bad`.
-__global__ void chol_step(double* G, double* L, int r, int j, int* bad) {
-  const int i = j + blockIdx.y * 16 + (threadIdx.x >> 4);
-  const int l = j + blockIdx.x * 16 + (threadIdx.x & 15);
-  if (i >= r || l > i) return;
-  const double d = G[(int64_t)j * r + j];
-  if (!(d > 0.0)) {
-    if (i == j && l == j) atomicExch(bad, 1);
-    return;
+// The same product by whichever form takes it: on the tensor cores by exact slices (gemm_f64_tc.cu)
+// from 2^20 multiply-adds on, with the caller's free scratch for the sliced operands, else on the
+// CUDA cores (one 64 x 64 tile of K = 128 keeps an SM's float64 pipe busy for about 130 us).
+int run_product(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t s) {
+  if (p.M <= 0 || p.N <= 0) return PIFA_OK;
+  if (gemm_f64_split_fits(p, bytes)) return gemm_f64_split(p, scratch, bytes, s);
+  return run_gemm_f64(p, 1, s);
+}
+
+// ---- Cholesky of G (r x r, pitch r, lower triangle used and overwritten) -------------------------
+// Blocked, right-looking: panels of 128 columns, each 32 columns at a time (chol_panel, then
+// chol_update for the rest of the panel), and the trailing matrix updated once per panel by a
+// K = 128 product. The predecessor, one rank-1 update of the whole trailing matrix with a division
+// per element and a launch per column, took 37.8 ms at r = 2048.
+constexpr int CB = 32;    // columns per chol_panel
+constexpr int CP = 128;   // columns per panel
+
+// Columns [j0, j0 + CB) of L. Every CTA factors the 32 x 32 diagonal block itself (as U D U^T with
+// unit-lower U, so that a column's critical path is one reciprocal, one multiply-add and one
+// barrier), then a thread per row below it substitutes that row. A non-positive pivot flags `bad`
+// and leaves its column of L zero.
+__global__ void __launch_bounds__(128) chol_panel(const double* G, double* L, int r, int j0, int* bad) {
+  __shared__ double D[CB][CB + 1];   // the block; column l of its lower part ends as d_l U[:, l]
+  __shared__ double rd[CB], rs[CB];  // 1 / d_l and 1 / sqrt(d_l), 0 where d_l is not positive
+  const int nb = min(CB, r - j0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = warp; i < CB; i += 4)
+    D[i][lane] = (i < nb && lane < nb) ? G[(int64_t)(j0 + i) * r + j0 + lane] : (i == lane ? 1.0 : 0.0);
+  __syncthreads();
+  for (int j = 0; j < CB; ++j) {
+    const double d = D[j][j];
+    const double inv = d > 0.0 ? 1.0 / d : 0.0;
+    const double f = D[lane][j] * inv;
+    if (threadIdx.x == 0) rd[j] = inv;
+    for (int l = j + 1 + ((warp - j - 1) & 3); l < CB; l += 4)
+      if (lane >= l) D[lane][l] = fma(-f, D[l][j], D[lane][l]);
+    __syncthreads();
   }
-  const double gij = G[(int64_t)i * r + j];
-  if (l == j) {
-    L[(int64_t)i * r + j] = gij / sqrt(d);
-  } else {
-    G[(int64_t)i * r + l] -= gij * G[(int64_t)l * r + j] / d;
+  if (warp == 0) {
+    const double d = D[lane][lane];
+    rs[lane] = d > 0.0 ? 1.0 / sqrt(d) : 0.0;
+    if (!(d > 0.0) && blockIdx.x == 0) atomicExch(bad, 1);
   }
+  __syncthreads();
+  if (blockIdx.x == 0)
+    for (int i = warp; i < nb; i += 4)
+      if (lane <= i) L[(int64_t)(j0 + i) * r + j0 + lane] = D[i][lane] * rs[lane];
+  const int64_t i = (int64_t)j0 + CB + (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= r) return;
+  const double* g = G + i * r + j0;
+  double y[CB];
+#pragma unroll
+  for (int l = 0; l < CB; ++l) y[l] = g[l];
+#pragma unroll
+  for (int l = 0; l < CB; ++l) {  // y_j -= (y_l / d_l) (d_l U_jl)
+    const double f = y[l] * rd[l];
+#pragma unroll
+    for (int j = l + 1; j < CB; ++j) y[j] = fma(-f, D[j][l], y[j]);
+  }
+  double* o = L + i * r + j0;
+#pragma unroll
+  for (int l = 0; l < CB; ++l) o[l] = y[l] * rs[l];
+}
+
+// G[i][l] -= sum over k in [j0, j0 + kn) of L[i][k] L[l][k] for l0 <= l < l1, i >= l (kn <= CB).
+// 64 x 32 tiles, 256 threads, 8 rows of one column each.
+__global__ void __launch_bounds__(256) chol_update(double* G, const double* L, int r, int j0, int kn, int l0, int l1) {
+  __shared__ double A[64][CB + 1];
+  __shared__ double B[CB][CB + 1];
+  const int i0 = l0 + blockIdx.y * 64, c0 = l0 + blockIdx.x * 32;
+  if (c0 > i0 + 63) return;  // wholly above the diagonal
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int u = warp; u < 64; u += 8) A[u][lane] = (i0 + u < r && lane < kn) ? L[(int64_t)(i0 + u) * r + j0 + lane] : 0.0;
+  for (int u = warp; u < 32; u += 8) B[u][lane] = (c0 + u < l1 && lane < kn) ? L[(int64_t)(c0 + u) * r + j0 + lane] : 0.0;
+  __syncthreads();
+  double acc[8] = {};
+#pragma unroll 8
+  for (int k = 0; k < CB; ++k) {
+    const double b = B[lane][k];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[u] = fma(A[warp * 8 + u][k], b, acc[u]);
+  }
+  const int l = c0 + lane;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = i0 + warp * 8 + u;
+    if (i < r && l < l1 && i >= l) G[(int64_t)i * r + l] -= acc[u];
+  }
+}
+
+// L (zeroed by the caller, pitch r) = the Cholesky factor of G; `scratch` for the sliced panels.
+int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t bytes, cudaStream_t s) {
+  const int ri = (int)r;
+  auto update = [&](int j0, int l0, int l1) {
+    const dim3 grid((unsigned)((l1 - l0 + 31) / 32), (unsigned)((ri - l0 + 63) / 64));
+    chol_update<<<grid, 256, 0, s>>>(G, L, ri, j0, ri - j0 < CB ? ri - j0 : CB, l0, l1);
+    pifa_count_launch();
+  };
+  for (int p0 = 0; p0 < ri; p0 += CP) {
+    const int p1 = p0 + CP < ri ? p0 + CP : ri;
+    GemmF64 t = {};  // the trailing update: G[p1:, p1:] -= L[p1:, p0:p1] L[p1:, p0:p1]^T
+    t.M = t.N = ri - p1; t.K = p1 - p0;
+    t.A = t.B = L + (int64_t)p1 * r + p0; t.sa_i = t.sb_j = r; t.sa_k = t.sb_k = 1;
+    t.C = G + (int64_t)p1 * r + p1; t.ldc = r; t.alpha = -1.0; t.beta = 1.0; t.lower = 1;
+    const bool split = t.M > 0 && gemm_f64_split_fits(t, bytes);
+    for (int j0 = p0; j0 < p1; j0 += CB) {
+      const int below = ri - j0 - CB;
+      chol_panel<<<below > 0 ? (unsigned)((below + 127) / 128) : 1u, 128, 0, s>>>(G, L, ri, j0, bad);
+      pifa_count_launch();
+      const int l1 = split ? p1 : ri;  // without the product, 32 columns at a time over everything
+      if (j0 + CB < l1) update(j0, j0 + CB, l1);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return pifa_fail_cuda("cholesky: launch", e);
+    if (split) {
+      const int st = gemm_f64_split(t, scratch, bytes, s);
+      if (st != PIFA_OK) return st;
+    }
+  }
+  return PIFA_OK;
 }
 
 // ---- greedy pivoted QR on the rows of Z -------------------------------------------------------
@@ -392,8 +477,9 @@ __global__ void max_abs(const double* C, int64_t rows, int64_t cols, int64_t ldc
 // Rinv = R^{-1} for an upper-triangular R (rp x rp, rp = 32 * 2^k; identity on any padding), by
 // doubling: the 32 x 32 diagonal blocks inverted directly, then, level by level, for every pair
 // of sz-blocks [[A, B], [0, D]] along the diagonal the off-diagonal block -A^{-1} (B D^{-1}).
-// Tt: scratch of rp * rp / 4 doubles.
-int upper_inverse(const double* R, double* Rinv, double* Tt, int rp, cudaStream_t s) {
+// Tt: scratch of rp * rp / 4 doubles; `scratch` for the sliced operands of the levels from 256 on
+// (below, all pairs of a level go in one batched launch on the CUDA cores).
+int upper_inverse(const double* R, double* Rinv, double* Tt, int rp, void* scratch, int64_t bytes, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(Rinv, 0, (size_t)rp * rp * 8, s);
   if (e != cudaSuccess) return pifa_fail_cuda("upper inverse: memset", e);
   inv_diag32<<<rp / 32, 32, 0, s>>>(R, Rinv, rp);
@@ -408,16 +494,24 @@ int upper_inverse(const double* R, double* Rinv, double* Tt, int rp, cudaStream_
     a.M = sz; a.N = sz; a.K = sz;
     a.A = R + sz; a.sa_i = rp; a.sa_k = 1;                        // B block
     a.B = Rinv + (int64_t)sz * rp + sz; a.sb_k = rp; a.sb_j = 1;  // D^{-1}
-    a.C = Tt; a.ldc = sz; a.alpha = 1.0; a.beta = 0.0;
+    a.C = Tt; a.ldc = sz; a.alpha = 1.0; a.beta = 0.0; a.tri = 2;
     a.za = step; a.zb = step; a.zc = (int64_t)sz * sz;
-    if ((st = run_gemm_f64(a, pairs, s)) != PIFA_OK) return st;
     GemmF64 b = {};
     b.M = sz; b.N = sz; b.K = sz;
     b.A = Rinv; b.sa_i = rp; b.sa_k = 1;                          // A^{-1}
     b.B = Tt; b.sb_k = sz; b.sb_j = 1;
-    b.C = Rinv + sz; b.ldc = rp; b.alpha = -1.0; b.beta = 0.0;
+    b.C = Rinv + sz; b.ldc = rp; b.alpha = -1.0; b.beta = 0.0; b.tri = 4;
     b.za = step; b.zb = (int64_t)sz * sz; b.zc = step;
-    if ((st = run_gemm_f64(b, pairs, s)) != PIFA_OK) return st;
+    if (sz < 256 || !gemm_f64_split_fits(a, bytes) || !gemm_f64_split_fits(b, bytes)) {
+      if ((st = run_gemm_f64(a, pairs, s)) != PIFA_OK || (st = run_gemm_f64(b, pairs, s)) != PIFA_OK) return st;
+      continue;
+    }
+    for (int z = 0; z < pairs; ++z) {
+      if ((st = gemm_f64_split(a, scratch, bytes, s)) != PIFA_OK || (st = gemm_f64_split(b, scratch, bytes, s)) != PIFA_OK)
+        return st;
+      a.A += a.za; a.B += a.zb; a.C += a.zc;
+      b.A += b.za; b.B += b.zb; b.C += b.zc;
+    }
   }
   return PIFA_OK;
 }
@@ -528,19 +622,16 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
   q.A = V; q.sa_i = 1; q.sa_k = r;
   q.B = V; q.sb_k = r; q.sb_j = 1;
   q.C = G; q.ldc = r; q.alpha = 1.0; q.beta = 0.0;
-  if ((st = run_gemm_f64(q, 1, s)) != PIFA_OK) return st;
-  for (int j = 0; j < ri; ++j) {
-    const int t = (ri - j + 15) / 16;
-    chol_step<<<dim3(t, t), 256, 0, s>>>(G, L, ri, j, flags);
-    pifa_count_launch();
-  }
-  PIFA_CK(cudaGetLastError(), "compress: cholesky launch");
+  q.lower = 1;  // G is symmetric
+  // scratch of the products: parts of the workspace that hold nothing yet, or nothing any more
+  if ((st = run_product(q, Z, Ly.blk - Ly.Z, s)) != PIFA_OK) return st;
+  if ((st = cholesky(G, L, r, flags, Z, Ly.blk - Ly.Z, s)) != PIFA_OK) return st;
   q = GemmF64{};
   q.M = mi; q.N = ri; q.K = ri;
   q.A = U; q.sa_i = r; q.sa_k = 1;
   q.B = L; q.sb_k = r; q.sb_j = 1;
   q.C = Z; q.ldc = r; q.alpha = 1.0; q.beta = 0.0; q.tri = 1;
-  if ((st = run_gemm_f64(q, 1, s)) != PIFA_OK) return st;
+  if ((st = run_product(q, R, Ly.blk - Ly.R, s)) != PIFA_OK) return st;
 
   // 2. r greedy steps
   greedy_init<<<Ly.nblk, 256, 0, s>>>(g);
@@ -563,7 +654,7 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
     const int64_t tot = (int64_t)rp * rp;
     build_r<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(g, R, rp);
     pifa_count_launch();
-    if ((st = upper_inverse(R, Rinv, Tt, rp, s)) != PIFA_OK) return st;
+    if ((st = upper_inverse(R, Rinv, Tt, rp, G, Ly.Z - Ly.G, s)) != PIFA_OK) return st;  // G and L are done with
   }
   if (has_np) {
     // C[a][asc[j]] = sum_{k >= j} Z[I^c[a]][k] Rinv[j][k]
@@ -572,7 +663,7 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
     c.A = Z; c.aidx = nonpivot_idx; c.sa_i = r; c.sa_k = 1;
     c.B = Rinv; c.sb_k = 1; c.sb_j = rp;
     c.C = C; c.cidx = asc; c.ldc = ldc; c.alpha = 1.0; c.beta = 0.0; c.tri = 1;
-    if ((st = run_gemm_f64(c, 1, s)) != PIFA_OK) return st;
+    if ((st = run_product(c, G, Ly.Z - Ly.G, s)) != PIFA_OK) return st;
     max_abs<<<4 * 152, 256, 0, s>>>(C, m - r, r, ldc, reinterpret_cast<unsigned long long*>(flags + 2));
     pifa_count_launch();
     PIFA_CK(cudaGetLastError(), "compress: max launch");
@@ -584,7 +675,7 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
     w.A = U; w.aidx = pivot_idx; w.sa_i = r; w.sa_k = 1;
     w.B = V; w.sb_k = 1; w.sb_j = r;
     w.C = Wp; w.ldc = ldwp; w.alpha = 1.0; w.beta = 0.0;
-    if ((st = run_gemm_f64(w, 1, s)) != PIFA_OK) return st;
+    if ((st = run_product(w, G, Ly.blk - Ly.G, s)) != PIFA_OK) return st;
   }
 
   // results for the rank check and the diagnostics
@@ -679,8 +770,7 @@ int64_t spd_scratch_doubles(int64_t k) {
   return 2 * k * k + 2 * rp * rp + rp * rp / 4 + 64;
 }
 
-// Sinv = S^{-1} for a symmetric positive definite S (k x k, pitch k): S = L L^T (Cholesky, one
-// column per launch), R = L^T, S^{-1} = R^{-1} R^{-T}. `bad` is set when a pivot is not positive.
+// Sinv = S^{-1} for a symmetric positive definite S (k x k, pitch k): S = L L^T, R = L^T, S^{-1} = R^{-1} R^{-T}. `bad` is set when a pivot is not positive.
 int spd_inverse(const double* S, int64_t k, double* Sinv, double* scratch, int* bad, cudaStream_t s) {
   const int rp = pad_pow2_32(k);
   double* G = scratch;
@@ -691,23 +781,20 @@ int spd_inverse(const double* S, int64_t k, double* Sinv, double* scratch, int* 
   cudaError_t e = cudaMemcpyAsync(G, S, (size_t)k * k * 8, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(L, 0, (size_t)k * k * 8, s);
   if (e != cudaSuccess) return pifa_fail_cuda("spd inverse: copy", e);
-  for (int j = 0; j < (int)k; ++j) {
-    const int t = ((int)k - j + 15) / 16;
-    chol_step<<<dim3(t, t), 256, 0, s>>>(G, L, (int)k, j, bad);
-    pifa_count_launch();
-  }
+  const int64_t gl = 2 * k * k * 8, rt = (2 * (int64_t)rp * rp + (int64_t)rp * rp / 4) * 8;  // bytes of G, L and of R .. Tt
+  int st = cholesky(G, L, k, bad, R, rt, s);
+  if (st != PIFA_OK) return st;
   transpose_pad_lower<<<grid_for((int64_t)rp * rp), 256, 0, s>>>(L, k, R, rp);
   pifa_count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return pifa_fail_cuda("spd inverse: launch", e);
-  int st = upper_inverse(R, Rinv, Tt, rp, s);
-  if (st != PIFA_OK) return st;
-  GemmF64 g = {};  // Sinv[i][j] = sum_t Rinv[i][t] Rinv[j][t]
+  if ((st = upper_inverse(R, Rinv, Tt, rp, G, gl, s)) != PIFA_OK) return st;  // G and L are done with
+  GemmF64 g = {};  // Sinv[i][j] = sum over t >= max(i, j) of Rinv[i][t] Rinv[j][t]
   g.M = (int)k; g.N = (int)k; g.K = (int)k;
   g.A = Rinv; g.sa_i = rp; g.sa_k = 1;
   g.B = Rinv; g.sb_k = 1; g.sb_j = rp;
-  g.C = Sinv; g.ldc = k; g.alpha = 1.0; g.beta = 0.0;
-  return run_gemm_f64(g, 1, s);
+  g.C = Sinv; g.ldc = k; g.alpha = 1.0; g.beta = 0.0; g.tri = 1 | 4;
+  return run_product(g, G, gl, s);
 }
 
 }  // namespace
@@ -758,6 +845,7 @@ extern "C" int pifa_m_reconstruct(const float* XXt, int64_t ldxx, const float* Y
   e = cudaGetLastError();
   if (e != cudaSuccess) return pifa_fail_cuda("reconstruct: launch", e);
   const int ni = (int)n, mi = (int)m, ri = (int)r;
+  const int64_t sbytes = spd_scratch_doubles(n) * 8;
   int st;
   auto gemm = [&](int M, int N, int K, const double* Ap, int64_t sai, int64_t sak, const double* Bp, int64_t sbk,
                   int64_t sbj, double* Cp, int64_t ldc) {
@@ -766,7 +854,7 @@ extern "C" int pifa_m_reconstruct(const float* XXt, int64_t ldxx, const float* Y
     g.A = Ap; g.sa_i = sai; g.sa_k = sak;
     g.B = Bp; g.sb_k = sbk; g.sb_j = sbj;
     g.C = Cp; g.ldc = ldc; g.alpha = 1.0; g.beta = 0.0;
-    return run_gemm_f64(g, 1, s);
+    return run_product(g, scratch, sbytes, s);  // between the inverses their scratch is free
   };
   // Eq. 4: U_r = (Y_t X^T) V (V^T (X X^T) V)^{-1}
   if ((st = gemm(ni, ri, ni, A, n, 1, V, r, 1, T1, r)) != PIFA_OK) return st;

@@ -1,0 +1,432 @@
+// gemm_f64_tc.cu -- float64 matrix products on the 5th-generation tensor cores, by exact slices,
+// for the float64 set-up paths (Algorithm 1 and the M reconstruction's solves).
+//
+// sm_103a issues about two float64 multiply-adds per clock and SM (1.1 TFLOP/s measured with the
+// CUDA-core gemm_f64), against 4096 bf16 ones, so a float64 product is computed as integers (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012): every row of A and column of B is
+// scaled by a power of two to below one in magnitude, rounded to 62 fractional bits (float64 keeps
+// 53 of its own), and cut into 8 balanced base-256 digits, each a whole number of at most 8 bits
+// and so exact in bf16. With a_p, b_q the digit matrices,
+//   A B = sum over d = p + q <= 7 of 2^-(12 + 8 d) V_d,   V_d = sum over p + q = d of a_p b_q,
+// where the dropped pairs (d > 7) lie below 2^-64 of the largest products. A V_d over K = 128
+// columns is a whole number of at most 8 128 128^2 = 2^24, which the fp32 accumulators in tensor
+// memory hold exactly; every 128 columns the 8 accumulators are drained into 64-bit integers. The
+// only roundings are the 62-bit one of the operands and the final one to float64: against quad
+// precision W_p = U V^T (K = 256 to 2048) is 4.7e-17 off, its float64 rounding, where a chain of
+// float64 multiply-adds is 5e-16 to 1.1e-15 off.
+//
+// Sliced operands are laid out [row][K block of 32][digit][32], so that a TMA box of 64 elements
+// holds two digits of one K block as one 128-byte swizzled row.
+//
+// One CTA per 128 x 64 output tile, 320 threads: warp 0 the TMA producer (two 96 KB stages of one K
+// block: 8 digits of 128 rows of A and 64 of B), warp 1 the MMA issuer (36 digit pairs x 2
+// instructions of M = 128, N = 64, K = 16 per stage, accumulators d = 0 .. 7 of 64 columns: all
+// 512 columns of tensor memory), warps 2-9 the drain. Within a stage the MMAs run in order of d and
+// each accumulator is committed and released by itself, so that the drain of one K = 128 chunk
+// overlaps the MMAs of the next. Every wait is bounded.
+#include <cuda_bf16.h>
+
+#include "pifa.h"
+#include "pifa_internal.h"
+#include "ptx.cuh"
+
+namespace {
+
+using namespace pifa;
+
+constexpr int SM_ = 128, SN = 64;        // output tile
+constexpr int KBLK = 32;                 // K columns per stage
+constexpr int NDIG = 8;                  // digits per value, and diagonals kept
+constexpr int CHUNK = 4;                 // stages per exact accumulation: 128 columns of K
+constexpr int ROWLEN = KBLK * NDIG;      // sliced elements per row and K block
+constexpr uint32_t A_BOX = SM_ * 128, B_BOX = SN * 128;  // two digits: 128-byte rows
+constexpr uint32_t STAGE = (NDIG / 2) * (A_BOX + B_BOX);
+constexpr int STAGES = 2;
+constexpr int DRAIN_WARPS = 8;
+constexpr int THREADS = 64 + 32 * DRAIN_WARPS;
+constexpr size_t SMEM = 1024 + STAGES * STAGE + 256;
+constexpr uint32_t TMEM_COLS = NDIG * SN;  // 512
+
+// ---- slicing -----------------------------------------------------------------------------------
+struct SliceArgs {
+  const double* X;     // element (i, k) at X[row(i) * s_row + k * s_k], row(i) = idx ? idx[i] : i
+  const int32_t* idx;
+  int64_t s_row, s_k;
+  int rows, K;
+  unsigned long long* mx;   // per row: the bits of max |x| over k
+  __nv_bfloat16* S;         // rows x (nkb ROWLEN)
+  int nkb;
+};
+
+// max |x| of each row as an unsigned bit pattern (non-negative float64 values order like their
+// bits, and every NaN and infinity orders above the finite ones). mx must be zero on entry.
+__global__ void __launch_bounds__(256) slice_row_max(SliceArgs a) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = blockIdx.x * 32;
+  const int per = (a.K + gridDim.y - 1) / gridDim.y;
+  const int k0 = blockIdx.y * per, k1 = min(a.K, k0 + per);
+  if (a.s_k == 1) {  // the lanes along K; a warp takes 4 of the block's 32 rows
+    for (int rr = warp; rr < 32; rr += 8) {
+      const int i = r0 + rr;
+      if (i >= a.rows) continue;
+      const double* x = a.X + (a.idx ? (int64_t)a.idx[i] : (int64_t)i) * a.s_row;
+      unsigned long long m = 0;
+#pragma unroll 4
+      for (int k = k0 + lane; k < k1; k += 32)
+        m = max(m, (unsigned long long)__double_as_longlong(x[k]) & 0x7fffffffffffffffull);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) atomicMax(a.mx + i, m);
+    }
+  } else {  // the lanes along the rows; the warps along K
+    const int i = r0 + lane;
+    if (i >= a.rows) return;
+    const double* x = a.X + (a.idx ? (int64_t)a.idx[i] : (int64_t)i) * a.s_row;
+    unsigned long long m = 0;
+#pragma unroll 4
+    for (int k = k0 + warp; k < k1; k += 8)
+      m = max(m, (unsigned long long)__double_as_longlong(x[(int64_t)k * a.s_k]) & 0x7fffffffffffffffull);
+    atomicMax(a.mx + i, m);
+  }
+}
+
+// The biased exponent of a row's scale: |x| < 2^(e - 1022) for every x of the row (1 for rows of
+// zeros and subnormals, 2047 for a row that holds an infinity or a NaN).
+__device__ __forceinline__ int row_exp(unsigned long long mx) {
+  const int e = (int)(mx >> 52);
+  return e < 1 ? 1 : e;
+}
+
+// The 8 digits of one 32 x 32 block of values per CTA of 128 threads: loaded with the lanes along
+// the contiguous index, then 4 threads a row, 8 values and 8 x 16 bytes of digits each.
+__global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
+  __shared__ unsigned long long t[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = blockIdx.y * 32, kb = blockIdx.x, k0 = kb * KBLK;
+  for (int u = warp; u < 32; u += 4) {
+    const int rr = a.s_k == 1 ? u : lane, kk = a.s_k == 1 ? lane : u;
+    const int i = r0 + rr, k = k0 + kk;
+    double x = 0.0;
+    if (i < a.rows && k < a.K) x = a.X[(a.idx ? (int64_t)a.idx[i] : (int64_t)i) * a.s_row + (int64_t)k * a.s_k];
+    t[rr][kk] = (unsigned long long)__double_as_longlong(x);
+  }
+  __syncthreads();
+  const int rr = threadIdx.x >> 2, kq = (threadIdx.x & 3) * 8;
+  const int i = r0 + rr;
+  if (i >= a.rows) return;
+  const int er = row_exp(a.mx[i]);
+  uint32_t w[NDIG][4];  // 8 bf16 digits per plane, packed in pairs
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const unsigned long long b = t[rr][kq + e];
+    int ex = (int)((b >> 52) & 2047);
+    unsigned long long mant = b & 0xfffffffffffffull;
+    if (ex) mant |= 0x10000000000000ull;
+    else ex = 1;
+    const int sh = ex - er + 9;  // mant 2^sh = |x| 2^62 / 2^(er - 1022)
+    unsigned long long mag = 0;
+    if (sh >= 0) mag = mant << sh;  // sh <= 9: ex <= er
+    else if (sh > -60) mag = (mant + (1ull << (-sh - 1))) >> -sh;
+    if (er == 2047) mag = 0;  // the drain writes NaN for this row
+    long long q = (b >> 63) ? -(long long)mag : (long long)mag;
+#pragma unroll
+    for (int p = NDIG - 1; p >= 0; --p) {
+      const int d = p > 0 ? (int)(signed char)(q & 255) : (int)q;
+      q = (q - d) >> 8;
+      const uint32_t h = __float_as_uint((float)d) >> 16;  // |d| <= 128: exact in bf16
+      if (e & 1) w[p][e >> 1] |= h << 16;
+      else w[p][e >> 1] = h;
+    }
+  }
+  __nv_bfloat16* s = a.S + (int64_t)i * a.nkb * ROWLEN + (int64_t)kb * ROWLEN + kq;
+#pragma unroll
+  for (int p = 0; p < NDIG; ++p) *reinterpret_cast<uint4*>(s + p * KBLK) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+}
+
+// ---- the products --------------------------------------------------------------------------------
+struct SplitArgs {
+  int M, N, kbase, K;  // this panel's columns [kbase, kbase + K) of the contraction
+  int tri, lower, first;
+  const unsigned long long *mxa, *mxb;
+  double* C;
+  const int32_t* cidx;
+  int64_t ldc;
+  double alpha, beta;
+  int* status;
+  uint64_t timeout_ns;
+};
+
+__global__ void __launch_bounds__(THREADS, 1)
+    gemm_f64_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
+  const int m0 = blockIdx.y * SM_, n0 = blockIdx.x * SN;
+  if (p.lower && n0 > m0 + SM_ - 1) return;  // tile wholly above the diagonal
+  // columns of K that can hold anything (triangular operands), as stages of this panel
+  int ka = 0, ke = p.kbase + p.K;
+  if (p.tri & 1) ka = max(ka, n0);
+  if (p.tri & 4) ka = max(ka, m0);
+  if (p.tri & 2) ke = min(ke, n0 + SN);
+  const int kb0 = max(0, ka - p.kbase) / KBLK, kb1 = ke > p.kbase ? (ke - p.kbase + KBLK - 1) / KBLK : 0;
+  const int nst = max(0, kb1 - kb0);
+  if (nst == 0 && !p.first) return;
+  const int nch = (nst + CHUNK - 1) / CHUNK;
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accf = empty + STAGES;
+  uint64_t* acce = accf + NDIG;
+  uint64_t* done = acce + NDIG;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int d = 0; d < NDIG; ++d) {
+      mbar_init(&accf[d], 1);
+      mbar_init(&acce[d], DRAIN_WARPS);
+    }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tmA);
+    prefetch_tmap(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int issued = 0;
+      for (int it = 0; it < nst; ++it) {
+        const int s = it % STAGES;
+        if ((it >= STAGES && !mbar_wait(&empty[s], (uint32_t)((it / STAGES) - 1) & 1u, p.timeout_ns)) || *abort_flag) {
+          latch_status(p.status, PIFA_ERR_TIMEOUT);
+          *abort_flag = 1;
+          break;
+        }
+        uint8_t* sa = smem + s * STAGE;
+        uint8_t* sb = sa + (NDIG / 2) * A_BOX;
+        const int x = (kb0 + it) * ROWLEN;
+        mbar_arrive_expect_tx(&full[s], STAGE);
+        for (int q = 0; q < NDIG / 2; ++q) {
+          tma_load_2d(smem_u32(sa + q * A_BOX), &tmA, x + 64 * q, m0, &full[s]);
+          tma_load_2d(smem_u32(sb + q * B_BOX), &tmB, x + 64 * q, n0, &full[s]);
+        }
+        issued = it + 1;
+      }
+      for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
+        if (!mbar_wait(&full[i % STAGES], (uint32_t)(i / STAGES) & 1u, 100000000ull))
+          latch_status(p.status, PIFA_ERR_TIMEOUT);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16_f32(SM_, SN);
+      bool dead = false;
+      for (int it = 0; it < nst && !dead; ++it) {
+        const int s = it % STAGES, ch = it / CHUNK, w = it % CHUNK;
+        const bool last = w == CHUNK - 1 || it == nst - 1;
+        if (!mbar_wait(&full[s], (uint32_t)(it / STAGES) & 1u, p.timeout_ns) || *abort_flag) {
+          dead = true;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a = smem_u32(smem + s * STAGE), b = a + (NDIG / 2) * A_BOX;
+        for (int d = 0; d < NDIG; ++d) {
+          if (w == 0 && ch > 0) {  // the drain has taken this accumulator's last chunk
+            if (!mbar_wait(&acce[d], (uint32_t)(ch - 1) & 1u, p.timeout_ns)) {
+              dead = true;
+              break;
+            }
+            tc_fence_after();
+          }
+          for (int i = 0; i <= d; ++i) {
+            const int j = d - i;
+            const uint32_t pa = a + (uint32_t)(i >> 1) * A_BOX + (uint32_t)(i & 1) * 64u;
+            const uint32_t pb = b + (uint32_t)(j >> 1) * B_BOX + (uint32_t)(j & 1) * 64u;
+#pragma unroll
+            for (int kk = 0; kk < KBLK / 16; ++kk)
+              mma_bf16_ss(tmem + (uint32_t)(d * SN), sw128_desc(pa + kk * 32), sw128_desc(pb + kk * 32), idesc,
+                          (w > 0 || i > 0 || kk > 0) ? 1u : 0u);
+          }
+          if (last) mma_commit(&accf[d]);
+        }
+        mma_commit(&empty[s]);
+      }
+      if (dead) {
+        latch_status(p.status, PIFA_ERR_TIMEOUT);
+        *abort_flag = 1;
+      }
+      mma_commit(done);
+      if (!mbar_wait(done, 0, 100000000ull)) latch_status(p.status, PIFA_ERR_TIMEOUT);
+    }
+  } else {
+    // drain: TMEM lane quarter warp % 4, 32 of the tile's 64 columns
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
+    long long hi[32], lo[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
+    bool ok = true;
+    for (int ch = 0; ch < nch; ++ch) {
+#pragma unroll
+      for (int d = 0; d < NDIG; ++d) {
+        if (ok && !mbar_wait(&accf[d], (uint32_t)ch & 1u, p.timeout_ns)) {
+          latch_status(p.status, PIFA_ERR_TIMEOUT);
+          *abort_flag = 1;
+          ok = false;
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t v[32];
+        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(d * SN + half * 32), v);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acce[d]);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const long long x = (long long)__float2int_rn(__uint_as_float(v[c]));
+          if (d < 4) hi[c] += x * (1ll << (8 * (3 - d)));
+          else lo[c] += x * (1ll << (8 * (7 - d)));
+        }
+      }
+      if (!ok) break;
+    }
+    // through shared memory (the ring: every MMA has completed and no copy is in flight once the
+    // last accumulator is full), so that the lanes store consecutive columns
+    if (ok) {
+      fence_proxy_async_smem();
+      double* tile = reinterpret_cast<double*>(smem) + (warp - 2) * 32 * 33;
+#pragma unroll
+      for (int c = 0; c < 32; ++c)
+        tile[lane * 33 + c] = (double)hi[c] * 0x1p-36 + (double)lo[c] * 0x1p-68;
+      __syncwarp();
+      const int j = n0 + half * 32 + lane;
+      const bool jn = j < p.N;
+      const int eb = jn ? row_exp(p.mxb[j]) : 1;
+      const int64_t cj = jn ? (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j) : 0;
+#pragma unroll 4
+      for (int rr = 0; rr < 32; ++rr) {
+        const int i = m0 + q4 * 32 + rr;
+        if (i >= p.M || !jn) continue;
+        const int ea = row_exp(p.mxa[i]);
+        double v = tile[rr * 33 + lane];
+        v = (ea == 2047 || eb == 2047) ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(v, ea + eb - 2044);
+        double* c = p.C + (int64_t)i * p.ldc + cj;
+        *c = (p.beta != 0.0 ? p.beta * *c : 0.0) + p.alpha * v;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, TMEM_COLS);
+  }
+}
+
+int64_t a1k(int64_t b) { return (b + 1023) / 1024 * 1024; }
+// scratch bytes of a product's two sliced operands over a panel of kp columns
+int64_t panel_bytes(int64_t M, int64_t N, int64_t kp, bool same) {
+  const int64_t row = (kp + KBLK - 1) / KBLK * ROWLEN * 2;
+  return a1k(M * row) + a1k(M * 8) + (same ? 0 : a1k(N * row) + a1k(N * 8));
+}
+
+int slice(const SliceArgs& a, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(a.mx, 0, (size_t)a.rows * 8, s);
+  if (e != cudaSuccess) return pifa_fail_cuda("f64 slices: memset", e);
+  const int rb = (a.rows + 31) / 32;
+  int ks = 608 / rb;
+  if (ks > (a.K + 127) / 128) ks = (a.K + 127) / 128;
+  if (ks < 1) ks = 1;
+  slice_row_max<<<dim3((unsigned)rb, (unsigned)ks), 256, 0, s>>>(a);
+  pifa_count_launch();
+  slice_digits<<<dim3((unsigned)a.nkb, (unsigned)rb), 128, 0, s>>>(a);
+  pifa_count_launch();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? PIFA_OK : pifa_fail_cuda("f64 slices: launch", e);
+}
+
+}  // namespace
+
+bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes) {
+  const int64_t work = (int64_t)p.M * p.N * p.K;
+  const bool same = p.A == p.B && p.sa_i == p.sb_j && p.sa_k == p.sb_k && p.M == p.N && !p.aidx;
+  return p.K >= 64 && work >= (int64_t)1 << 20 && (p.M + 31) / 32 <= 65535 && (p.N + 31) / 32 <= 65535 &&
+         panel_bytes(p.M, p.N, p.K < 128 ? p.K : 128, same) <= bytes - 256;  // 256: alignment of the scratch
+}
+
+int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream) {
+  cudaError_t e = cudaSuccess;
+  int* status = pifa_status_word(&e);
+  if (!status) return pifa_fail_cuda("device status word", e);
+  const int64_t shift = (int64_t)((256 - (reinterpret_cast<uintptr_t>(scratch) & 255u)) & 255u);
+  scratch = static_cast<uint8_t*>(scratch) + shift;
+  bytes -= shift;
+  const bool same = p.A == p.B && p.sa_i == p.sb_j && p.sa_k == p.sb_k && p.M == p.N && !p.aidx;
+  int64_t kp = p.K;  // the widest panel of whole 128-column chunks that fits the scratch
+  if (panel_bytes(p.M, p.N, kp, same) > bytes) {
+    kp = (kp + 127) / 128 * 128;
+    while (kp > 128 && panel_bytes(p.M, p.N, kp, same) > bytes) kp -= 128;
+  }
+  e = cudaFuncSetAttribute(gemm_f64_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+  if (e != cudaSuccess) return pifa_fail_cuda("cudaFuncSetAttribute(gemm_f64_split)", e);
+  for (int64_t k0 = 0; k0 < p.K; k0 += kp) {
+    const int kn = (int)(p.K - k0 < kp ? p.K - k0 : kp);
+    const int nkb = (kn + KBLK - 1) / KBLK;
+    const int64_t row = (int64_t)nkb * ROWLEN * 2;
+    uint8_t* w = static_cast<uint8_t*>(scratch);
+    SliceArgs a = {p.A + k0 * p.sa_k, p.aidx, p.sa_i, p.sa_k, p.M, kn, nullptr, nullptr, nkb};
+    a.S = reinterpret_cast<__nv_bfloat16*>(w);
+    w += a1k(p.M * row);
+    a.mx = reinterpret_cast<unsigned long long*>(w);
+    w += a1k((int64_t)p.M * 8);
+    SliceArgs b = a;
+    int st = slice(a, stream);
+    if (st != PIFA_OK) return st;
+    if (!same) {
+      b = SliceArgs{p.B + k0 * p.sb_k, nullptr, p.sb_j, p.sb_k, p.N, kn, nullptr, nullptr, nkb};
+      b.S = reinterpret_cast<__nv_bfloat16*>(w);
+      w += a1k(p.N * row);
+      b.mx = reinterpret_cast<unsigned long long*>(w);
+      if ((st = slice(b, stream)) != PIFA_OK) return st;
+    }
+    CUtensorMap tA, tB;
+    if ((st = make_tmap_2d(&tA, PIFA_DTYPE_BF16, a.S, p.M, row / 2, row / 2, 64, SM_)) != PIFA_OK) return st;
+    if ((st = make_tmap_2d(&tB, PIFA_DTYPE_BF16, b.S, p.N, row / 2, row / 2, 64, SN)) != PIFA_OK) return st;
+    SplitArgs g = {};
+    g.M = p.M;
+    g.N = p.N;
+    g.kbase = (int)k0;
+    g.K = kn;
+    g.tri = p.tri;
+    g.lower = p.lower;
+    g.first = k0 == 0;
+    g.mxa = a.mx;
+    g.mxb = b.mx;
+    g.C = p.C;
+    g.cidx = p.cidx;
+    g.ldc = p.ldc;
+    g.alpha = p.alpha;
+    g.beta = k0 == 0 ? p.beta : 1.0;
+    g.status = status;
+    g.timeout_ns = pifa_wait_timeout_ns();
+    const dim3 grid((unsigned)((p.N + SN - 1) / SN), (unsigned)((p.M + SM_ - 1) / SM_));
+    if (grid.y > 65535u) return pifa_fail(PIFA_ERR_UNSUPPORTED, "gemm_f64_split: more than 65535 row tiles");
+    gemm_f64_split_kernel<<<grid, THREADS, SMEM, stream>>>(tA, tB, g);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return pifa_fail_cuda("gemm_f64_split launch", e);
+    pifa_count_launch();
+  }
+  return PIFA_OK;
+}

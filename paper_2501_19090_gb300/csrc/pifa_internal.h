@@ -159,6 +159,34 @@ struct GemmTc {
 };
 int gemm_tc(const GemmTc& g, int* status, uint64_t timeout_ns, cudaStream_t stream);
 
+// ---- float64 products (compress_gpu.cu, gemm_f64_tc.cu) -------------------------------------------
+// C[i][ccol(j)] = beta C + alpha sum_k A(i, k) B(k, j), with
+//   A(i, k) = A[arow(i) * sa_i + k * sa_k],  arow(i) = aidx ? aidx[i] : i
+//   B(k, j) = B[k * sb_k + j * sb_j]
+//   C at C[i * ldc + (cidx ? cidx[j] : j)]
+// and, on the CUDA cores, a batch index z (blockIdx.z) offsetting A, B and C by za, zb, zc elements.
+// `tri` (bits): 1 B(k, j) = 0 for k < j, 2 B(k, j) = 0 for k > j, 4 A(i, k) = 0 for k < i; the k loop
+// skips those zeros. `lower`: only the tiles that hold some i >= j are computed.
+struct GemmF64 {
+  int M, N, K;
+  const double* A;
+  const int32_t* aidx;
+  int64_t sa_i, sa_k;
+  const double* B;
+  int64_t sb_k, sb_j;
+  double* C;
+  const int32_t* cidx;
+  int64_t ldc;
+  double alpha, beta;
+  int tri;
+  int64_t za, zb, zc;
+  int lower;
+};
+// The same on the tensor cores by exact slices (no batch), in `bytes` of scratch:
+// whether that form takes the product, and the product.
+bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes);
+int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream);
+
 // ---- prefill (prefill.cu) --------------------------------------------------------------------
 int64_t prefill_split_workspace_bytes(const PifaShape& s);
 int launch_prefill_split(const PifaShape& s, const PifaPointers& p, int* status, uint64_t timeout_ns,

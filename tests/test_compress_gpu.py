@@ -125,3 +125,30 @@ def test_llama70b_gate_up_compresses_on_the_gpu():
     Wnp = Ud[nonp[rows]] @ Vd.T
     assert np.linalg.norm(C[rows] @ Wp - Wnp) / np.linalg.norm(Wnp) <= 1e-10
     print(f"pifa_compress_device 28672 x 8192, r = 4096: {dt:.2f} s, min gap {info.min_pivot_gap:.3e}")
+
+
+@pytest.mark.parametrize("m,n,r", [(300, 129, 97), (257, 320, 128), (400, 191, 161), (520, 260, 257)])
+def test_float64_products_by_slices_are_exact_on_whole_numbers(m, n, r):
+    """W_p = U[I] V^T runs on the tensor cores by exact slices from 2^20 multiply-adds on. Whole
+    numbers below 2^20 in magnitude have products and sums below 257 * 2^40 < 2^49, exact in
+    float64 whatever the order, so W_p must equal the host's product bit for bit (sizes around the
+    128 x 64 tiles, the 32-column K blocks and the 128-column exact accumulations)."""
+    rng = np.random.default_rng(m)
+    U = rng.integers(-(1 << 20), 1 << 20, (m, r)).astype(np.float64)
+    V = rng.integers(-(1 << 20), 1 << 20, (n, r)).astype(np.float64)
+    assert r * n * r >= 1 << 20
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert P.pifa_device_status() == P.PIFA_OK
+    assert np.array_equal(Wp, U[piv] @ V.T)
+    _check_eqs(U, V, piv, nonp, Wp, C)
+
+
+@pytest.mark.parametrize("r", [31, 32, 33, 127, 129, 160, 257, 300])
+def test_blocked_cholesky_edges_match_the_greedy_oracle(r):
+    """Ranks around the 32-column blocks and 128-column panels of the Cholesky factorisation."""
+    m, n = r + 150, r + 90
+    U, V, _ = inputs.make_factors(m, n, r, r)
+    L = oracle.compress(U, V, r, "greedy")
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert np.array_equal(piv, L.pivots) and np.array_equal(nonp, L.nonpivots)
+    _check_eqs(U, V, piv, nonp, Wp, C)
