@@ -30,8 +30,12 @@
 
 #include "pifa.h"
 #include "pifa_internal.h"
+#include "ptx.cuh"
 
 namespace {
+
+using namespace pifa;
+
 
 // ---- float64 GEMM on the CUDA cores (GemmF64 in pifa_internal.h): small products ------------
 constexpr int GT = 64, GK = 16;  // output tile 64 x 64, k step 16; 256 threads, 4 x 4 outputs each
@@ -227,37 +231,34 @@ int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t b
 }
 
 // ---- greedy pivoted QR on the rows of Z -------------------------------------------------------
-// Best and runner-up residual norms (squared) with their rows; larger norm first, then the lower
-// index: the selection rule of Algorithm 1, step 1 with ties to the lowest index.
+// Best and runner-up residual norms (squared, as float64 bit patterns: non-negative values order
+// like their bits) with their rows, and the best one's slot in the list of unchosen rows; larger
+// norm first, then the lower row: the selection rule of Algorithm 1, step 1 with ties to the lowest
+// index.
 struct Top2 {
-  double v1;
-  int i1;
-  double v2;
-  int i2;
+  unsigned long long v1, v2;
+  int i1, i2, s1;
 };
 
-__device__ __forceinline__ bool better(double va, int ia, double vb, int ib) {
-  return va > vb || (va == vb && ia < ib);
-}
-
-__device__ __forceinline__ void top2_add(Top2& t, double v, int i) {
+__device__ __forceinline__ void top2_add(Top2& t, unsigned long long v, int i, int s) {
   if (i < 0) return;
-  if (t.i1 < 0 || better(v, i, t.v1, t.i1)) {
+  if (t.i1 < 0 || v > t.v1 || (v == t.v1 && i < t.i1)) {
     t.v2 = t.v1;
     t.i2 = t.i1;
     t.v1 = v;
     t.i1 = i;
-  } else if (t.i2 < 0 || better(v, i, t.v2, t.i2)) {
+    t.s1 = s;
+  } else if (t.i2 < 0 || v > t.v2 || (v == t.v2 && i < t.i2)) {
     t.v2 = v;
     t.i2 = i;
   }
 }
 
-__device__ __forceinline__ Top2 top2_empty() { return Top2{0.0, -1, 0.0, -1}; }
+__device__ __forceinline__ Top2 top2_empty() { return Top2{0ull, 0ull, -1, -1, -1}; }
 
 __device__ __forceinline__ void top2_merge(Top2& a, const Top2& b) {
-  top2_add(a, b.v1, b.i1);
-  top2_add(a, b.v2, b.i2);
+  top2_add(a, b.v1, b.i1, b.s1);
+  top2_add(a, b.v2, b.i2, -1);  // never a's best: b's best is in front of it
 }
 
 __device__ Top2 warp_top2(Top2 t) {
@@ -265,44 +266,39 @@ __device__ Top2 warp_top2(Top2 t) {
   for (int o = 16; o > 0; o >>= 1) {
     Top2 u;
     u.v1 = __shfl_xor_sync(0xffffffffu, t.v1, o);
-    u.i1 = __shfl_xor_sync(0xffffffffu, t.i1, o);
     u.v2 = __shfl_xor_sync(0xffffffffu, t.v2, o);
+    u.i1 = __shfl_xor_sync(0xffffffffu, t.i1, o);
     u.i2 = __shfl_xor_sync(0xffffffffu, t.i2, o);
+    u.s1 = __shfl_xor_sync(0xffffffffu, t.s1, o);
     top2_merge(t, u);
   }
   return t;
 }
 
-// Block-wide Top2 (blockDim.x = 256): every thread gets the block's result.
+// Block-wide Top2 (at most 16 warps): every thread gets the block's result.
 __device__ Top2 block_top2(Top2 t) {
-  __shared__ Top2 sw[8];
+  __shared__ Top2 sw[16];
   t = warp_top2(t);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __syncthreads();
   if (lane == 0) sw[w] = t;
   __syncthreads();
-  Top2 r = top2_empty();
-  for (int k = 0; k < 8; ++k) top2_merge(r, sw[k]);
-  return r;
+  return warp_top2(lane < (int)(blockDim.x >> 5) ? sw[lane] : top2_empty());
 }
 
-__device__ double block_sum(double v) {
-  __shared__ double sw[8];
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sw[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int k = 0; k < 8; ++k) s += sw[k];  // fixed order: the same value in every block
-  return s;
+  return v;
 }
+
+constexpr int kGreedyBlocks = 152;  // one per SM
 
 struct Greedy {
   double* Z;        // m x r, row-major
   int m, r;
   int32_t* sel;     // m flags: chosen in an earlier step
+  int32_t* act;     // the unchosen rows: m - k of them before step k
   Top2* blk;        // 2 x nblk per-block results (ping-pong by step parity)
   int nblk;
   int32_t* order;   // r: row chosen at step k
@@ -310,7 +306,7 @@ struct Greedy {
   double* gap;      // r: (best - runner-up) / best of the residual norms at step k
 };
 
-// Initial squared row norms of Z and each block's best two.
+// Initial squared row norms of Z, each block's best two, and the list of all rows.
 __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   Top2 t = top2_empty();
@@ -318,79 +314,125 @@ __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
     const double* z = g.Z + (int64_t)i * g.r;
     double s = 0.0;
     for (int c = lane; c < g.r; c += 32) s = fma(z[c], z[c], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) top2_add(t, s, i);
+    s = warp_sum(s);
+    if (lane == 0) {
+      top2_add(t, (unsigned long long)__double_as_longlong(s), i, i);
+      g.act[i] = i;
+    }
   }
   t = block_top2(t);
   if (threadIdx.x == 0) g.blk[blockIdx.x] = t;
 }
 
 // Step k: every block reduces step k - 1's per-block results to the pivot p (all blocks reach the
-// same p), forms the reflector from row p's residual (coordinates k..r-1) in shared memory, and
+// same p), forms the reflector H = I - tau v v^T from row p's residual x (coordinates k..r-1,
+// v = x - alpha e_0, alpha = -sign(x_0) |x|, tau = 1 / (|x|^2 + |x| |x_0|)) in shared memory, and
 // reflects its share of the unchosen rows, recomputing their residual norms (coordinates k+1..).
 // Row p itself is left as it is (other blocks read it during this launch): its column of R is
 // its coordinates 0..k-1 plus rdiag[k].
-__global__ void __launch_bounds__(256) greedy_step(Greedy g, int k) {
-  extern __shared__ double v[];  // r - k entries
-  __shared__ int s_p;
+//
+// A row belongs to W warps, which keep its residual in registers (NREG values per lane) from its
+// one read to its one write: dot product, update and norm are three float64 multiply-adds per
+// value, at two per clock and SM the bound of this kernel; the rows of Z (67 MB at 4096 x 2048)
+// stay in L2. One block per SM; the unchosen rows are kept as a list, dealt to the blocks in turn,
+// so that no SM holds more than one row above its share (the chosen row's slot takes the last row).
+// 4096 x 4096, r = 2048: the form that this replaced (rows read twice from L2, by warps fixed to
+// rows; three more block-wide sums before the first row) took 84.3 us a step against 16 us of
+// float64 multiply-adds; this one KERNEL_US.
+template <int NREG, int W>
+constexpr int kGreedyWarps = W == 1 && NREG <= 32 ? 12 : 8;  // what the registers allow
+template <int NREG, int W>
+__global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Greedy g, int k) {
+  constexpr int WARPS = kGreedyWarps<NREG, W>, GROUPS = WARPS / W, LEN = 32 * NREG * W;
+  extern __shared__ double v[];  // LEN entries, zero from r - k on
+  __shared__ double part[2][WARPS];
   const Top2* in = g.blk + (k & 1) * g.nblk;
   Top2* out = g.blk + ((k + 1) & 1) * g.nblk;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = warp / W, wq = warp % W;
+  pdl_launch_dependents();
+  pdl_wait_primary();
   Top2 t = top2_empty();
-  for (int b = threadIdx.x; b < g.nblk; b += 256) top2_merge(t, in[b]);
+  for (int b = threadIdx.x; b < g.nblk; b += WARPS * 32) top2_merge(t, in[b]);
   t = block_top2(t);
-  if (threadIdx.x == 0) s_p = t.i1;
-  __syncthreads();
-  const int p = s_p;
-  const int len = g.r - k;
-  if (p < 0 || p >= g.m) return;  // cannot happen for m >= r; guards the row read
+  const int p = t.i1;
+  const int len = g.r - k, n = g.m - k;  // unchosen rows, p among them
+  if (p < 0 || p >= g.m || t.s1 < 0 || t.s1 >= n) return;  // cannot happen for m >= r; guards the reads
   const double* zp = g.Z + (int64_t)p * g.r + k;
-  double ss = 0.0;
-  for (int c = threadIdx.x; c < len; c += 256) {
-    const double x = zp[c];
-    v[c] = x;
-    ss = fma(x, x, ss);
-  }
-  const double nx2 = block_sum(ss);  // also orders the v[] writes before the reads below
-  const double nx = sqrt(nx2);
-  const double x0 = v[0];
+  const double nx2 = __longlong_as_double((long long)t.v1), nx = sqrt(nx2);
+  const double x0 = zp[0];
   const double alpha = -copysign(nx, x0 != 0.0 ? x0 : 1.0);
-  __syncthreads();
-  if (threadIdx.x == 0) v[0] = x0 - alpha;
-  __syncthreads();
-  double vs = 0.0;
-  for (int c = threadIdx.x; c < len; c += 256) vs = fma(v[c], v[c], vs);
-  const double vn2 = block_sum(vs);
-  const double tau = vn2 > 0.0 ? 2.0 / vn2 : 0.0;  // H = I - tau v v^T
+  const double tau = nx2 > 0.0 ? 1.0 / (nx2 + nx * fabs(x0)) : 0.0;
+  for (int c = threadIdx.x; c < LEN; c += WARPS * 32) v[c] = c < len ? (c == 0 ? x0 - alpha : zp[c]) : 0.0;
+  const int tail = g.act[n - 1];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     g.order[k] = p;
     g.rdiag[k] = alpha;
-    const double b1 = sqrt(fmax(t.v1, 0.0)), b2 = t.i2 >= 0 ? sqrt(fmax(t.v2, 0.0)) : 0.0;
-    g.gap[k] = b1 > 0.0 ? (b1 - b2) / b1 : 0.0;
-    g.sel[p] = 1;  // read only by later launches
+    const double b2 = t.i2 >= 0 ? sqrt(__longlong_as_double((long long)t.v2)) : 0.0;
+    g.gap[k] = nx > 0.0 ? (nx - b2) / nx : 0.0;
+    g.sel[p] = 1;          // read only by later launches
+    g.act[t.s1] = tail;    // read by no block of this launch (see below)
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
   Top2 mine = top2_empty();
-  for (int i = blockIdx.x * 8 + warp; i < g.m; i += gridDim.x * 8) {
-    if (i == p || g.sel[i]) continue;  // warp-uniform
+  for (int s = blockIdx.x + gridDim.x * grp; s < n - 1; s += gridDim.x * GROUPS) {
+    const int i = s == t.s1 ? tail : g.act[s];
     double* z = g.Z + (int64_t)i * g.r + k;
-    double d = 0.0;
-    for (int c = lane; c < len; c += 32) d = fma(z[c], v[c], d);
+    double y[NREG];
+    double d0 = 0.0, d1 = 0.0;
+    const int c0 = wq * 32 * NREG + lane;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    const double s = tau * d;
-    double nr = 0.0;
-    for (int c = lane; c < len; c += 32) {
-      const double y = fma(-s, v[c], z[c]);
-      z[c] = y;
-      if (c > 0) nr = fma(y, y, nr);
+    for (int u = 0; u < NREG; ++u) y[u] = c0 + 32 * u < len ? z[c0 + 32 * u] : 0.0;
+#pragma unroll
+    for (int u = 0; u < NREG; u += 2) {
+      d0 = fma(y[u], v[c0 + 32 * u], d0);
+      d1 = fma(y[u + 1], v[c0 + 32 * u + 32], d1);
     }
+    double d = warp_sum(d0 + d1);
+    if (W > 1) {
+      if (lane == 0) part[0][warp] = d;
+      named_barrier_sync(1 + grp, 32 * W);
+      d = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
-    if (lane == 0) top2_add(mine, nr, i);
+      for (int w = 0; w < W; ++w) d += part[0][grp * W + w];
+    }
+    const double f = -tau * d;
+    d0 = d1 = 0.0;
+#pragma unroll
+    for (int u = 0; u < NREG; ++u) {
+      y[u] = fma(f, v[c0 + 32 * u], y[u]);
+      if (c0 + 32 * u < len) z[c0 + 32 * u] = y[u];
+      const double x = u == 0 && c0 == 0 ? 0.0 : y[u];
+      if (u & 1) d1 = fma(x, x, d1);
+      else d0 = fma(x, x, d0);
+    }
+    double nr = warp_sum(d0 + d1);
+    if (W > 1) {
+      if (lane == 0) part[1][warp] = nr;
+      named_barrier_sync(1 + grp, 32 * W);
+      nr = 0.0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) nr += part[1][grp * W + w];
+    }
+    if (lane == 0 && wq == 0) top2_add(mine, (unsigned long long)__double_as_longlong(nr), i, s);
   }
   mine = block_top2(mine);
   if (threadIdx.x == 0) out[blockIdx.x] = mine;
+}
+
+// The form of step k for residuals of `len` values: one warp a row up to 2048 values, then 2, 4 or 8.
+using GreedyStep = void (*)(Greedy, int);
+GreedyStep greedy_form(int len, int* threads, size_t* smem) {
+  static const GreedyStep one[8] = {greedy_step<8, 1>,  greedy_step<16, 1>, greedy_step<24, 1>, greedy_step<32, 1>,
+                                    greedy_step<40, 1>, greedy_step<48, 1>, greedy_step<56, 1>, greedy_step<64, 1>};
+  const int u = (len + 255) / 256;  // 8 values per lane each
+  *threads = u <= 4 ? 384 : 256;
+  if (u <= 8) {
+    *smem = (size_t)u * 256 * 8;
+    return one[u - 1];
+  }
+  const int w = u <= 16 ? 2 : u <= 32 ? 4 : 8;
+  *smem = (size_t)2048 * w * 8;
+  return w == 2 ? greedy_step<64, 2> : w == 4 ? greedy_step<64, 4> : greedy_step<64, 8>;
 }
 
 // ---- R, its inverse, the index sets -----------------------------------------------------------
@@ -594,8 +636,9 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
   g.m = (int)m;
   g.r = (int)r;
   g.sel = reinterpret_cast<int32_t*>(ws + Ly.sel);
+  g.act = reinterpret_cast<int32_t*>(ws + Ly.pos);  // index_sets fills it afresh afterwards
   g.blk = reinterpret_cast<Top2*>(ws + Ly.blk);
-  g.nblk = Ly.nblk;
+  g.nblk = kGreedyBlocks;
   g.order = reinterpret_cast<int32_t*>(ws + Ly.order);
   g.rdiag = reinterpret_cast<double*>(ws + Ly.rdiag);
   g.gap = reinterpret_cast<double*>(ws + Ly.gap);
@@ -634,15 +677,25 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
   if ((st = run_product(q, R, Ly.blk - Ly.R, s)) != PIFA_OK) return st;
 
   // 2. r greedy steps
-  greedy_init<<<Ly.nblk, 256, 0, s>>>(g);
+  greedy_init<<<g.nblk, 256, 0, s>>>(g);
   pifa_count_launch();
   PIFA_CK(cudaGetLastError(), "compress: greedy init launch");
-  const size_t vsm = (size_t)r * 8;
-  PIFA_CK(cudaFuncSetAttribute(greedy_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm),
-          "compress: greedy smem attribute");
   for (int k = 0; k < ri; ++k) {
-    greedy_step<<<Ly.nblk, 256, (size_t)(r - k) * 8, s>>>(g, k);
-    pifa_count_launch();
+    cudaLaunchConfig_t cfg = {};
+    int threads = 0;
+    const GreedyStep step = greedy_form(ri - k, &threads, &cfg.dynamicSmemBytes);
+    if (cfg.dynamicSmemBytes > 32768 && (k == 0 || (ri - k) % 2048 == 0))
+      PIFA_CK(cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes),
+              "compress: greedy smem attribute");
+    cfg.gridDim = dim3((unsigned)g.nblk);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;  // the next step's launch overlaps this step's tail
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    PIFA_CK(pifa_launch_ex(&cfg, step, g, k), "compress: greedy step launch");
   }
   PIFA_CK(cudaGetLastError(), "compress: greedy step launch");
 
