@@ -338,50 +338,63 @@ __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
 // so that no SM holds more than one row above its share (the chosen row's slot takes the last row).
 // 4096 x 4096, r = 2048: the form that this replaced (rows read twice from L2, by warps fixed to
 // rows; three more block-wide sums before the first row) took 84.3 us a step against 16 us of
-// float64 multiply-adds; this one KERNEL_US.
+// float64 multiply-adds; this one takes 34 us.
 template <int NREG, int W>
-constexpr int kGreedyWarps = W == 1 && NREG <= 32 ? 12 : 8;  // what the registers allow
+constexpr int kGreedyWarps = NREG <= 32 ? 12 : 8;  // what the registers allow
 template <int NREG, int W>
 __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Greedy g, int k) {
   constexpr int WARPS = kGreedyWarps<NREG, W>, GROUPS = WARPS / W, LEN = 32 * NREG * W;
   extern __shared__ double v[];  // LEN entries, zero from r - k on
-  __shared__ double part[2][WARPS];
+  __shared__ double part[2][WARPS], s_tau;
   const Top2* in = g.blk + (k & 1) * g.nblk;
   Top2* out = g.blk + ((k + 1) & 1) * g.nblk;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = warp / W, wq = warp % W;
   pdl_launch_dependents();
   pdl_wait_primary();
+  const int len = g.r - k, n = g.m - k;  // unchosen rows, p among them
+  const int c0 = wq * 32 * NREG + lane;
+  double y[NREG];
+  auto load = [&](int i) {
+    const double* z = g.Z + (int64_t)i * g.r + k;
+#pragma unroll
+    for (int u = 0; u < NREG; ++u) y[u] = c0 + 32 * u < len ? z[c0 + 32 * u] : 0.0;
+  };
+  const int s0 = blockIdx.x + gridDim.x * grp;
+  if (s0 < n - 1) load(g.act[s0]);  // this warp's first row, under the reduction (p's own is replaced)
   Top2 t = top2_empty();
   for (int b = threadIdx.x; b < g.nblk; b += WARPS * 32) top2_merge(t, in[b]);
   t = block_top2(t);
   const int p = t.i1;
-  const int len = g.r - k, n = g.m - k;  // unchosen rows, p among them
   if (p < 0 || p >= g.m || t.s1 < 0 || t.s1 >= n) return;  // cannot happen for m >= r; guards the reads
   const double* zp = g.Z + (int64_t)p * g.r + k;
-  const double nx2 = __longlong_as_double((long long)t.v1), nx = sqrt(nx2);
-  const double x0 = zp[0];
-  const double alpha = -copysign(nx, x0 != 0.0 ? x0 : 1.0);
-  const double tau = nx2 > 0.0 ? 1.0 / (nx2 + nx * fabs(x0)) : 0.0;
-  for (int c = threadIdx.x; c < LEN; c += WARPS * 32) v[c] = c < len ? (c == 0 ? x0 - alpha : zp[c]) : 0.0;
   const int tail = g.act[n - 1];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    g.order[k] = p;
-    g.rdiag[k] = alpha;
-    const double b2 = t.i2 >= 0 ? sqrt(__longlong_as_double((long long)t.v2)) : 0.0;
-    g.gap[k] = nx > 0.0 ? (nx - b2) / nx : 0.0;
-    g.sel[p] = 1;          // read only by later launches
-    g.act[t.s1] = tail;    // read by no block of this launch (see below)
+  for (int c = threadIdx.x; c < LEN; c += WARPS * 32)
+    if (c > 0) v[c] = c < len ? zp[c] : 0.0;
+  if (threadIdx.x < 32) {  // one warp: a float64 square root and division by each would delay the rows
+    const double nx2 = __longlong_as_double((long long)t.v1), nx = sqrt(nx2);
+    const double x0 = zp[0];
+    const double alpha = -copysign(nx, x0 != 0.0 ? x0 : 1.0);
+    if (threadIdx.x == 0) {
+      v[0] = x0 - alpha;
+      s_tau = nx2 > 0.0 ? 1.0 / (nx2 + nx * fabs(x0)) : 0.0;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      g.order[k] = p;
+      g.rdiag[k] = alpha;
+      const double b2 = t.i2 >= 0 ? sqrt(__longlong_as_double((long long)t.v2)) : 0.0;
+      g.gap[k] = nx > 0.0 ? (nx - b2) / nx : 0.0;
+      g.sel[p] = 1;          // read only by later launches
+      g.act[t.s1] = tail;    // a row loaded early from that slot is loaded again below
+    }
   }
   __syncthreads();
+  const double tau = s_tau;
   Top2 mine = top2_empty();
-  for (int s = blockIdx.x + gridDim.x * grp; s < n - 1; s += gridDim.x * GROUPS) {
+  for (int s = s0; s < n - 1; s += gridDim.x * GROUPS) {
     const int i = s == t.s1 ? tail : g.act[s];
     double* z = g.Z + (int64_t)i * g.r + k;
-    double y[NREG];
+    if (s != s0 || s == t.s1) load(i);
     double d0 = 0.0, d1 = 0.0;
-    const int c0 = wq * 32 * NREG + lane;
-#pragma unroll
-    for (int u = 0; u < NREG; ++u) y[u] = c0 + 32 * u < len ? z[c0 + 32 * u] : 0.0;
 #pragma unroll
     for (int u = 0; u < NREG; u += 2) {
       d0 = fma(y[u], v[c0 + 32 * u], d0);
