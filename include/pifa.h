@@ -270,11 +270,7 @@ int64_t pifa_compress_device_workspace_size(int64_t m, int64_t n, int64_t r);
  *   hi + lo pairs of bf16. Alignment as pifa_forward (fp32 pitches multiples of 4 elements).
  *   T == 0 writes zero dW_p and dC. Asynchronous on cuda_stream; out-of-range indices latch
  *   PIFA_ERR_DEVICE_INDEX (read with pifa_device_status()).
- *   Concurrency: independent products run on two side streams that the library keeps per host
- *   thread and device, forked from cuda_stream and joined back into it inside the call (also on
- *   failure), so the call orders like one kernel sequence on cuda_stream and can be captured into a
- *   CUDA graph. The first call on a thread and device creates those streams: make it before a
- *   stream capture that contains the call.
+ *   The call is one sequence of kernels on cuda_stream and can be captured into a CUDA graph.
  */
 int pifa_backward(const void* X, int64_t T, int64_t n, int64_t ldx,
                   const void* Wp, int64_t r, int64_t ldwp,
@@ -306,8 +302,7 @@ int64_t pifa_backward_workspace_size(int64_t T, int64_t m, int64_t n, int64_t r)
  *   workspace    DEVICE scratch of pifa_m_accumulate_workspace_size(T, m, n) bytes, 256-byte
  *                aligned (X_u^T, the mixed input and Y_t^T in bf16).
  *   Numerics: bf16 operands, fp32 accumulation; the mixed input and Y_t pass as hi + lo bf16 pairs.
- *   T == 0 is a no-op. Asynchronous on cuda_stream; X X^T runs beside the Y_t chain on a side
- *   stream, as in pifa_backward (same ordering and capture rules).
+ *   T == 0 is a no-op. Asynchronous on cuda_stream (ordering and capture as pifa_backward).
  */
 int pifa_m_accumulate(const void* Xo, const void* Xu, int64_t T, int64_t n, int64_t ldx,
                       const void* W, int64_t m, int64_t ldw, float lambda,

@@ -269,42 +269,37 @@ extern "C" int pifa_backward(const void* X, int64_t T, int64_t n, int64_t ldx, c
                                          ldnp, status);
     if (e != cudaSuccess) return pifa_fail_cuda("backward: split dY", e);
   }
-  // Independent products run concurrently: Y_p and then dC on side stream 0 (after the split),
-  // dY_p and then dX on the caller's stream, dW_p on side stream 1 once dY_p is done. Each product
-  // alone fills one or two waves of the GPU; together they keep it busy (the side streams rejoin
-  // the caller's stream before this call returns, also on failure).
-  PifaSides sides(s);
-  cudaStream_t s_yp = s, s_dw = s;
-  // Y_p = X W_p^T as hi + lo planes (only dC needs it)
-  if (dC && has_np) {
-    if ((st = sides.fork(0, &s_yp)) != PIFA_OK) return st;
-    GemmTc g = {T, r, n, X, ldx, false, Wp, ldwp, false, Yp, ldr, 3, 1.0f, nullptr, nullptr, 0, 0};
-    g.D2 = Yp_lo;
-    if ((st = gemm_tc(g, status, tmo, s_yp)) != PIFA_OK) return st;
-  }
-  // dY_p = dY_I + dY_np C, as hi + lo planes (dY_p = dY_I when r = m)
-  if (has_np) {
-    GemmTc g = {T, r, m - r, dYnp, ldnp, false, C, ldc, true, dYp, ldr, 3, 1.0f, dYi, nullptr, ldr, r};
+  // Two launches of independent products: those that dY and X give, then those that need them. (One
+  // stream per product instead left the last wave of each launch's tiles on a part of the SMs.)
+  GemmTc first[2], second[3];
+  int n1 = 0, n2 = 0;
+  if (has_np) {  // dY_p = dY_I + dY_np C, as hi + lo planes (dY_p = dY_I when r = m)
+    GemmTc g = {T, r, m - r, dYnp, ldnp, false, C, ldc, true, dYp, ldr, 3, 1.0f, dYi, ldr};
     g.D2 = dYp_lo;
-    if ((st = gemm_tc(g, status, tmo, s)) != PIFA_OK) return st;
+    first[n1++] = g;
   }
-  if (dWp) {  // dW_p = (dY_p,hi + dY_p,lo)^T X
-    if ((st = sides.fork(1, &s_dw)) != PIFA_OK) return st;
-    GemmTc g = {r, n, T, dYp, ldr, true, X, ldx, true, dWp, lddwp, 1, 1.0f, nullptr, nullptr, 0, 0};
-    if (has_np) g.A2 = dYp_lo;
-    if ((st = gemm_tc(g, status, tmo, s_dw)) != PIFA_OK) return st;
+  if (dC && has_np) {  // Y_p = X W_p^T as hi + lo planes (only dC needs it)
+    GemmTc g = {T, r, n, X, ldx, false, Wp, ldwp, false, Yp, ldr, 3, 1.0f, nullptr, 0};
+    g.D2 = Yp_lo;
+    first[n1++] = g;
   }
   if (dX) {  // dX = (dY_p,hi + dY_p,lo) W_p  (dY_p exact in bf16 when r == m)
-    GemmTc g = {T, n, r, dYp, ldr, false, Wp, ldwp, true, dX, lddx, 0, 1.0f, nullptr, nullptr, 0, 0};
+    GemmTc g = {T, n, r, dYp, ldr, false, Wp, ldwp, true, dX, lddx, 0, 1.0f, nullptr, 0};
     if (has_np) g.A2 = dYp_lo;
-    if ((st = gemm_tc(g, status, tmo, s)) != PIFA_OK) return st;
+    second[n2++] = g;
   }
-  if (dC && has_np) {  // dC = dY_np^T (Y_p,hi + Y_p,lo), after Y_p on its side stream
-    GemmTc g = {m - r, r, T, dYnp, ldnp, true, Yp, ldr, true, dC, lddc, 1, 1.0f, nullptr, nullptr, 0, 0};
+  if (dWp) {  // dW_p = (dY_p,hi + dY_p,lo)^T X
+    GemmTc g = {r, n, T, dYp, ldr, true, X, ldx, true, dWp, lddwp, 1, 1.0f, nullptr, 0};
+    if (has_np) g.A2 = dYp_lo;
+    second[n2++] = g;
+  }
+  if (dC && has_np) {  // dC = dY_np^T (Y_p,hi + Y_p,lo)
+    GemmTc g = {m - r, r, T, dYnp, ldnp, true, Yp, ldr, true, dC, lddc, 1, 1.0f, nullptr, 0};
     g.B2 = Yp_lo;
-    if ((st = gemm_tc(g, status, tmo, s_yp)) != PIFA_OK) return st;
+    second[n2++] = g;
   }
-  return PIFA_OK;
+  if ((st = gemm_tc_group(first, n1, status, tmo, s)) != PIFA_OK) return st;
+  return gemm_tc_group(second, n2, status, tmo, s);
 }
 
 extern "C" int64_t pifa_m_accumulate_workspace_size(int64_t T, int64_t m, int64_t n) {
@@ -355,40 +350,29 @@ extern "C" int pifa_m_accumulate(const void* Xo, const void* Xu, int64_t T, int6
                                              (int)n, XuT, ldT);
     if (e != cudaSuccess) return pifa_fail_cuda("m_accumulate: transpose", e);
   }
-  // X X^T on the caller's stream and, concurrently, the mix, Y_t^T and Y_t X^T on a side stream
-  // (both read X_u^T; the side stream rejoins before this call returns, also on failure)
-  PifaSides sides(s);
-  if (YtXt) {
-    cudaStream_t s2 = s;
-    if ((st = sides.fork(0, &s2)) != PIFA_OK) return st;
-    bf16* Xmix = reinterpret_cast<bf16*>(ws + Ly.xmix);
-    bf16* Xmix_lo = reinterpret_cast<bf16*>(ws + Ly.xmix_lo);
-    bf16* YtT = reinterpret_cast<bf16*>(ws + Ly.ytt);
-    bf16* YtT_lo = reinterpret_cast<bf16*>(ws + Ly.ytt_lo);
-    {  // X_mix = lambda X_o + (1 - lambda) X_u, as hi + lo planes
-      int Ti = (int)T, ni = (int)n;
-      float a = lambda, b = 1.0f - lambda;
-      void* args[] = {(void*)&Xo, (void*)&Xu, (void*)&ldx, (void*)&Ti, (void*)&ni, (void*)&a, (void*)&b, (void*)&Xmix,
-                      (void*)&Xmix_lo, (void*)&ldn};
-      if ((st = launch_small((const void*)axpby_rows, args, T, (n + 7) / 8, s2, "m_accumulate: mix")) != PIFA_OK)
-        return st;
-    }
-    {  // Y_t^T = W (X_mix,hi + X_mix,lo)^T, as hi + lo planes (m x T)
-      GemmTc g = {m, T, n, W, ldw, false, Xmix, ldn, false, YtT, ldT, 3, 1.0f, nullptr, nullptr, 0, 0};
-      g.B2 = Xmix_lo;
-      g.D2 = YtT_lo;
-      if ((st = gemm_tc(g, status, tmo, s2)) != PIFA_OK) return st;
-    }
-    {  // YtXt += (Y_t^T,hi + Y_t^T,lo) X_u
-      GemmTc g = {m, n, T, YtT, ldT, false, XuT, ldT, false, YtXt, ldyx, 2, 1.0f, nullptr, nullptr, 0, 0};
-      g.A2 = YtT_lo;
-      if ((st = gemm_tc(g, status, tmo, s2)) != PIFA_OK) return st;
-    }
+  // XXt += X_u^T X_u, its upper triangle (the product is symmetric: half the tiles)
+  GemmTc xx = {n, n, T, XuT, ldT, false, XuT, ldT, false, XXt, ldxx, 2, 1.0f, nullptr, 0};
+  xx.upper = true;
+  if (!YtXt) return gemm_tc_group(&xx, 1, status, tmo, s);
+  bf16* Xmix = reinterpret_cast<bf16*>(ws + Ly.xmix);
+  bf16* Xmix_lo = reinterpret_cast<bf16*>(ws + Ly.xmix_lo);
+  bf16* YtT = reinterpret_cast<bf16*>(ws + Ly.ytt);
+  bf16* YtT_lo = reinterpret_cast<bf16*>(ws + Ly.ytt_lo);
+  {  // X_mix = lambda X_o + (1 - lambda) X_u, as hi + lo planes
+    int Ti = (int)T, ni = (int)n;
+    float a = lambda, b = 1.0f - lambda;
+    void* args[] = {(void*)&Xo, (void*)&Xu, (void*)&ldx, (void*)&Ti, (void*)&ni, (void*)&a, (void*)&b, (void*)&Xmix,
+                    (void*)&Xmix_lo, (void*)&ldn};
+    if ((st = launch_small((const void*)axpby_rows, args, T, (n + 7) / 8, s, "m_accumulate: mix")) != PIFA_OK) return st;
   }
-  {  // XXt += X_u^T X_u, its upper triangle (the product is symmetric: half the tiles)
-    GemmTc g = {n, n, T, XuT, ldT, false, XuT, ldT, false, XXt, ldxx, 2, 1.0f, nullptr, nullptr, 0, 0};
-    g.upper = true;
-    if ((st = gemm_tc(g, status, tmo, s)) != PIFA_OK) return st;
-  }
-  return PIFA_OK;
+  // Y_t^T = W (X_mix,hi + X_mix,lo)^T, as hi + lo planes (m x T), beside X X^T, whose tiles fill the
+  // SMs that Y_t^T's last wave leaves; then YtXt += (Y_t^T,hi + Y_t^T,lo) X_u
+  GemmTc yt = {m, T, n, W, ldw, false, Xmix, ldn, false, YtT, ldT, 3, 1.0f, nullptr, 0};
+  yt.B2 = Xmix_lo;
+  yt.D2 = YtT_lo;
+  GemmTc yx = {m, n, T, YtT, ldT, false, XuT, ldT, false, YtXt, ldyx, 2, 1.0f, nullptr, 0};
+  yx.A2 = YtT_lo;
+  const GemmTc first[2] = {yt, xx};
+  if ((st = gemm_tc_group(first, 2, status, tmo, s)) != PIFA_OK) return st;
+  return gemm_tc_group(&yx, 1, status, tmo, s);
 }

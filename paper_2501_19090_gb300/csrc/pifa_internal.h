@@ -24,23 +24,6 @@ uint64_t pifa_wait_timeout_ns();
 // per successful launch; pifa_launch_count() reads the total.
 void pifa_count_launch();
 
-// Up to two side streams for independent work inside one call (status.cu): fork(i) makes side
-// stream i wait for the work enqueued on the caller's stream so far and returns it; the destructor
-// makes the caller's stream wait for every side stream that was forked. Per host thread and device.
-class PifaSides {
- public:
-  explicit PifaSides(cudaStream_t main) : main_(main) {}
-  ~PifaSides();
-  PifaSides(const PifaSides&) = delete;
-  PifaSides& operator=(const PifaSides&) = delete;
-  int fork(int i, cudaStream_t* side);  // PIFA_OK or PIFA_ERR_CUDA
-
- private:
-  cudaStream_t main_;
-  void* state_ = nullptr;
-  bool forked_[2] = {false, false};
-};
-
 #ifdef __CUDACC__
 #include <utility>
 // cudaLaunchKernelEx, counted.
@@ -131,10 +114,8 @@ int launch_decode_tc(const DecodeTcPhase& ph, int* status, uint64_t timeout_ns, 
 // is K-major (a_mn = false: element (i, k) at [i * ld + k]) or MN-major (true: at [k * ld + i]).
 // out_mode 0: D bf16; 1: D fp32; 2: D fp32 += result; 3: D = bf16 hi, D2 = bf16 lo of the result.
 // A2 / B2 (optional, A's / B's layout and pitch): a second K pass with A2 for A and / or B2 for B,
-// D = (A + A2) B^T or A (B + B2)^T. Optional addend:
-// D[i][j] += add[i * ldadd + (add_idx ? add_idx[j] : j)] (bf16; add_idx values must lie in
-// [0, add_bound)). Pointers 16-byte aligned, leading dimensions multiples of 8 elements (the caller
-// checks).
+// D = (A + A2) B^T or A (B + B2)^T. Optional addend (out_mode 0 and 3): D[i][j] += add[i * ldadd + j]
+// (bf16). Pointers 16-byte aligned, leading dimensions multiples of 8 elements (the caller checks).
 struct GemmTc {
   int64_t M, N, K;
   const void* A;
@@ -148,16 +129,14 @@ struct GemmTc {
   int out_mode;
   float alpha;
   const void* add;
-  const int32_t* add_idx;
   int64_t ldadd;
-  int64_t add_bound;
   const void* A2 = nullptr;
   const void* B2 = nullptr;
   void* D2 = nullptr;
-  bool d_trans = false;  // store D^T: element (i, j) at D[j * ldd + i] (out_mode 0, 1 or 3 only)
-  bool upper = false;    // M == N: skip tiles wholly below the diagonal (a symmetric product's upper triangle)
+  bool upper = false;    // M == N: skip 128 x 128 blocks wholly below the diagonal (a symmetric product)
 };
-int gemm_tc(const GemmTc& g, int* status, uint64_t timeout_ns, cudaStream_t stream);
+// Up to three independent products in one launch.
+int gemm_tc_group(const GemmTc* gs, int n, int* status, uint64_t timeout_ns, cudaStream_t stream);
 
 // ---- float64 products (compress_gpu.cu, gemm_f64_tc.cu) -------------------------------------------
 // C[i][ccol(j)] = beta C + alpha sum_k A(i, k) B(k, j), with

@@ -250,3 +250,32 @@ def test_backward_and_m_accumulate_under_graph_capture():
     torch.cuda.synchronize()
     assert P.pifa_device_status() == P.PIFA_OK
     assert torch.equal(torch.triu(XXt1), torch.triu(XXt0)) and torch.equal(Y1, Y0)
+
+
+@pytest.mark.parametrize("m,n,r,T", [(384, 264, 136, 65), (1032, 776, 300, 130), (4104, 4096, 264, 300), (300, 4000, 129, 2100)])
+def test_backward_tile_edges(m, n, r, T):
+    """Products of one tile, of ragged last tiles, of more tiles than SMs and of every tile width, dealt
+    over the persistent grid, against the oracle (random layer: the tiling is what matters)."""
+    piv, nonp, Wp32, C32 = inputs.synthetic_layer(m, n, r, 31)
+    rng = np.random.default_rng(32)
+    X32, dY32 = inputs.make_activations(rng, T, n, "bf16"), inputs.make_activations(rng, T, m, "bf16")
+    pd = torch.from_numpy(piv).to(DEV)
+    nd = torch.from_numpy(nonp).to(DEV)
+    dX, dWp, dC = P.pifa_backward(dev_bf16(X32), dev_bf16(Wp32), dev_bf16(C32), pd, nd, dev_bf16(dY32))
+    assert P.pifa_device_status() == P.PIFA_OK
+    for got, ref, what in zip((dX, dWp, dC), oracle.backward(X32, Wp32, C32, piv, nonp, dY32), ("dX", "dW_p", "dC")):
+        check(got.float().cpu().numpy(), ref, what)
+
+
+@pytest.mark.parametrize("m,n,T", [(130, 4200, 70), (2050, 136, 300), (264, 520, 2100)])
+def test_m_accumulate_tile_edges(m, n, T):
+    """X X^T keeps exactly its 128 x 128 blocks on and above the diagonal, whatever the tile width."""
+    Xo, Xu, W = _macc_inputs(T, n, m, 41)
+    XXt = torch.zeros((n, n), dtype=torch.float32, device=DEV)
+    YtXt = torch.zeros((m, n), dtype=torch.float32, device=DEV)
+    P.pifa_m_accumulate(dev_bf16(Xo), dev_bf16(Xu), dev_bf16(W), 0.25, XXt, YtXt)
+    assert P.pifa_device_status() == P.PIFA_OK
+    a, b = oracle.m_accumulate(Xo, Xu, W, 0.25)
+    blk = np.arange(n) // 128
+    check(XXt.cpu().numpy(), np.where(blk[:, None] <= blk[None, :], a, 0.0), "X X^T")
+    check(YtXt.cpu().numpy(), b, "Y_t X^T")
