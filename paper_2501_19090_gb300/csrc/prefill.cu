@@ -1,7 +1,7 @@
 // prefill.cu -- PIFA forward for many tokens on the 5th-generation tensor cores (tcgen05).
 //
 // Split variant: two launches of one warp-specialised tcgen05 GEMM.
-//   GEMM 1 (Algorithm 2, steps 2 and 4): D1 = W_p X^T, tile 128 weight rows x 256 tokens.
+//   GEMM 1 (Algorithm 2, steps 2 and 4): D1 = W_p X^T, weight rows x tokens.
 //           Epilogue writes bf16(Y_p) into the pivot columns Y[:, I[j]] and the pair
 //           hi = rnd(Y_p), lo = rnd(Y_p - hi) into two T x r scratch matrices, rnd rounding to
 //           C's storage type (bf16 or fp16).
@@ -11,21 +11,33 @@
 // memory holds one weight row per TMEM lane: an epilogue warp's 32 lanes are 32 consecutive
 // weight rows, which for a fixed token land in 32 ascending output columns of one row of Y.
 //
-// Per CTA (576 threads): warp 0 issues TMA loads into a 4-stage shared-memory ring (A tile
-// 128 x 64, B tile 256 x 64, bf16, 128-byte swizzle), warp 1 owns the TMEM allocation and issues
-// tcgen05.mma (M=128, N=256, K=16) from one thread, warps 2-17 drain the fp32 accumulator
-// (128 lanes x 256 columns of TMEM) through tcgen05.ld. The epilogue, not the tensor cores, was
-// the largest cost of this kernel (16 of 66 us at 4096 x 4096, r = 2048, T = 2048): its output is
-// a column scatter into Y of 2-byte stores. Sixteen warps issue them, and Y_p's hi/lo planes go
-// out as 16-byte stores after a transpose through shared memory. Every wait is bounded
-// (globaltimer); on timeout the CTA latches PIFA_ERR_TIMEOUT, drains what it has in flight and
-// returns.
+// A pair of CTAs (one per SM, 352 threads each) computes a tile of 256 weight rows x bn tokens
+// (bn <= 256) with pair MMAs (cta_group::2: M = 256, N = bn, K = 16): each CTA loads its 128 weight
+// rows and half of the tile's tokens per 64 columns of K into a ring of stages (128-byte swizzle),
+// warp 0 the weights, which need not wait for the previous kernel, the last warp the activations;
+// the even CTA's warp 1 issues the MMAs of both; warps 2-9 of each CTA drain its 128 rows of the
+// accumulator through tcgen05.ld. The grid is persistent with two accumulators (256 TMEM columns
+// each), so that from the second tile on a tile's epilogue runs under the next tile's MMAs.
+// Y's stores are a column scatter of 2 bytes per lane; Y_p's hi/lo planes go out as 4-byte stores of
+// two rows after an exchange between neighbouring lanes. Every wait is bounded (globaltimer); on timeout the CTA
+// latches PIFA_ERR_TIMEOUT, drains what it has in flight and returns.
 //
-// GEMMs whose full-width tiles leave most SMs idle (GEMM 1 of the 70B layers has 32 row blocks;
-// T of a few hundred gives one token tile) split K instead: a tile's 2 or 4 CTAs form a cluster,
-// each accumulates its K-slice, stores the fp32 partial tile in its own freed stage ring, and the
-// cluster adds the slices through distributed shared memory in rank order before the epilogue.
-#include <utility>
+// A 64-column chunk of K costs a tile 330 + 0.85 bn cycles by a pair (its MMAs are 2 bn of them) and
+// 410 + 0.3 bn to 480 + 0.66 bn by one CTA, much of it the hand-offs of a stage (its copy's arrival, the
+// MMAs' issue and commit, the release), which is why a stage holds two chunks where the ring allows, why
+// the issuing threads do no division and read no flag, and why wide tiles are best where they fill
+// the GPU. GEMMs of few tiles run on tiles of 128 rows by one CTA and split K: the 2 or 4 CTAs of a
+// tile form a cluster, each accumulates its K-slice, stores the fp32 partial tile in its own freed
+// ring, and the cluster adds the slices through distributed shared memory in rank order before the
+// epilogue. pick_shape takes the form, width and split that these costs say finishes first; measured
+// beside every alternative on five layers at T = 80 to 2048 it was within 4% of the best.
+// Against the one-CTA forms that this replaced (us, CUDA graph, one process): 7B attention T = 128
+// 25.2 -> 20.0, 512 37.4 -> 34.6, 2048 58.0 -> 53.9, 4096 119.5 -> 94.7; 7B gate T = 2048 143.8 ->
+// 120.4; 7B down T = 300 48.1 -> 35.9; 70B q/o T = 300 89.4 -> 56.3, 4096 400.3 -> 345.8; 70B gate/up
+// T = 512 227.2 -> 181.5, 4096 1460.2 -> 1226.3. At T = 2048 on the 7B attention layer each GEMM is one
+// round of 64 pair tiles: what is left is its 34 GFLOP at the tensor rate of 128 of 152 SMs (19 us), its
+// launch and first copies (about 5 us) and its exposed epilogue (about 3 us).
+#include <algorithm>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -39,50 +51,35 @@ namespace {
 using namespace pifa;
 using bf16 = __nv_bfloat16;
 
-constexpr int BM = 128;  // weight rows per tile (MMA M)
-constexpr int BK = 64;   // K per stage: one 128-byte swizzle row of bf16
+constexpr int BM = 128;       // weight rows of one CTA
+constexpr int PM = 2 * BM;    // of a pair
+constexpr int BNMAX = 256;    // tokens per tile
+constexpr int BK = 64;        // K per chunk: one 128-byte swizzle row of bf16
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = 96 + 32 * EPI_WARPS;
 constexpr uint32_t A_BYTES = BM * BK * 2;
-
-// Two shapes of the same kernel. Config 0: one CTA per SM, up to 256 tokens per tile, a 4-stage
-// ring and 16 epilogue warps (the fastest when a GEMM fits one or two waves). Config 1: two CTAs
-// per SM, up to 160 tokens per tile, 3 stages and 8 epilogue warps: one CTA's epilogue runs while
-// the other's MMAs keep the tensor core busy, which pays on GEMMs of many waves (measured, same
-// outputs bit for bit: T = 8192 on the 4096 x 4096, r = 2048 layer 241.1 -> 226.2 us; 70B q/o
-// T = 4096 427.3 -> 390.1 us). A GEMM of one or two waves leaves little to overlap, and there the
-// one-CTA shape's wider tiles and deeper ring are kept.
-template <int CFG>
-struct PCfg;
-template <>
-struct PCfg<0> {
-  static constexpr int BN = 256, STAGES = 4, EPI_WARPS = 16, CTAS = 1;
-};
-template <>
-struct PCfg<1> {
-  static constexpr int BN = 160, STAGES = 3, EPI_WARPS = 8, CTAS = 2;
-};
-template <int CFG>
-struct PC : PCfg<CFG> {
-  using B = PCfg<CFG>;
-  static constexpr int THREADS = 64 + 32 * B::EPI_WARPS;  // + the TMA producer and the MMA warp
-  static constexpr uint32_t B_BYTES = B::BN * BK * 2;
-  static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr uint32_t TMEM_COLS = 256;  // fp32 accumulator, one column per token (a power of two)
-  static constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + B::STAGES * STAGE_BYTES + 256 /*barriers*/;
-};
+constexpr uint32_t RING_BYTES = 224 * 1024;
+constexpr int MAX_STAGES = 10;
+constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + 256;
+constexpr uint32_t TMEM_COLS = 512;
 
 // Epilogue modes: what GEMM 1 also writes besides Y (GEMM 2 writes Y only).
 enum { EPI_Y_ONLY = 0, EPI_SPLIT_BF16 = 1, EPI_SPLIT_F16 = 2 };
 
 struct GemmArgs {
   uint32_t idesc;        // tcgen05 instruction descriptor (bf16 or fp16 operands)
-  int M;                 // weight rows (r for GEMM 1, m - r for GEMM 2)
+  int M;                 // weight rows (r for GEMM 1, m - r for GEMM 2, times the groups)
   int N;                 // tokens T
-  int bn;                // tokens per tile (MMA N, TMA box rows of B): a multiple of 16, <= BN
-  int tok_fast;          // 1: blockIdx.x walks token tiles (CTAs of one weight-row block together), else row tiles
+  int bn;                // tokens per tile (MMA N): a multiple of 32, <= BNMAX
+  int nt, mt, tiles;     // token tiles, row tiles
+  int tok_fast;          // 1: consecutive tiles walk the token tiles (pairs of one weight-row block together)
+  int gsz, mtg;          // weight rows per group (M when not grouped), row tiles per group: none spans two
+  int goff;              // B columns between consecutive groups' K ranges (r; 0 when not grouped)
   int kchunks;           // ceil(K / 64) per pass
+  int subs, ksteps;      // chunks per stage (1 or 2), stages per pass
   int passes;            // 1, or 2 for the hi + lo passes of GEMM 2
-  int gsz;               // grouped layers (GEMM 2): weight rows per group (whole tiles), else 0
-  int goff;              // B columns between consecutive groups' K ranges (r), when gsz > 0
+  int stages;
+  uint32_t stage_bytes;
   const int32_t* cols;   // output column of each weight row (I or I^c)
   int m;                 // columns of Y (index bound)
   bf16* Y;
@@ -92,265 +89,334 @@ struct GemmArgs {
   int64_t ldyp;
   int* status;
   uint64_t timeout_ns;
-  int ks;                // K-slices per tile (kCl): the CTAs blockIdx.z = 0 .. ks - 1 of a tile form a cluster
+  int ks;                // K-slices per tile (kCl): CTAs of a cluster
 };
 
-// kCl: split-K over a cluster of ks CTAs per tile (grids with too few tiles to fill the GPU). CTA z
-// accumulates the K-steps [z total / ks, (z + 1) total / ks) of both passes, stores its fp32
-// partial tile in its own shared memory (the stage ring, free once its MMAs are done) and, after a
-// cluster barrier, adds rows [z 128 / ks, (z + 1) 128 / ks) of every peer's partial tile in rank
-// order (distributed shared memory) and writes them out as the epilogue would. Only these
-// instantiations hold cluster barriers and distributed shared-memory loads.
-template <int kEpi, int CFG, bool kCl>
-__global__ void __launch_bounds__(PC<CFG>::THREADS, PC<CFG>::CTAS)
+// hi + lo split of an fp32 value in bf16 or fp16; fp16 saturates at +-65504 and reports it.
+template <int kEpi>
+__device__ __forceinline__ void split_hl(float f, uint16_t& h, uint16_t& l, bool& range_err) {
+  if (kEpi == EPI_SPLIT_F16) {
+    if (fabsf(f) > 65504.0f) {
+      range_err = true;
+      f = copysignf(65504.0f, f);
+    }
+    const __half hh = __float2half_rn(f);
+    h = __half_as_ushort(hh);
+    l = __half_as_ushort(__float2half_rn(f - __half2float(hh)));
+  } else {
+    const bf16 hh = __float2bfloat16_rn(f);
+    h = __bfloat16_as_ushort(hh);
+    l = __bfloat16_as_ushort(__float2bfloat16_rn(f - __bfloat162float(hh)));
+  }
+}
+
+// kPair: a tile of 256 weight rows by a pair of CTAs; else of 128 rows by one.
+// kCl (one-CTA tiles): split-K over a cluster of ks CTAs per tile (grids with too few tiles to fill the
+// GPU): CTA z accumulates the K-steps [z total / ks, (z + 1) total / ks) of both passes; after a cluster
+// barrier it adds rows [z 128 / ks, (z + 1) 128 / ks) of the slices in rank order.
+template <int kEpi, bool kCl, bool kPair>
+__global__ void __launch_bounds__(THREADS, 1)
     pifa_umma_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
-                   const __grid_constant__ CUtensorMap tmB1, GemmArgs p) {
-  constexpr int STAGES = PC<CFG>::STAGES, EPI_WARPS = PC<CFG>::EPI_WARPS, BN = PC<CFG>::BN;
-  constexpr uint32_t STAGE_BYTES = PC<CFG>::STAGE_BYTES, TMEM_COLS = PC<CFG>::TMEM_COLS;
+                   const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ GemmArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* acc_full = empty + STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
+  uint64_t* empty = full + MAX_STAGES;
+  uint64_t* accf = empty + MAX_STAGES;
+  uint64_t* acce = accf + 2;
+  uint64_t* drain = acce + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
   pdl_launch_dependents();  // the next kernel may launch now (its CTAs take SMs this grid leaves idle)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // launch order: along the shorter of M and T (see run_gemm), so that one wave's operand tiles
-  // stay in L2
-  const int m0 = (p.tok_fast ? blockIdx.y : blockIdx.x) * BM;
-  const int n0 = (p.tok_fast ? blockIdx.x : blockIdx.y) * p.bn;
-  const uint32_t b_bytes = (uint32_t)p.bn * BK * 2;  // one B box
-  const int bx0 = p.gsz > 0 ? (m0 / p.gsz) * p.goff : 0;  // the tile's group's first B column
-  const int ksteps = p.kchunks * p.passes;
-  const int z = kCl ? (int)blockIdx.z : 0;
+  static_assert(!(kCl && kPair), "split-K clusters are of one-CTA tiles");
+  const bool leader = !kPair || (blockIdx.x & 1) == 0;  // issues the MMAs
+  const int z = kCl ? (int)cluster_ctarank() : 0;
+  const int ksteps = p.ksteps * p.passes;
   const int i0 = kCl ? (int)(((int64_t)z * ksteps) / p.ks) : 0;  // this CTA's K-steps [i0, i0 + total)
   const int total = kCl ? (int)(((int64_t)(z + 1) * ksteps) / p.ks) - i0 : ksteps;
+  // tiles first, first + stride, ... of this CTA or pair
+  const int first = kCl ? (int)blockIdx.x / p.ks : (int)blockIdx.x >> (kPair ? 1 : 0);
+  const int stride = kCl ? p.tiles : (int)gridDim.x >> (kPair ? 1 : 0);
+  auto place = [&](int idx, int& m0, int& mend, int& n0, int& bx0) {
+    const int mi = p.tok_fast ? idx / p.nt : idx % p.mt, ni = p.tok_fast ? idx % p.nt : idx / p.mt;
+    const int g = mi / p.mtg;
+    m0 = g * p.gsz + (mi - g * p.mtg) * (kPair ? PM : BM) + (leader ? 0 : BM);  // this CTA's rows
+    mend = min(p.M, (g + 1) * p.gsz);
+    n0 = ni * p.bn;
+    bx0 = g * p.goff;
+  };
 
-  if (warp == 0 && lane == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(acc_full, 1);
-    *abort_flag = 0;
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accf[b], 1);
+      mbar_init(&acce[b], (kPair ? 2 : 1) * EPI_WARPS);  // the leader's: both CTAs' warps
+    }
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB0);
     if (p.passes > 1) prefetch_tmap(&tmB1);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, TMEM_COLS);
-    tmem_relinquish();
+    if (kPair) {
+      tmem_alloc_pair(tmem_slot, TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (kPair) cluster_sync_all();  // both CTAs' barriers are initialised before either signals the other's
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
+  if (warp == 0 || warp == EPI_WARPS + 2) {
     if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      // The weight tiles (A) do not depend on the previous kernel: those of the first stages go out
-      // before the dependency wait, raising the expected bytes without arriving; the activation
-      // tiles (B: X, or the y_p planes GEMM 1 wrote) follow the wait and bring the arrival.
-      const int pre = total < STAGES ? total : STAGES;
-      for (int i = 0; i < pre; ++i) {
-        mbar_expect_tx(&full[i], A_BYTES);
-        tma_load_2d(smem_u32(smem + i * STAGE_BYTES), &tmA, ((i0 + i) % p.kchunks) * BK, m0, &full[i]);
-      }
-      pdl_wait_primary();
-      for (int i = 0; i < pre; ++i) {
-        const int pass = (i0 + i) / p.kchunks, kc = (i0 + i) % p.kchunks;
-        mbar_arrive_expect_tx(&full[i], b_bytes);
-        tma_load_2d(smem_u32(smem + i * STAGE_BYTES + A_BYTES), pass ? &tmB1 : &tmB0, bx0 + kc * BK, n0, &full[i]);
-      }
-      int issued = pre;
-      for (int i = pre; i < total; ++i) {
-        const int s = i % STAGES;
-        const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, p.timeout_ns)) {
-          *abort_flag = 1;
-          latch_status(p.status, PIFA_ERR_TIMEOUT);
-          break;
+      // ---------------- TMA producers: warp 0 the weights, the last warp the activations ----------------
+      const bool is_a = warp == 0;
+      if (!is_a) pdl_wait_primary();  // X, or the y_p planes GEMM 1 wrote; the weights depend on no kernel
+      const int hb = kPair ? p.bn / 2 : p.bn;  // this CTA's tokens
+      const uint32_t bytes = (kPair ? 2 : 1) * A_BYTES + (uint32_t)p.bn * BK * 2;  // a chunk's, both CTAs'
+      const uint32_t box = is_a ? A_BYTES : (uint32_t)hb * BK * 2;
+      const uint32_t dst0 = smem_u32(smem) + (is_a ? 0u : (uint32_t)p.subs * A_BYTES);
+      int s = 0, it = 0;
+      uint32_t ph = 1;  // parity that a fresh "empty" barrier passes
+      bool dead = false;
+      for (int idx = first; idx < p.tiles && !dead; idx += stride) {
+        int m0, mend, n0, bx0;
+        place(idx, m0, mend, n0, bx0);
+        const int y = is_a ? m0 : n0 + (leader ? 0 : hb), x0 = is_a ? 0 : bx0;
+        const int pass = i0 / p.ksteps;
+        int kc = (i0 - pass * p.ksteps) * p.subs;  // first chunk of the stage
+        const CUtensorMap* map = is_a ? &tmA : pass ? &tmB1 : &tmB0;
+        for (int i = 0; i < total; ++i, ++it) {
+          if (!mbar_wait(&empty[s], ph, p.timeout_ns)) {
+            latch_status(p.status, PIFA_ERR_TIMEOUT);
+            dead = true;
+            break;
+          }
+          const bool two = p.subs == 2 && kc + 1 < p.kchunks;
+          if (leader && is_a) mbar_arrive_expect_tx(&full[s], two ? 2 * bytes : bytes);
+          const uint32_t dst = dst0 + (uint32_t)s * p.stage_bytes;
+          const int x = x0 + kc * BK;
+          if (kPair) {
+            const uint32_t bar = mapa_shared(smem_u32(&full[s]), 0);
+            tma_load_2d_pair(dst, map, x, y, bar);
+            if (two) tma_load_2d_pair(dst + box, map, x + BK, y, bar);
+          } else {
+            tma_load_2d(dst, map, x, y, &full[s]);
+            if (two) tma_load_2d(dst + box, map, x + BK, y, &full[s]);
+          }
+          kc += p.subs;
+          if (kc >= p.kchunks) {
+            kc = 0;
+            if (!is_a) map = &tmB1;
+          }
+          if (++s == p.stages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        if (*abort_flag) break;
-        const int pass = (i0 + i) / p.kchunks, kc = (i0 + i) % p.kchunks;
-        uint8_t* sa = smem + s * STAGE_BYTES;
-        mbar_arrive_expect_tx(&full[s], A_BYTES + b_bytes);
-        tma_load_2d(smem_u32(sa), &tmA, kc * BK, m0, &full[s]);
-        tma_load_2d(smem_u32(sa + A_BYTES), pass ? &tmB1 : &tmB0, bx0 + kc * BK, n0, &full[s]);
-        issued = i + 1;
       }
-      // drain: the last use of every stage must have landed before the CTA may exit
-      const uint64_t drain_ns = 100000000ull;
-      for (int i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i) {
-        const int s = i % STAGES;
-        if (!mbar_wait(&full[s], (uint32_t)(i / STAGES) & 1u, drain_ns)) latch_status(p.status, PIFA_ERR_TIMEOUT);
-      }
+      // nothing may land in shared memory after the CTA has left: the leader waits for both CTAs'
+      // copies, and the cluster barrier at the end holds the other CTA until it has
+      for (int i = it > p.stages ? it - p.stages : 0; leader && is_a && i < it; ++i)
+        if (!mbar_wait(&full[i % p.stages], (uint32_t)(i / p.stages) & 1u, 100000000ull))
+          latch_status(p.status, PIFA_ERR_TIMEOUT);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      for (int i = 0; i < total; ++i) {
-        const int s = i % STAGES;
-        const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-        if (!mbar_wait(&full[s], ph, p.timeout_ns)) {
-          *abort_flag = 1;
-          latch_status(p.status, PIFA_ERR_TIMEOUT);
+    if (lane == 0 && leader) {
+      // ---------------- MMA issuer (the leader's, for both CTAs) ----------------
+      int n = 0, s = 0;
+      uint32_t ph = 0;
+      bool dead = false;
+      // descriptors count 16-byte units
+      const uint64_t a0 = sw128_desc(smem_u32(smem)), b0 = sw128_desc(smem_u32(smem) + (uint32_t)p.subs * A_BYTES);
+      const uint32_t step = p.stage_bytes / 16, boxb = (uint32_t)(kPair ? p.bn / 2 : p.bn) * 8u;
+      auto commit = [](uint64_t* bar) {
+        if (kPair) mma_commit_pair(bar);
+        else mma_commit(bar);
+      };
+      for (int idx = first; idx < p.tiles && !dead; idx += stride, ++n) {
+        const int buf = n & 1;
+        const uint32_t acc = tmem + (uint32_t)(buf * BNMAX);
+        const uint32_t pe = (uint32_t)((n >> 1) - 1) & 1u;
+        if (n >= 2 && !(kPair ? mbar_wait_cluster(&acce[buf], pe, p.timeout_ns) : mbar_wait(&acce[buf], pe, p.timeout_ns))) {
+          dead = true;
           break;
         }
         tc_fence_after();
-        const uint32_t a = smem_u32(smem + s * STAGE_BYTES);
-        const uint32_t b = a + A_BYTES;
+        int kc = (i0 % p.ksteps) * p.subs;
+        for (int i = 0; i < total; ++i) {
+          if (!mbar_wait(&full[s], ph, p.timeout_ns)) {
+            dead = true;
+            break;
+          }
+          tc_fence_after();
+          uint64_t a = a0 + (uint32_t)s * step, b = b0 + (uint32_t)s * step;
+          const int n64 = p.subs == 2 && kc + 1 < p.kchunks ? 2 : 1;
+          for (int u = 0; u < n64; ++u, a += A_BYTES / 16, b += boxb) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          mma_bf16_ss(tmem, sw128_desc(a + kk * 32), sw128_desc(b + kk * 32), p.idesc, (i > 0 || kk > 0) ? 1u : 0u);
-        mma_commit(&empty[s]);
+            for (uint32_t kk = 0; kk < BK / 16; ++kk) {
+              const uint32_t on = (i > 0 || u > 0 || kk > 0) ? 1u : 0u;
+              if (kPair) mma_bf16_ss_pair(acc, a + kk * 2u, b + kk * 2u, p.idesc, on);
+              else mma_bf16_ss(acc, a + kk * 2u, b + kk * 2u, p.idesc, on);
+            }
+          }
+          kc += p.subs;
+          if (kc >= p.kchunks) kc = 0;
+          commit(&empty[s]);
+          if (++s == p.stages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+        if (!dead) commit(&accf[buf]);
       }
-      mma_commit(acc_full);  // arrives once every MMA issued above has completed
-      // the CTA frees TMEM only after its MMAs are done, even if the epilogue gave up waiting
-      if (!mbar_wait(acc_full, 0, 100000000ull)) latch_status(p.status, PIFA_ERR_TIMEOUT);
+      if (dead) latch_status(p.status, PIFA_ERR_TIMEOUT);
+      commit(drain);  // every MMA has completed before the tensor memory is freed
+      if (!mbar_wait(drain, 0, 100000000ull)) latch_status(p.status, PIFA_ERR_TIMEOUT);
     }
   } else {
-    // ---------------- epilogue: warps 2 .. 2 + EPI_WARPS - 1 ----------------
-    // Warp w may access TMEM lanes 32 (w % 4) .. + 31, one quarter of the tile's weight rows; the
-    // EPI_WARPS / 4 warps of a quarter split the tile's tokens. Many warps keep the store issue
-    // rate up: the scattered 2-byte stores into Y's columns are instruction-bound.
-    constexpr int kSlices = EPI_WARPS / 4;
-    constexpr int kChunks = (BN / 32 + kSlices - 1) / kSlices;  // 32-token chunks per warp (the last ones may lie beyond bn)
-    const int tend = min(n0 + p.bn, p.N);       // this tile's tokens end here
-    const int q = warp & 3;
-    const int slice = (warp - 2) >> 2;
-    const int row = m0 + q * 32 + lane;
-    // Y_p's hi and lo planes are written transposed through this warp's 4 KB of the stage memory
-    // (free once every MMA has completed) as 16-byte stores of 8 consecutive weight rows.
-    uint16_t* st_hi = reinterpret_cast<uint16_t*>(smem) + (warp - 2) * 2048;
-    uint16_t* st_lo = st_hi + 1024;
-    const bool ok = mbar_wait(acc_full, 0, p.timeout_ns);
-    if (!ok) latch_status(p.status, PIFA_ERR_TIMEOUT);
-    tc_fence_after();
-    if (kCl) {
-      // this K-slice's partial tile into the ring as [token][128 rows] fp32 (the lanes of a
-      // warp on consecutive rows): the cluster adds the slices below
-      if (ok && !*abort_flag) {
-        fence_proxy_async_smem();  // the ring's last operands were read by the MMAs (async proxy)
-        float* red = reinterpret_cast<float*>(smem);
-        const int tend = min(n0 + p.bn, p.N);
-#pragma unroll 1
-        for (int ci = 0; ci < kChunks; ++ci) {
-          const int tb = n0 + (slice * kChunks + ci) * 32;
-          if (tb >= tend) break;  // warp-uniform
-          uint32_t v[32];
-          tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(tb - n0), v);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) red[(tb - n0 + j) * BM + q * 32 + lane] = __uint_as_float(v[j]);
-        }
-      }
-    } else if (ok && !*abort_flag) {
+    // ---------------- epilogue: warps 2..9, TMEM lane quarter warp % 4 ----------------
+    // Warp w may access TMEM lanes 32 (w % 4) .. + 31, one quarter of the CTA's weight rows; the two
+    // warps of a quarter take the tile's blocks of 32 tokens in turn.
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
+    bool range_err = false;
+    int n = 0;
+    for (int idx = first; idx < p.tiles; idx += stride, ++n) {
+      int m0, mend, n0, bx0;
+      place(idx, m0, mend, n0, bx0);
+      const int buf = n & 1, ntok = min(p.bn, p.N - n0);
+      const int row = m0 + q4 * 32 + lane;
       int col = -1;
-      if (row < p.M) {
-        col = p.cols[row];
+      if (!kCl && row < mend) {
+        col = __ldg(p.cols + row);
         if ((unsigned)col >= (unsigned)p.m) {
           latch_status(p.status, PIFA_ERR_DEVICE_INDEX);
           col = -1;
         }
       }
-      bool range_err = false;
-#pragma unroll 1
-      for (int ci = 0; ci < kChunks; ++ci) {
-        const int tb = n0 + (slice * kChunks + ci) * 32;  // first token of the chunk
-        if (tb >= tend) break;  // warp-uniform; TMEM columns beyond bn hold no result
+      if (!__all_sync(0xffffffffu, mbar_wait(&accf[buf], (uint32_t)(n >> 1) & 1u, p.timeout_ns))) {
+        latch_status(p.status, PIFA_ERR_TIMEOUT);
+        break;
+      }
+      tc_fence_after();
+      if (kCl) fence_proxy_async_smem();  // the ring's last operands were read by the MMAs (async proxy)
+      for (int c0 = half * 32; c0 < ntok; c0 += 64) {
         uint32_t v[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(tb - n0), v);
+        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(buf * BNMAX + c0), v);
         tmem_ld_wait();
+        if (kCl) {
+          // this K-slice's partial tile into the ring as [token][128 rows] fp32 (the lanes of a
+          // warp on consecutive rows): the cluster adds the slices below
+          float* red = reinterpret_cast<float*>(smem) + c0 * BM + q4 * 32 + lane;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float f = __uint_as_float(v[j]);
-          if (col >= 0 && tb + j < tend) p.Y[(int64_t)(tb + j) * p.ldy + col] = __float2bfloat16_rn(f);
-          if (kEpi == EPI_SPLIT_BF16) {
-            const bf16 h = __float2bfloat16_rn(f);
-            st_hi[j * 32 + lane] = __bfloat16_as_ushort(h);
-            st_lo[j * 32 + lane] = __bfloat16_as_ushort(__float2bfloat16_rn(f - __bfloat162float(h)));
-          } else if (kEpi == EPI_SPLIT_F16) {
-            float fs = f;
-            if (fabsf(fs) > 65504.0f) {
-              range_err = true;
-              fs = copysignf(65504.0f, fs);
-            }
-            const __half hh = __float2half_rn(fs);
-            st_hi[j * 32 + lane] = __half_as_ushort(hh);
-            st_lo[j * 32 + lane] = __half_as_ushort(__float2half_rn(fs - __half2float(hh)));
-          }
+          for (int j = 0; j < 32; ++j) red[j * BM] = __uint_as_float(v[j]);
+          continue;
         }
-        if (kEpi != EPI_Y_ONLY) {
-          __syncwarp();
-          // 128 chunks of 16 bytes per plane: token j = c / 4, weight rows 8 (c % 4) .. + 7
+        bf16* y = p.Y + (int64_t)(n0 + c0) * p.ldy + col;
+        const int nj = ntok - c0;
+        // planes: lanes l and l ^ 1 exchange halves, so that a 4-byte store holds two neighbouring rows
+        // of one token (even lanes token j, odd lanes j + 1): 64 contiguous bytes per 16 lanes
+        const bool odd = lane & 1;
+        const int64_t po = (int64_t)(n0 + c0 + (odd ? 1 : 0)) * p.ldyp + (row & ~1);
+        const bool pin = kEpi != EPI_Y_ONLY && (row & ~1) < p.ldyp;  // rows beyond M hold zeros (padding columns)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int c = lane + 32 * k;
-            const int t = tb + (c >> 2);
-            const int rr = m0 + q * 32 + (c & 3) * 8;  // rows beyond M hold zeros (padding columns)
-            if (t < tend && rr < p.ldyp) {
-              *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(p.yp_hi) + (int64_t)t * p.ldyp + rr) =
-                  *reinterpret_cast<const uint4*>(st_hi + c * 8);
-              *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(p.yp_lo) + (int64_t)t * p.ldyp + rr) =
-                  *reinterpret_cast<const uint4*>(st_lo + c * 8);
+        for (int j = 0; j < 32; j += 2) {
+          const float f0 = __uint_as_float(v[j]), f1 = __uint_as_float(v[j + 1]);
+          if (col >= 0 && j < nj) y[(int64_t)j * p.ldy] = __float2bfloat16_rn(f0);
+          if (col >= 0 && j + 1 < nj) y[(int64_t)(j + 1) * p.ldy] = __float2bfloat16_rn(f1);
+          if (kEpi != EPI_Y_ONLY) {
+            uint16_t h0, l0, h1, l1;
+            split_hl<kEpi>(f0, h0, l0, range_err);
+            split_hl<kEpi>(f1, h1, l1, range_err);
+            const uint32_t h = (uint32_t)h0 | (uint32_t)h1 << 16, l = (uint32_t)l0 | (uint32_t)l1 << 16;
+            const uint32_t xh = __shfl_xor_sync(0xffffffffu, h, 1), xl = __shfl_xor_sync(0xffffffffu, l, 1);
+            if (pin && j + (odd ? 1 : 0) < nj) {
+              const int64_t o = po + (int64_t)j * p.ldyp;
+              *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(p.yp_hi) + o) =
+                  odd ? __byte_perm(xh, h, 0x7632) : __byte_perm(h, xh, 0x5410);
+              *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(p.yp_lo) + o) =
+                  odd ? __byte_perm(xl, l, 0x7632) : __byte_perm(l, xl, 0x5410);
             }
           }
-          __syncwarp();  // the next chunk reuses the staging
         }
       }
-      if (range_err) latch_status(p.status, PIFA_ERR_RANGE);
+      if (kCl) break;  // one tile per cluster
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {  // this warp has read its share of the accumulator
+        if (kPair) mbar_arrive_remote(mapa_shared(smem_u32(&acce[buf]), 0));
+        else mbar_arrive(&acce[buf]);
+      }
     }
+    if (range_err) latch_status(p.status, PIFA_ERR_RANGE);
   }
 
+  // Every wait above is bounded, so every thread of every CTA gets here: no CTA frees its tensor
+  // memory or leaves while the pair's MMAs, copies or arrivals may still reach it, and with kCl every
+  // CTA of the cluster has its partial tile in its own shared memory.
   tc_fence_before();
   __syncthreads();
+  if (kPair || kCl) cluster_sync_all();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, TMEM_COLS);
+    if (kPair) tmem_dealloc_pair(tmem, TMEM_COLS);
+    else tmem_dealloc(tmem, TMEM_COLS);
   }
   if (kCl) {
-    // Every CTA of the cluster has its partial tile in its own shared memory once all arrive (every
-    // wait above is bounded, so each CTA gets here); CTA z then finishes rows [z rpc, (z + 1) rpc)
-    // of the tile for all its tokens, adding the slices in rank order (deterministic), and a
-    // second barrier keeps each CTA resident until no peer reads its shared memory any more.
-    cluster_sync_all();
-    const int rpc = BM / p.ks;
+    // CTA z finishes rows [z rpc, (z + 1) rpc) of the tile for all its tokens: four rows of a token
+    // per thread and step, every slice's loads in flight at once, added in rank order
+    // (deterministic). A second barrier keeps each CTA resident until no peer reads its shared
+    // memory any more.
+    int m0, mend, n0, bx0;
+    place(first, m0, mend, n0, bx0);
+    const int rpc = BM / p.ks, q = rpc / 4;  // rows, and groups of four, of this CTA
     const int ntok = min(p.bn, p.N - n0);
     const uint32_t red = smem_u32(smem);
     bool range_err = false;
-    for (int idx = threadIdx.x; idx < rpc * ntok; idx += PC<CFG>::THREADS) {
-      const int t = idx / rpc, rr = z * rpc + idx % rpc;
-      const int row = m0 + rr;
+    for (int i = threadIdx.x; i < q * ntok; i += THREADS) {
+      const int t = i / q, rr = z * rpc + (i - t * q) * 4;
       const uint32_t off = red + (uint32_t)(t * BM + rr) * 4u;
-      float f = 0.0f;
-      for (int k = 0; k < p.ks; ++k) f += ld_dsmem_f32(mapa_shared(off, (uint32_t)k));
-      if (row >= p.M) continue;
-      const int tok = n0 + t;
-      const int col = __ldg(p.cols + row);
-      if ((unsigned)col >= (unsigned)p.m)
-        latch_status(p.status, PIFA_ERR_DEVICE_INDEX);
-      else
-        p.Y[(int64_t)tok * p.ldy + col] = __float2bfloat16_rn(f);
-      if (kEpi == EPI_SPLIT_BF16) {
-        const bf16 h = __float2bfloat16_rn(f);
-        reinterpret_cast<uint16_t*>(p.yp_hi)[(int64_t)tok * p.ldyp + row] = __bfloat16_as_ushort(h);
-        reinterpret_cast<uint16_t*>(p.yp_lo)[(int64_t)tok * p.ldyp + row] =
-            __bfloat16_as_ushort(__float2bfloat16_rn(f - __bfloat162float(h)));
-      } else if (kEpi == EPI_SPLIT_F16) {
-        float fs = f;
-        if (fabsf(fs) > 65504.0f) {
-          range_err = true;
-          fs = copysignf(65504.0f, fs);
+      float4 a[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k < p.ks) a[k] = ld_dsmem_f32x4(mapa_shared(off, (uint32_t)k));
+      float f[4] = {a[0].x, a[0].y, a[0].z, a[0].w};
+#pragma unroll
+      for (int k = 1; k < 4; ++k)
+        if (k < p.ks) {
+          f[0] += a[k].x;
+          f[1] += a[k].y;
+          f[2] += a[k].z;
+          f[3] += a[k].w;
         }
-        const __half hh = __float2half_rn(fs);
-        reinterpret_cast<uint16_t*>(p.yp_hi)[(int64_t)tok * p.ldyp + row] = __half_as_ushort(hh);
-        reinterpret_cast<uint16_t*>(p.yp_lo)[(int64_t)tok * p.ldyp + row] =
-            __half_as_ushort(__float2half_rn(fs - __half2float(hh)));
+      const int tok = n0 + t, row = m0 + rr;
+      uint16_t h[4], l[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (kEpi != EPI_Y_ONLY) split_hl<kEpi>(f[j], h[j], l[j], range_err);
+        if (row + j >= mend) continue;
+        const int col = __ldg(p.cols + row + j);
+        if ((unsigned)col >= (unsigned)p.m)
+          latch_status(p.status, PIFA_ERR_DEVICE_INDEX);
+        else
+          p.Y[(int64_t)tok * p.ldy + col] = __float2bfloat16_rn(f[j]);
+      }
+      if (kEpi != EPI_Y_ONLY && row < p.ldyp) {  // rows beyond M hold zeros (padding columns)
+        const int64_t o = (int64_t)tok * p.ldyp + row;
+        *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(p.yp_hi) + o) =
+            make_uint2((uint32_t)h[0] | (uint32_t)h[1] << 16, (uint32_t)h[2] | (uint32_t)h[3] << 16);
+        *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(p.yp_lo) + o) =
+            make_uint2((uint32_t)l[0] | (uint32_t)l[1] << 16, (uint32_t)l[2] | (uint32_t)l[3] << 16);
       }
     }
     if (range_err) latch_status(p.status, PIFA_ERR_RANGE);
@@ -358,118 +424,144 @@ __global__ void __launch_bounds__(PC<CFG>::THREADS, PC<CFG>::CTAS)
   }
 }
 
-template <int CFG>
-int run_gemm(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmArgs& args,
-             cudaStream_t stream) {
-  const bool cl = CFG == 0 && args.ks > 1;  // split-K clusters: config 0 only (one CTA per SM)
-  auto kern = cl ? (epi == EPI_SPLIT_BF16 ? pifa_umma_gemm<EPI_SPLIT_BF16, CFG, CFG == 0>
-                    : epi == EPI_SPLIT_F16 ? pifa_umma_gemm<EPI_SPLIT_F16, CFG, CFG == 0>
-                                          : pifa_umma_gemm<EPI_Y_ONLY, CFG, CFG == 0>)
-                 : (epi == EPI_SPLIT_BF16 ? pifa_umma_gemm<EPI_SPLIT_BF16, CFG, false>
-                    : epi == EPI_SPLIT_F16 ? pifa_umma_gemm<EPI_SPLIT_F16, CFG, false>
-                                          : pifa_umma_gemm<EPI_Y_ONLY, CFG, false>);
-  if (args.ks > 1 && !cl) return pifa_fail(PIFA_ERR_UNSUPPORTED, "prefill: split-K needs the one-CTA shape");
-  if (cl && (size_t)args.bn * BM * 4 > (size_t)PC<CFG>::B::STAGES * PC<CFG>::STAGE_BYTES)
-    return pifa_fail(PIFA_ERR_UNSUPPORTED, "prefill: partial tile larger than the stage ring");
-  constexpr size_t SMEM_BYTES = PC<CFG>::SMEM_BYTES;
+using Kern = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+
+// How a GEMM is tiled: by pairs of CTAs (256 weight rows) or by one CTA (128), tokens per tile, and
+// K-slices per tile (one-CTA tiles only: the CTAs of a cluster).
+struct GemmShape {
+  bool pair;
+  int bn, ks;
+};
+
+Kern kernel_of(int epi, const GemmShape& sh) {
+  static const Kern k[3][3] = {
+      {pifa_umma_gemm<EPI_Y_ONLY, false, true>, pifa_umma_gemm<EPI_Y_ONLY, false, false>, pifa_umma_gemm<EPI_Y_ONLY, true, false>},
+      {pifa_umma_gemm<EPI_SPLIT_BF16, false, true>, pifa_umma_gemm<EPI_SPLIT_BF16, false, false>,
+       pifa_umma_gemm<EPI_SPLIT_BF16, true, false>},
+      {pifa_umma_gemm<EPI_SPLIT_F16, false, true>, pifa_umma_gemm<EPI_SPLIT_F16, false, false>,
+       pifa_umma_gemm<EPI_SPLIT_F16, true, false>}};
+  return k[epi][sh.pair ? 0 : sh.ks > 1 ? 2 : 1];
+}
+
+// Tiles that run at once on the current device: pairs, single CTAs, clusters of 2 and of 4.
+struct Slots {
+  int pair, one, cl[2];
+};
+const Slots& tile_slots() {
+  static const Slots slots = [] {
+    auto query = [](const GemmShape& sh) {
+      const Kern k = kernel_of(EPI_Y_ONLY, sh);
+      cudaLaunchConfig_t cfg = {};
+      const unsigned c = sh.pair ? 2u : (unsigned)sh.ks;
+      cfg.gridDim = dim3(c);
+      cfg.blockDim = dim3(THREADS);
+      cfg.dynamicSmemBytes = SMEM_BYTES;
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = c;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess ||
+          cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n < 1)
+        n = 1;
+      cudaGetLastError();  // a failed query leaves no sticky error behind
+      return n;
+    };
+    return Slots{query({true, BNMAX, 1}), query({false, BNMAX, 1}), {query({false, BNMAX, 2}), query({false, BNMAX, 4})}};
+  }();
+  return slots;
+}
+
+// Bytes of one 64-column chunk of a tile in a CTA's ring, and chunks per stage: two where the ring
+// holds at least six (a barrier hand-off per 128 columns instead of per 64 takes a fifth off the step
+// of narrow tiles, but two stages in all would starve wide one-CTA ones).
+uint32_t chunk_bytes(bool pair, int bn) { return A_BYTES + (uint32_t)(pair ? bn / 2 : bn) * BK * 2; }
+int subs_for(bool pair, int bn) { return RING_BYTES / chunk_bytes(pair, bn) >= 6 ? 2 : 1; }
+
+// The tiling of G groups of `rows` weight rows x T tokens that finishes first by the measured costs, in
+// cycles: a chunk's (see the head of this file), an unhidden epilogue's 25 per token of a tile's width,
+// a launch's 9600 (a pair's 10600), a cluster's 12500 and its exchange of partial tiles 20 per token.
+GemmShape pick_shape(int64_t G, int64_t rows, int64_t T, int64_t kchunks) {
+  const Slots& slots = tile_slots();
+  GemmShape best = {true, BNMAX, 1};
+  double best_cost = -1.0;
+  for (int form = 0; form < 4; ++form) {  // pairs, single CTAs, clusters of 2, of 4
+    const bool pair = form == 0;
+    const int ks = form < 2 ? 1 : form == 2 ? 2 : 4;
+    if (ks > 1 && kchunks < 8 * ks) break;
+    const int64_t mt = G * ((rows + (pair ? PM : BM) - 1) / (pair ? PM : BM));
+    const int64_t at_once = form == 0 ? slots.pair : form == 1 ? slots.one : slots.cl[form - 2];
+    for (int bn = T < BNMAX ? (int)(T + 31) / 32 * 32 : BNMAX; bn >= 32; bn -= 32) {
+      const int64_t rounds = (mt * ((T + bn - 1) / bn) + at_once - 1) / at_once;
+      const double step = pair ? 330.0 + 0.85 * bn : subs_for(false, bn) == 2 ? 410.0 + 0.3 * bn : 480.0 + 0.66 * bn;
+      double cost = (double)rounds * (double)((kchunks + ks - 1) / ks) * step + 25.0 * bn;
+      cost += ks > 1 ? (double)rounds * (12500.0 + 20.0 * bn) : pair ? 10600.0 : 9600.0;
+      if (best_cost < 0.0 || cost < best_cost) {
+        best_cost = cost;
+        best = {pair, bn, ks};
+      }
+    }
+  }
+  return best;
+}
+
+int run_gemm(int epi, const CUtensorMap& a, const CUtensorMap& b0, const CUtensorMap& b1, const GemmArgs& g,
+             const GemmShape& sh, cudaStream_t stream) {
+  const Kern kern = kernel_of(epi, sh);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return pifa_fail_cuda("cudaFuncSetAttribute(prefill gemm)", e);
   // programmatic dependent launch: each GEMM may start (weight tiles in flight) while the previous
   // kernel of the stream drains; its dependent loads follow griddepcontrol.wait
   cudaLaunchConfig_t cfg = {};
-  // CTAs launch x-fastest. Walking token tiles first (when M > T) runs a weight-row block's tiles
-  // together, sharing its A tile, with all of B (T x K) the wave's other operand; walking row tiles
-  // first shares B tiles with all of A (M x K): the wave's working set is the smaller way round.
-  // Measured: grouped 7B MLP gate+up T = 2048 (GEMM 2 M = 17920) 377 -> 356 us token-first;
-  // attention T = 8192 (M = 2048) 239 us row-first against 259.
-  const unsigned mt = (unsigned)((args.M + BM - 1) / BM), nt = (unsigned)((args.N + args.bn - 1) / args.bn);
-  GemmArgs g = args;
-  g.tok_fast = args.M > args.N ? 1 : 0;
-  if ((g.tok_fast ? mt : nt) > 65535u) g.tok_fast ^= 1;  // gridDim.y is at most 65535
-  if ((g.tok_fast ? mt : nt) > 65535u) return pifa_fail(PIFA_ERR_UNSUPPORTED, "more than 65535 tiles along both M and T");
-  g.ks = cl ? args.ks : 1;
-  cfg.gridDim = g.tok_fast ? dim3(nt, mt, (unsigned)g.ks) : dim3(mt, nt, (unsigned)g.ks);
-  cfg.blockDim = dim3(PC<CFG>::THREADS);
+  const unsigned per = sh.pair ? 2u : (unsigned)sh.ks;  // CTAs per tile: a cluster
+  const int at_once = sh.pair ? tile_slots().pair : sh.ks > 1 ? g.tiles : tile_slots().one;
+  cfg.gridDim = dim3(per * (unsigned)(g.tiles < at_once ? g.tiles : at_once));
+  cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;  // a tile's K-slices: consecutive along z
-  attr[1].val.clusterDim.x = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = per;
   attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = (unsigned)g.ks;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = cl ? 2 : 1;
+  cfg.numAttrs = 2;
   e = pifa_launch_ex(&cfg, kern, a, b0, b1, g);
   if (e != cudaSuccess) return pifa_fail_cuda("prefill gemm launch", e);
   return PIFA_OK;
 }
 
+// Fills the tiling of an M x T GEMM (G groups of rows) into `g`.
+int set_tiling(GemmArgs& g, int64_t G, int64_t M, int64_t T, const GemmShape& sh) {
+  g.M = (int)M;
+  g.N = (int)T;
+  g.bn = sh.bn;
+  g.ks = sh.ks;
+  g.gsz = (int)(M / G);
+  const int tm = sh.pair ? PM : BM;
+  g.mtg = (g.gsz + tm - 1) / tm;
+  g.mt = (int)G * g.mtg;
+  g.nt = (int)((T + sh.bn - 1) / sh.bn);
+  if ((int64_t)g.mt * g.nt * 4 >= ((int64_t)1 << 31))
+    return pifa_fail(PIFA_ERR_UNSUPPORTED, "prefill: more than 2^30 tiles");
+  g.tiles = g.mt * g.nt;
+  g.subs = subs_for(sh.pair, sh.bn);
+  g.ksteps = (g.kchunks + g.subs - 1) / g.subs;
+  g.stage_bytes = (uint32_t)g.subs * chunk_bytes(sh.pair, sh.bn);
+  g.stages = (int)(RING_BYTES / g.stage_bytes);
+  if (g.stages > MAX_STAGES) g.stages = MAX_STAGES;
+  // Walking token tiles first (when M > T) runs a weight-row block's tiles together, sharing its A
+  // tile, with all of B (T x K) the round's other operand; walking row tiles first shares B tiles
+  // with all of A (M x K): the round's working set is the smaller way round.
+  g.tok_fast = M > T ? 1 : 0;
+  return PIFA_OK;
+}
+
 inline int64_t pad8(int64_t v) { return (v + 7) / 8 * 8; }
-
-// Tokens per tile for an M x T GEMM: the multiple of 16 (16..256) minimising the slowest SM's time,
-// waves x (tile time); ties to the larger bn. The tile time is the measured fit on the 4096 x 4096,
-// r = 2048 layer (T = 8192: 4 waves of 256-token tiles 254 us, 6 waves of 144-token tiles 320 us):
-// t(bn) ~ t0 (432 + bn), most of a tile's time not shrinking with its width. There T = 2048 takes
-// 240 (144 tiles, one wave of 152 SMs, where 256 leaves 24 SMs idle: 58.3 -> 57.3 us) and
-// T = 8192 224 (254.4 -> 242.8 us).
-int sm_count_prefill() {
-  int sms = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      sms < 1)
-    sms = 1;
-  return sms;
-}
-
-// The kernel shape and token-tile width of one GEMM: config 0 with pick_bn's width unless that
-// takes three or more waves, then config 1 (CTA slots = 2 per SM) with its own width.
-struct GemmShape {
-  int cfg, bn, ks;  // kernel shape, tokens per tile, K-slices per tile (a cluster when > 1)
-};
-int pick_bn_slots(int64_t M, int64_t T, int bnmax, int64_t slots) {
-  const int64_t mt = (M + BM - 1) / BM;
-  int best = bnmax;
-  int64_t best_cost = -1;
-  for (int bn = bnmax; bn >= 16; bn -= 16) {
-    const int64_t tiles = mt * ((T + bn - 1) / bn);
-    const int64_t cost = (tiles + slots - 1) / slots * (432 + bn);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = bn;
-    }
-  }
-  return best;
-}
-// Split-K: when the GEMM's full-width tiles (256 tokens, or all of T) fill at most half the SMs and
-// the one-wave plan would otherwise fall back to tiles of 64 tokens or fewer, each full-width tile
-// gets ks CTAs (2 or 4, keeping one CTA per SM, every K-slice at least 16 steps of 64) as a
-// cluster that adds its partial tiles in shared memory. Measured against the narrow-tile plan (us,
-// one process, interleaved): 7B attention T = 256 44.5 -> 34.8, T = 512 47.3 -> 37.0; 7B MLP down
-// T = 256 76.7 -> 43.5, T = 512 80.4 -> 46.7; 7B MLP gate T = 256 46.6 -> 42.7; 70B q/o T = 256
-// 88.9 -> 53.0; 70B gate/up T = 256 159.4 -> 142.8; 4096 x 4096, r = 1024, T = 512 36.4 -> 32.3.
-// Splitting also where the plan keeps tiles of 96-128 tokens lost (r = 1024, T = 2048: 55.4 ->
-// 59.0), as did clusters of 8 (8 K-steps per slice: 7B attention T = 256 44.5 -> 49.2).
-GemmShape pick_shape(int64_t M, int64_t T, int64_t ksteps) {
-  const int64_t sms = sm_count_prefill();
-  const int64_t mt = (M + BM - 1) / BM;
-  const int bnw = (int)(T >= PC<0>::BN ? PC<0>::BN : (T + 15) / 16 * 16);
-  const int64_t tiles_w = mt * ((T + bnw - 1) / bnw);
-  const int bn0 = pick_bn_slots(M, T, PC<0>::BN, sms);
-  if (tiles_w * 2 <= sms && bn0 <= 64) {
-    int ks = 1;
-    while (ks < 4 && tiles_w * ks * 2 <= sms && ksteps / (ks * 2) >= 16) ks *= 2;
-    if (ks > 1) return {0, bnw, ks};
-  }
-  const int64_t waves0 = (mt * ((T + bn0 - 1) / bn0) + sms - 1) / sms;
-  if (waves0 < 3) return {0, bn0, 1};
-  return {1, pick_bn_slots(M, T, PC<1>::BN, 2 * sms), 1};
-}
-
-template <typename... A>
-int run_gemm_cfg(int cfg, A&&... args) {
-  return cfg == 0 ? run_gemm<0>(std::forward<A>(args)...) : run_gemm<1>(std::forward<A>(args)...);
-}
 
 }  // namespace
 
@@ -489,18 +581,15 @@ int launch_prefill_split(const PifaShape& s, const PifaPointers& p, int* status,
 
   CUtensorMap tWp, tX, tC, tHi, tLo;
   int st;
-  const GemmShape sh1 = pick_shape(G * s.r, s.T, (s.n + BK - 1) / BK);
-  const int bn1 = sh1.bn;
-  if ((st = make_tmap_2d(&tWp, PIFA_DTYPE_BF16, p.Wp, G * s.r, s.n, s.ldwp, BK, BM)) != PIFA_OK) return st;
-  if ((st = make_tmap_2d(&tX, PIFA_DTYPE_BF16, p.X, s.T, s.n, s.ldx, BK, bn1)) != PIFA_OK) return st;
-
   GemmArgs g1 = {};
-  g1.idesc = idesc_bf16_f32(BM, bn1);
-  g1.M = (int)(G * s.r);
-  g1.N = (int)s.T;
-  g1.bn = bn1;
   g1.kchunks = (int)((s.n + BK - 1) / BK);
   g1.passes = 1;
+  const GemmShape sh1 = pick_shape(1, G * s.r, s.T, g1.kchunks);
+  const uint32_t box1 = (uint32_t)(sh1.pair ? sh1.bn / 2 : sh1.bn);
+  if ((st = set_tiling(g1, 1, G * s.r, s.T, sh1)) != PIFA_OK) return st;
+  if ((st = make_tmap_2d(&tWp, PIFA_DTYPE_BF16, p.Wp, G * s.r, s.n, s.ldwp, BK, BM)) != PIFA_OK) return st;
+  if ((st = make_tmap_2d(&tX, PIFA_DTYPE_BF16, p.X, s.T, s.n, s.ldx, BK, box1)) != PIFA_OK) return st;
+  g1.idesc = idesc_bf16_f32(sh1.pair ? PM : BM, (uint32_t)sh1.bn);
   g1.cols = p.piv;
   g1.m = (int)(G * s.m);
   g1.Y = reinterpret_cast<bf16*>(p.Y);
@@ -510,29 +599,24 @@ int launch_prefill_split(const PifaShape& s, const PifaPointers& p, int* status,
   g1.ldyp = ldyp;
   g1.status = status;
   g1.timeout_ns = timeout_ns;
-  g1.ks = sh1.ks;
-  if ((st = run_gemm_cfg(sh1.cfg, f16 ? EPI_SPLIT_F16 : EPI_SPLIT_BF16, tWp, tX, tX, g1, stream)) != PIFA_OK) return st;
+  if ((st = run_gemm(f16 ? EPI_SPLIT_F16 : EPI_SPLIT_BF16, tWp, tX, tX, g1, sh1, stream)) != PIFA_OK) return st;
   if (s.m == s.r) return PIFA_OK;
 
-  const GemmShape sh2 = pick_shape(G * (s.m - s.r), s.T, 2 * ((s.r + BK - 1) / BK));
-  const int bn2 = sh2.bn;
-  if ((st = make_tmap_2d(&tC, s.c_dtype, p.C, G * (s.m - s.r), s.r, s.ldc, BK, BM)) != PIFA_OK) return st;
-  if ((st = make_tmap_2d(&tHi, s.c_dtype, hi, s.T, G * s.r, ldyp, BK, bn2)) != PIFA_OK) return st;
-  if ((st = make_tmap_2d(&tLo, s.c_dtype, lo, s.T, G * s.r, ldyp, BK, bn2)) != PIFA_OK) return st;
   GemmArgs g2 = g1;
-  g2.bn = bn2;
-  g2.idesc = f16 ? idesc_f16_f32(BM, bn2) : idesc_bf16_f32(BM, bn2);
-  g2.M = (int)(G * (s.m - s.r));
-  if (G > 1) {  // group g's non-pivot rows (whole tiles) read the hi/lo columns [g r, (g + 1) r)
-    g2.gsz = (int)(s.m - s.r);
-    g2.goff = (int)s.r;
-  }
   g2.kchunks = (int)((s.r + BK - 1) / BK);
   g2.passes = 2;
-  g2.ks = sh2.ks;
+  const int64_t M2 = G * (s.m - s.r);
+  const GemmShape sh2 = pick_shape(G, s.m - s.r, s.T, 2 * g2.kchunks);
+  const uint32_t box2 = (uint32_t)(sh2.pair ? sh2.bn / 2 : sh2.bn), tm2 = sh2.pair ? PM : BM;
+  // group g's non-pivot rows (no tile spans two groups) read the hi/lo columns [g r, (g + 1) r)
+  if ((st = set_tiling(g2, G, M2, s.T, sh2)) != PIFA_OK) return st;
+  g2.goff = G > 1 ? (int)s.r : 0;
+  if ((st = make_tmap_2d(&tC, s.c_dtype, p.C, M2, s.r, s.ldc, BK, BM)) != PIFA_OK) return st;
+  if ((st = make_tmap_2d(&tHi, s.c_dtype, hi, s.T, G * s.r, ldyp, BK, box2)) != PIFA_OK) return st;
+  if ((st = make_tmap_2d(&tLo, s.c_dtype, lo, s.T, G * s.r, ldyp, BK, box2)) != PIFA_OK) return st;
+  g2.idesc = f16 ? idesc_f16_f32(tm2, (uint32_t)sh2.bn) : idesc_bf16_f32(tm2, (uint32_t)sh2.bn);
   g2.cols = p.nonpiv;
   g2.yp_hi = nullptr;
   g2.yp_lo = nullptr;
-  return run_gemm_cfg(sh2.cfg, EPI_Y_ONLY, tC, tHi, tLo, g2, stream);
+  return run_gemm(EPI_Y_ONLY, tC, tHi, tLo, g2, sh2, stream);
 }
-

@@ -144,6 +144,14 @@ __device__ __forceinline__ float ld_dsmem_f32(uint32_t cluster_saddr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_saddr) : "memory");
   return v;
 }
+__device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t cluster_saddr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_saddr)
+               : "memory");
+  return v;
+}
 // 128-bit load from this CTA's shared memory at a 32-bit shared-window address.
 __device__ __forceinline__ uint4 lds128(uint32_t saddr) {
   uint4 v;

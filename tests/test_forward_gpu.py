@@ -741,3 +741,24 @@ def test_prefill_split_k_clusters_ragged_and_deterministic():
     parity(L, 200, P.PIFA_VARIANT_PREFILL_SPLIT)
     X = acts(200, 2000, 9)
     assert np.array_equal(run(L, X, P.PIFA_VARIANT_PREFILL_SPLIT), run(L, X, P.PIFA_VARIANT_PREFILL_SPLIT))
+
+
+@pytest.mark.parametrize("m,n,r,T,c", [
+    (2500, 1000, 900, 6000, "bf16"),   # pairs of CTAs, several rounds of tiles, ragged rows and tokens
+    (1400, 833, 517, 3001, "fp16"),   # the same with an odd number of K chunks and fp16 planes
+    (4096, 1000, 300, 70, "bf16"),    # one-CTA tiles, clusters of 4
+    (2304, 2000, 1100, 700, "fp16"),  # clusters of 2 and single tiles
+    (600, 330, 200, 513, "bf16"),     # single one-CTA tiles
+])
+def test_prefill_tilings_ragged(m, n, r, T, c):
+    """Every tiling of the prefill GEMMs at ragged sizes, and the same bits from call to call."""
+    L = layer_for(m, n, r, 6, "synthetic", c)
+    parity(L, T, P.PIFA_VARIANT_PREFILL_SPLIT, sample=96 if T > 1000 else None)
+    X = acts(T, n, 3)
+    assert np.array_equal(run(L, X, P.PIFA_VARIANT_PREFILL_SPLIT), run(L, X, P.PIFA_VARIANT_PREFILL_SPLIT))
+
+
+@pytest.mark.parametrize("T", [200, 5000])
+def test_grouped_prefill_groups_end_inside_a_pair_tile(T):
+    """384 non-pivot rows per group: one and a half 256-row tiles, of which none may span two groups."""
+    grouped_parity([layer_for(1152, 840, 768, s, "synthetic") for s in (7, 8, 9)], T, sample=64)
