@@ -300,7 +300,7 @@ int64_t pifa_backward_workspace_size(int64_t T, int64_t m, int64_t n, int64_t r)
  *                that straddle the diagonal are accumulated too and the rest are left as they were.
  *   YtXt         DEVICE in/out, fp32, m x n, pitch ldyx >= n (NULL: only XXt is accumulated).
  *   workspace    DEVICE scratch of pifa_m_accumulate_workspace_size(T, m, n) bytes, 256-byte
- *                aligned (X_u^T, the mixed input and Y_t^T in bf16).
+ *                aligned (the mixed input and Y_t^T in bf16).
  *   Numerics: bf16 operands, fp32 accumulation; the mixed input and Y_t pass as hi + lo bf16 pairs.
  *   T == 0 is a no-op. Asynchronous on cuda_stream (ordering and capture as pifa_backward).
  */
@@ -367,7 +367,7 @@ int pifa_set_wait_timeout(int64_t ns);
  * grid of co-resident clusters that stream their tiles through a ring of TMA-filled stages; and
  * split-K on the tensor cores. The latter gives a phase of at most two 128-row blocks per SM 1, 2,
  * 4 or 8 CTAs per row block, each one K-slice of it, as a thread-block cluster that adds up its
- * slices in shared memory in rank order and writes the outputs itself (one kernel); a taller
+ * slices in shared memory in a fixed order and writes the outputs itself (one kernel); a taller
  * phase deals equal ranges of 128 x 64 weight tiles to a persistent grid and a second kernel sums
  * the fp32 partial sums in a fixed order.
  * PIFA_DECODE_GRID_AUTO (0, the default) picks per phase from its shape and T: split-K when

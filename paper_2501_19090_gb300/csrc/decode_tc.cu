@@ -12,12 +12,13 @@
 // the largest multiple of 64 that keeps a unit no longer than a CTA's range, so a unit is split
 // between at most two CTAs: its head (chunk 0 on) goes to P, its tail (if split) to P2.
 //
-// Partial kernel (two CTAs per SM, 192 threads each):
-//   warp 0     TMA producer: per chunk, the weight tile (128 rows x 64 columns, 128-byte swizzle)
-//              and the matching 64 columns of B (a token tile of TNT = 16, 32, 64 or 128 rows per
-//              plane, the smallest that holds T; rows >= T zero-filled)
-//              into one stage of a ring; the first weight tiles go out before the dependency wait
-//              (the weights do not depend on the previous kernel), their B boxes after it.
+// Partial kernel (two CTAs per SM, 256 threads each):
+//   warp 0     TMA producer of the weights: per chunk, the weight tile (128 rows x 64 columns, 128-byte
+//              swizzle) into one stage of a ring, the first ones before the dependency wait (the
+//              weights do not depend on the previous kernel).
+//   warp 6     TMA producer of B, after the dependency wait: the matching 64 columns (a token tile of
+//              TNT = 16, 32, 64 or 128 rows per plane, the smallest that holds T; rows >= T
+//              zero-filled) into the same stage.
 //   warp 1     owns 256 TMEM columns (two segments in flight) and issues tcgen05.mma.kind::f16
 //              M = 128, K = 16, N = TNT (one B plane) or 2 TNT (the y_p hi and lo planes as one
 //              operand) from one thread, dealing a segment's MMAs round-robin over independent
@@ -36,8 +37,15 @@
 // cs = 1 the epilogue's sums are the outputs. With cs > 1 the block's CTAs form a thread-block
 // cluster: each stores its slice's sums in its own shared memory (the stage ring, free once its
 // MMAs are done), and after a cluster barrier CTA k reads rows [k 128 / cs, (k + 1) 128 / cs) of
-// every peer's sums through distributed shared memory, adds them in rank order and writes Y and
+// every peer's sums through distributed shared memory, adds them in a fixed order and writes Y and
 // y_p's planes. One kernel per phase: no partial sums in global memory and no reduce kernel.
+// A producer per operand, issuing loops without divisions or a shared flag, the cluster's sums as
+// 16-byte loads of all peers at once from a different peer on per CTA, and their output columns read
+// at the start took 4096 x 4096 layers at r = 2458, T = 50 from 23.2 to 20.9 us a layer, 11008 x 4096 at
+// T = 32 from 21.9 to 19.1 and 28672 x 8192 at T = 16 from 55.6 to 54.1 (CUDA graphs of 2 and 3 layers).
+// A call of T = 64 on a 4096 x 4096 layer spends, per phase: 1.1 us from the dependency's release to the
+// first B box, 1.3-2.4 in the MMAs, 0.7 in storing the slice, 0.7 in the barrier, 1.6-3 in the sums, and
+// 1.8 in the second barrier and the next kernel's release.
 // Every wait is bounded (globaltimer); on timeout the CTA latches PIFA_ERR_TIMEOUT, drains what
 // it has in flight and returns.
 #include <cuda_bf16.h>
@@ -58,7 +66,7 @@ constexpr int kMaxTokensTc = 128;               // token tiles of 32, 64 and 128
 constexpr int KB = 64;                          // K per chunk: one 128-byte swizzle row
 constexpr uint32_t A_BYTES = TM * KB * 2;       // one weight tile
 constexpr int MAX_STAGES = 10;
-constexpr int THREADS = 192;
+constexpr int THREADS = 256;  // two producers, the MMA warp, four epilogue warps, one that only helps to sum
 // A segment's MMAs are dealt round-robin over NACC independent accumulators (summed in the
 // epilogue), so that consecutive MMAs do not wait for each other. With two B planes (y_p hi and
 // lo) one MMA of N = 2 TNT covers both: the lo box follows the hi box in shared memory, making one
@@ -202,9 +210,6 @@ __device__ __forceinline__ void split_hi_lo(float f, uint16_t& h, uint16_t& l, b
   }
 }
 
-// Column (within the unit's K-slice) of the c-th chunk a CTA loads for segment q.
-__device__ __forceinline__ int seg_col(const Seg& q, int c) { return (q.c0 + c) * KB; }
-
 // kCl: the row-block plan with cs > 1 (a cluster per row block); only these instantiations hold
 // cluster barriers and distributed shared-memory loads.
 template <int NB, int TNT, bool kCl>
@@ -219,7 +224,6 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   uint64_t* acce = accf + 2;
   uint64_t* drain = acce + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -244,7 +248,6 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       mbar_init(&acce[b], 4);
     }
     mbar_init(drain, 1);
-    *abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB0);
@@ -258,60 +261,64 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // kCl: the four rows of the block that this thread adds up over the cluster at the end (the same for
+  // all its tokens), and their output columns, read now: behind the sums they cost a memory round trip
+  const int rpr = kCl ? TM / a.cs : TM, rgrp = rpr / 4;
+  const int myrow = kCl ? ((int)blockIdx.x / a.cs) * TM + ((int)blockIdx.x % a.cs) * rpr + ((int)threadIdx.x % rgrp) * 4 : 0;
+  int mycol[4];
+  if (kCl) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mycol[j] = myrow + j < a.R ? __ldg(a.cols + myrow + j) : 0;
+  }
 
-  if (warp == 0) {
+  if (warp == 0 || warp == 6) {
     if (lane == 0) {
-      // ---------------- producer ----------------
-      const int total = (int)(g1 - g0);
-      const int pre = min(total, a.stages);
-      {  // weight tiles of the first stages, before the dependency wait; their B boxes follow it
-        int it = 0;
-        for (int64_t g = g0; it < pre;) {
-          const Seg q = seg_at(a, g, g1);
-          for (int c = 0; c < q.nc && it < pre; ++c, ++it) {
-            mbar_arrive_expect_tx(&full[it], a.stage_bytes);
-            tma_load_2d(smem_u32(ring + (size_t)it * a.stage_bytes), &tmA, q.s * a.ncf * KB + seg_col(q, c),
-                        q.rb * TM, &full[it]);
-          }
-          g += q.nc;
-        }
-      }
-      pdl_wait_primary();
-      int it = 0;
+      // ---------------- producers: warp 0 the weight tiles, warp 6 the B boxes ----------------
+      // The first weight tiles go out before the dependency wait, the B boxes after it. A stage's
+      // barrier takes one arrival, with the weight tile, for all its bytes.
+      const bool is_a = warp == 0;
+      if (!is_a) pdl_wait_primary();
+      int st = 0, it = 0;
+      uint32_t ph = 1;  // parity that a fresh "empty" barrier passes
       bool dead = false;
       for (int64_t g = g0; g < g1 && !dead;) {
         const Seg q = seg_at(a, g, g1);
         g += q.nc;
-        const int x0 = (a.gsz > 0 ? ((q.rb * TM) / a.gsz) * a.goff : 0) + q.s * a.ncf * KB;
+        const int k0 = q.s * a.ncf * KB + q.c0 * KB, row = q.rb * TM;
+        const int x0 = k0 + (!is_a && a.gsz > 0 ? (row / a.gsz) * a.goff : 0);
         for (int c = 0; c < q.nc; ++c, ++it) {
-          const int st = it % a.stages;
-          uint8_t* stage = ring + (size_t)st * a.stage_bytes;
-          const int kx = seg_col(q, c);
-          if (it >= pre) {
-            if (!mbar_wait(&empty[st], (uint32_t)((it / a.stages) - 1) & 1u, a.timeout_ns) || *abort_flag) {
-              latch_status(a.status, PIFA_ERR_TIMEOUT);
-              *abort_flag = 1;
-              dead = true;
-              break;
-            }
-            mbar_arrive_expect_tx(&full[st], a.stage_bytes);
-            tma_load_2d(smem_u32(stage), &tmA, q.s * a.ncf * KB + kx, q.rb * TM, &full[st]);
+          if (!mbar_wait(&empty[st], ph, a.timeout_ns)) {
+            latch_status(a.status, PIFA_ERR_TIMEOUT);
+            dead = true;
+            break;
           }
-          tma_load_2d(smem_u32(stage + A_BYTES), &tmB0, x0 + kx, 0, &full[st]);
-          if (NB > 1) tma_load_2d(smem_u32(stage + A_BYTES + (uint32_t)TNT * KB * 2), &tmB1, x0 + kx, 0, &full[st]);
+          const uint32_t stage = smem_u32(ring + (size_t)st * a.stage_bytes);
+          if (is_a) {
+            mbar_arrive_expect_tx(&full[st], a.stage_bytes);
+            tma_load_2d(stage, &tmA, x0 + c * KB, row, &full[st]);
+          } else {
+            tma_load_2d(stage + A_BYTES, &tmB0, x0 + c * KB, 0, &full[st]);
+            if (NB > 1) tma_load_2d(stage + A_BYTES + (uint32_t)TNT * KB * 2, &tmB1, x0 + c * KB, 0, &full[st]);
+          }
+          if (++st == a.stages) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
       }
-      int issued = dead ? it : total;
-      if (issued < pre) issued = pre;
       // nothing may land in shared memory once the CTA has left: the last use of every stage
-      for (int j = issued > a.stages ? issued - a.stages : 0; j < issued; ++j)
+      for (int j = it > a.stages ? it - a.stages : 0; is_a && j < it; ++j)
         if (!mbar_wait(&full[j % a.stages], (uint32_t)(j / a.stages) & 1u, 100000000ull))
           latch_status(a.status, PIFA_ERR_TIMEOUT);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // ---------------- MMA issuer ----------------
-      int it = 0, j = 0;
+      constexpr int NACC = kNacc<NB, TNT>;
+      const uint64_t a0 = sw128_desc(smem_u32(ring)), b0 = sw128_desc(smem_u32(ring) + A_BYTES);
+      const uint32_t step = a.stage_bytes / 16;  // descriptors count 16-byte units
+      int j = 0, st = 0;
+      uint32_t ph = 0;
       bool dead = false;
       for (int64_t g = g0; g < g1; ++j) {
         const Seg q = seg_at(a, g, g1);
@@ -322,34 +329,33 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           break;
         }
         tc_fence_after();
-        constexpr int NACC = kNacc<NB, TNT>;
         const uint32_t dacc = tmem + (uint32_t)(acc * NACC * TNT * NB);
         int e = 0;  // MMAs of this segment so far: accumulator e % NACC, first use overwrites
-        for (int c = 0; c < q.nc; ++c, ++it) {
-          const int st = it % a.stages;
-          if (!mbar_wait(&full[st], (uint32_t)(it / a.stages) & 1u, a.timeout_ns) || *abort_flag) {
+        for (int c = 0; c < q.nc; ++c) {
+          if (!mbar_wait(&full[st], ph, a.timeout_ns)) {
             dead = true;
             break;
           }
           tc_fence_after();
-          const uint32_t at = smem_u32(ring + (size_t)st * a.stage_bytes);
+          const uint32_t so = (uint32_t)st * step;
 #pragma unroll
-          for (int kk = 0; kk < KB / 16; ++kk, ++e)
-            mma_bf16_ss(dacc + (uint32_t)((e % NACC) * TNT * NB), sw128_desc(at + kk * 32),
-                        sw128_desc(at + A_BYTES + kk * 32), a.idesc, e >= NACC ? 1u : 0u);
+          for (uint32_t kk = 0; kk < KB / 16; ++kk, ++e)
+            mma_bf16_ss(dacc + (uint32_t)((e % NACC) * TNT * NB), a0 + (so + kk * 2u), b0 + (so + kk * 2u), a.idesc,
+                        e >= NACC ? 1u : 0u);
           mma_commit(&empty[st]);  // the stage is free once these MMAs have read it
+          if (++st == a.stages) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
         if (dead) break;
         mma_commit(&accf[acc]);
       }
-      if (dead) {
-        latch_status(a.status, PIFA_ERR_TIMEOUT);
-        *abort_flag = 1;
-      }
+      if (dead) latch_status(a.status, PIFA_ERR_TIMEOUT);
       mma_commit(drain);  // every MMA issued above has completed before TMEM and SMEM are released
       if (!mbar_wait(drain, 0, 100000000ull)) latch_status(a.status, PIFA_ERR_TIMEOUT);
     }
-  } else {
+  } else if (warp < 6) {
     // ---------------- epilogue: warps 2..5, TMEM lane quarter warp % 4 ----------------
     const int q4 = warp & 3;
     int j = 0;
@@ -357,9 +363,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       const Seg q = seg_at(a, g, g1);
       g += q.nc;
       const int acc = j & 1;
-      if (!mbar_wait(&accf[acc], (uint32_t)(j >> 1) & 1u, a.timeout_ns) || *abort_flag) {
+      if (!mbar_wait(&accf[acc], (uint32_t)(j >> 1) & 1u, a.timeout_ns)) {
         latch_status(a.status, PIFA_ERR_TIMEOUT);
-        *abort_flag = 1;
         break;
       }
       tc_fence_after();
@@ -438,7 +443,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
         }
       } else {
         // wider token tiles: accumulator a, plane nb, tokens 16 g .. 16 g + 15 at column
-        // (a NB + nb) TNT + 16 g; one (a, nb) pair's TNT / 16 loads in flight at a time
+        // (a NB + nb) TNT + 16 g; one (a, nb) pair's loads in flight at a time
         for (int a2 = 0; a2 < used; ++a2)
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb) {
@@ -517,36 +522,55 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   }
   if (kCl) {
     // Every CTA of the cluster has its slice's sums in its own shared memory once all arrive;
-    // CTA k then finishes rows [k rpr, (k + 1) rpr) of the block, adding the slices in rank
-    // order (deterministic). Every wait above is bounded, so each CTA reaches both barriers; the
-    // second keeps each CTA resident until no peer reads its shared memory any more.
+    // CTA k then finishes rows [k rpr, (k + 1) rpr) of the block, adding the slices in a fixed
+    // order (from its own on, so that the CTAs do not all read one peer at a time). Every wait above is
+    // bounded, so each CTA reaches both barriers; the second keeps each CTA resident until no peer
+    // reads its shared memory any more.
     cluster_sync_all();
-    const int k = (int)blockIdx.x % a.cs, rb = (int)blockIdx.x / a.cs;
-    const int rpr = TM / a.cs;
     const int nsrc = a.ns < a.cs ? a.ns : a.cs;
-    const uint32_t red = smem_u32(ring);
+    const int first = ((int)blockIdx.x % a.cs) % nsrc;  // each CTA starts at another peer
+    const uint32_t red = smem_u32(ring) + (uint32_t)(myrow % TM) * 4u;
     bool range_err = false;
-    for (int idx = threadIdx.x; idx < rpr * a.T; idx += THREADS) {
-      const int t = idx / rpr, rr = k * rpr + idx % rpr;
-      const int row = rb * TM + rr;
-      const uint32_t off = red + (uint32_t)(t * TM + rr) * 4u;
-      float sum = 0.0f;
-      for (int p = 0; p < nsrc; ++p) sum += ld_dsmem_f32(mapa_shared(off, (uint32_t)p));
-      if (row >= a.R) continue;
-      if (a.yph) {
-        uint16_t hi, lo;
-        if (a.split_f16)
-          split_hi_lo<true>(sum, hi, lo, range_err);
-        else
-          split_hi_lo<false>(sum, hi, lo, range_err);
-        a.yph[(int64_t)t * a.ldyp + row] = hi;
-        a.ypl[(int64_t)t * a.ldyp + row] = lo;
+    // four rows of a token per thread and step, every slice's loads in flight at once
+    for (int t = (int)threadIdx.x / rgrp; t < a.T; t += THREADS / rgrp) {
+      const uint32_t off = red + (uint32_t)(t * TM) * 4u;
+      float4 v[MAX_CLUSTER_TC];
+#pragma unroll
+      for (int p = 0; p < MAX_CLUSTER_TC; ++p) {
+        const int src = first + p < nsrc ? first + p : first + p - nsrc;
+        if (p < nsrc) v[p] = ld_dsmem_f32x4(mapa_shared(off, (uint32_t)src));
       }
-      const int col = __ldg(a.cols + row);
-      if ((unsigned)col >= (unsigned)a.m)
-        latch_status(a.status, PIFA_ERR_DEVICE_INDEX);
-      else
-        a.Y[(int64_t)t * a.ldy + col] = __float2bfloat16_rn(sum);
+      float sum[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+      for (int p = 1; p < MAX_CLUSTER_TC; ++p)
+        if (p < nsrc) {
+          sum[0] += v[p].x;
+          sum[1] += v[p].y;
+          sum[2] += v[p].z;
+          sum[3] += v[p].w;
+        }
+      if (myrow >= a.R) continue;
+      if (a.yph) {  // rows beyond R hold zeros (padding columns: pitches are multiples of 8)
+        uint16_t h[4], l[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (a.split_f16)
+            split_hi_lo<true>(sum[j], h[j], l[j], range_err);
+          else
+            split_hi_lo<false>(sum[j], h[j], l[j], range_err);
+        }
+        const int64_t o = (int64_t)t * a.ldyp + myrow;
+        *reinterpret_cast<uint2*>(a.yph + o) = make_uint2((uint32_t)h[0] | (uint32_t)h[1] << 16, (uint32_t)h[2] | (uint32_t)h[3] << 16);
+        *reinterpret_cast<uint2*>(a.ypl + o) = make_uint2((uint32_t)l[0] | (uint32_t)l[1] << 16, (uint32_t)l[2] | (uint32_t)l[3] << 16);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (myrow + j >= a.R) break;
+        if ((unsigned)mycol[j] >= (unsigned)a.m)
+          latch_status(a.status, PIFA_ERR_DEVICE_INDEX);
+        else
+          a.Y[(int64_t)t * a.ldy + mycol[j]] = __float2bfloat16_rn(sum[j]);
+      }
     }
     if (range_err) latch_status(a.status, PIFA_ERR_RANGE);
     cluster_sync_all();

@@ -28,7 +28,7 @@
 // the issuing threads do no division and read no flag, and why wide tiles are best where they fill
 // the GPU. GEMMs of few tiles run on tiles of 128 rows by one CTA and split K: the 2 or 4 CTAs of a
 // tile form a cluster, each accumulates its K-slice, stores the fp32 partial tile in its own freed
-// ring, and the cluster adds the slices through distributed shared memory in rank order before the
+// ring, and the cluster adds the slices through distributed shared memory in a fixed order before the
 // epilogue. pick_shape takes the form, width and split that these costs say finishes first; measured
 // beside every alternative on five layers at T = 80 to 2048 it was within 4% of the best.
 // Against the one-CTA forms that this replaced (us, CUDA graph, one process): 7B attention T = 128
@@ -113,7 +113,7 @@ __device__ __forceinline__ void split_hl(float f, uint16_t& h, uint16_t& l, bool
 // kPair: a tile of 256 weight rows by a pair of CTAs; else of 128 rows by one.
 // kCl (one-CTA tiles): split-K over a cluster of ks CTAs per tile (grids with too few tiles to fill the
 // GPU): CTA z accumulates the K-steps [z total / ks, (z + 1) total / ks) of both passes; after a cluster
-// barrier it adds rows [z 128 / ks, (z + 1) 128 / ks) of the slices in rank order.
+// barrier it adds rows [z 128 / ks, (z + 1) 128 / ks) of the slices in a fixed order.
 template <int kEpi, bool kCl, bool kPair>
 __global__ void __launch_bounds__(THREADS, 1)
     pifa_umma_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
   if (kCl) {
     // CTA z finishes rows [z rpc, (z + 1) rpc) of the tile for all its tokens: four rows of a token
-    // per thread and step, every slice's loads in flight at once, added in rank order
-    // (deterministic). A second barrier keeps each CTA resident until no peer reads its shared
+    // per thread and step, every slice's loads in flight at once, added in a fixed order (from its
+    // own on, so that the CTAs do not all read one peer at a time). A second barrier keeps each CTA resident until no peer reads its shared
     // memory any more.
     int m0, mend, n0, bx0;
     place(first, m0, mend, n0, bx0);
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       float4 a[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        if (k < p.ks) a[k] = ld_dsmem_f32x4(mapa_shared(off, (uint32_t)k));
+        if (k < p.ks) a[k] = ld_dsmem_f32x4(mapa_shared(off, (uint32_t)((z + k) & (p.ks - 1))));
       float f[4] = {a[0].x, a[0].y, a[0].z, a[0].w};
 #pragma unroll
       for (int k = 1; k < 4; ++k)
