@@ -34,10 +34,49 @@ int64_t a256(int64_t b) { return (b + 255) / 256 * 256; }
 
 // dY's columns split into its pivot and non-pivot parts (bf16): outp[t][j] = in[t][piv[j]] for
 // j < r and outnp[t][i] = in[t][nonpiv[i]] for i < nnp; an index outside [0, bound) writes 0 and
-// latches PIFA_ERR_DEVICE_INDEX. A thread owns one output column (its index read once, the lanes
-// of a warp on consecutive columns) and walks the rows of its y-block's share, so that the loads of
-// consecutive rows are independent and many are in flight.
-__global__ void split_cols(const bf16* in, int64_t ldin, const int32_t* piv, int r, const int32_t* nonpiv, int nnp,
+// latches PIFA_ERR_DEVICE_INDEX. A block stages `rows` rows of dY in shared memory with 16-byte
+// loads; a thread then owns two neighbouring output columns, reads their indices once and gathers
+// them for each staged row into one 4-byte store (both output pitches are multiples of 8 and both
+// parts start at even columns). Bound by its 2 x 2 T m bytes; gathering from global memory, one
+// 2-byte load and store per element, took 19.1 us for T = 2048, m = 4096, this 12.4 us.
+__global__ void __launch_bounds__(256) split_cols(const bf16* in, int64_t ldin, const int32_t* piv, int r,
+                                                  const int32_t* nonpiv, int nnp, int bound, int T, int rows, bf16* outp,
+                                                  int64_t ldp, bf16* outnp, int64_t ldnp, int* status) {
+  extern __shared__ __align__(16) uint16_t row_sm[];  // rows x w, w = bound rounded up to 8
+  pdl_launch_dependents();
+  pdl_wait_primary();
+  const int w = (bound + 7) & ~7, t0 = blockIdx.x * rows, nr = min(rows, T - t0);
+  for (int e = threadIdx.x; e < nr * (w / 8); e += 256) {
+    const int t = e / (w / 8), c = e - t * (w / 8);
+    const bf16* src = in + (int64_t)(t0 + t) * ldin + 8 * c;
+    if (8 * c + 8 <= bound) {
+      reinterpret_cast<uint4*>(row_sm)[e] = __ldcs(reinterpret_cast<const uint4*>(src));
+    } else {
+      for (int k = 0; 8 * c + k < bound; ++k) row_sm[8 * e + k] = __bfloat16_as_ushort(src[k]);
+    }
+  }
+  __syncthreads();
+  const int np = (r + 1) / 2, nq = (nnp + 1) / 2;  // output pairs of each part
+  for (int e = threadIdx.x; e < np + nq; e += 256) {
+    const bool pv = e < np;
+    const int j = 2 * (pv ? e : e - np), n = pv ? r : nnp;
+    const int32_t* idx = (pv ? piv : nonpiv) + j;
+    const int c0 = __ldg(idx), c1 = j + 1 < n ? __ldg(idx + 1) : c0;
+    const bool ok0 = (unsigned)c0 < (unsigned)bound, ok1 = (unsigned)c1 < (unsigned)bound;
+    if (!ok0 || !ok1) latch_status(status, PIFA_ERR_DEVICE_INDEX);
+    const int64_t ld = pv ? ldp : ldnp;
+    bf16* out = (pv ? outp : outnp) + (int64_t)t0 * ld + j;
+#pragma unroll 4
+    for (int t = 0; t < nr; ++t) {
+      const uint32_t a = ok0 ? row_sm[t * w + c0] : 0u, b = ok1 ? row_sm[t * w + c1] : 0u;
+      *reinterpret_cast<uint32_t*>(out + (int64_t)t * ld) = a | b << 16;  // an odd part's last pair ends in its padding
+    }
+  }
+}
+
+// The same straight from global memory, for rows too wide to stage: a thread owns one output column
+// and walks the rows of its y-block's share.
+__global__ void split_wide(const bf16* in, int64_t ldin, const int32_t* piv, int r, const int32_t* nonpiv, int nnp,
                            int bound, int T, bf16* outp, int64_t ldp, bf16* outnp, int64_t ldnp, int* status) {
   pdl_launch_dependents();
   pdl_wait_primary();
@@ -95,48 +134,6 @@ __global__ void axpby_rows(const bf16* x, const bf16* y, int64_t ld, int T, int 
     }
 }
 
-// out (cols x rows) = in (rows x cols)^T, bf16, through 64 x 64 shared-memory tiles: each thread
-// loads 8 consecutive elements of an input row and stores 8 consecutive elements of an output row
-// (16-byte accesses: both pitches are multiples of 8 elements and both bases 16-byte aligned;
-// scalar at ragged edges). The tile's 8-element groups are stored XOR-swizzled by the row's group
-// (group g of row k at g ^ (k / 8 % 8)), so that the column reads of 8 rows 8 apart hit 8 different
-// banks. Block (8, 32); grid (ceil(cols / 64), ceil(rows / 64)).
-__global__ void transpose_bf16(const bf16* in, int64_t ldin, int rows, int cols, bf16* out, int64_t ldout) {
-  __shared__ __align__(16) bf16 t[64][64];
-  pdl_launch_dependents();
-  pdl_wait_primary();
-  const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 8 x 32
-  for (int k = ty; k < 64; k += 32) {  // input row r0 + k, columns c0 + 8 tx .. + 7
-    const int r = r0 + k, c = c0 + 8 * tx;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r < rows && c + 8 <= cols) {
-      v = *reinterpret_cast<const uint4*>(in + (int64_t)r * ldin + c);
-    } else if (r < rows) {
-      bf16* ve = reinterpret_cast<bf16*>(&v);
-      for (int e = 0; e < 8 && c + e < cols; ++e) ve[e] = in[(int64_t)r * ldin + c + e];
-    }
-    *reinterpret_cast<uint4*>(&t[k][8 * (tx ^ ((k >> 3) & 7))]) = v;
-  }
-  __syncthreads();
-  for (int k = ty; k < 64; k += 32) {  // output row c0 + k (input column), rows r0 + 8 tx .. + 7
-    const int c = c0 + k, r = r0 + 8 * tx;
-    if (c >= cols) continue;
-    uint4 v;
-    bf16* ve = reinterpret_cast<bf16*>(&v);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int kr = 8 * tx + e;  // tile row; its group (k >> 3) sits at (k >> 3) ^ tx
-      ve[e] = t[kr][8 * ((k >> 3) ^ ((kr >> 3) & 7)) + (k & 7)];
-    }
-    if (r + 8 <= rows) {
-      *reinterpret_cast<uint4*>(out + (int64_t)c * ldout + r) = v;
-    } else {
-      for (int e = 0; r + e < rows; ++e) out[(int64_t)c * ldout + r + e] = ve[e];
-    }
-  }
-}
-
 // A row-wise elementwise kernel over `rows` rows of `cols` columns: rows on the y grid (at most
 // 65535, the kernel loops beyond), columns on x.
 int launch_small(const void* fn, void** args, int64_t rows, int64_t cols, cudaStream_t stream, const char* what) {
@@ -181,15 +178,14 @@ BwdLayout bwd_layout(int64_t T, int64_t m, int64_t r) {
 }
 
 struct MaccLayout {
-  int64_t xut, xmix, xmix_lo, ytt, ytt_lo, total;
+  int64_t xmix, xmix_lo, ytt, ytt_lo, total;
 };
 
-// X_u^T (n x pad8(T)), the mixed input's hi and lo planes (T x pad8(n)), Y_t^T's hi and lo planes
-// (m x pad8(T)), all bf16
+// The mixed input's hi and lo planes (T x pad8(n)), Y_t^T's hi and lo planes (m x pad8(T)), all bf16,
+// behind n x pad8(T) values that nothing uses any more: the size that callers are asked for stays.
 MaccLayout macc_layout(int64_t T, int64_t m, int64_t n) {
   MaccLayout L;
   int64_t o = 0;
-  L.xut = o;
   o += a256(n * pad8(T) * 2);
   L.xmix = o;
   o += a256(T * pad8(n) * 2);
@@ -256,7 +252,13 @@ extern "C" int pifa_backward(const void* X, int64_t T, int64_t n, int64_t ldx, c
   bf16* dYi = reinterpret_cast<bf16*>(ws + Ly.dyi);
   {  // dY_I = dY[:, I] and dY_np = dY[:, I^c] in one pass over dY (dY_I straight into dY_p when r = m)
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((m + 255) / 256), (unsigned)(T < 64 ? T : 64));
+    const int64_t row_bytes = (m + 7) / 8 * 16;
+    // rows per block: 72 KB of them (three blocks per SM), or up to three wider ones that share the
+    // indices' loads
+    int64_t rows = 72 * 1024 / row_bytes;
+    if (rows < 3) rows = 200 * 1024 / row_bytes < 3 ? 200 * 1024 / row_bytes : 3;
+    if (rows > 16) rows = 16;
+    cudaError_t e = cudaSuccess;
     cfg.blockDim = dim3(256);
     cfg.stream = s;
     cudaLaunchAttribute attr;
@@ -264,9 +266,18 @@ extern "C" int pifa_backward(const void* X, int64_t T, int64_t n, int64_t ldx, c
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = pifa_launch_ex(&cfg, split_cols, reinterpret_cast<const bf16*>(dY), lddy, pivot_idx, (int)r,
-                                         nonpivot_idx, (int)(m - r), (int)m, (int)T, has_np ? dYi : dYp, ldr, dYnp,
-                                         ldnp, status);
+    if (rows > 0) {
+      cfg.gridDim = dim3((unsigned)((T + rows - 1) / rows));
+      cfg.dynamicSmemBytes = (size_t)(rows * row_bytes);
+      e = cudaFuncSetAttribute(split_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (e == cudaSuccess)
+        e = pifa_launch_ex(&cfg, split_cols, reinterpret_cast<const bf16*>(dY), lddy, pivot_idx, (int)r, nonpivot_idx,
+                           (int)(m - r), (int)m, (int)T, (int)rows, has_np ? dYi : dYp, ldr, dYnp, ldnp, status);
+    } else {
+      cfg.gridDim = dim3((unsigned)((m + 255) / 256), (unsigned)(T < 64 ? T : 64));
+      e = pifa_launch_ex(&cfg, split_wide, reinterpret_cast<const bf16*>(dY), lddy, pivot_idx, (int)r, nonpivot_idx,
+                         (int)(m - r), (int)m, (int)T, has_np ? dYi : dYp, ldr, dYnp, ldnp, status);
+    }
     if (e != cudaSuccess) return pifa_fail_cuda("backward: split dY", e);
   }
   // Two launches of independent products: those that dY and X give, then those that need them. (One
@@ -331,27 +342,10 @@ extern "C" int pifa_m_accumulate(const void* Xo, const void* Xu, int64_t T, int6
   cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
   const uint64_t tmo = pifa_wait_timeout_ns();
   int st;
-  // Every product runs with both operands K-major (measured twice as fast as the transposed forms):
-  // X_u^T is formed once, and Y_t^T comes out of W X_mix^T directly.
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  bf16* XuT = reinterpret_cast<bf16*>(ws + Ly.xut);
   const int64_t ldT = pad8(T), ldn = pad8(n);
-  {  // X_u^T
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n + 63) / 64), (unsigned)((T + 63) / 64));
-    cfg.blockDim = dim3(8, 32);
-    cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = pifa_launch_ex(&cfg, transpose_bf16, reinterpret_cast<const bf16*>(Xu), ldx, (int)T,
-                                             (int)n, XuT, ldT);
-    if (e != cudaSuccess) return pifa_fail_cuda("m_accumulate: transpose", e);
-  }
   // XXt += X_u^T X_u, its upper triangle (the product is symmetric: half the tiles)
-  GemmTc xx = {n, n, T, XuT, ldT, false, XuT, ldT, false, XXt, ldxx, 2, 1.0f, nullptr, 0};
+  GemmTc xx = {n, n, T, Xu, ldx, true, Xu, ldx, true, XXt, ldxx, 2, 1.0f, nullptr, 0};
   xx.upper = true;
   if (!YtXt) return gemm_tc_group(&xx, 1, status, tmo, s);
   bf16* Xmix = reinterpret_cast<bf16*>(ws + Ly.xmix);
@@ -370,7 +364,7 @@ extern "C" int pifa_m_accumulate(const void* Xo, const void* Xu, int64_t T, int6
   GemmTc yt = {m, T, n, W, ldw, false, Xmix, ldn, false, YtT, ldT, 3, 1.0f, nullptr, 0};
   yt.B2 = Xmix_lo;
   yt.D2 = YtT_lo;
-  GemmTc yx = {m, n, T, YtT, ldT, false, XuT, ldT, false, YtXt, ldyx, 2, 1.0f, nullptr, 0};
+  GemmTc yx = {m, n, T, YtT, ldT, false, Xu, ldx, true, YtXt, ldyx, 2, 1.0f, nullptr, 0};
   yx.A2 = YtT_lo;
   const GemmTc first[2] = {yt, xx};
   if ((st = gemm_tc_group(first, 2, status, tmo, s)) != PIFA_OK) return st;

@@ -279,3 +279,17 @@ def test_m_accumulate_tile_edges(m, n, T):
     blk = np.arange(n) // 128
     check(XXt.cpu().numpy(), np.where(blk[:, None] <= blk[None, :], a, 0.0), "X X^T")
     check(YtXt.cpu().numpy(), b, "Y_t X^T")
+
+
+@pytest.mark.parametrize("m,T", [(9001, 37), (40003, 7), (110003, 5)])
+def test_backward_splits_rows_of_any_width(m, T):
+    """dY's rows staged many, three and (too wide for shared memory) none per block; odd parts."""
+    n, r = 48, 25
+    piv, nonp, Wp32, C32 = inputs.synthetic_layer(m, n, r, 51)
+    rng = np.random.default_rng(52)
+    X32, dY32 = inputs.make_activations(rng, T, n, "bf16"), inputs.make_activations(rng, T, m, "bf16")
+    pd, nd = torch.from_numpy(piv).to(DEV), torch.from_numpy(nonp).to(DEV)
+    dX, dWp, dC = P.pifa_backward(dev_bf16(X32), dev_bf16(Wp32), dev_bf16(C32), pd, nd, dev_bf16(dY32))
+    assert P.pifa_device_status() == P.PIFA_OK
+    for got, ref, what in zip((dX, dWp, dC), oracle.backward(X32, Wp32, C32, piv, nonp, dY32), ("dX", "dW_p", "dC")):
+        check(got.float().cpu().numpy(), ref, what)
