@@ -371,8 +371,8 @@ int pifa_set_wait_timeout(int64_t ns);
  * phase deals equal ranges of 128 x 64 weight tiles to a persistent grid and a second kernel sums
  * the fp32 partial sums in a fixed order.
  * PIFA_DECODE_GRID_AUTO (0, the default) picks per phase from its shape and T: split-K when
- * T > 2 and R >= 4096, else waves while the phase takes at most two of them, else the persistent
- * grid. PIFA_DECODE_GRID_WAVES (1), PIFA_DECODE_GRID_PERSISTENT (2) and PIFA_DECODE_GRID_SPLITK
+ * T > 2 and R >= 4096 or T > 8 and the waves would need more CTAs than there are SMs, else waves
+ * while the phase takes at most two of them, else the persistent grid. PIFA_DECODE_GRID_WAVES (1), PIFA_DECODE_GRID_PERSISTENT (2) and PIFA_DECODE_GRID_SPLITK
  * (3) force one form for both phases (a tuning and test knob: all compute the same result up to
  * the summation order of fp32 partial sums; forced split-K runs the persistent grid instead when the
  * workspace is too small for its partial sums). For 16 < T <= 128 only the split-K form exists

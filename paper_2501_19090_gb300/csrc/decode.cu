@@ -1008,6 +1008,12 @@ int launch_one_phase(DecodeArgs& a, uint32_t budget, int dtype, const SplitKScra
   // decode_rows in waves while a phase takes at most two of them (its weights staged at launch,
   // before the dependency wait, outweigh the persistent grid's streaming); else decode_stream
   const int tiles = (a.R + kRows - 1) / kRows;
+  // For T > 8 (two token tiles) a phase whose waves need more CTAs than there are SMs is faster in
+  // split-K whatever its rows: 4096 x 11008, r = 2048 (512 and 256 CTAs) T = 16 22.5 -> 19.5 us,
+  // 4096 x 4096, r = 3072 (192 and 128 CTAs) 18.9 -> 15.6; one CTA per SM stays with waves (4096 x
+  // 4096, r = 2048: 13.2 against 14.5). Up to T = 8 the two are within 2%.
+  if (mode == PIFA_DECODE_GRID_AUTO && a.T > 8 && tc_fits && tiles * a.ks > sm_count())
+    return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
   if (mode == PIFA_DECODE_GRID_WAVES ||
       (mode == PIFA_DECODE_GRID_AUTO && tiles <= 2 * max_clusters(reinterpret_cast<const void*>(kr), a.ks, smem)))
     return launch_phase(kr, kRows, a, smem, stream, what);

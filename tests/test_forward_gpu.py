@@ -762,3 +762,18 @@ def test_prefill_tilings_ragged(m, n, r, T, c):
 def test_grouped_prefill_groups_end_inside_a_pair_tile(T):
     """384 non-pivot rows per group: one and a half 256-row tiles, of which none may span two groups."""
     grouped_parity([layer_for(1152, 840, 768, s, "synthetic") for s in (7, 8, 9)], T, sample=64)
+
+
+def test_decode_selector_splits_k_where_waves_exceed_the_sms():
+    """For T > 8 a phase whose waves would take more CTAs than the GPU has SMs runs split-K, whatever
+    its rows (here 3072 per phase): bit for bit the forced form; at T = 8 the same layer keeps waves."""
+    L = layer_for(6144, 4096, 3072, 6, "synthetic")
+    for T, forced in ((9, P.PIFA_DECODE_GRID_SPLITK), (16, P.PIFA_DECODE_GRID_SPLITK), (8, P.PIFA_DECODE_GRID_WAVES)):
+        X = acts(T, 4096, 6)
+        auto = run(L, X, P.PIFA_VARIANT_DECODE)
+        check(auto, oracle.forward(X, L.Wp, L.C, L.pivots, L.nonpivots), f"T={T}")
+        P.pifa_set_decode_grid(forced)
+        try:
+            assert np.array_equal(auto, run(L, X, P.PIFA_VARIANT_DECODE)), T
+        finally:
+            P.pifa_set_decode_grid(P.PIFA_DECODE_GRID_AUTO)
