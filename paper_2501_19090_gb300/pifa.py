@@ -8,6 +8,7 @@ missing or unloadable library raises -- there is no fallback path.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -198,12 +199,17 @@ def pifa_select_variant(T: int, m: int, n: int, r: int, c_dtype: int = PIFA_DTYP
     return v
 
 
-def pifa_workspace_size(T: int, m: int, n: int, r: int, variant: int = PIFA_VARIANT_AUTO,
-                        c_dtype: int = PIFA_DTYPE_BF16) -> int:
+@functools.lru_cache(maxsize=1024)  # host arithmetic on the arguments alone
+def _workspace_size(T, m, n, r, variant, c_dtype) -> int:
     v = _lib().pifa_workspace_size(T, m, n, r, c_dtype, variant)
     if v < 0:
         _check(int(v), "pifa_workspace_size")
     return int(v)
+
+
+def pifa_workspace_size(T: int, m: int, n: int, r: int, variant: int = PIFA_VARIANT_AUTO,
+                        c_dtype: int = PIFA_DTYPE_BF16) -> int:
+    return _workspace_size(T, m, n, r, variant, c_dtype)
 
 
 def pifa_validate_indices(pivot_idx: np.ndarray, nonpivot_idx: np.ndarray, m: int, r: int) -> int:
@@ -277,6 +283,8 @@ def pifa_compress_device(U, V, stream=None):
 def _stream_ptr(stream):
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():  # the current device's current stream, without a Stream object
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         if not torch.cuda.is_available():
             return None
         return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
@@ -304,9 +312,10 @@ def workspace(nbytes: int, device, stream=None, tag: str = ""):
 
 
 def _ld(t) -> int:
-    if t.dim() != 2 or t.stride(1) != 1:
+    s = t.stride()
+    if len(s) != 2 or s[1] != 1:
         raise ValueError("expected a row-major 2-D tensor with unit column stride")
-    return t.stride(0)
+    return s[0]
 
 
 def c_dtype_of(C) -> int:
@@ -319,11 +328,46 @@ def c_dtype_of(C) -> int:
     raise TypeError(f"C must be bfloat16 or float16, got {C.dtype}")
 
 
+def _operands_ok(G: int, X, Wp, C, pivot_idx, nonpivot_idx, Y, ws, c_fp16_ok):
+    """_operands' checks without its messages: (T, n, r, m) if every operand is as it should be, else
+    None (a call of a small layer spends as long in the checks as in its kernels)."""
+    import torch
+    Tensor, bf16, i32 = torch.Tensor, torch.bfloat16, torch.int32
+    if not (isinstance(X, Tensor) and isinstance(Wp, Tensor) and isinstance(pivot_idx, Tensor)):
+        return None
+    xs, ws_, dev = X.shape, Wp.shape, X.device
+    if len(xs) != 2 or len(ws_) != 2 or ws_[0] % G or ws_[1] != xs[1] or dev.type != "cuda":
+        return None
+    r = ws_[0] // G
+    if (X.dtype is not bf16 or Wp.dtype is not bf16 or Wp.device != dev or pivot_idx.dtype is not i32
+            or pivot_idx.shape != (G * r,) or not pivot_idx.is_contiguous() or pivot_idx.device != dev):
+        return None
+    nnp = 0
+    if nonpivot_idx is not None:
+        if not isinstance(nonpivot_idx, Tensor) or nonpivot_idx.dtype is not i32 or nonpivot_idx.dim() != 1:
+            return None
+        nnp = nonpivot_idx.numel()
+        if nnp % G or not nonpivot_idx.is_contiguous() or nonpivot_idx.device != dev:
+            return None
+    m = r + nnp // G
+    if nnp and (not isinstance(C, Tensor) or C.shape != (nnp, r) or C.device != dev
+                or not (C.dtype is bf16 or (c_fp16_ok and C.dtype is torch.float16))):
+        return None
+    if Y is not None and (not isinstance(Y, Tensor) or Y.dtype is not bf16 or Y.shape != (xs[0], G * m) or Y.device != dev):
+        return None
+    if ws is not None and (not isinstance(ws, Tensor) or ws.device != dev):
+        return None
+    return xs[0], xs[1], r, m
+
+
 def _operands(G: int, X, Wp, C, pivot_idx, nonpivot_idx, Y, workspace_tensor=None, c_fp16_ok=True):
     """Check what the C ABI cannot see -- tensor type, dtype, shape and device -- before any
     pointer reaches the library (a host or mistyped buffer would otherwise be read as device
     bf16). Types and shapes first, then that every tensor sits on X's CUDA device. Returns
     (T, n, r, m) of one group. Raises ValueError."""
+    ok = _operands_ok(G, X, Wp, C, pivot_idx, nonpivot_idx, Y, workspace_tensor, c_fp16_ok)
+    if ok is not None:
+        return ok
     import torch
 
     def fail(msg):

@@ -777,3 +777,25 @@ def test_decode_selector_splits_k_where_waves_exceed_the_sms():
             assert np.array_equal(auto, run(L, X, P.PIFA_VARIANT_DECODE)), T
         finally:
             P.pifa_set_decode_grid(P.PIFA_DECODE_GRID_AUTO)
+
+
+def test_binding_refuses_bad_cuda_operands_before_the_library():
+    """One operand at a time of the wrong type, dtype, shape, layout or device: ValueError, and no kernel."""
+    L = layer_for(300, 200, 77, 3, "synthetic")
+    Wp, C, piv, nonp = L.dev()
+    X = _pad_dev(acts(5, 200, 1))
+    Y = torch.empty((5, 304), dtype=torch.bfloat16, device=DEV)[:, :300]
+    good = dict(X=X, Wp=Wp, C=C, pivot_idx=piv, nonpivot_idx=nonp, Y=Y)
+    P.pifa_forward(**good)
+    c0 = P.pifa_launch_count()
+    bad = [dict(X=X.float()), dict(X=X.cpu()), dict(X=X[0]), dict(X=None), dict(Wp=Wp[:, :192]), dict(Wp=Wp.half()),
+           dict(Wp=Wp.cpu()), dict(C=C[:-1]), dict(C=C.float()), dict(C=None), dict(C=C.cpu()), dict(pivot_idx=piv[:-1]),
+           dict(pivot_idx=piv.long()), dict(pivot_idx=piv.cpu()), dict(pivot_idx=piv.repeat(2)[::2]),
+           dict(nonpivot_idx=nonp.cpu()), dict(nonpivot_idx=nonp.long()), dict(nonpivot_idx=nonp[:-1]),
+           dict(Y=Y.float()), dict(Y=Y[:4]), dict(Y=Y.cpu()), dict(workspace_tensor=torch.empty(1 << 20, dtype=torch.uint8))]
+    for change in bad:
+        with pytest.raises(ValueError):
+            P.pifa_forward(**{**good, **change})
+    with pytest.raises(ValueError):  # the allocation-free entry point takes bf16 C only
+        P.pifa_forward_decode_noalloc(X, Wp, C.half(), piv, nonp, Y=Y)
+    assert P.pifa_launch_count() == c0
