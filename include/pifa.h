@@ -236,8 +236,8 @@ int pifa_compress(const double* U, const double* V, int64_t m, int64_t n, int64_
  *                (threads = 0).
  *   cuda_stream  the stream the work is enqueued on; the call synchronizes it before returning.
  *
- *   Pivot rule exactly as pifa_compress (greedy Businger-Golub on W'^T, residual norms recomputed
- *   every step, ties to the lowest index), computed in the r-dimensional row space Z = U L with
+ *   Pivot rule exactly as pifa_compress (greedy Businger-Golub on W'^T, ties to the lowest index;
+ *   residual norms recomputed every step for all rows that the step could choose), computed in the r-dimensional row space Z = U L with
  *   L L^T = V^T V (Cholesky), which has the row inner products of W'. C = Z[I^c] R^{-T} from the
  *   triangular factor R of that pivoted QR; W_p = U[I] V^T. Requires 1 <= r <= min(m, n) and
  *   r <= 16384 (PIFA_ERR_UNSUPPORTED otherwise); PIFA_ERR_RANK_DEFICIENT when V^T V is not

@@ -7,9 +7,10 @@
 //      pivoting on W'^T (Algorithm 1, step 1) selects the same rows when run on Z^T, whose columns
 //      are r long instead of n.
 //   2. r greedy Businger-Golub steps on the rows of Z: step k picks the unchosen row of largest
-//      residual norm (norms recomputed from the reflected rows every step, no downdating; ties to
-//      the lowest index), builds the Householder reflector that maps the pivot row's residual onto
-//      e_k, and applies it to every unchosen row. After r steps a chosen row holds its column of
+//      residual norm (norms recomputed from the reflected rows, no downdating; ties to the lowest
+//      index), builds the Householder reflector that maps the pivot row's residual onto e_k, and
+//      applies it to every unchosen row; on large layers, at first to the candidates of up to 64
+//      steps only and then to the other rows in one product ("candidate blocks" below). After r steps a chosen row holds its column of
 //      the triangular factor R (selection order) and every other row i holds c_i = Q^T z_i.
 //   3. Eq. 2 in Z-space: Z_np = C Z_p, with Z_p = R^T Q^T and Z_np = Cmat Q^T (rows c_i), so
 //      C = Cmat R^{-T} -- one GEMM against the explicit inverse of R (computed by doubling:
@@ -18,10 +19,11 @@
 //   4. W_p = U[I, :] V^T (Eq. 1).
 // Products of 2^20 multiply-adds and more run on the tensor cores by exact slices (gemm_f64_tc.cu);
 // small ones, the panels of the Cholesky factorisation and the greedy steps run on the CUDA cores,
-// bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured on the two
-// parts that this replaced (all products on the CUDA cores; Cholesky by rank-1 updates):
-// 4096 x 4096, r = 2048: products 90.4 ms, Cholesky 37.8 ms of 310 ms; now 190 ms in all;
-// the M solves at m = n = 2048, r = 1024: 142.1 -> 21.3 ms. No kernel waits on another CTA.
+// bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
+// this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
+// row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
+// with their slices 25, Cholesky 4.0 and steps 37 of 71.5 ms. The M solves at m = n = 2048, r = 1024:
+// 141.5 -> 20.6 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -254,6 +256,11 @@ __device__ __forceinline__ void top2_add(Top2& t, unsigned long long v, int i, i
   }
 }
 
+// The key of a squared norm; a NaN (a row of U that holds one) ranks below every number.
+__device__ __forceinline__ unsigned long long norm_key(double v) {
+  return v >= 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+}
+
 __device__ __forceinline__ Top2 top2_empty() { return Top2{0ull, 0ull, -1, -1, -1}; }
 
 __device__ __forceinline__ void top2_merge(Top2& a, const Top2& b) {
@@ -304,9 +311,20 @@ struct Greedy {
   int32_t* order;   // r: row chosen at step k
   double* rdiag;    // r: R_kk of the pivoted QR
   double* gap;      // r: (best - runner-up) / best of the residual norms at step k
+  struct GreedyCtl* ctl;
+  double* tau;      // r: the reflectors' tau (candidate blocks only, else null)
 };
 
-// Initial squared row norms of Z, each block's best two, and the list of all rows.
+// The rows that a run of steps works on, set by greedy_select.
+struct GreedyCtl {
+  int stop, k_end;           // set by the step that could not be sure of its pivot
+  int count;                 // rows in the list at the run's first step
+  int all;                   // 1: every unchosen row is in the list
+  unsigned long long theta;  // else: no other row's squared norm exceeded this at the run's first step
+};
+
+// Initial squared row norms of Z, each block's best two, and the list of all rows (the exhaustive
+// steps from 0 on, without a norm's scratch per row).
 __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   Top2 t = top2_empty();
@@ -316,20 +334,116 @@ __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
     for (int c = lane; c < g.r; c += 32) s = fma(z[c], z[c], s);
     s = warp_sum(s);
     if (lane == 0) {
-      top2_add(t, (unsigned long long)__double_as_longlong(s), i, i);
+      top2_add(t, norm_key(s), i, i);
       g.act[i] = i;
     }
   }
   t = block_top2(t);
   if (threadIdx.x == 0) g.blk[blockIdx.x] = t;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *g.ctl = GreedyCtl{0, 0, g.m, 1, 0ull};
 }
 
-// Step k: every block reduces step k - 1's per-block results to the pivot p (all blocks reach the
+// Squared residual norms (coordinates k..r-1) of the unchosen rows; -1 marks a chosen one.
+__global__ void __launch_bounds__(256) greedy_norms(Greedy g, int k, double* norms) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = blockIdx.x * 8 + warp; i < g.m; i += gridDim.x * 8) {
+    const double* z = g.Z + (int64_t)i * g.r;
+    double s0 = 0.0, s1 = 0.0;
+    if (!g.sel[i]) {
+      int c = k + lane;
+      for (; c + 32 < g.r; c += 64) {
+        s0 = fma(z[c], z[c], s0);
+        s1 = fma(z[c + 32], z[c + 32], s1);
+      }
+      if (c < g.r) s0 = fma(z[c], z[c], s0);
+    }
+    s0 = warp_sum(s0 + s1);
+    if (lane == 0) norms[i] = g.sel[i] ? -1.0 : s0;
+  }
+}
+
+// The list for the steps from k on and their first best two: the rows of the `want` or somewhat fewer
+// largest norms (a threshold found by bisection; in_list marks them), or, with want = 0 or where
+// ties leave fewer than a quarter of them above any threshold, all unchosen rows. One block of 1024.
+__global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const double* norms, int want, uint8_t* in_list) {
+  __shared__ int s_n[32];
+  __shared__ double s_m[32];
+  __shared__ Top2 s_t[32];
+  __shared__ int s_count;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto count_above = [&](double th) {
+    int n = 0;
+    for (int i = threadIdx.x; i < g.m; i += 1024) n += norms[i] > th ? 1 : 0;
+    n = __reduce_add_sync(0xffffffffu, n);
+    __syncthreads();
+    if (lane == 0) s_n[warp] = n;
+    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, s_n[lane]);
+  };
+  double mx = 0.0;
+  for (int i = threadIdx.x; i < g.m; i += 1024) mx = fmax(mx, norms[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) s_m[warp] = mx;
+  __syncthreads();
+  mx = s_m[lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  double lo = -0.5, hi = mx;  // count above lo: all unchosen rows; above hi: none
+  bool all = want == 0 || count_above(lo) <= 2 * want;
+  double th = lo;
+  for (int it = 0; it < 48 && !all; ++it) {
+    const double mid = it == 0 ? 0.5 * mx : 0.5 * (fmax(lo, 0.0) + hi);
+    const int n = count_above(mid);
+    if (n > want) {
+      lo = mid;
+    } else {
+      hi = mid;
+      th = mid;
+      if (n >= want - want / 4) break;
+    }
+  }
+  if (!all && (th < 0.0 || count_above(th) < want / 4)) all = true;
+  if (all) th = -0.5;
+  if (threadIdx.x == 0) s_count = 0;
+  __syncthreads();
+  Top2 t = top2_empty();
+  for (int i0 = 0; i0 < g.m; i0 += 1024) {
+    const int i = i0 + (int)threadIdx.x;
+    const bool in = i < g.m && (all ? norms[i] != -1.0 : norms[i] > th);
+    if (in_list && i < g.m) in_list[i] = in ? 1 : 0;
+    const unsigned ballot = __ballot_sync(0xffffffffu, in);
+    int at = 0;
+    if (lane == 0 && ballot) at = atomicAdd(&s_count, __popc(ballot));  // the list's order changes no result
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(ballot & ((1u << lane) - 1u));
+    if (in) {
+      g.act[at] = i;
+      top2_add(t, norm_key(norms[i]), i, at);
+    }
+  }
+  t = warp_top2(t);
+  if (lane == 0) s_t[warp] = t;
+  __syncthreads();
+  t = warp_top2(s_t[lane]);
+  for (int b = threadIdx.x; b < g.nblk; b += 1024) g.blk[(k & 1) * g.nblk + b] = b == 0 ? t : top2_empty();
+  if (threadIdx.x == 0) {
+    g.ctl->stop = 0;
+    g.ctl->k_end = 0;
+    g.ctl->count = s_count;
+    g.ctl->all = all ? 1 : 0;
+    g.ctl->theta = (unsigned long long)__double_as_longlong(all ? 0.0 : th);
+  }
+}
+
+// Step k of a run from step k0 on: every block reduces step k - 1's per-block results to the pivot p (all blocks reach the
 // same p), forms the reflector H = I - tau v v^T from row p's residual x (coordinates k..r-1,
 // v = x - alpha e_0, alpha = -sign(x_0) |x|, tau = 1 / (|x|^2 + |x| |x_0|)) in shared memory, and
-// reflects its share of the unchosen rows, recomputing their residual norms (coordinates k+1..).
+// reflects its share of the listed rows, recomputing their residual norms (coordinates k+1..).
 // Row p itself is left as it is (other blocks read it during this launch): its column of R is
-// its coordinates 0..k-1 plus rdiag[k].
+// its coordinates 0..k-1 plus rdiag[k]. Where the list does not hold every unchosen row, the run
+// stops (ctl) before a step whose best two listed norms do not both exceed every other row's norm at
+// the run's start: a reflection never adds to a row's residual, so until then they are the best two
+// of all rows (the margin of 1e-10 is far above the norms' rounding).
 //
 // A row belongs to W warps, which keep its residual in registers (NREG values per lane) from its
 // one read to its one write: dot product, update and norm are three float64 multiply-adds per
@@ -342,7 +456,7 @@ __global__ void __launch_bounds__(256) greedy_init(Greedy g) {
 template <int NREG, int W>
 constexpr int kGreedyWarps = NREG <= 32 ? 12 : 8;  // what the registers allow
 template <int NREG, int W>
-__global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Greedy g, int k) {
+__global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Greedy g, int k, int k0) {
   constexpr int WARPS = kGreedyWarps<NREG, W>, GROUPS = WARPS / W, LEN = 32 * NREG * W;
   extern __shared__ double v[];  // LEN entries, zero from r - k on
   __shared__ double part[2][WARPS], s_tau;
@@ -351,7 +465,9 @@ __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Gre
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = warp / W, wq = warp % W;
   pdl_launch_dependents();
   pdl_wait_primary();
-  const int len = g.r - k, n = g.m - k;  // unchosen rows, p among them
+  if (g.ctl->stop) return;
+  const bool all = g.ctl->all;
+  const int len = g.r - k, n = g.ctl->count - (k - k0);  // listed rows still unchosen, p among them
   const int c0 = wq * 32 * NREG + lane;
   double y[NREG];
   auto load = [&](int i) {
@@ -365,6 +481,14 @@ __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Gre
   for (int b = threadIdx.x; b < g.nblk; b += WARPS * 32) top2_merge(t, in[b]);
   t = block_top2(t);
   const int p = t.i1;
+  if (!all && (t.i2 < 0 || !(__longlong_as_double((long long)t.v2) >
+                             __longlong_as_double((long long)g.ctl->theta) * (1.0 + 1e-10)))) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // every block finds the same, or the flag set
+      g.ctl->k_end = k;
+      g.ctl->stop = 1;
+    }
+    return;
+  }
   if (p < 0 || p >= g.m || t.s1 < 0 || t.s1 >= n) return;  // cannot happen for m >= r; guards the reads
   const double* zp = g.Z + (int64_t)p * g.r + k;
   const int tail = g.act[n - 1];
@@ -377,6 +501,7 @@ __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Gre
     if (threadIdx.x == 0) {
       v[0] = x0 - alpha;
       s_tau = nx2 > 0.0 ? 1.0 / (nx2 + nx * fabs(x0)) : 0.0;
+      if (blockIdx.x == 0 && g.tau) g.tau[k] = s_tau;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       g.order[k] = p;
@@ -426,14 +551,16 @@ __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Gre
 #pragma unroll
       for (int w = 0; w < W; ++w) nr += part[1][grp * W + w];
     }
-    if (lane == 0 && wq == 0) top2_add(mine, (unsigned long long)__double_as_longlong(nr), i, s);
+    if (lane == 0 && wq == 0) top2_add(mine, norm_key(nr), i, s);
   }
   mine = block_top2(mine);
   if (threadIdx.x == 0) out[blockIdx.x] = mine;
 }
 
-// The form of step k for residuals of `len` values: one warp a row up to 2048 values, then 2, 4 or 8.
-using GreedyStep = void (*)(Greedy, int);
+// The form of step k for residuals of `len` values: one warp a row up to 2048 values, then 2, 4 or 8
+// (2 or 4 warps a row from the start cost 92 / 99 ms of steps against 70 at 4096 x 4096, r = 2048; four
+// warps a row for candidate blocks alone gain nothing, 73.3 against 72.6 ms of call).
+using GreedyStep = void (*)(Greedy, int, int);
 GreedyStep greedy_form(int len, int* threads, size_t* smem) {
   static const GreedyStep one[8] = {greedy_step<8, 1>,  greedy_step<16, 1>, greedy_step<24, 1>, greedy_step<32, 1>,
                                     greedy_step<40, 1>, greedy_step<48, 1>, greedy_step<56, 1>, greedy_step<64, 1>};
@@ -447,6 +574,90 @@ GreedyStep greedy_form(int len, int* threads, size_t* smem) {
   *smem = (size_t)2048 * w * 8;
   return w == 2 ? greedy_step<64, 2> : w == 4 ? greedy_step<64, 4> : greedy_step<64, 8>;
 }
+
+// ---- candidate blocks ----------------------------------------------------------------------------
+// A step over every unchosen row costs three float64 multiply-adds per value of Z, but only rows of
+// large residual can be chosen, and no residual grows. So, while Z is large, a run of up to kRun steps
+// works on the rows of the largest norms alone (greedy_select, greedy_step) and ends when another row
+// might come into play; the other rows then take the run's reflectors at once, Z -= W T V^T with
+// W = Z V (the compact WY form of Schreiber and Van Loan, 1989; T^-1 = diag(1 / tau) + the strictly upper
+// part of V^T V), as two products on the tensor cores and a substitution per row, and all norms are
+// recomputed. The pivots, and the order of every comparison that decides one, are those of the
+// exhaustive steps. 4096 x 4096, r = 2048: the call 86.1 -> 71.5 ms.
+constexpr int kRun = 64;
+constexpr int kCandidates = 512;
+constexpr int kRunSlices = 4;  // K-slices of Z V, whose tiles (128 rows each) are few
+// Values of Z left (unchosen rows x coordinates) from which on a candidate block pays.
+constexpr int64_t kRunFrom = 2000000;
+
+// V (kRun x len, row-major): row j the reflector of step k0 + j over coordinates k0..r-1, zero rows
+// from `steps` on.
+__global__ void run_vectors(Greedy g, int k0, int steps, double* V) {
+  const int len = g.r - k0, j = blockIdx.y;
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= len) return;
+  double v = 0.0;
+  if (j < steps && c >= j) {
+    v = g.Z[(int64_t)g.order[k0 + j] * g.r + k0 + c];
+    if (c == j) v -= g.rdiag[k0 + j];
+  }
+  V[(int64_t)j * len + c] = v;
+}
+
+// S[i][j] = v_i . v_j for i < j < kRun, a warp each.
+__global__ void __launch_bounds__(256) run_gram(const double* V, int len, double* S) {
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int i = w / kRun, j = w % kRun;
+  if (i >= kRun || i >= j) return;
+  const double *a = V + (int64_t)i * len, *b = V + (int64_t)j * len;
+  double s0 = 0.0, s1 = 0.0;
+  int c = lane;
+  for (; c + 32 < len; c += 64) {
+    s0 = fma(a[c], b[c], s0);
+    s1 = fma(a[c + 32], b[c + 32], s1);
+  }
+  if (c < len) s0 = fma(a[c], b[c], s0);
+  s0 = warp_sum(s0 + s1);
+  if (lane == 0) S[i * kRun + j] = s0;
+}
+
+// W (m x kRun, the sum of its slices) becomes W T by forward substitution, w_j = tau_j (w_j - sum over i < j of w_i S[i][j]),
+// and zero for the rows that already carry the run's reflectors (listed) or must not (chosen before).
+// Four lanes a row, each with every fourth column.
+__global__ void __launch_bounds__(128) run_substitute(Greedy g, int k0, int steps, const double* S, const uint8_t* in_list,
+                                                      double* W, int slices) {
+  __shared__ double s_S[kRun * kRun];
+  __shared__ double s_tau[kRun];
+  for (int e = threadIdx.x; e < kRun * kRun; e += 128) s_S[e] = e / kRun < e % kRun ? S[e] : 0.0;
+  if (threadIdx.x < kRun) s_tau[threadIdx.x] = (int)threadIdx.x < steps ? g.tau[k0 + threadIdx.x] : 0.0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, q = lane & 3;
+  const int row = blockIdx.x * 32 + (threadIdx.x >> 2);
+  const bool live = row < g.m && !g.sel[row] && !in_list[row];
+  double w[kRun / 4];
+  double* p = W + (int64_t)row * kRun;
+#pragma unroll
+  for (int u = 0; u < kRun / 4; ++u) w[u] = live ? p[4 * u + q] : 0.0;
+  for (int z = 1; z < slices; ++z)  // Z V came in K-slices
+#pragma unroll
+    for (int u = 0; u < kRun / 4; ++u)
+      if (live) w[u] += p[(int64_t)z * g.m * kRun + 4 * u + q];
+#pragma unroll
+  for (int j = 0; j < kRun; ++j) {
+    const double x = __shfl_sync(0xffffffffu, w[j / 4], (lane & ~3) | (j & 3)) * s_tau[j];
+    if (q == (j & 3)) w[j / 4] = x;
+#pragma unroll
+    for (int u = j / 4; u < kRun / 4; ++u)
+      if (4 * u + q > j) w[u] = fma(-x, s_S[j * kRun + 4 * u + q], w[u]);
+  }
+  if (row < g.m)
+#pragma unroll
+    for (int u = 0; u < kRun / 4; ++u) p[4 * u + q] = w[u];
+}
+
+// Doubles of scratch a candidate block needs beside the sliced operands: V, S, W, tau; and, for every
+// form, the rows' norms and flags.
+int64_t run_doubles(int64_t m, int64_t r) { return kRun * r + kRun * kRun + kRunSlices * kRun * m + r + 64; }
 
 // ---- R, its inverse, the index sets -----------------------------------------------------------
 // R (rp x rp, row-major, upper triangular, selection order): R[c][k] = Z[order[k]][c] for c < k,
@@ -690,27 +901,98 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
   if ((st = run_product(q, R, Ly.blk - Ly.R, s)) != PIFA_OK) return st;
 
   // 2. r greedy steps
-  greedy_init<<<g.nblk, 256, 0, s>>>(g);
-  pifa_count_launch();
-  PIFA_CK(cudaGetLastError(), "compress: greedy init launch");
-  for (int k = 0; k < ri; ++k) {
-    cudaLaunchConfig_t cfg = {};
-    int threads = 0;
-    const GreedyStep step = greedy_form(ri - k, &threads, &cfg.dynamicSmemBytes);
-    if (cfg.dynamicSmemBytes > 32768 && (k == 0 || (ri - k) % 2048 == 0))
-      PIFA_CK(cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes),
-              "compress: greedy smem attribute");
-    cfg.gridDim = dim3((unsigned)g.nblk);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr;  // the next step's launch overlaps this step's tail
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    PIFA_CK(pifa_launch_ex(&cfg, step, g, k), "compress: greedy step launch");
+  g.ctl = reinterpret_cast<GreedyCtl*>(flags + 4);
+  auto run_steps = [&](int from, int to) {
+    for (int j = from; j < to; ++j) {
+      cudaLaunchConfig_t cfg = {};
+      int threads = 0;
+      const GreedyStep step = greedy_form(ri - j, &threads, &cfg.dynamicSmemBytes);
+      if (cfg.dynamicSmemBytes > 32768 &&
+          (e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes)) != cudaSuccess)
+        return pifa_fail_cuda("compress: greedy smem attribute", e);
+      cfg.gridDim = dim3((unsigned)g.nblk);
+      cfg.blockDim = dim3((unsigned)threads);
+      cfg.stream = s;
+      cudaLaunchAttribute attr;  // the next step's launch overlaps this step's tail
+      attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr.val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if ((e = pifa_launch_ex(&cfg, step, g, j, from)) != cudaSuccess)
+        return pifa_fail_cuda("compress: greedy step launch", e);
+    }
+    return (int)PIFA_OK;
+  };
+  // Candidate blocks: the norms and flags where R goes later, the sliced operands behind them, the
+  // small matrices where G and L were.
+  double* norms = R;
+  uint8_t* in_list = reinterpret_cast<uint8_t*>(norms + m);
+  uint8_t* slices = ws + Ly.R + a256(m * 9);
+  const int64_t slice_bytes = Ly.blk - Ly.R - a256(m * 9);
+  double *V_run = G, *S_run = V_run + kRun * r, *W_run = S_run + kRun * kRun, *tau_run = W_run + kRunSlices * kRun * m;
+  const bool runs = r >= 256 && slice_bytes > 0 && run_doubles(m, r) * 8 <= Ly.Z - Ly.G && m * r >= kRunFrom;
+  int k = 0, guess = kRun;
+  for (bool more = runs; more;) {
+    const bool block = (int64_t)(mi - k) * (ri - k) >= kRunFrom;  // else: every row, to the end
+    const int most = guess < kRun ? guess : kRun;  // a run's length changes slowly: few launches find it over
+    const int steps = block && ri - k > most ? most : ri - k;
+    g.tau = block ? tau_run : nullptr;
+    greedy_norms<<<4 * kGreedyBlocks, 256, 0, s>>>(g, k, norms);
+    pifa_count_launch();
+    greedy_select<<<1, 1024, 0, s>>>(g, k, norms, block ? kCandidates : 0, block ? in_list : nullptr);
+    pifa_count_launch();
+    PIFA_CK(cudaGetLastError(), "compress: greedy selection launch");
+    if ((st = run_steps(k, k + steps)) != PIFA_OK) return st;
+    if (!block) {
+      k = ri;
+      break;
+    }
+    GreedyCtl c = {};
+    PIFA_CK(cudaMemcpyAsync(&c, g.ctl, sizeof c, cudaMemcpyDeviceToHost, s), "compress: read back");
+    PIFA_CK(cudaStreamSynchronize(s), "compress: synchronize");
+    const int done = c.stop ? c.k_end - k : steps;
+    if (done <= 0 || done > steps) break;  // no step was sure: the rest exhaustively
+    if (!c.all) {  // the other rows take the run's reflectors
+      const int len = ri - k;
+      run_vectors<<<dim3((unsigned)((len + 255) / 256), kRun), 256, 0, s>>>(g, k, done, V_run);
+      pifa_count_launch();
+      run_gram<<<kRun * kRun / 8, 256, 0, s>>>(V_run, len, S_run);
+      pifa_count_launch();
+      GemmF64 w = {};  // W = Z V
+      w.M = mi; w.N = kRun; w.K = len;
+      w.A = Z + k; w.sa_i = r; w.sa_k = 1;
+      w.B = V_run; w.sb_k = 1; w.sb_j = len;
+      w.C = W_run; w.ldc = kRun; w.alpha = 1.0; w.beta = 0.0;
+      const int parts = gemm_f64_split_fits(w, slice_bytes) ? kRunSlices : 1;
+      st = parts > 1 ? gemm_f64_split(w, slices, slice_bytes, s, parts, m * kRun) : run_gemm_f64(w, 1, s);
+      if (st != PIFA_OK) return st;
+      run_substitute<<<(unsigned)((m + 31) / 32), 128, 0, s>>>(g, k, done, S_run, in_list, W_run, parts);
+      pifa_count_launch();
+      GemmF64 u = {};  // Z -= (W T) V^T
+      u.M = mi; u.N = len; u.K = kRun;
+      u.A = W_run; u.sa_i = kRun; u.sa_k = 1;
+      u.B = V_run; u.sb_k = len; u.sb_j = 1;
+      u.C = Z + k; u.ldc = r; u.alpha = -1.0; u.beta = 1.0;
+      if ((st = run_product(u, slices, slice_bytes, s)) != PIFA_OK) return st;
+      PIFA_CK(cudaGetLastError(), "compress: candidate block launch");
+    }
+    k += done;
+    guess = done + 8;
+    more = k < ri;
   }
-  PIFA_CK(cudaGetLastError(), "compress: greedy step launch");
+  if (k < ri) {  // every step over every row
+    g.tau = nullptr;
+    if (k == 0) {
+      greedy_init<<<g.nblk, 256, 0, s>>>(g);
+    } else {
+      greedy_norms<<<4 * kGreedyBlocks, 256, 0, s>>>(g, k, norms);
+      pifa_count_launch();
+      greedy_select<<<1, 1024, 0, s>>>(g, k, norms, 0, nullptr);
+    }
+    pifa_count_launch();
+    PIFA_CK(cudaGetLastError(), "compress: greedy init launch");
+    if ((st = run_steps(k, ri)) != PIFA_OK) return st;
+  }
 
   // 3. index sets, R, R^{-1}, C = Z[I^c] R^{-T} in ascending-I columns
   index_sets<<<1, 1024, 0, s>>>(g.sel, mi, g.order, ri, pivot_idx, has_np ? nonpivot_idx : pos, pos, asc);

@@ -97,6 +97,42 @@ __device__ __forceinline__ int row_exp(unsigned long long mx) {
   return e < 1 ? 1 : e;
 }
 
+// (hi 2^-36 + lo 2^-68) 2^e rounded to the nearest float64 (ties to even), in integer arithmetic: a
+// float64 instruction costs an SM as much issue time as some 30 integer ones.
+__device__ __forceinline__ double fixed_to_f64(long long hi, long long lo, int e) {
+  unsigned long long l = ((unsigned long long)hi << 32) + (unsigned long long)lo;  // hi 2^32 + lo, 128 bits
+  long long h = (hi >> 32) + (lo >> 63) + (l < (unsigned long long)lo ? 1 : 0);
+  const bool neg = h < 0;
+  if (neg) {
+    l = ~l + 1ull;
+    h = ~h + (l == 0ull ? 1 : 0);
+  }
+  unsigned long long m = (unsigned long long)h, rest = l;
+  int ex = 127;
+  if (m == 0ull) {
+    m = l;
+    rest = 0ull;
+    ex = 63;
+  }
+  if (m == 0ull) return 0.0;
+  const int lz = __clzll((long long)m);
+  ex -= lz;
+  if (lz) {
+    m = (m << lz) | (rest >> (64 - lz));
+    rest <<= lz;
+  }
+  const unsigned int low = (unsigned int)m & 0x7ffu;
+  m >>= 11;  // 53 bits
+  if (low > 0x400u || (low == 0x400u && (rest != 0ull || (m & 1ull)))) ++m;
+  const int be = ex - 68 + e + 1023;
+  double v;
+  if (be > 1 && be < 2045)
+    v = __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + m));
+  else
+    v = scalbn((double)m, be - 1023 - 52);
+  return neg ? -v : v;
+}
+
 // The 8 digits of one 32 x 32 block of values per CTA of 128 threads: loaded with the lanes along
 // the contiguous index, then 4 threads a row, 8 values and 8 x 16 bytes of digits each.
 __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
@@ -127,7 +163,7 @@ __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
     unsigned long long mag = 0;
     if (sh >= 0) mag = mant << sh;  // sh <= 9: ex <= er
     else if (sh > -60) mag = (mant + (1ull << (-sh - 1))) >> -sh;
-    if (er == 2047) mag = 0;  // the drain writes NaN for this row
+    if (er == 2047) mag = 0;  // the drain computes this row by plain_dot
     long long q = (b >> 63) ? -(long long)mag : (long long)mag;
 #pragma unroll
     for (int p = NDIG - 1; p >= 0; --p) {
@@ -146,15 +182,27 @@ __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
 // ---- the products --------------------------------------------------------------------------------
 struct SplitArgs {
   int M, N, kbase, K;  // this panel's columns [kbase, kbase + K) of the contraction
+  SliceArgs a, b;      // the panel's operands before slicing
   int tri, lower, first;
-  const unsigned long long *mxa, *mxb;
   double* C;
   const int32_t* cidx;
   int64_t ldc;
+  int64_t zc;  // elements between the partial results of consecutive K-slices (blockIdx.z)
   double alpha, beta;
   int* status;
   uint64_t timeout_ns;
 };
+
+// Element (i, j) over the panel's columns [k0, k1) by float64 multiply-adds: rows and columns that hold
+// an infinity or a NaN have no slices, and which elements they turn into which of the two is for the
+// arithmetic to say.
+__device__ __noinline__ double plain_dot(const SliceArgs& a, const SliceArgs& b, int i, int j, int k0, int k1) {
+  const double* x = a.X + (a.idx ? (int64_t)a.idx[i] : (int64_t)i) * a.s_row;
+  const double* y = b.X + (b.idx ? (int64_t)b.idx[j] : (int64_t)j) * b.s_row;
+  double s = 0.0;
+  for (int k = k0; k < k1; ++k) s = fma(x[(int64_t)k * a.s_k], y[(int64_t)k * b.s_k], s);
+  return s;
+}
 
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_f64_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
@@ -166,8 +214,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (p.tri & 4) ka = max(ka, m0);
   if (p.tri & 2) ke = min(ke, n0 + SN);
   const int kb0 = max(0, ka - p.kbase) / KBLK, kb1 = ke > p.kbase ? (ke - p.kbase + KBLK - 1) / KBLK : 0;
-  const int nst = max(0, kb1 - kb0);
+  const int nall = max(0, kb1 - kb0);
+  // this K-slice's stages (whole chunks, so that the last one of a slice is not cut short)
+  const int per = ((nall + CHUNK - 1) / CHUNK + (int)gridDim.z - 1) / (int)gridDim.z * CHUNK;
+  const int sb0 = kb0 + min(nall, (int)blockIdx.z * per), nst = min(nall, ((int)blockIdx.z + 1) * per) - (sb0 - kb0);
   if (nst == 0 && !p.first) return;
+  double* const Cz = p.C + blockIdx.z * p.zc;
   const int nch = (nst + CHUNK - 1) / CHUNK;
 
   extern __shared__ uint8_t smem_raw[];
@@ -216,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         uint8_t* sa = smem + s * STAGE;
         uint8_t* sb = sa + (NDIG / 2) * A_BOX;
-        const int x = (kb0 + it) * ROWLEN;
+        const int x = (sb0 + it) * ROWLEN;
         mbar_arrive_expect_tx(&full[s], STAGE);
         for (int q = 0; q < NDIG / 2; ++q) {
           tma_load_2d(smem_u32(sa + q * A_BOX), &tmA, x + 64 * q, m0, &full[s]);
@@ -307,23 +359,38 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (ok) {
       fence_proxy_async_smem();
       double* tile = reinterpret_cast<double*>(smem) + (warp - 2) * 32 * 33;
-#pragma unroll
-      for (int c = 0; c < 32; ++c)
-        tile[lane * 33 + c] = (double)hi[c] * 0x1p-36 + (double)lo[c] * 0x1p-68;
-      __syncwarp();
-      const int j = n0 + half * 32 + lane;
+      const int j = n0 + half * 32 + lane, r0 = m0 + q4 * 32, nr = min(32, p.M - r0);
       const bool jn = j < p.N;
-      const int eb = jn ? row_exp(p.mxb[j]) : 1;
-      const int64_t cj = jn ? (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j) : 0;
-#pragma unroll 4
-      for (int rr = 0; rr < 32; ++rr) {
-        const int i = m0 + q4 * 32 + rr;
-        if (i >= p.M || !jn) continue;
-        const int ea = row_exp(p.mxa[i]);
-        double v = tile[rr * 33 + lane];
-        v = (ea == 2047 || eb == 2047) ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(v, ea + eb - 2044);
-        double* c = p.C + (int64_t)i * p.ldc + cj;
-        *c = (p.beta != 0.0 ? p.beta * *c : 0.0) + p.alpha * v;
+      const int ea = lane < nr ? row_exp(p.a.mx[r0 + lane]) : 1, eb = jn ? row_exp(p.b.mx[j]) : 1;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        const int e2 = __shfl_sync(0xffffffffu, eb, c);
+        tile[lane * 33 + c] = fixed_to_f64(hi[c], lo[c], ea + e2 - 2044);
+      }
+      __syncwarp();
+      if (__any_sync(0xffffffffu, ea == 2047 || eb == 2047)) {
+        const int kc = (p.tri & 4) ? ((r0 & ~63) - p.kbase) : 0;  // a triangular A: from its rows' block of 64 on
+        const int c0 = max(sb0 * KBLK, kc), c1 = min(p.K, min((sb0 + nst) * KBLK, ke - p.kbase));
+        for (int g = 0; g < nr; ++g) {
+          const int e1 = __shfl_sync(0xffffffffu, ea, g);
+          if (jn && (e1 == 2047 || eb == 2047)) tile[g * 33 + lane] = plain_dot(p.a, p.b, r0 + g, j, c0, c1);
+        }
+      }
+      const bool neg = p.alpha == -1.0, one = neg || p.alpha == 1.0;
+      double* c = Cz + (int64_t)r0 * p.ldc + (jn ? (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j) : 0);
+      for (int g8 = 0; g8 < nr; g8 += 8) {
+        double old[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) old[u] = p.beta != 0.0 && jn && g8 + u < nr ? c[(int64_t)(g8 + u) * p.ldc] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (!jn || g8 + u >= nr) continue;
+          double v = tile[(g8 + u) * 33 + lane];
+          if (!one) v *= p.alpha;
+          else if (neg) v = -v;
+          if (p.beta != 0.0) v += p.beta == 1.0 ? old[u] : p.beta * old[u];
+          c[(int64_t)(g8 + u) * p.ldc] = v;
+        }
       }
     }
   }
@@ -366,7 +433,7 @@ bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes) {
          panel_bytes(p.M, p.N, p.K < 128 ? p.K : 128, same) <= bytes - 256;  // 256: alignment of the scratch
 }
 
-int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream) {
+int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream, int slices, int64_t zc) {
   cudaError_t e = cudaSuccess;
   int* status = pifa_status_word(&e);
   if (!status) return pifa_fail_cuda("device status word", e);
@@ -412,16 +479,17 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
     g.tri = p.tri;
     g.lower = p.lower;
     g.first = k0 == 0;
-    g.mxa = a.mx;
-    g.mxb = b.mx;
+    g.a = a;
+    g.b = b;
     g.C = p.C;
     g.cidx = p.cidx;
     g.ldc = p.ldc;
     g.alpha = p.alpha;
     g.beta = k0 == 0 ? p.beta : 1.0;
+    g.zc = zc;
     g.status = status;
     g.timeout_ns = pifa_wait_timeout_ns();
-    const dim3 grid((unsigned)((p.N + SN - 1) / SN), (unsigned)((p.M + SM_ - 1) / SM_));
+    const dim3 grid((unsigned)((p.N + SN - 1) / SN), (unsigned)((p.M + SM_ - 1) / SM_), (unsigned)slices);
     if (grid.y > 65535u) return pifa_fail(PIFA_ERR_UNSUPPORTED, "gemm_f64_split: more than 65535 row tiles");
     gemm_f64_split_kernel<<<grid, THREADS, SMEM, stream>>>(tA, tB, g);
     e = cudaGetLastError();

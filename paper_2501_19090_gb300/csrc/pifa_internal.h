@@ -162,9 +162,11 @@ struct GemmF64 {
   int lower;
 };
 // The same on the tensor cores by exact slices (no batch), in `bytes` of scratch:
-// whether that form takes the product, and the product.
+// whether that form takes the product, and the product. slices > 1: the contraction cut into that many
+// partial results, zc elements apart, each added to or stored in its own C, for the caller to add up
+// (products of few tiles).
 bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes);
-int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream);
+int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream, int slices = 1, int64_t zc = 0);
 
 // ---- prefill (prefill.cu) --------------------------------------------------------------------
 int64_t prefill_split_workspace_bytes(const PifaShape& s);

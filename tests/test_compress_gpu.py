@@ -152,3 +152,54 @@ def test_blocked_cholesky_edges_match_the_greedy_oracle(r):
     piv, nonp, Wp, C, _ = _device_compress(U, V)
     assert np.array_equal(piv, L.pivots) and np.array_equal(nonp, L.nonpivots)
     _check_eqs(U, V, piv, nonp, Wp, C)
+
+
+@pytest.mark.parametrize("m,n,r", [(7901, 300, 256), (3700, 700, 650), (2500, 1111, 1100)])
+@pytest.mark.parametrize("kind", ["plain", "twins", "nan"])
+def test_candidate_blocks_match_the_greedy_oracle(m, n, r, kind):
+    """Layers with 2e6 unchosen values of Z and more step over the rows of the largest norms and give
+    the others each block's reflectors at once. Rows that appear twice tie at every step (the first
+    copies must be chosen, in the order of the layer without the second ones); a row that holds a NaN
+    is never chosen and leaves every other row as it is."""
+    U, V, _ = inputs.make_factors(m, n, r, r)
+    keep = np.arange(m)
+    if kind == "twins":
+        U = np.concatenate([U, U[::-1]])
+    elif kind == "nan":
+        keep = np.delete(keep, 5)
+        U[5, 3] = np.nan
+    L = oracle.compress(U[keep], V, r, "lapack")
+    piv, nonp, Wp, C, info = _device_compress(U, V)
+    assert P.pifa_device_status() == P.PIFA_OK
+    assert np.array_equal(piv, keep[L.pivots])
+    assert P.pifa_validate_indices(piv, nonp, U.shape[0], r) == P.PIFA_OK
+    if kind == "nan":
+        assert np.isnan(C[np.searchsorted(nonp, 5)]).all()
+    _check_eqs(U, V, piv, nonp, Wp, C, rows=np.flatnonzero(nonp != 5)[:: 7])
+    assert 0 < info.r_ratio <= 1 and info.min_pivot_gap >= 0
+
+
+@pytest.mark.parametrize("m,n,r", [(7901, 300, 256), (300, 200, 77), (2500, 1111, 1100)])
+def test_an_infinity_in_u_does_what_float64_arithmetic_does(m, n, r):
+    """Z = U L with a triangular L: an infinity in the last column of U gives its row of Z infinities
+    only and with them an infinite norm, refused; in column 2 it meets L's zeros, and the row of NaN
+    that this makes is never chosen."""
+    U, V, _ = inputs.make_factors(m, n, r, 1)
+    U[7, r - 1] = np.inf
+    with pytest.raises(P.PifaError) as e:
+        _device_compress(U, V)
+    assert e.value.status == P.PIFA_ERR_RANK_DEFICIENT
+    U[7, r - 1], U[7, 2] = 0.0, np.inf
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert 7 in nonp and np.isnan(C[np.searchsorted(nonp, 7)]).all()
+    _check_eqs(U, V, piv, nonp, Wp, C, rows=np.flatnonzero(nonp != 7)[::7])
+
+
+def test_equal_norms_are_taken_from_the_lowest_index():
+    """Rows of +-1 on V = [I; 0] have exactly equal norms: no threshold separates the candidates."""
+    m, n, r = 3600, 620, 600
+    U = np.random.default_rng(0).integers(0, 2, (m, r)) * 2.0 - 1.0
+    V = np.eye(n, r)
+    piv, nonp, Wp, C, info = _device_compress(U, V)
+    assert piv[0] == 0 and info.min_pivot_gap == 0.0
+    _check_eqs(U, V, piv, nonp, Wp, C, rows=np.arange(0, nonp.size, 7))
