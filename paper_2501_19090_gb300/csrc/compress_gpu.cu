@@ -22,8 +22,8 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 25, Cholesky 4.0 and steps 37 of 71.5 ms. The M solves at m = n = 2048, r = 1024:
-// 141.5 -> 20.6 ms. No kernel waits on another CTA.
+// with their slices 25, Cholesky 2.2 and steps 37 of 69.3 ms. The M solves at m = n = 2048, r = 1024:
+// 141.5 -> 17.0 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -127,25 +127,66 @@ int run_product(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t s) 
 constexpr int CB = 32;    // columns per chol_panel
 constexpr int CP = 128;   // columns per panel
 
+constexpr int CR = 32;    // rows below the diagonal block per CTA of chol_panel
+
+// 1 / d for d > 0: the float32 reciprocal of d's significand, good to 2^-22, and one step of Halley's
+// third-order iteration r (1 + e + e^2), e = 1 - d r: three float64 instructions, of 64 cycles each for
+// a warp alone on its scheduler, where the division takes about ten.
+__device__ __forceinline__ double recip(double d) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+  const int ex = (int)(b >> 52);
+  if (ex < 64 || ex > 1982) return 1.0 / d;  // the scale below would leave the normal range
+  const float m = __uint_as_float(0x3f800000u | (uint32_t)((b >> 29) & 0x7fffffu));  // [1, 2)
+  const uint32_t q = __float_as_uint(__frcp_rn(m));                                   // (0.5, 1]
+  const unsigned long long rb =
+      ((unsigned long long)((int)(q >> 23) - 127 + 1023 - (ex - 1023)) << 52) | ((unsigned long long)(q & 0x7fffffu) << 29);
+  const double r = __longlong_as_double((long long)rb);
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // Columns [j0, j0 + CB) of L. Every CTA factors the 32 x 32 diagonal block itself (as U D U^T with
-// unit-lower U, so that a column's critical path is one reciprocal, one multiply-add and one
-// barrier), then a thread per row below it substitutes that row. A non-positive pivot flags `bad`
-// and leaves its column of L zero.
+// unit-lower U): the warp that holds column j + 1 finishes it first and takes its reciprocal while the
+// other three update the rest, so that a column's critical path is one multiply-add, one reciprocal,
+// one multiplication and one barrier. Then four lanes per row below it substitute that row. A
+// non-positive pivot flags `bad` and leaves its column of L zero.
+// Bound by the float64 pipe (one warp instruction per 64 cycles and scheduler). r = 2048: 45 -> 27 us
+// against a division per column in every warp and a thread per row.
 __global__ void __launch_bounds__(128) chol_panel(const double* G, double* L, int r, int j0, int* bad) {
-  __shared__ double D[CB][CB + 1];   // the block; column l of its lower part ends as d_l U[:, l]
+  __shared__ double D[CB][CB + 1];  // the block; column l of its lower part ends as d_l U[:, l]
+  __shared__ double U[CB][CB + 1];
   __shared__ double rd[CB], rs[CB];  // 1 / d_l and 1 / sqrt(d_l), 0 where d_l is not positive
   const int nb = min(CB, r - j0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = warp; i < CB; i += 4)
-    D[i][lane] = (i < nb && lane < nb) ? G[(int64_t)(j0 + i) * r + j0 + lane] : (i == lane ? 1.0 : 0.0);
+  // this lane's share of a row below: columns 4 u + lane % 4
+  const int64_t i = (int64_t)j0 + CB + (int64_t)blockIdx.x * CR + (threadIdx.x >> 2);
+  const int q = lane & 3;
+  double y[CB / 4];
+#pragma unroll
+  for (int u = 0; u < CB / 4; ++u) y[u] = i < r ? G[i * r + j0 + 4 * u + q] : 0.0;
+  for (int k = warp; k < CB; k += 4)
+    D[k][lane] = (k < nb && lane < nb) ? G[(int64_t)(j0 + k) * r + j0 + lane] : (k == lane ? 1.0 : 0.0);
+  __syncthreads();
+  if (warp == 0) {
+    const double d = D[0][0], inv = d > 0.0 ? recip(d) : 0.0;
+    if (lane == 0) rd[0] = inv;
+  }
   __syncthreads();
   for (int j = 0; j < CB; ++j) {
-    const double d = D[j][j];
-    const double inv = d > 0.0 ? 1.0 / d : 0.0;
-    const double f = D[lane][j] * inv;
-    if (threadIdx.x == 0) rd[j] = inv;
-    for (int l = j + 1 + ((warp - j - 1) & 3); l < CB; l += 4)
-      if (lane >= l) D[lane][l] = fma(-f, D[l][j], D[lane][l]);
+    const double f = D[lane][j] * rd[j];
+    if (warp == (j & 3)) {  // column j + 1 and its reciprocal; it has a warp to itself
+      U[lane][j] = f;
+      if (j + 1 < CB) {
+        const double x = fma(-f, D[j + 1][j], D[lane][j + 1]);
+        if (lane >= j + 1) D[lane][j + 1] = x;
+        const double d = __shfl_sync(0xffffffffu, x, j + 1), inv = d > 0.0 ? recip(d) : 0.0;
+        if (lane == 0) rd[j + 1] = inv;
+      }
+    } else {
+      const int w = (warp - j + 3) & 3;  // 0, 1, 2 among the others
+      for (int l = j + 2 + w; l < CB; l += 3)
+        if (lane >= l) D[lane][l] = fma(-f, D[l][j], D[lane][l]);
+    }
     __syncthreads();
   }
   if (warp == 0) {
@@ -153,49 +194,48 @@ __global__ void __launch_bounds__(128) chol_panel(const double* G, double* L, in
     rs[lane] = d > 0.0 ? 1.0 / sqrt(d) : 0.0;
     if (!(d > 0.0) && blockIdx.x == 0) atomicExch(bad, 1);
   }
-  __syncthreads();
-  if (blockIdx.x == 0)
-    for (int i = warp; i < nb; i += 4)
-      if (lane <= i) L[(int64_t)(j0 + i) * r + j0 + lane] = D[i][lane] * rs[lane];
-  const int64_t i = (int64_t)j0 + CB + (int64_t)blockIdx.x * 128 + threadIdx.x;
-  if (i >= r) return;
-  const double* g = G + i * r + j0;
-  double y[CB];
 #pragma unroll
-  for (int l = 0; l < CB; ++l) y[l] = g[l];
+  for (int l = 0; l < CB; ++l) {  // y_j -= y_l U_jl
+    const double x = __shfl_sync(0xffffffffu, y[l / 4], (lane & ~3) | (l & 3));
 #pragma unroll
-  for (int l = 0; l < CB; ++l) {  // y_j -= (y_l / d_l) (d_l U_jl)
-    const double f = y[l] * rd[l];
-#pragma unroll
-    for (int j = l + 1; j < CB; ++j) y[j] = fma(-f, D[j][l], y[j]);
+    for (int u = l / 4; u < CB / 4; ++u)
+      if (4 * u + q > l) y[u] = fma(-x, U[4 * u + q][l], y[u]);
   }
-  double* o = L + i * r + j0;
+  __syncthreads();
+  if (i < r) {
+    double* o = L + i * r + j0;
 #pragma unroll
-  for (int l = 0; l < CB; ++l) o[l] = y[l] * rs[l];
+    for (int u = 0; u < CB / 4; ++u) o[4 * u + q] = y[u] * rs[4 * u + q];
+  }
+  if (blockIdx.x == 0)
+    for (int k = warp; k < nb; k += 4)
+      if (lane <= k) L[(int64_t)(j0 + k) * r + j0 + lane] = D[k][lane] * rs[lane];
 }
 
 // G[i][l] -= sum over k in [j0, j0 + kn) of L[i][k] L[l][k] for l0 <= l < l1, i >= l (kn <= CB).
-// 64 x 32 tiles, 256 threads, 8 rows of one column each.
+// 16 x 32 tiles, 256 threads, 2 rows of one column each: bound by the float64 pipe of the SM that has
+// the most tiles (r = 2048: 22 -> 8.4 us against 64 x 32 tiles, fewer than SMs).
+constexpr int CU = 16;
 __global__ void __launch_bounds__(256) chol_update(double* G, const double* L, int r, int j0, int kn, int l0, int l1) {
-  __shared__ double A[64][CB + 1];
+  __shared__ double A[CU][CB + 1];
   __shared__ double B[CB][CB + 1];
-  const int i0 = l0 + blockIdx.y * 64, c0 = l0 + blockIdx.x * 32;
-  if (c0 > i0 + 63) return;  // wholly above the diagonal
+  const int i0 = l0 + blockIdx.y * CU, c0 = l0 + blockIdx.x * 32;
+  if (c0 > i0 + CU - 1) return;  // wholly above the diagonal
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int u = warp; u < 64; u += 8) A[u][lane] = (i0 + u < r && lane < kn) ? L[(int64_t)(i0 + u) * r + j0 + lane] : 0.0;
+  for (int u = warp; u < CU; u += 8) A[u][lane] = (i0 + u < r && lane < kn) ? L[(int64_t)(i0 + u) * r + j0 + lane] : 0.0;
   for (int u = warp; u < 32; u += 8) B[u][lane] = (c0 + u < l1 && lane < kn) ? L[(int64_t)(c0 + u) * r + j0 + lane] : 0.0;
   __syncthreads();
-  double acc[8] = {};
+  double acc[CU / 8] = {};
 #pragma unroll 8
   for (int k = 0; k < CB; ++k) {
     const double b = B[lane][k];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) acc[u] = fma(A[warp * 8 + u][k], b, acc[u]);
+    for (int u = 0; u < CU / 8; ++u) acc[u] = fma(A[warp * (CU / 8) + u][k], b, acc[u]);
   }
   const int l = c0 + lane;
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const int i = i0 + warp * 8 + u;
+  for (int u = 0; u < CU / 8; ++u) {
+    const int i = i0 + warp * (CU / 8) + u;
     if (i < r && l < l1 && i >= l) G[(int64_t)i * r + l] -= acc[u];
   }
 }
@@ -204,7 +244,7 @@ __global__ void __launch_bounds__(256) chol_update(double* G, const double* L, i
 int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t bytes, cudaStream_t s) {
   const int ri = (int)r;
   auto update = [&](int j0, int l0, int l1) {
-    const dim3 grid((unsigned)((l1 - l0 + 31) / 32), (unsigned)((ri - l0 + 63) / 64));
+    const dim3 grid((unsigned)((l1 - l0 + 31) / 32), (unsigned)((ri - l0 + CU - 1) / CU));
     chol_update<<<grid, 256, 0, s>>>(G, L, ri, j0, ri - j0 < CB ? ri - j0 : CB, l0, l1);
     pifa_count_launch();
   };
@@ -217,7 +257,7 @@ int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t b
     const bool split = t.M > 0 && gemm_f64_split_fits(t, bytes);
     for (int j0 = p0; j0 < p1; j0 += CB) {
       const int below = ri - j0 - CB;
-      chol_panel<<<below > 0 ? (unsigned)((below + 127) / 128) : 1u, 128, 0, s>>>(G, L, ri, j0, bad);
+      chol_panel<<<below > 0 ? (unsigned)((below + CR - 1) / CR) : 1u, 128, 0, s>>>(G, L, ri, j0, bad);
       pifa_count_launch();
       const int l1 = split ? p1 : ri;  // without the product, 32 columns at a time over everything
       if (j0 + CB < l1) update(j0, j0 + CB, l1);
