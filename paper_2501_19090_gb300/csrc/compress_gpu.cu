@@ -22,7 +22,7 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 25, Cholesky 2.2 and steps 37 of 69.3 ms. The M solves at m = n = 2048, r = 1024:
+// with their slices 20, Cholesky 2.2 and steps 38 of 65.4 ms. The M solves at m = n = 2048, r = 1024:
 // 141.5 -> 17.0 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const dou
     } else {
       hi = mid;
       th = mid;
-      if (n >= want - want / 4) break;
+      if (n >= want - want / 10) break;
     }
   }
   if (!all && (th < 0.0 || count_above(th) < want / 4)) all = true;
@@ -540,19 +540,22 @@ __global__ void __launch_bounds__(32 * kGreedyWarps<NREG, W>, 1) greedy_step(Gre
     const double alpha = -copysign(nx, x0 != 0.0 ? x0 : 1.0);
     if (threadIdx.x == 0) {
       v[0] = x0 - alpha;
-      s_tau = nx2 > 0.0 ? 1.0 / (nx2 + nx * fabs(x0)) : 0.0;
+      s_tau = nx2 > 0.0 ? recip(fma(nx, fabs(x0), nx2)) : 0.0;
       if (blockIdx.x == 0 && g.tau) g.tau[k] = s_tau;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       g.order[k] = p;
       g.rdiag[k] = alpha;
-      const double b2 = t.i2 >= 0 ? sqrt(__longlong_as_double((long long)t.v2)) : 0.0;
-      g.gap[k] = nx > 0.0 ? (nx - b2) / nx : 0.0;
       g.sel[p] = 1;          // read only by later launches
       g.act[t.s1] = tail;    // a row loaded early from that slot is loaded again below
     }
   }
   __syncthreads();
+  if (blockIdx.x == gridDim.x - 1 && warp == WARPS - 1) {  // the warp with the fewest rows
+    const double nx = sqrt(__longlong_as_double((long long)t.v1));
+    const double b2 = t.i2 >= 0 ? sqrt(__longlong_as_double((long long)t.v2)) : 0.0;
+    if (lane == 0) g.gap[k] = nx > 0.0 ? (nx - b2) / nx : 0.0;
+  }
   const double tau = s_tau;
   Top2 mine = top2_empty();
   for (int s = s0; s < n - 1; s += gridDim.x * GROUPS) {
@@ -623,9 +626,11 @@ GreedyStep greedy_form(int len, int* threads, size_t* smem) {
 // W = Z V (the compact WY form of Schreiber and Van Loan, 1989; T^-1 = diag(1 / tau) + the strictly upper
 // part of V^T V), as two products on the tensor cores and a substitution per row, and all norms are
 // recomputed. The pivots, and the order of every comparison that decides one, are those of the
-// exhaustive steps. 4096 x 4096, r = 2048: the call 86.1 -> 71.5 ms.
+// exhaustive steps. 4096 x 4096, r = 2048: the call 86.1 -> 67.8 ms.
 constexpr int kRun = 64;
-constexpr int kCandidates = 512;
+// Rows of a run: six for every SM. More make a run longer, fewer a step shorter: 65.3 ms of call at
+// 4096 x 4096, r = 2048; with 512 rows 69.0, 608 66.2, 760 65.9, 1216 66.2.
+constexpr int kCandidates = 912;
 constexpr int kRunSlices = 4;  // K-slices of Z V, whose tiles (128 rows each) are few
 // Values of Z left (unchosen rows x coordinates) from which on a candidate block pays.
 constexpr int64_t kRunFrom = 2000000;
