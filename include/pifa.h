@@ -370,9 +370,12 @@ int pifa_set_wait_timeout(int64_t ns);
  * slices in shared memory in a fixed order and writes the outputs itself (one kernel); a taller
  * phase deals equal ranges of 128 x 64 weight tiles to a persistent grid and a second kernel sums
  * the fp32 partial sums in a fixed order.
- * PIFA_DECODE_GRID_AUTO (0, the default) picks per phase from its shape and T: split-K when
- * T > 2 and R >= 4096 or T > 8 and the waves would need more CTAs than there are SMs, else waves
- * while the phase takes at most two of them, else the persistent grid. PIFA_DECODE_GRID_WAVES (1), PIFA_DECODE_GRID_PERSISTENT (2) and PIFA_DECODE_GRID_SPLITK
+ * PIFA_DECODE_GRID_AUTO (0, the default) picks per phase from its shape and T: waves while an SM can
+ * stage its share of the weights at launch (about 24 MB in phase 1, 12 MB in phase 2, at most two
+ * rounds); beyond, the persistent grid for T <= 2 and split-K for T > 2, which also takes a phase 1 of
+ * R >= 4096, and for T > 8 phases whose waves would need more CTAs than there are SMs. The waves' tile
+ * height (16, 32 or 64 rows) and K split follow from shape and T in every mode.
+ * PIFA_DECODE_GRID_WAVES (1), PIFA_DECODE_GRID_PERSISTENT (2) and PIFA_DECODE_GRID_SPLITK
  * (3) force one form for both phases (a tuning and test knob: all compute the same result up to
  * the summation order of fp32 partial sums; forced split-K runs the persistent grid instead when the
  * workspace is too small for its partial sums). For 16 < T <= 128 only the split-K form exists

@@ -8,7 +8,7 @@
 //                                                                     (Algorithm 2, steps 3 and 5)
 //
 // Both phases have one shape. A CTA owns a tile of 16 RG consecutive weight rows (RG m16 MMA row
-// groups; RG = 1 or 4 by token count) and a K range; a thread-block cluster of up to 8 CTAs
+// groups; RG = 1, 2 or 4 by shape and T) and a K range; a thread-block cluster of up to 8 CTAs
 // splits K when a tile's rows do not fit one stage, so each CTA reads only
 // its slice of the broadcast operand (x or y_p). Every CTA of the grid reads the whole broadcast
 // slice of its K range once, so taller tiles mean proportionally less of that L2 traffic, which
@@ -60,8 +60,7 @@ using bf16 = __nv_bfloat16;
 
 // Weight rows per CTA: RG MMA row groups of 16. Taller tiles read less of the broadcast operand
 // per weight byte (RG = 4 reads 4x less than RG = 1) but split K over larger clusters whose
-// partial tiles must be summed; RG = 1 (no cluster) wins at T <= 2, RG = 4 up to T = 8, RG = 2
-// with two token tiles.
+// partial tiles must be summed; rows_form chooses by the phase's shape and T.
 template <int RG>
 constexpr int kRowsOf = 16 * RG;
 constexpr int kChunk = 32;          // K elements per warp step (two k16 MMAs)
@@ -782,20 +781,27 @@ int launch_phase(Kern kernel, int rows, const DecodeArgs& args, size_t smem, cud
   return PIFA_OK;
 }
 
-// The K split and the stages of one phase: the fewest CTAs per cluster (1, 2, 4, 8) whose K range
-// fits one stage within `budget`; else 8 CTAs, each streaming its range through two stages.
-void plan_phase(int kRows, uint32_t budget, DecodeArgs& a) {
-  for (int ks = 1; ks <= kMaxCluster; ks *= 2) {
-    const int kcta = ((a.K + ks - 1) / ks + kChunk - 1) / kChunk * kChunk;
-    if ((uint64_t)kRows * row_pitch(kcta) <= budget) {
-      a.ks = ks;
-      a.kcta = a.kc = kcta;
-      a.stages = 1;
-      return;
-    }
+int kcta_of(int K, int ks) { return ((K + ks - 1) / ks + kChunk - 1) / kChunk * kChunk; }
+
+// The fewest CTAs per cluster (1, 2, 4, 8) whose K range of 16 rg rows fits one stage within
+// `budget`; 0 if none.
+int least_split(int rg, int K, uint32_t budget) {
+  for (int ks = 1; ks <= kMaxCluster; ks *= 2)
+    if ((uint64_t)(16 * rg) * row_pitch(kcta_of(K, ks)) <= budget) return ks;
+  return 0;
+}
+
+// The stages of one phase: the whole K range of one of ks CTAs; ks = 0: 8 CTAs, each streaming its
+// range through two stages.
+void plan_phase(int kRows, int ks, uint32_t budget, DecodeArgs& a) {
+  if (ks > 0) {
+    a.ks = ks;
+    a.kcta = a.kc = kcta_of(a.K, ks);
+    a.stages = 1;
+    return;
   }
   a.ks = kMaxCluster;
-  a.kcta = ((a.K + kMaxCluster - 1) / kMaxCluster + kChunk - 1) / kChunk * kChunk;
+  a.kcta = kcta_of(a.K, kMaxCluster);
   a.stages = 2;
   int kc = kChunk;
   while (kc + kChunk <= a.kcta && 2ull * kRows * row_pitch(kc + kChunk) <= budget) kc += kChunk;
@@ -849,8 +855,6 @@ int max_clusters(const void* fn, int ks, size_t smem, int threads = kWarps * 32)
 }
 
 std::atomic<int> g_decode_grid{PIFA_DECODE_GRID_AUTO};  // pifa_set_decode_grid
-
-int kcta_of(int K, int ks) { return ((K + ks - 1) / ks + kChunk - 1) / kChunk * kChunk; }
 
 int sm_count() {
   static int n = 0;
@@ -932,10 +936,6 @@ int launch_stream(Kern kernel, const CUtensorMap& tm, const CUtensorMap& tb0, co
   return PIFA_OK;
 }
 
-// One phase: decode_rows (16 RG-row tiles) or decode_stream (16 RGS-row tiles, over a TMA map of
-// the weights in their storage type `dtype`). The stream reads its B operand once per CTA, so its
-// tiles can be taller than decode_rows': 32 rows make 4 KB TMA boxes (2 KB boxes of 16 rows
-// issue too many copies per byte).
 // Scratch of the split-K tensor-core form (decode_tc.cu): where its partial sums go, and how many
 // bytes are available there.
 struct SplitKScratch {
@@ -973,9 +973,106 @@ int launch_phase_tc(const DecodeArgs& a, int dtype, const SplitKScratch& sk, cud
   return launch_decode_tc(ph, a.status, a.timeout_ns, stream);
 }
 
-template <int PHASE, int NT, bool kF16C, int RG, int RGS>
-int launch_one_phase(DecodeArgs& a, uint32_t budget, int dtype, const SplitKScratch& sk, cudaStream_t stream) {
+// ---- which form, by shape and T (T <= 16) ------------------------------------------------------
+// Measured over 27 layer shapes from 256 x 256 to 8192 x 8192 (ranks 0.12 to 0.75 of the smaller side,
+// grouped ones among them) and T = 1 to 16, weights from HBM, each pair of forms of the two phases
+// and each RG and K split of decode_rows that fits; us per layer below. Against one tile height per T
+// (16, 64 and 32 rows up to T = 2, 8 and 16), split-K for T > 2 from 4096 rows on and waves else:
+// 1024 x 1024, r = 512, T = 8: 6.4 -> 5.2; 4096 x 4096, r = 1024, T = 8: 9.2 -> 8.0; 4096 x 11008,
+// r = 1024, T = 3: 24.0 -> 10.2; 5120 x 5120, r = 2560, T = 8: 22.4 -> 16.9; over all of them 1.12x, none more than 2% slower.
+enum Form { kFormRows, kFormStream, kFormSplitK };
+struct PhasePlan {
+  Form form;
+  int rg, ks;  // decode_rows' tile height and K split; ks = 0: see plan_phase
+};
+
+// The tile height and K split of decode_rows for a phase of R rows and K columns. `other` is the other
+// phase's form; `first` (phase 2) phase 1's plan.
+PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan* first) {
+  const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
+  const int sms = sm_count();
+  const int64_t work = (int64_t)R * K;
+  const int k1 = least_split(1, K, budget), k2 = least_split(2, K, budget);
+  const int tiles = (R + 31) / 32, tall = (R + 63) / 64 * 4;  // 32-row tiles; CTAs of 64 rows split four ways
+  const bool fits4 = (uint64_t)64 * row_pitch(kcta_of(K, 4)) <= budget;
+  // 64 rows split four ways where that is one round of most SMs (in phase 2 behind such a phase 1,
+  // whose CTAs leave room for its own): 4096 x 4096, r = 2048, T = 8: 9.3, 32 rows split two ways 10.0
+  const bool behind = first && first->rg == 4 && first->ks == 4;
+  const bool round = fits4 && tall * 3 >= sms * 2 && (phase == 1 ? tall <= sms : behind && tall * 4 <= sms * 5);
+  if (T <= 2) {
+    if (phase == 1 && round && tall * 5 >= sms * 4 && other == kFormRows) return {kFormRows, 4, 4};  // T = 1: 8.9 -> 8.2
+    // x is short: 16 rows, unless the phase is so small that half the CTAs do, or K needs a split
+    const int rg = (work < (1 << 22) && k2 == 1) || k1 != 1 ? 2 : 1;
+    return {kFormRows, rg, rg == 2 ? k2 : k1};
+  }
+  if (T <= 8) {
+    if (round && other != kFormSplitK) return {kFormRows, 4, 4};
+    // several rounds of clusters of four: clusters of eight of the tall tiles read half of x
+    if (k2 == 4 && tiles * 16 > sms * 5 && least_split(4, K, budget) == 8) return {kFormRows, 4, 8};
+    // a small phase needs no more SMs, and a split-K phase behind this one wants the free ones
+    if (work < (1 << 22) || other == kFormSplitK) return {kFormRows, 2, k2};
+  } else {
+    if (work < (1 << 20)) return {kFormRows, 1, k1};
+    if (phase == 1 && round && other != kFormSplitK) return {kFormRows, 4, 4};
+  }
+  int ks = k2;
+  while (ks > 0 && ks < 4 && tiles * ks * 2 <= sms) ks *= 2;  // as many CTAs as make one round
+  return {kFormRows, 2, ks};
+}
+
+// The form of a phase. Waves of decode_rows win while an SM stages its share of the weights at launch
+// (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds.
+Form phase_form(int phase, int R, int K, int T, int ngrp) {
+  const int64_t bytes = (int64_t)R * K * 2;
+  const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
+  const int sms = sm_count();
+  if (phase == 2 && bytes <= 12000000) {
+    // with two token tiles a K split in more CTAs than SMs loses to split-K (4096 x 4096, r = 2458,
+    // T = 12: 15.8 against 15.0)
+    const int k2 = least_split(2, K, budget);
+    return T > 8 && k2 != 1 && (R + 31) / 32 * k2 > sms ? kFormSplitK : kFormRows;
+  }
+  if (T <= 2) {
+    // decode_stream, whose x / y_p stay resident (8192 x 8192, r = 2048, T = 1: 20.3 -> 18.0); a K of
+    // 1024 or less is too short for its ring (11008 x 4096, r = 1024: split-K 10.8, stream 12.1), and
+    // many groups' y_p split it over clusters (three of 4096 x 4096, r = 2048, T = 2: 24.0 against 21.4)
+    if (phase == 2 && R >= 32 * 128 && K <= 1024) return kFormSplitK;
+    if (ngrp > 1 && (uint64_t)ngrp * 2 * T * row_pitch(K) > kStreamBudget / 3) return kFormRows;
+    return phase == 2 || bytes > 26000000 ? kFormStream : kFormRows;
+  }
+  if (phase == 2 || R >= 32 * 128) return kFormSplitK;
+  const int k2 = least_split(2, K, budget);
+  if (T <= 8) {
+    // clusters of eight of 64 rows stay ahead for two rounds (8192 x 8192, r = 2048, T = 8: 20.8, split-K 21.5)
+    const bool two = k2 == 4 && least_split(4, K, budget) == 8 && (R + 63) / 64 * 8 <= 2 * sms;
+    return bytes > 26000000 && !two ? kFormSplitK : kFormRows;
+  }
+  // two token tiles: 4096 x 4096, r = 3072, T = 16: 18.9 -> 15.1; few row blocks keep split-K slow
+  // (4096 x 11008, r = 1024, T = 16: 16.7, waves 14.2)
+  return k2 == 0 || bytes > 24000000 || (R >= 2048 && (R + 31) / 32 * k2 > sms) ? kFormSplitK : kFormRows;
+}
+
+// decode_rows on one phase, if its clusters take at most two rounds (or `always`): its weights staged
+// at launch, before the dependency wait, then outweigh the persistent grid's streaming.
+template <int PHASE, int NT, bool kF16C, int RG>
+int launch_rows(DecodeArgs& a, int ks, uint32_t budget, bool always, cudaStream_t stream, const char* what, bool* taken) {
   constexpr int kRows = kRowsOf<RG>;
+  const auto kr = decode_rows<PHASE, NT, kF16C, RG>;
+  plan_phase(kRows, ks, budget, a);
+  const size_t smem = smem_bytes(kRows, a, NT);
+  const int st = prepare_kernel(reinterpret_cast<const void*>(kr), smem, what);
+  *taken = true;
+  if (st != PIFA_OK) return st;
+  const int tiles = (a.R + kRows - 1) / kRows;
+  if (always || tiles <= 2 * max_clusters(reinterpret_cast<const void*>(kr), a.ks, smem))
+    return launch_phase(kr, kRows, a, smem, stream, what);
+  *taken = false;
+  return PIFA_OK;
+}
+
+// One phase of T <= 128 tokens.
+template <int PHASE, int NT, bool kF16C>
+int launch_one_phase(DecodeArgs& a, uint32_t budget, int dtype, const SplitKScratch& sk, const PhasePlan& plan, cudaStream_t stream) {
   const char* what = PHASE == 1 ? "decode phase 1 launch" : "decode phase 2 launch";
   const int mode = g_decode_grid.load(std::memory_order_relaxed);
   const bool tc_fits = sk.P != nullptr && decode_tc_partial_bytes(a.R, a.K, a.T, PHASE == 1 ? 1 : 2) <= sk.bytes;
@@ -983,40 +1080,23 @@ int launch_one_phase(DecodeArgs& a, uint32_t budget, int dtype, const SplitKScra
     if (!tc_fits) return pifa_fail(PIFA_ERR_INVALID_ARG, "decode with T > 16 needs the split-K workspace");
     return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
   }
-  if (mode == PIFA_DECODE_GRID_SPLITK && tc_fits) return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
-  // Auto, keyed on the phase's shape and T (phase 1: r rows of K = n; phase 2: m - r rows of
-  // K = r): for T > 2 a phase of at least 32 blocks of 128 rows runs split-K on the tensor cores
-  // (decode_tc.cu); a shorter one gives the grid too few row blocks, so that each CTA's range
-  // spans many K-slices and the partial sums grow with them. Measured per phase, every
-  // combination of the three forms (us, T = 4 / 8 / 16):
-  //   70B gate/up 28672x8192 r4096 (4096 and 24576 rows): tc+tc 51.5 / 54.1 / 56.9, best of all
-  //   70B q/o     8192x8192 r4096  (4096 and 4096 rows):  tc+tc 27.6 / 27.1 / 28.9, best within 1%
-  //   7B gate     11008x4096 r2048 (2048 and 8960 rows):  waves+tc 16.1 / 17.5 / 20.8 (was 19.0 /
-  //                                                       19.5 / 21.1 in waves+waves)
-  //   7B down     4096x11008 r2048 (2048 and 2048 rows):  stream+waves 18.9 / 19.1 / 22.6 (was
-  //                                                       21.4 / 22.3 / 22.3 with phase 1 on tc)
-  //   7B attn     4096x4096 r2048  (2048 and 2048 rows):  waves+waves 8.6 / 8.7 / 13.0
-  // For T <= 2 decode_stream's resident x / y_p and short loop win (70B gate/up, T = 1: 46.9
-  // against 51.7 us on the tensor cores).
-  if (mode == PIFA_DECODE_GRID_AUTO && a.T > 2 && a.R >= 32 * 128 && tc_fits)
-    return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
-  const auto kr = decode_rows<PHASE, NT, kF16C, RG>;
-  plan_phase(kRows, budget, a);
-  const size_t smem = smem_bytes(kRows, a, NT);
-  int st = prepare_kernel(reinterpret_cast<const void*>(kr), smem, what);
-  if (st != PIFA_OK) return st;
-  // decode_rows in waves while a phase takes at most two of them (its weights staged at launch,
-  // before the dependency wait, outweigh the persistent grid's streaming); else decode_stream
-  const int tiles = (a.R + kRows - 1) / kRows;
-  // For T > 8 (two token tiles) a phase whose waves need more CTAs than there are SMs is faster in
-  // split-K whatever its rows: 4096 x 11008, r = 2048 (512 and 256 CTAs) T = 16 22.5 -> 19.5 us,
-  // 4096 x 4096, r = 3072 (192 and 128 CTAs) 18.9 -> 15.6; one CTA per SM stays with waves (4096 x
-  // 4096, r = 2048: 13.2 against 14.5). Up to T = 8 the two are within 2%.
-  if (mode == PIFA_DECODE_GRID_AUTO && a.T > 8 && tc_fits && tiles * a.ks > sm_count())
-    return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
-  if (mode == PIFA_DECODE_GRID_WAVES ||
-      (mode == PIFA_DECODE_GRID_AUTO && tiles <= 2 * max_clusters(reinterpret_cast<const void*>(kr), a.ks, smem)))
-    return launch_phase(kr, kRows, a, smem, stream, what);
+  const Form form = mode == PIFA_DECODE_GRID_WAVES        ? kFormRows
+                    : mode == PIFA_DECODE_GRID_PERSISTENT ? kFormStream
+                    : mode == PIFA_DECODE_GRID_SPLITK     ? kFormSplitK
+                                                          : plan.form;
+  if (form == kFormSplitK && tc_fits) return launch_phase_tc<PHASE, kF16C>(a, dtype, sk, stream);
+  int st = PIFA_OK;
+  if (form == kFormRows || (mode == PIFA_DECODE_GRID_AUTO && form == kFormSplitK)) {  // (without its scratch)
+    const bool always = mode == PIFA_DECODE_GRID_WAVES;
+    bool taken = false;
+    st = plan.rg == 1   ? launch_rows<PHASE, NT, kF16C, 1>(a, plan.ks, budget, always, stream, what, &taken)
+         : plan.rg == 2 ? launch_rows<PHASE, NT, kF16C, 2>(a, plan.ks, budget, always, stream, what, &taken)
+                        : launch_rows<PHASE, NT, kF16C, 4>(a, plan.ks, budget, always, stream, what, &taken);
+    if (taken) return st;
+  }
+  // The stream reads its B operand once per CTA; its tiles of 32 rows make 4 KB TMA boxes (2 KB boxes
+  // of 16 rows issue too many copies per byte).
+  constexpr int RGS = 2;
   const auto ks = decode_stream<PHASE, NT, kF16C, RGS>;
   const size_t smem_s =
       plan_stream(reinterpret_cast<const void*>(ks), kRowsOf<RGS>, NT, PHASE == 1 ? 1 : 2, a, what, &st);
@@ -1035,7 +1115,7 @@ int64_t decode_planes_bytes(const PifaShape& s) {
   return ((s.T * ((s.groups * s.r + 7) / 8 * 8) * 4 + 255) / 256) * 256;
 }
 
-template <int NT, bool kF16C, int RG, int RGS>
+template <int NT, bool kF16C>
 int launch_decode_t(const PifaShape& s, const PifaPointers& p, int* status, cudaStream_t stream) {
   const int64_t G = s.groups;                      // layers sharing X (1: one layer)
   const int64_t ldyp = (G * s.r + 7) / 8 * 8;  // 16-byte rows keep the fragment loads aligned
@@ -1065,7 +1145,11 @@ int launch_decode_t(const PifaShape& s, const PifaPointers& p, int* status, cuda
   a.T = (int)s.T;
   a.status = status;
   a.timeout_ns = pifa_wait_timeout_ns();
-  int st = launch_one_phase<1, NT, kF16C, RG, RGS>(a, kStageBudget1, PIFA_DTYPE_BF16, sk, stream);
+  const int R2 = (int)(G * (s.m - s.r)), K2 = (int)s.r, T = a.T;
+  const Form f1 = phase_form(1, a.R, a.K, T, 1), f2 = R2 > 0 ? phase_form(2, R2, K2, T, (int)G) : kFormRows;
+  PhasePlan plan1 = plan_rows(1, a.R, a.K, T, f2, nullptr);
+  plan1.form = f1;
+  int st = launch_one_phase<1, NT, kF16C>(a, kStageBudget1, PIFA_DTYPE_BF16, sk, plan1, stream);
   if (st != PIFA_OK || s.m == s.r) return st;
   DecodeArgs b = a;
   b.A = reinterpret_cast<const uint16_t*>(p.C);
@@ -1083,7 +1167,9 @@ int launch_decode_t(const PifaShape& s, const PifaPointers& p, int* status, cuda
   }
   b.yph = b.ypl = nullptr;
   b.cols = p.nonpiv;
-  return launch_one_phase<2, NT, kF16C, RG, RGS>(b, kStageBudget2, (int)s.c_dtype, sk, stream);
+  PhasePlan plan2 = plan_rows(2, R2, K2, T, f1, f1 == kFormRows ? &plan1 : nullptr);
+  plan2.form = f2;
+  return launch_one_phase<2, NT, kF16C>(b, kStageBudget2, (int)s.c_dtype, sk, plan2, stream);
 }
 
 }  // namespace
@@ -1110,14 +1196,8 @@ int64_t decode_workspace_bytes(const PifaShape& s) {
 
 int launch_decode(const PifaShape& s, const PifaPointers& p, int* status, cudaStream_t stream) {
   const bool f16 = s.c_dtype == PIFA_DTYPE_FP16;
-  // Tile height by token count (measured on the 4096 x 4096, r = 2048 layer): 16 rows for T <= 2,
-  // 64 rows for T <= 8, 32 rows for T <= 16 (two token tiles).
-  // Persistent-grid tiles (layers beyond two waves): 32 rows (4 KB TMA boxes) at any T.
-  if (s.T <= 2)
-    return f16 ? launch_decode_t<1, true, 1, 2>(s, p, status, stream) : launch_decode_t<1, false, 1, 2>(s, p, status, stream);
-  if (s.T <= 8)
-    return f16 ? launch_decode_t<1, true, 4, 2>(s, p, status, stream) : launch_decode_t<1, false, 4, 2>(s, p, status, stream);
-  return f16 ? launch_decode_t<2, true, 2, 2>(s, p, status, stream) : launch_decode_t<2, false, 2, 2>(s, p, status, stream);
+  if (s.T <= 8) return f16 ? launch_decode_t<1, true>(s, p, status, stream) : launch_decode_t<1, false>(s, p, status, stream);
+  return f16 ? launch_decode_t<2, true>(s, p, status, stream) : launch_decode_t<2, false>(s, p, status, stream);
 }
 
 // ---- allocation-free decode entry point -------------------------------------------------------

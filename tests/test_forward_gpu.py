@@ -766,17 +766,35 @@ def test_grouped_prefill_groups_end_inside_a_pair_tile(T):
 
 def test_decode_selector_splits_k_where_waves_exceed_the_sms():
     """For T > 8 a phase whose waves would take more CTAs than the GPU has SMs runs split-K, whatever
-    its rows (here 3072 per phase): bit for bit the forced form; at T = 8 the same layer keeps waves."""
+    its rows (here 3072 per phase): bit for bit the forced form."""
     L = layer_for(6144, 4096, 3072, 6, "synthetic")
-    for T, forced in ((9, P.PIFA_DECODE_GRID_SPLITK), (16, P.PIFA_DECODE_GRID_SPLITK), (8, P.PIFA_DECODE_GRID_WAVES)):
+    for T in (9, 16):
         X = acts(T, 4096, 6)
         auto = run(L, X, P.PIFA_VARIANT_DECODE)
         check(auto, oracle.forward(X, L.Wp, L.C, L.pivots, L.nonpivots), f"T={T}")
-        P.pifa_set_decode_grid(forced)
+        P.pifa_set_decode_grid(P.PIFA_DECODE_GRID_SPLITK)
         try:
             assert np.array_equal(auto, run(L, X, P.PIFA_VARIANT_DECODE)), T
         finally:
             P.pifa_set_decode_grid(P.PIFA_DECODE_GRID_AUTO)
+
+
+@pytest.mark.parametrize("m,n,r,Ts", [
+    (513, 250, 130, (1, 2, 3, 8, 9, 16)),    # 32 rows, no split; 16 rows from T = 9 on
+    (4096, 4096, 2048, (1, 2)),              # 64 rows split four ways, then 16 rows
+    (4096, 4100, 2010, (9, 16)),             # 64 and 32 rows at two token tiles, ragged
+    (4000, 4090, 1001, (3, 8, 9, 16)),       # 32 rows, the split raised to four; ragged tiles and K
+    (2300, 8202, 1545, (3, 8, 9)),           # 64 rows split eight ways; split-K at T = 9
+    (1700, 11003, 611, (1, 3, 8, 16)),       # 32 rows split eight ways
+    (5121, 2569, 2560, (1, 2, 3, 8)),        # 13 MB of C: persistent grid, then split-K
+    (9003, 1030, 515, (1, 8, 16)),           # many rows of a short K: waves, several CTAs per SM
+])
+def test_decode_plans_by_shape(m, n, r, Ts):
+    """Every tile height and K split that the plan of a phase can take, and both sides of its lines."""
+    L = layer_for(m, n, r, 8, "synthetic")
+    for T in Ts:
+        X = acts(T, n, 8)
+        check(run(L, X, P.PIFA_VARIANT_DECODE), oracle.forward(X, L.Wp, L.C, L.pivots, L.nonpivots), f"T={T}")
 
 
 def test_binding_refuses_bad_cuda_operands_before_the_library():
