@@ -22,8 +22,8 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 20, Cholesky 2.2 and steps 38 of 65.4 ms. The M solves at m = n = 2048, r = 1024:
-// 141.5 -> 17.0 ms. No kernel waits on another CTA.
+// with their slices 15, Cholesky 2.2 and steps 38 of 59.8 ms. The M solves at m = n = 2048, r = 1024:
+// 141.5 -> 13.2 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 

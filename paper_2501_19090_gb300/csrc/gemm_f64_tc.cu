@@ -19,11 +19,14 @@
 // holds two digits of one K block as one 128-byte swizzled row.
 //
 // One CTA per 128 x 64 output tile, 320 threads: warp 0 the TMA producer (two 96 KB stages of one K
-// block: 8 digits of 128 rows of A and 64 of B), warp 1 the MMA issuer (36 digit pairs x 2
-// instructions of M = 128, N = 64, K = 16 per stage, accumulators d = 0 .. 7 of 64 columns: all
-// 512 columns of tensor memory), warps 2-9 the drain. Within a stage the MMAs run in order of d and
-// each accumulator is committed and released by itself, so that the drain of one K = 128 chunk
-// overlaps the MMAs of the next. Every wait is bounded.
+// block: 8 digits of 128 rows of A and 64 of B), warp 1 the MMA issuer (accumulators d = 0 .. 7 of 64
+// columns: all 512 columns of tensor memory; a digit of A times up to four digits of B in one
+// instruction of M = 128, N = 64 to 256, K = 16: 30 instructions a stage for the 36 digit pairs), warps
+// 2-9 the drain. In the last stage of a K = 128 chunk accumulator i is complete, and committed by
+// itself, after A's digit i, so that most of the drain runs under the chunk's own MMAs. Every wait is
+// bounded. 2048 x 2048 x 2048: 645 -> 302 us against one N = 64 instruction per pair (each 66 cycles, of
+// which its multiply-adds are 33), 2.0 PFLOP/s of the tensor cores; feeding those from a pair of CTAs
+// changed nothing (641).
 #include <cuda_bf16.h>
 
 #include "pifa.h"
@@ -46,6 +49,8 @@ constexpr int DRAIN_WARPS = 8;
 constexpr int THREADS = 64 + 32 * DRAIN_WARPS;
 constexpr size_t SMEM = 1024 + STAGES * STAGE + 256;
 constexpr uint32_t TMEM_COLS = NDIG * SN;  // 512
+// First column of accumulator d: the even ones, then the odd ones (see the MMA issuer).
+__host__ __device__ constexpr uint32_t acc_col(int d) { return (uint32_t)((d & 1) * (NDIG / 2) + (d >> 1)) * SN; }
 
 // ---- slicing -----------------------------------------------------------------------------------
 struct SliceArgs {
@@ -282,7 +287,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(SM_, SN);
+      // A digit i times the even digits of B is one MMA: box q of B holds digits 2 q and 2 q + 1 side by
+      // side, so every second digit is 64 rows further on, and accumulators i, i + 2, .. are
+      // adjacent columns; and so the odd digits. An MMA costs at least the 64 cycles of reading its
+      // 128 rows of A: 36 pairs one by one took twice the time of their multiply-adds.
       bool dead = false;
       for (int it = 0; it < nst && !dead; ++it) {
         const int s = it % STAGES, ch = it / CHUNK, w = it % CHUNK;
@@ -293,24 +301,25 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         tc_fence_after();
         const uint32_t a = smem_u32(smem + s * STAGE), b = a + (NDIG / 2) * A_BOX;
-        for (int d = 0; d < NDIG; ++d) {
-          if (w == 0 && ch > 0) {  // the drain has taken this accumulator's last chunk
-            if (!mbar_wait(&acce[d], (uint32_t)(ch - 1) & 1u, p.timeout_ns)) {
-              dead = true;
-              break;
-            }
-            tc_fence_after();
+        for (int d = 0; w == 0 && ch > 0 && d < NDIG; ++d)  // the drain has taken the last chunk
+          if (!mbar_wait(&acce[d], (uint32_t)(ch - 1) & 1u, p.timeout_ns)) {
+            dead = true;
+            break;
           }
-          for (int i = 0; i <= d; ++i) {
-            const int j = d - i;
-            const uint32_t pa = a + (uint32_t)(i >> 1) * A_BOX + (uint32_t)(i & 1) * 64u;
-            const uint32_t pb = b + (uint32_t)(j >> 1) * B_BOX + (uint32_t)(j & 1) * 64u;
+        if (dead) break;
+        tc_fence_after();
 #pragma unroll
-            for (int kk = 0; kk < KBLK / 16; ++kk)
-              mma_bf16_ss(tmem + (uint32_t)(d * SN), sw128_desc(pa + kk * 32), sw128_desc(pb + kk * 32), idesc,
-                          (w > 0 || i > 0 || kk > 0) ? 1u : 0u);
+        for (int i = 0; i < NDIG; ++i) {
+          const uint32_t pa = a + (uint32_t)(i >> 1) * A_BOX + (uint32_t)(i & 1) * 64u;
+          const uint32_t even = idesc_bf16_f32(SM_, SN * ((NDIG + 1 - i) / 2)), odd = idesc_bf16_f32(SM_, SN * ((NDIG - i) / 2));
+#pragma unroll
+          for (int kk = 0; kk < KBLK / 16; ++kk) {
+            const uint32_t acc = (w > 0 || i > 0 || kk > 0) ? 1u : 0u;
+            mma_bf16_ss(tmem + acc_col(i), sw128_desc(pa + kk * 32), sw128_desc(b + kk * 32), even, acc);
+            if (i + 1 < NDIG)
+              mma_bf16_ss(tmem + acc_col(i + 1), sw128_desc(pa + kk * 32), sw128_desc(b + 64u + kk * 32), odd, acc);
           }
-          if (last) mma_commit(&accf[d]);
+          if (last) mma_commit(&accf[i]);  // accumulator i has no terms of the later digits of A
         }
         mma_commit(&empty[s]);
       }
@@ -340,7 +349,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!ok) break;
         tc_fence_after();
         uint32_t v[32];
-        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(d * SN + half * 32), v);
+        tmem_ld_32x32b_x32(tmem + ((uint32_t)(q4 * 32) << 16) + acc_col(d) + (uint32_t)(half * 32), v);
         tmem_ld_wait();
         tc_fence_before();
         __syncwarp();
