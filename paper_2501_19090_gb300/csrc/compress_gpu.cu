@@ -22,8 +22,8 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 15, Cholesky 2.2 and steps 38 of 59.8 ms. The M solves at m = n = 2048, r = 1024:
-// 141.5 -> 13.2 ms. No kernel waits on another CTA.
+// with their slices 15, Cholesky 2.2 and steps 38 of 59.6 ms. The M solves at m = n = 2048, r = 1024:
+// 141.3 -> 12.1 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -40,9 +40,16 @@ using namespace pifa;
 
 
 // ---- float64 GEMM on the CUDA cores (GemmF64 in pifa_internal.h): small products ------------
-constexpr int GT = 64, GK = 16;  // output tile 64 x 64, k step 16; 256 threads, 4 x 4 outputs each
+// GT x GT output tiles, K step 16; 256 threads of (GT / 16)^2 outputs each. Tiles of 32 where those of
+// 64 are fewer than the SMs, each bound by its SM's float64 pipe (a tile of 64 and K = 128: 130 us): the
+// levels of a triangular inverse below 256, r = 1024 or 2048: 86 -> 25 us a launch.
+constexpr int GK = 16;
+constexpr int kSms = 152;
+constexpr int kZeroBlock = 64;  // triangular operands: zeros are skipped in blocks of 64, whatever the tile
 
+template <int GT>
 __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
+  constexpr int U = GT / 16;
   __shared__ double As[GK][GT + 1];
   __shared__ double Bs[GK][GT + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -52,10 +59,11 @@ __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
   double* C = p.C + blockIdx.z * p.zc;
   if (p.lower && j0 > i0 + GT - 1) return;
   int kbeg = 0, kend = p.K;
-  if (p.tri & 1) kbeg = (j0 / GK) * GK;
-  if (p.tri & 4) kbeg = max(kbeg, (i0 / GK) * GK);
-  if (p.tri & 2) kend = min(p.K, j0 + GT);
-  double acc[4][4] = {};
+  const int ib = i0 / kZeroBlock * kZeroBlock, jb = j0 / kZeroBlock * kZeroBlock;
+  if (p.tri & 1) kbeg = jb;
+  if (p.tri & 4) kbeg = max(kbeg, ib);
+  if (p.tri & 2) kend = min(p.K, jb + kZeroBlock);
+  double acc[U][U] = {};
   for (int k0 = kbeg; k0 < kend; k0 += GK) {
     for (int e = threadIdx.x; e < GT * GK; e += 256) {
       const int ii = e % GT, kk = e / GT;  // consecutive threads: consecutive rows of the A tile
@@ -74,25 +82,25 @@ __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
+      double a[U], b[U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < U; ++u) {
         a[u] = As[kk][ty + 16 * u];
         b[u] = Bs[kk][tx + 16 * u];
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+        for (int v = 0; v < U; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int i = i0 + ty + 16 * u;
     if (i >= p.M) continue;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < U; ++v) {
       const int j = j0 + tx + 16 * v;
       if (j >= p.N) continue;
       double* c = C + (int64_t)i * p.ldc + (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j);
@@ -103,8 +111,10 @@ __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
 
 int run_gemm_f64(const GemmF64& p, int batch, cudaStream_t s) {
   if (p.M <= 0 || p.N <= 0 || batch <= 0) return PIFA_OK;
-  dim3 grid((unsigned)((p.N + GT - 1) / GT), (unsigned)((p.M + GT - 1) / GT), (unsigned)batch);
-  gemm_f64<<<grid, 256, 0, s>>>(p);
+  const auto grid = [&](int gt) { return dim3((unsigned)((p.N + gt - 1) / gt), (unsigned)((p.M + gt - 1) / gt), (unsigned)batch); };
+  const int64_t tiles = (int64_t)((p.N + 63) / 64) * ((p.M + 63) / 64) * batch;
+  if (tiles < kSms) gemm_f64<32><<<grid(32), 256, 0, s>>>(p);
+  else gemm_f64<64><<<grid(64), 256, 0, s>>>(p);
   pifa_count_launch();
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? PIFA_OK : pifa_fail_cuda("compress: gemm launch", e);
