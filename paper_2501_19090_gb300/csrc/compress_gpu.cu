@@ -22,8 +22,8 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 15, Cholesky 2.2 and steps 38 of 59.6 ms. The M solves at m = n = 2048, r = 1024:
-// 141.3 -> 12.1 ms. No kernel waits on another CTA.
+// with their slices 15, Cholesky 2.2 and steps 38 of 58.9 ms. The M solves at m = n = 2048, r = 1024:
+// 141.4 -> 11.7 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -798,8 +798,9 @@ __global__ void max_abs(const double* C, int64_t rows, int64_t cols, int64_t ldc
 // Rinv = R^{-1} for an upper-triangular R (rp x rp, rp = 32 * 2^k; identity on any padding), by
 // doubling: the 32 x 32 diagonal blocks inverted directly, then, level by level, for every pair
 // of sz-blocks [[A, B], [0, D]] along the diagonal the off-diagonal block -A^{-1} (B D^{-1}).
-// Tt: scratch of rp * rp / 4 doubles; `scratch` for the sliced operands of the levels from 256 on
-// (below, all pairs of a level go in one batched launch on the CUDA cores).
+// Tt: scratch of rp * rp / 4 doubles; `scratch` for the sliced operands of the levels from 512 on
+// (below, all pairs of a level go in one batched launch on the CUDA cores: 256-blocks, r = 2048, eight
+// products 260 us in two launches, one by one in slices 376).
 int upper_inverse(const double* R, double* Rinv, double* Tt, int rp, void* scratch, int64_t bytes, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(Rinv, 0, (size_t)rp * rp * 8, s);
   if (e != cudaSuccess) return pifa_fail_cuda("upper inverse: memset", e);
@@ -823,7 +824,7 @@ int upper_inverse(const double* R, double* Rinv, double* Tt, int rp, void* scrat
     b.B = Tt; b.sb_k = sz; b.sb_j = 1;
     b.C = Rinv + sz; b.ldc = rp; b.alpha = -1.0; b.beta = 0.0; b.tri = 4;
     b.za = step; b.zb = (int64_t)sz * sz; b.zc = step;
-    if (sz < 256 || !gemm_f64_split_fits(a, bytes) || !gemm_f64_split_fits(b, bytes)) {
+    if (sz < 512 || !gemm_f64_split_fits(a, bytes) || !gemm_f64_split_fits(b, bytes)) {
       if ((st = run_gemm_f64(a, pairs, s)) != PIFA_OK || (st = run_gemm_f64(b, pairs, s)) != PIFA_OK) return st;
       continue;
     }
