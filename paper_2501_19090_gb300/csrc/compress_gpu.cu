@@ -23,7 +23,7 @@
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
 // with their slices 15, Cholesky 2.2 and steps 38 of 58.9 ms. The M solves at m = n = 2048, r = 1024:
-// 141.4 -> 11.7 ms. No kernel waits on another CTA.
+// 141.4 -> 11.3 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -166,6 +166,8 @@ __global__ void __launch_bounds__(128) chol_panel(const double* G, double* L, in
   __shared__ double D[CB][CB + 1];  // the block; column l of its lower part ends as d_l U[:, l]
   __shared__ double U[CB][CB + 1];
   __shared__ double rd[CB], rs[CB];  // 1 / d_l and 1 / sqrt(d_l), 0 where d_l is not positive
+  pdl_launch_dependents();
+  pdl_wait_primary();
   const int nb = min(CB, r - j0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // this lane's share of a row below: columns 4 u + lane % 4
@@ -230,6 +232,8 @@ __global__ void __launch_bounds__(256) chol_update(double* G, const double* L, i
   __shared__ double A[CU][CB + 1];
   __shared__ double B[CB][CB + 1];
   const int i0 = l0 + blockIdx.y * CU, c0 = l0 + blockIdx.x * 32;
+  pdl_launch_dependents();
+  pdl_wait_primary();
   if (c0 > i0 + CU - 1) return;  // wholly above the diagonal
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int u = warp; u < CU; u += 8) A[u][lane] = (i0 + u < r && lane < kn) ? L[(int64_t)(i0 + u) * r + j0 + lane] : 0.0;
@@ -253,10 +257,19 @@ __global__ void __launch_bounds__(256) chol_update(double* G, const double* L, i
 // L (zeroed by the caller, pitch r) = the Cholesky factor of G; `scratch` for the sliced panels.
 int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t bytes, cudaStream_t s) {
   const int ri = (int)r;
-  auto update = [&](int j0, int l0, int l1) {
-    const dim3 grid((unsigned)((l1 - l0 + 31) / 32), (unsigned)((ri - l0 + CU - 1) / CU));
-    chol_update<<<grid, 256, 0, s>>>(G, L, ri, j0, ri - j0 < CB ? ri - j0 : CB, l0, l1);
-    pifa_count_launch();
+  cudaError_t e = cudaSuccess;
+  // each launch under the tail of the one before (224 launches of the M solves at n = 2048: 11.7 -> 11.3 ms)
+  auto launch = [&](auto kernel, dim3 grid, int threads, auto... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (e == cudaSuccess) e = pifa_launch_ex(&cfg, kernel, args...);
   };
   for (int p0 = 0; p0 < ri; p0 += CP) {
     const int p1 = p0 + CP < ri ? p0 + CP : ri;
@@ -267,12 +280,13 @@ int cholesky(double* G, double* L, int64_t r, int* bad, void* scratch, int64_t b
     const bool split = t.M > 0 && gemm_f64_split_fits(t, bytes);
     for (int j0 = p0; j0 < p1; j0 += CB) {
       const int below = ri - j0 - CB;
-      chol_panel<<<below > 0 ? (unsigned)((below + CR - 1) / CR) : 1u, 128, 0, s>>>(G, L, ri, j0, bad);
-      pifa_count_launch();
+      launch(chol_panel, dim3(below > 0 ? (unsigned)((below + CR - 1) / CR) : 1u), 128, (const double*)G, L, ri, j0, bad);
       const int l1 = split ? p1 : ri;  // without the product, 32 columns at a time over everything
-      if (j0 + CB < l1) update(j0, j0 + CB, l1);
+      const int l0 = j0 + CB;
+      if (l0 < l1)
+        launch(chol_update, dim3((unsigned)((l1 - l0 + 31) / 32), (unsigned)((ri - l0 + CU - 1) / CU)), 256, G, (const double*)L,
+               ri, j0, ri - j0 < CB ? ri - j0 : CB, l0, l1);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return pifa_fail_cuda("cholesky: launch", e);
     if (split) {
       const int st = gemm_f64_split(t, scratch, bytes, s);
