@@ -62,7 +62,7 @@ NCU_TRAFFIC = {
     # profiles/decode_tc_gateup70b_T16_traffic.md: phase 1 in clusters of 8 CTAs per row block,
     # phase 2 one CTA per row block; two kernels, no partial sums in global memory
     ("llama2_70b_gate_up_28672x8192_r4096", 16): {
-        "sha": {"decode_tc.cu": "7e6777523b40bb13", "decode.cu": "08cc4130ffbb131e"},
+        "sha": {"decode_tc.cu": "7e6777523b40bb13", "decode.cu": "0614a1bef5baa62d"},
         "bytes": 269364992,
     },
 }

@@ -30,7 +30,7 @@
 // memory and finishes 16 RG / ks rows itself. Both sums run in a fixed order, so the result is
 // deterministic.
 //
-// Layers with more row tiles than one wave of clusters holds run a second kernel, decode_stream:
+// Phases for T <= 2 whose weights are more than the SMs can stage run a second kernel, decode_stream:
 // a persistent grid (as many clusters as are co-resident) in which every cluster streams the
 // K-chunks of its tiles through a ring of shared-memory stages filled by 2-D TMA boxes (few large
 // copies: per-row bulk copies of 1-2 KB stream well below the HBM rate), with the CTA's K range

@@ -21,8 +21,8 @@
 // The main loop is bound by the threads that issue: a flag read from shared memory per step, the
 // stage index by division and the MN-major boxes in a loop cost it up to 45%. Measured, K-major,
 // 4864 x 4096 x 8192 (four whole rounds of tiles): 1925 TFLOP/s, cuBLAS's burst rate; 4096 x 4096,
-// r = 2048, T = 2048: backward 316.5 -> 169.1 us and the M accumulators of two batches 860.2 ->
-// 453.2 us against the form that this replaced (a launch and a CTA per tile of up to 128 x 256 with
+// r = 2048, T = 2048: backward 316.5 -> 164 to 170 us and the M accumulators of two batches 860 ->
+// 440 us against the form that this replaced (a launch and a CTA per tile of up to 128 x 256 with
 // the epilogue exposed, products on side streams), every output bit for bit the same; one-CTA MMAs
 // on the same persistent grid took 253.6 and 538.1 us.
 // Every wait is bounded (globaltimer); on timeout the CTA latches PIFA_ERR_TIMEOUT, drains what it
