@@ -22,7 +22,7 @@
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 15, Cholesky 2.2 and steps 38 of 58.9 ms. The M solves at m = n = 2048, r = 1024:
+// with their slices 15, Cholesky 2.2 and steps 38 of 58.3 ms. The M solves at m = n = 2048, r = 1024:
 // 141.4 -> 11.3 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
@@ -429,35 +429,52 @@ __global__ void __launch_bounds__(256) greedy_norms(Greedy g, int k, double* nor
 // The list for the steps from k on and their first best two: the rows of the `want` or somewhat fewer
 // largest norms (a threshold found by bisection; in_list marks them), or, with want = 0 or where
 // ties leave fewer than a quarter of them above any threshold, all unchosen rows. One block of 1024.
+// The norms are compared as integers (their bits; -1 for a chosen row, 0 for a NaN), the first 4096 of
+// them kept in registers: float64 comparisons of values read again at each step took 35 us, these 17 (m = 4096).
 __global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const double* norms, int want, uint8_t* in_list) {
   __shared__ int s_n[32];
-  __shared__ double s_m[32];
+  __shared__ long long s_m[32];
   __shared__ Top2 s_t[32];
   __shared__ int s_count;
+  constexpr int HELD = 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto count_above = [&](double th) {
+  auto key = [&](int i) {
+    const long long b = __double_as_longlong(norms[i]), a = b & 0x7fffffffffffffffll;
+    return b == (long long)0xbff0000000000000ull ? -1ll : a > 0x7ff0000000000000ll ? 0ll : a;  // -1.0: chosen
+  };
+  long long held[HELD], mx = 0;
+#pragma unroll
+  for (int u = 0; u < HELD; ++u) {
+    const int i = threadIdx.x + 1024 * u;
+    held[u] = i < g.m ? key(i) : -1ll;
+    mx = max(mx, held[u]);
+  }
+  for (int i = threadIdx.x + 1024 * HELD; i < g.m; i += 1024) mx = max(mx, key(i));
+  auto count_above = [&](long long th) {
     int n = 0;
-    for (int i = threadIdx.x; i < g.m; i += 1024) n += norms[i] > th ? 1 : 0;
+#pragma unroll
+    for (int u = 0; u < HELD; ++u) n += held[u] > th ? 1 : 0;
+    for (int i = threadIdx.x + 1024 * HELD; i < g.m; i += 1024) n += key(i) > th ? 1 : 0;
     n = __reduce_add_sync(0xffffffffu, n);
     __syncthreads();
     if (lane == 0) s_n[warp] = n;
     __syncthreads();
     return __reduce_add_sync(0xffffffffu, s_n[lane]);
   };
-  double mx = 0.0;
-  for (int i = threadIdx.x; i < g.m; i += 1024) mx = fmax(mx, norms[i]);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, (long long)__shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) s_m[warp] = mx;
   __syncthreads();
   mx = s_m[lane];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  double lo = -0.5, hi = mx;  // count above lo: all unchosen rows; above hi: none
-  bool all = want == 0 || count_above(lo) <= 2 * want;
-  double th = lo;
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, (long long)__shfl_xor_sync(0xffffffffu, mx, o));
+  // count above -1: all unchosen rows; above hi: none. Midpoints of the values, not of their bits.
+  long long lo = -1, hi = mx;
+  bool all = want == 0 || count_above(-1) <= 2 * want;
+  long long th = lo;
   for (int it = 0; it < 48 && !all; ++it) {
-    const double mid = it == 0 ? 0.5 * mx : 0.5 * (fmax(lo, 0.0) + hi);
+    const double a = lo < 0 ? 0.0 : __longlong_as_double(lo);
+    const long long mid = __double_as_longlong(0.5 * (a + __longlong_as_double(hi)));
     const int n = count_above(mid);
     if (n > want) {
       lo = mid;
@@ -467,14 +484,15 @@ __global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const dou
       if (n >= want - want / 10) break;
     }
   }
-  if (!all && (th < 0.0 || count_above(th) < want / 4)) all = true;
-  if (all) th = -0.5;
+  if (!all && (th < 0 || count_above(th) < want / 4)) all = true;
+  if (all) th = -1;
   if (threadIdx.x == 0) s_count = 0;
   __syncthreads();
   Top2 t = top2_empty();
   for (int i0 = 0; i0 < g.m; i0 += 1024) {
     const int i = i0 + (int)threadIdx.x;
-    const bool in = i < g.m && (all ? norms[i] != -1.0 : norms[i] > th);
+    const long long ki = i < g.m ? key(i) : -1ll;
+    const bool in = ki > th;
     if (in_list && i < g.m) in_list[i] = in ? 1 : 0;
     const unsigned ballot = __ballot_sync(0xffffffffu, in);
     int at = 0;
@@ -482,7 +500,7 @@ __global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const dou
     at = __shfl_sync(0xffffffffu, at, 0) + __popc(ballot & ((1u << lane) - 1u));
     if (in) {
       g.act[at] = i;
-      top2_add(t, norm_key(norms[i]), i, at);
+      top2_add(t, (unsigned long long)ki, i, at);
     }
   }
   t = warp_top2(t);
@@ -495,7 +513,7 @@ __global__ void __launch_bounds__(1024) greedy_select(Greedy g, int k, const dou
     g.ctl->k_end = 0;
     g.ctl->count = s_count;
     g.ctl->all = all ? 1 : 0;
-    g.ctl->theta = (unsigned long long)__double_as_longlong(all ? 0.0 : th);
+    g.ctl->theta = all ? 0ull : (unsigned long long)th;
   }
 }
 
