@@ -239,7 +239,8 @@ int pifa_compress(const double* U, const double* V, int64_t m, int64_t n, int64_
  *   Pivot rule exactly as pifa_compress (greedy Businger-Golub on W'^T, ties to the lowest index;
  *   residual norms recomputed every step for all rows that the step could choose), computed in the r-dimensional row space Z = U L with
  *   L L^T = V^T V (Cholesky), which has the row inner products of W'. C = Z[I^c] R^{-T} from the
- *   triangular factor R of that pivoted QR; W_p = U[I] V^T. Requires 1 <= r <= min(m, n) and
+ *   triangular factor R of that pivoted QR; W_p = U[I] V^T. Products run in float64 or on the tensor
+ *   cores where that is within float64 arithmetic's error bounds. Requires 1 <= r <= min(m, n) and
  *   r <= 16384 (PIFA_ERR_UNSUPPORTED otherwise); PIFA_ERR_RANK_DEFICIENT when V^T V is not
  *   positive definite or |R_(r-1,r-1)| < 1e-8 |R_00|. Synchronous; no device memory is allocated.
  */

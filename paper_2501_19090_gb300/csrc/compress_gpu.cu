@@ -17,13 +17,14 @@
 //      inverted 32 x 32 diagonal blocks, then off-diagonal blocks -A^{-1} B D^{-1} level by level).
 //      Columns go from selection order to ascending I as they are written.
 //   4. W_p = U[I, :] V^T (Eq. 1).
-// Products of 2^20 multiply-adds and more run on the tensor cores by exact slices (gemm_f64_tc.cu);
+// Products of 2^20 multiply-adds and more run on the tensor cores by exact slices (gemm_f64_tc.cu), the
+// elements for which those are less exact than float64 arithmetic excepted (gemm_f64_masked);
 // small ones, the panels of the Cholesky factorisation and the greedy steps run on the CUDA cores,
 // bound by the float64 issue rate (about two multiply-adds per clock and SM). Measured against what
 // this replaced (all products on the CUDA cores; Cholesky by rank-1 updates; every step over every
 // row), 4096 x 4096, r = 2048: products 90.4, Cholesky 37.8 and steps 173 of 308 ms; now products
-// with their slices 15, Cholesky 2.2 and steps 38 of 58.3 ms. The M solves at m = n = 2048, r = 1024:
-// 141.4 -> 11.3 ms. No kernel waits on another CTA.
+// with their slices and checks 16, Cholesky 2.2 and steps 38 of 59.6 ms. The M solves at m = n = 2048, r = 1024:
+// 141.4 -> 11.7 ms. No kernel waits on another CTA.
 #include <cmath>
 #include <cstdio>
 
@@ -47,23 +48,27 @@ constexpr int GK = 16;
 constexpr int kSms = 152;
 constexpr int kZeroBlock = 64;  // triangular operands: zeros are skipped in blocks of 64, whatever the tile
 
+// Columns of the contraction that hold anything in the GT x GT tile at (i0, j0), of 0 .. K.
+__device__ __forceinline__ void k_range(const GemmF64& p, int i0, int j0, int& kbeg, int& kend) {
+  kbeg = 0;
+  kend = p.K;
+  const int ib = i0 / kZeroBlock * kZeroBlock, jb = j0 / kZeroBlock * kZeroBlock;
+  if (p.tri & 1) kbeg = max(0, jb - p.kbase);
+  if (p.tri & 4) kbeg = max(kbeg, ib - p.kbase);
+  if (p.tri & 2) kend = min(p.K, jb + kZeroBlock - p.kbase);
+}
+
+// The tile's sums, one chain of multiply-adds per element, in the order of k: thread (tx, ty) of 16 x 16
+// gets elements (i0 + ty + 16 u, j0 + tx + 16 v).
 template <int GT>
-__global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
+__device__ __forceinline__ void tile_f64(const GemmF64& p, const double* A, const double* B, int i0, int j0,
+                                         double (&acc)[GT / 16][GT / 16]) {
   constexpr int U = GT / 16;
   __shared__ double As[GK][GT + 1];
   __shared__ double Bs[GK][GT + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int i0 = blockIdx.y * GT, j0 = blockIdx.x * GT;
-  const double* A = p.A + blockIdx.z * p.za;
-  const double* B = p.B + blockIdx.z * p.zb;
-  double* C = p.C + blockIdx.z * p.zc;
-  if (p.lower && j0 > i0 + GT - 1) return;
-  int kbeg = 0, kend = p.K;
-  const int ib = i0 / kZeroBlock * kZeroBlock, jb = j0 / kZeroBlock * kZeroBlock;
-  if (p.tri & 1) kbeg = jb;
-  if (p.tri & 4) kbeg = max(kbeg, ib);
-  if (p.tri & 2) kend = min(p.K, jb + kZeroBlock);
-  double acc[U][U] = {};
+  int kbeg, kend;
+  k_range(p, i0, j0, kbeg, kend);
   for (int k0 = kbeg; k0 < kend; k0 += GK) {
     for (int e = threadIdx.x; e < GT * GK; e += 256) {
       const int ii = e % GT, kk = e / GT;  // consecutive threads: consecutive rows of the A tile
@@ -95,18 +100,83 @@ __global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
     }
     __syncthreads();
   }
+}
+
+__device__ __forceinline__ void store_f64(const GemmF64& p, double* C, int i, int j, double sum) {
+  double* c = C + (int64_t)i * p.ldc + (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j);
+  *c = (p.beta != 0.0 ? p.beta * *c : 0.0) + p.alpha * sum;
+}
+
+template <int GT>
+__global__ void __launch_bounds__(256) gemm_f64(GemmF64 p) {
+  constexpr int U = GT / 16;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int i0 = blockIdx.y * GT, j0 = blockIdx.x * GT;
+  double* C = p.C + blockIdx.z * p.zc;
+  if (p.lower && j0 > i0 + GT - 1) return;
+  double acc[U][U] = {};
+  tile_f64<GT>(p, p.A + blockIdx.z * p.za, p.B + blockIdx.z * p.zb, i0, j0, acc);
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int i = i0 + ty + 16 * u;
-    if (i >= p.M) continue;
+  for (int u = 0; u < U; ++u)
 #pragma unroll
     for (int v = 0; v < U; ++v) {
-      const int j = j0 + tx + 16 * v;
-      if (j >= p.N) continue;
-      double* c = C + (int64_t)i * p.ldc + (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j);
-      *c = (p.beta != 0.0 ? p.beta * *c : 0.0) + p.alpha * acc[u][v];
+      const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
+      if (i < p.M && j < p.N) store_f64(p, C, i, j, acc[u][v]);
     }
+}
+
+// The flagged elements of a 32 x 32 tile per CTA: the tile's sums where many are flagged, else a thread per
+// element with the same chain, so that an element's value does not depend on its neighbours' flags (equal
+// rows keep equal values). Bound by the float64 pipe: a tile of K columns holds its SM for 512 K cycles,
+// up to kFewFlags elements alone for 64 K.
+constexpr int kFewFlags = 64;
+__global__ void __launch_bounds__(256) gemm_f64_masked(GemmF64 p, const uint32_t* mask, int words) {
+  __shared__ uint32_t s_mask[32];
+  __shared__ int s_at[33];
+  __shared__ uint16_t s_list[kFewFlags];
+  const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    const uint32_t w = i0 + lane < p.M ? mask[(int64_t)(i0 + lane) * words + blockIdx.x] : 0u;
+    s_mask[lane] = w;
+    int at = __popc(w);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += x;
+    }
+    s_at[lane + 1] = at;
+    if (lane == 0) s_at[0] = 0;
   }
+  __syncthreads();
+  const int n = s_at[32];
+  if (n == 0) return;
+  if (n > kFewFlags) {
+    double acc[2][2] = {};
+    tile_f64<32>(p, p.A, p.B, i0, j0, acc);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+        if (s_mask[ty + 16 * u] >> (tx + 16 * v) & 1u) store_f64(p, p.C, i0 + ty + 16 * u, j0 + tx + 16 * v, acc[u][v]);
+    return;
+  }
+  if (threadIdx.x < 32) {
+    int at = s_at[threadIdx.x];
+    for (uint32_t w = s_mask[threadIdx.x]; w; w &= w - 1) s_list[at++] = (uint16_t)(threadIdx.x * 32 + __ffs(w) - 1);
+  }
+  __syncthreads();
+  if ((int)threadIdx.x >= n) return;
+  const int i = i0 + (s_list[threadIdx.x] >> 5), j = j0 + (s_list[threadIdx.x] & 31);
+  int kbeg, kend;
+  k_range(p, i0, j0, kbeg, kend);
+  const double* a = p.A + (p.aidx ? (int64_t)p.aidx[i] : (int64_t)i) * p.sa_i;
+  const double* b = p.B + (int64_t)j * p.sb_j;
+  double sum = 0.0;
+#pragma unroll 8
+  for (int k = kbeg; k < kend; ++k) sum = fma(a[(int64_t)k * p.sa_k], b[(int64_t)k * p.sb_k], sum);
+  store_f64(p, p.C, i, j, sum);
 }
 
 int run_gemm_f64(const GemmF64& p, int batch, cudaStream_t s) {
@@ -912,6 +982,13 @@ constexpr int64_t kMaxRank = 16384;  // the reflector lives in shared memory (r 
 
 }  // namespace
 
+int gemm_f64_flagged(const GemmF64& p, const uint32_t* mask, int words, cudaStream_t s) {
+  gemm_f64_masked<<<dim3((unsigned)((p.N + 31) / 32), (unsigned)((p.M + 31) / 32)), 256, 0, s>>>(p, mask, words);
+  pifa_count_launch();
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? PIFA_OK : pifa_fail_cuda("float64 products: flagged elements", e);
+}
+
 extern "C" int64_t pifa_compress_device_workspace_size(int64_t m, int64_t n, int64_t r) {
   pifa_clear_error();
   if (m < 1 || n < 1 || r < 1 || r > m || r > n) return pifa_fail(PIFA_ERR_INVALID_ARG, "need 1 <= r <= min(m, n)");
@@ -1050,7 +1127,7 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
       w.M = mi; w.N = kRun; w.K = len;
       w.A = Z + k; w.sa_i = r; w.sa_k = 1;
       w.B = V_run; w.sb_k = 1; w.sb_j = len;
-      w.C = W_run; w.ldc = kRun; w.alpha = 1.0; w.beta = 0.0;
+      w.C = W_run; w.ldc = kRun; w.alpha = 1.0; w.beta = 0.0; w.normwise = 1;
       const int parts = gemm_f64_split_fits(w, slice_bytes) ? kRunSlices : 1;
       st = parts > 1 ? gemm_f64_split(w, slices, slice_bytes, s, parts, m * kRun) : run_gemm_f64(w, 1, s);
       if (st != PIFA_OK) return st;
@@ -1060,7 +1137,7 @@ extern "C" int pifa_compress_device(const double* U, const double* V, int64_t m,
       u.M = mi; u.N = len; u.K = kRun;
       u.A = W_run; u.sa_i = kRun; u.sa_k = 1;
       u.B = V_run; u.sb_k = len; u.sb_j = 1;
-      u.C = Z + k; u.ldc = r; u.alpha = -1.0; u.beta = 1.0;
+      u.C = Z + k; u.ldc = r; u.alpha = -1.0; u.beta = 1.0; u.normwise = 1;
       if ((st = run_product(u, slices, slice_bytes, s)) != PIFA_OK) return st;
       PIFA_CK(cudaGetLastError(), "compress: candidate block launch");
     }

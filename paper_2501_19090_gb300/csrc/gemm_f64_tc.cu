@@ -7,13 +7,26 @@
 // scaled by a power of two to below one in magnitude, rounded to 62 fractional bits (float64 keeps
 // 53 of its own), and cut into 8 balanced base-256 digits, each a whole number of at most 8 bits
 // and so exact in bf16. With a_p, b_q the digit matrices,
-//   A B = sum over d = p + q <= 7 of 2^-(12 + 8 d) V_d,   V_d = sum over p + q = d of a_p b_q,
-// where the dropped pairs (d > 7) lie below 2^-64 of the largest products. A V_d over K = 128
-// columns is a whole number of at most 8 128 128^2 = 2^24, which the fp32 accumulators in tensor
-// memory hold exactly; every 128 columns the 8 accumulators are drained into 64-bit integers. The
-// only roundings are the 62-bit one of the operands and the final one to float64: against quad
-// precision W_p = U V^T (K = 256 to 2048) is 4.7e-17 off, its float64 rounding, where a chain of
-// float64 multiply-adds is 5e-16 to 1.1e-15 off.
+//   A B = sum over d = p + q <= 7 of 2^-(12 + 8 d) V_d,   V_d = sum over p + q = d of a_p b_q.
+// A V_d over K = 128 columns is a whole number of at most 8 128 128^2 = 2^24, which the fp32 accumulators
+// in tensor memory hold exactly; every 128 columns the 8 accumulators are drained into 64-bit integers.
+// Beside the final rounding to float64, element (i, j) is off by the operands' rounding and the dropped
+// pairs (d > 7). With A_i and B_j the scales of row i and column j (powers of two above their largest
+// magnitudes) that is at most 2^-59 A_i B_j per term (seven pairs d = 8 of up to 2^14 2^-76, and 2^-62),
+// and 2^-62.2 A_i B_j sqrt(K) in the root mean square. The bound is relative to the largest entries, not to
+// the terms themselves: where small entries meet large ones, or one entry of a row towers above the
+// others, a chain of float64 multiply-adds, off by up to K 2^-53 S_ij with S_ij = sum over k of |a_ik b_kj|,
+// can be far better. So the elements with S_ij < sqrt(K) / 128 A_i B_j (K: the terms that triangular
+// operands leave) are computed by such a chain, in the order of the CUDA-core products; the others are off
+// by at most 2 sqrt(K) 2^-53 S_ij, and by 0.22 2^-53 S_ij in the root mean square, less than one rounding.
+// S comes from the operands' magnitudes in bf16 (truncated, and not below 2^-60, so that S = 0 means that
+// every term is zero), one more product of bf16 matrices (gemm_tc.cu) whose epilogue writes a bit per
+// element: 1 / 36 of the digits' multiply-adds. Products with themselves (A = B^T) need none: theirs enter
+// or leave a Cholesky factorisation, whose own error in element (i, j) is a multiple of 2^-53 times the
+// geometric mean of the diagonal elements i and j, each at least its scale's square over four.
+// Against quad precision W_p = U V^T (K = 256 to 2048, N(0, 1) factors) is 4.7e-17 off, its float64
+// rounding, where the chain is 5e-16 to 1.1e-15 off; so it is with U D and V / D for any diagonal D of powers
+// of two, for which slices alone lose all digits at D = 2^-30 to 2^30.
 //
 // Sliced operands are laid out [row][K block of 32][digit][32], so that a TMA box of 64 elements
 // holds two digits of one K block as one 128-byte swizzled row.
@@ -61,6 +74,7 @@ struct SliceArgs {
   unsigned long long* mx;   // per row: the bits of max |x| over k
   __nv_bfloat16* S;         // rows x (nkb ROWLEN)
   int nkb;
+  __nv_bfloat16* mag;       // rows x (nkb KBLK): the magnitudes over the row's scale (null: not needed)
 };
 
 // max |x| of each row as an unsigned bit pattern (non-negative float64 values order like their
@@ -157,6 +171,7 @@ __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
   if (i >= a.rows) return;
   const int er = row_exp(a.mx[i]);
   uint32_t w[NDIG][4];  // 8 bf16 digits per plane, packed in pairs
+  uint32_t mg[4];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     const unsigned long long b = t[rr][kq + e];
@@ -169,6 +184,11 @@ __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
     if (sh >= 0) mag = mant << sh;  // sh <= 9: ex <= er
     else if (sh > -60) mag = (mant + (1ull << (-sh - 1))) >> -sh;
     if (er == 2047) mag = 0;  // the drain computes this row by plain_dot
+    // |x| / 2^(er - 1022) = mant 2^(ex - er - 53), truncated to bf16; at least 2^-60 unless x = 0
+    float f = __uint2float_rz((uint32_t)(mant >> 22)) * __uint_as_float((uint32_t)max(ex - er - 31 + 127, 1) << 23);
+    f = mant == 0ull || er == 2047 ? 0.0f : fmaxf(f, 0x1p-60f);
+    if (e & 1) mg[e >> 1] |= __float_as_uint(f) & 0xffff0000u;
+    else mg[e >> 1] = __float_as_uint(f) >> 16;
     long long q = (b >> 63) ? -(long long)mag : (long long)mag;
 #pragma unroll
     for (int p = NDIG - 1; p >= 0; --p) {
@@ -182,6 +202,7 @@ __global__ void __launch_bounds__(128) slice_digits(SliceArgs a) {
   __nv_bfloat16* s = a.S + (int64_t)i * a.nkb * ROWLEN + (int64_t)kb * ROWLEN + kq;
 #pragma unroll
   for (int p = 0; p < NDIG; ++p) *reinterpret_cast<uint4*>(s + p * KBLK) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+  if (a.mag) *reinterpret_cast<uint4*>(a.mag + ((int64_t)i * a.nkb + kb) * KBLK + kq) = make_uint4(mg[0], mg[1], mg[2], mg[3]);
 }
 
 // ---- the products --------------------------------------------------------------------------------
@@ -194,6 +215,8 @@ struct SplitArgs {
   int64_t ldc;
   int64_t zc;  // elements between the partial results of consecutive K-slices (blockIdx.z)
   double alpha, beta;
+  const uint32_t* mask;  // the elements to leave alone, a bit each (null: none); gemm_f64_flagged computes them
+  int words;             // its pitch
   int* status;
   uint64_t timeout_ns;
 };
@@ -386,6 +409,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       const bool neg = p.alpha == -1.0, one = neg || p.alpha == 1.0;
+      const uint32_t skip = p.mask && lane < nr && n0 + half * 32 < p.N
+                                ? p.mask[(int64_t)(r0 + lane) * p.words + (n0 >> 5) + half] : 0u;
       double* c = Cz + (int64_t)r0 * p.ldc + (jn ? (p.cidx ? (int64_t)p.cidx[j] : (int64_t)j) : 0);
       for (int g8 = 0; g8 < nr; g8 += 8) {
         double old[8];
@@ -393,7 +418,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int u = 0; u < 8; ++u) old[u] = p.beta != 0.0 && jn && g8 + u < nr ? c[(int64_t)(g8 + u) * p.ldc] : 0.0;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          if (!jn || g8 + u >= nr) continue;
+          const uint32_t sk = __shfl_sync(0xffffffffu, skip, g8 + u);
+          if (!jn || g8 + u >= nr || (sk >> lane & 1u)) continue;
           double v = tile[(g8 + u) * 33 + lane];
           if (!one) v *= p.alpha;
           else if (neg) v = -v;
@@ -412,10 +438,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 int64_t a1k(int64_t b) { return (b + 1023) / 1024 * 1024; }
-// scratch bytes of a product's two sliced operands over a panel of kp columns
-int64_t panel_bytes(int64_t M, int64_t N, int64_t kp, bool same) {
-  const int64_t row = (kp + KBLK - 1) / KBLK * ROWLEN * 2;
-  return a1k(M * row) + a1k(M * 8) + (same ? 0 : a1k(N * row) + a1k(N * 8));
+constexpr float kLeast = 1.0f / 128.0f;  // S_ij / (A_i B_j sqrt(K)) below which an element is recomputed
+
+bool with_itself(const GemmF64& p) {
+  return p.A == p.B && p.sa_i == p.sb_j && p.sa_k == p.sb_k && p.M == p.N && !p.aidx;
+}
+bool checked(const GemmF64& p) { return !with_itself(p) && !p.normwise; }
+int mask_words(const GemmF64& p) { return (p.N + 31) / 32; }
+
+// scratch bytes of a product's sliced operands, their magnitudes and the mask over a panel of kp columns
+int64_t panel_bytes(const GemmF64& p, int64_t kp) {
+  const int64_t nkb = (kp + KBLK - 1) / KBLK, row = nkb * ROWLEN * 2, mag = checked(p) ? nkb * KBLK * 2 : 0;
+  return a1k(p.M * row) + a1k(p.M * 8ll) + a1k(p.M * mag) +
+         (with_itself(p) ? 0 : a1k(p.N * row) + a1k(p.N * 8ll) + a1k(p.N * mag)) +
+         (checked(p) ? a1k((int64_t)p.M * mask_words(p) * 4) : 0);
 }
 
 int slice(const SliceArgs& a, cudaStream_t s) {
@@ -437,9 +473,8 @@ int slice(const SliceArgs& a, cudaStream_t s) {
 
 bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes) {
   const int64_t work = (int64_t)p.M * p.N * p.K;
-  const bool same = p.A == p.B && p.sa_i == p.sb_j && p.sa_k == p.sb_k && p.M == p.N && !p.aidx;
   return p.K >= 64 && work >= (int64_t)1 << 20 && (p.M + 31) / 32 <= 65535 && (p.N + 31) / 32 <= 65535 &&
-         panel_bytes(p.M, p.N, p.K < 128 ? p.K : 128, same) <= bytes - 256;  // 256: alignment of the scratch
+         panel_bytes(p, p.K < 128 ? p.K : 128) <= bytes - 256;  // 256: alignment of the scratch
 }
 
 int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream, int slices, int64_t zc) {
@@ -449,11 +484,12 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
   const int64_t shift = (int64_t)((256 - (reinterpret_cast<uintptr_t>(scratch) & 255u)) & 255u);
   scratch = static_cast<uint8_t*>(scratch) + shift;
   bytes -= shift;
-  const bool same = p.A == p.B && p.sa_i == p.sb_j && p.sa_k == p.sb_k && p.M == p.N && !p.aidx;
+  const bool same = with_itself(p), check = checked(p);
+  if (check && slices > 1) return pifa_fail(PIFA_ERR_INVALID_ARG, "gemm_f64_split: a checked product in K-slices");
   int64_t kp = p.K;  // the widest panel of whole 128-column chunks that fits the scratch
-  if (panel_bytes(p.M, p.N, kp, same) > bytes) {
+  if (panel_bytes(p, kp) > bytes) {
     kp = (kp + 127) / 128 * 128;
-    while (kp > 128 && panel_bytes(p.M, p.N, kp, same) > bytes) kp -= 128;
+    while (kp > 128 && panel_bytes(p, kp) > bytes) kp -= 128;
   }
   e = cudaFuncSetAttribute(gemm_f64_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
   if (e != cudaSuccess) return pifa_fail_cuda("cudaFuncSetAttribute(gemm_f64_split)", e);
@@ -462,20 +498,35 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
     const int nkb = (kn + KBLK - 1) / KBLK;
     const int64_t row = (int64_t)nkb * ROWLEN * 2;
     uint8_t* w = static_cast<uint8_t*>(scratch);
-    SliceArgs a = {p.A + k0 * p.sa_k, p.aidx, p.sa_i, p.sa_k, p.M, kn, nullptr, nullptr, nkb};
-    a.S = reinterpret_cast<__nv_bfloat16*>(w);
-    w += a1k(p.M * row);
-    a.mx = reinterpret_cast<unsigned long long*>(w);
-    w += a1k((int64_t)p.M * 8);
+    auto take = [&](int64_t n) {
+      uint8_t* at = w;
+      w += a1k(n);
+      return at;
+    };
+    const int64_t mag = (int64_t)nkb * KBLK * 2;
+    SliceArgs a = {p.A + k0 * p.sa_k, p.aidx, p.sa_i, p.sa_k, p.M, kn, nullptr, nullptr, nkb, nullptr};
+    a.S = reinterpret_cast<__nv_bfloat16*>(take(p.M * row));
+    a.mx = reinterpret_cast<unsigned long long*>(take((int64_t)p.M * 8));
+    if (check) a.mag = reinterpret_cast<__nv_bfloat16*>(take(p.M * mag));
     SliceArgs b = a;
     int st = slice(a, stream);
     if (st != PIFA_OK) return st;
     if (!same) {
-      b = SliceArgs{p.B + k0 * p.sb_k, nullptr, p.sb_j, p.sb_k, p.N, kn, nullptr, nullptr, nkb};
-      b.S = reinterpret_cast<__nv_bfloat16*>(w);
-      w += a1k(p.N * row);
-      b.mx = reinterpret_cast<unsigned long long*>(w);
+      b = SliceArgs{p.B + k0 * p.sb_k, nullptr, p.sb_j, p.sb_k, p.N, kn, nullptr, nullptr, nkb, nullptr};
+      b.S = reinterpret_cast<__nv_bfloat16*>(take(p.N * row));
+      b.mx = reinterpret_cast<unsigned long long*>(take((int64_t)p.N * 8));
+      if (check) b.mag = reinterpret_cast<__nv_bfloat16*>(take(p.N * mag));
       if ((st = slice(b, stream)) != PIFA_OK) return st;
+    }
+    uint32_t* mask = nullptr;
+    const int words = mask_words(p);
+    if (check) {  // one bit per element: S_ij < kLeast sqrt(terms), S in units of A_i B_j
+      mask = reinterpret_cast<uint32_t*>(take((int64_t)p.M * words * 4));
+      GemmTc c = {p.M, p.N, kn, a.mag, mag / 2, false, b.mag, mag / 2, false, mask, words, 4, kLeast, nullptr, 0};
+      c.tri = p.tri;
+      c.k0 = (int)k0;
+      c.k1 = (int)k0 + kn;
+      if ((st = gemm_tc_group(&c, 1, status, pifa_wait_timeout_ns(), stream)) != PIFA_OK) return st;
     }
     CUtensorMap tA, tB;
     if ((st = make_tmap_2d(&tA, PIFA_DTYPE_BF16, a.S, p.M, row / 2, row / 2, 64, SM_)) != PIFA_OK) return st;
@@ -496,6 +547,8 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
     g.alpha = p.alpha;
     g.beta = k0 == 0 ? p.beta : 1.0;
     g.zc = zc;
+    g.mask = mask;
+    g.words = words;
     g.status = status;
     g.timeout_ns = pifa_wait_timeout_ns();
     const dim3 grid((unsigned)((p.N + SN - 1) / SN), (unsigned)((p.M + SM_ - 1) / SM_), (unsigned)slices);
@@ -504,6 +557,15 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
     e = cudaGetLastError();
     if (e != cudaSuccess) return pifa_fail_cuda("gemm_f64_split launch", e);
     pifa_count_launch();
+    if (check) {
+      GemmF64 f = p;
+      f.A += k0 * p.sa_k;
+      f.B += k0 * p.sb_k;
+      f.K = kn;
+      f.kbase = (int)k0;
+      f.beta = g.beta;
+      if ((st = gemm_f64_flagged(f, mask, words, stream)) != PIFA_OK) return st;
+    }
   }
   return PIFA_OK;
 }

@@ -9,7 +9,8 @@
 //   D (M x N, fp32 accumulate) is written as bf16, as fp32, added into an fp32 matrix, or as a
 //   hi + lo pair of bf16 matrices (hi = bf16(D), lo = bf16(D - hi)) for a later contraction that must
 //   not lose D's low bits. A second K pass into the same accumulator with A2 in place of A and/or
-//   B2 in place of B (same layouts) consumes such a pair: D = (A + A2) B^T or A (B + B2)^T.
+//   B2 in place of B (same layouts) consumes such a pair: D = (A + A2) B^T or A (B + B2)^T. For the sliced
+//   float64 products D can also be one bit per element, whether it is small against its terms.
 //
 // One launch computes up to three independent products on a persistent grid of CTA pairs (clusters of
 // two, one CTA of 352 threads per SM). A pair computes 256 x bn tiles (bn <= 256) with pair MMAs
@@ -66,6 +67,7 @@ struct Problem {
   float alpha;
   const bf16* add;    // optional addend: D[i][j] += add[i * ldadd + j] (out_mode 0 or 3)
   int64_t ldadd;
+  int tri, k0, k1;    // out_mode 4: which terms of the contraction can be other than zero
   int wide;           // every base and pitch of D, D2 and add is a multiple of 32 bytes
   // which pair computes which tile: tiles [0, lo_tiles) are dealt in turn to the lo_n pairs from
   // lo_first on (those with less work so far), the rest to all pairs in turn from rr0 on
@@ -94,6 +96,15 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr) {
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
+}
+
+// Terms of element (i, j) over the contraction's columns [k0, k1) (triangular operands: GemmF64::tri).
+__device__ __forceinline__ int terms(const Problem& q, int i, int j) {
+  int a = q.k0, b = q.k1;
+  if (q.tri & 1) a = max(a, j);
+  if (q.tri & 4) a = max(a, i);
+  if (q.tri & 2) b = min(b, j + 1);
+  return max(b - a, 0);
 }
 
 // One lane's up to 32 consecutive values of a row: whole 32-byte sectors when `wide`, else 16-byte
@@ -390,6 +401,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             v[j] = __float_as_uint(f);
           }
           store_f32(reinterpret_cast<float*>(q.D) + o, nc, q.wide, v);
+        } else if (mode == 4) {  // one word of 32 columns per lane
+          uint32_t word = 0;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float f = __uint_as_float(v[j]);
+            const bool low = f != 0.0f && !(f * f >= alpha * alpha * (float)terms(q, row, col + j));
+            word |= (low && j < nc ? 1u : 0u) << j;
+          }
+          reinterpret_cast<uint32_t*>(q.D)[(int64_t)row * q.ldd + (col >> 5)] = word;
         } else {
           uint32_t h[16], l[16];
 #pragma unroll
@@ -482,7 +502,7 @@ int gemm_tc_group(const GemmTc* gs, int n, int* status, uint64_t timeout_ns, cud
     if (g.K <= 0) return pifa_fail(PIFA_ERR_INVALID_ARG, "gemm_tc: K must be positive");
     if (g.M >= lim || g.N >= lim || g.K >= lim) return pifa_fail(PIFA_ERR_INVALID_ARG, "gemm_tc: size >= 2^30");
     if (g.upper && g.M != g.N) return pifa_fail(PIFA_ERR_INVALID_ARG, "gemm_tc: upper triangle of a non-square product");
-    if (g.add && (g.out_mode == 1 || g.out_mode == 2))
+    if (g.add && g.out_mode != 0 && g.out_mode != 3)
       return pifa_fail(PIFA_ERR_UNSUPPORTED, "gemm_tc: addend of an fp32 product");
     order[np++] = &g;
   }
@@ -567,6 +587,9 @@ int gemm_tc_group(const GemmTc* gs, int n, int* status, uint64_t timeout_ns, cud
     q.alpha = g.alpha;
     q.add = reinterpret_cast<const bf16*>(g.add);
     q.ldadd = g.ldadd;
+    q.tri = g.tri;
+    q.k0 = g.k0;
+    q.k1 = g.k1;
     const int64_t esz = (g.out_mode == 1 || g.out_mode == 2) ? 4 : 2;
     q.wide = ((reinterpret_cast<uintptr_t>(g.D) | reinterpret_cast<uintptr_t>(g.D2) | (uintptr_t)(g.ldd * esz) |
                reinterpret_cast<uintptr_t>(g.add) | (uintptr_t)(g.add ? g.ldadd * 2 : 0)) & 31u) == 0;

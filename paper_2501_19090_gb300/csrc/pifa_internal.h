@@ -112,7 +112,9 @@ int launch_decode_tc(const DecodeTcPhase& ph, int* status, uint64_t timeout_ns, 
 // ---- general tensor-core contraction (gemm_tc.cu) ------------------------------------------------
 // D (M x N) = alpha A B^T (+ addend), bf16 operands, fp32 accumulation. A is M x K, B is N x K; each
 // is K-major (a_mn = false: element (i, k) at [i * ld + k]) or MN-major (true: at [k * ld + i]).
-// out_mode 0: D bf16; 1: D fp32; 2: D fp32 += result; 3: D = bf16 hi, D2 = bf16 lo of the result.
+// out_mode 0: D bf16; 1: D fp32; 2: D fp32 += result; 3: D = bf16 hi, D2 = bf16 lo of the result;
+// 4: D = one bit per element, uint32 words of 32 columns, ldd words a row: whether the result S is
+// neither zero nor at least alpha sqrt(k), k the element's terms (GemmF64's check, see `tri`).
 // A2 / B2 (optional, A's / B's layout and pitch): a second K pass with A2 for A and / or B2 for B,
 // D = (A + A2) B^T or A (B + B2)^T. Optional addend (out_mode 0 and 3): D[i][j] += add[i * ldadd + j]
 // (bf16). Pointers 16-byte aligned, leading dimensions multiples of 8 elements (the caller checks).
@@ -134,6 +136,7 @@ struct GemmTc {
   const void* B2 = nullptr;
   void* D2 = nullptr;
   bool upper = false;    // M == N: skip 128 x 128 blocks wholly below the diagonal (a symmetric product)
+  int tri = 0, k0 = 0, k1 = 0;  // out_mode 4: the columns [k0, k1) of a contraction with GemmF64's zeros `tri`
 };
 // Up to three independent products in one launch.
 int gemm_tc_group(const GemmTc* gs, int n, int* status, uint64_t timeout_ns, cudaStream_t stream);
@@ -145,7 +148,9 @@ int gemm_tc_group(const GemmTc* gs, int n, int* status, uint64_t timeout_ns, cud
 //   C at C[i * ldc + (cidx ? cidx[j] : j)]
 // and, on the CUDA cores, a batch index z (blockIdx.z) offsetting A, B and C by za, zb, zc elements.
 // `tri` (bits): 1 B(k, j) = 0 for k < j, 2 B(k, j) = 0 for k > j, 4 A(i, k) = 0 for k < i; the k loop
-// skips those zeros. `lower`: only the tiles that hold some i >= j are computed.
+// skips those zeros (k counts from kbase on). `lower`: only the tiles that hold some i >= j are computed.
+// `normwise`: an error of a small multiple of 2^-62 sqrt(K) max_k |A(i, k)| max_k |B(k, j)| in element (i, j)
+// is as good as float64's for the caller (see gemm_f64_split).
 struct GemmF64 {
   int M, N, K;
   const double* A;
@@ -160,6 +165,8 @@ struct GemmF64 {
   int tri;
   int64_t za, zb, zc;
   int lower;
+  int normwise;
+  int kbase;
 };
 // The same on the tensor cores by exact slices (no batch), in `bytes` of scratch:
 // whether that form takes the product, and the product. slices > 1: the contraction cut into that many
@@ -167,6 +174,8 @@ struct GemmF64 {
 // (products of few tiles).
 bool gemm_f64_split_fits(const GemmF64& p, int64_t bytes);
 int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t stream, int slices = 1, int64_t zc = 0);
+// The elements of p whose bit is set in `mask` (uint32 words of 32 columns, `words` a row), on the CUDA cores.
+int gemm_f64_flagged(const GemmF64& p, const uint32_t* mask, int words, cudaStream_t stream);
 
 // ---- prefill (prefill.cu) --------------------------------------------------------------------
 int64_t prefill_split_workspace_bytes(const PifaShape& s);

@@ -203,3 +203,42 @@ def test_equal_norms_are_taken_from_the_lowest_index():
     piv, nonp, Wp, C, info = _device_compress(U, V)
     assert piv[0] == 0 and info.min_pivot_gap == 0.0
     _check_eqs(U, V, piv, nonp, Wp, C, rows=np.arange(0, nonp.size, 7))
+
+
+@pytest.mark.parametrize("m,n,r", [(1000, 700, 640), (400, 191, 161), (2500, 1111, 1100)])
+@pytest.mark.parametrize("s", [8, 20, 40])
+def test_a_diagonal_between_the_factors_changes_nothing(m, n, r, s):
+    """U D and V / D with D = 2^-s .. 2^s make the same W' as U and V, term by term, so Algorithm 1 has
+    to give the same pivots, W_p within a float64 chain's bound r 2^-53 (|U| |V|^T) of each element (the
+    host's product has that error too) and C with Eq. 2's residual of float64 arithmetic, although the
+    large entries of a row of U D meet the small ones of V / D."""
+    U, V, _ = inputs.make_factors(m, n, r, r)
+    D = np.ldexp(1.0, np.random.default_rng(s).permutation(np.linspace(-s, s, r).astype(int)))
+    L = oracle.compress(U, V, r, "lapack")
+    piv, nonp, Wp, C, _ = _device_compress(U.astype(np.float64) * D, V.astype(np.float64) / D)
+    assert P.pifa_device_status() == P.PIFA_OK
+    assert np.array_equal(piv, L.pivots)
+    Ud, Vd = U.astype(np.float64), V.astype(np.float64)
+    bound = r * 2.0 ** -53 * (np.abs(Ud[piv]) @ np.abs(Vd).T)
+    assert (np.abs(Wp - Ud[piv] @ Vd.T) / bound).max() <= 2.0
+    Wnp = Ud[nonp] @ Vd.T
+    assert np.linalg.norm(C @ (Ud[piv] @ Vd.T) - Wnp) / np.linalg.norm(Wnp) <= 8 * r * 2.0 ** -53
+
+
+@pytest.mark.parametrize("spread,where", [(1e3, "U"), (1e7, "V"), (1e7, "both")])
+def test_graded_singular_values_keep_the_residual_of_float64(spread, where):
+    """W' = P diag(sigma) Q^T with sigma from 1 to 1 / spread, as layers' factors are: Eq. 2 holds to a
+    small multiple of r 2^-53 however the values are shared out (rank check: 1e-8)."""
+    m, n, r = 1000, 700, 640
+    rng = np.random.default_rng(7)
+    p = np.linalg.qr(rng.standard_normal((m, r)))[0]
+    q = np.linalg.qr(rng.standard_normal((n, r)))[0]
+    sig = np.logspace(0.0, -np.log10(spread), r)
+    U = p * {"U": sig, "V": 1.0, "both": np.sqrt(sig)}[where]
+    V = q * {"U": 1.0, "V": sig, "both": np.sqrt(sig)}[where]
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert P.pifa_device_status() == P.PIFA_OK
+    bound = r * 2.0 ** -53 * (np.abs(U[piv]) @ np.abs(V).T)
+    assert (np.abs(Wp - U[piv] @ V.T) / bound).max() <= 2.0
+    W = U @ V.T
+    assert np.linalg.norm(C @ W[piv] - W[nonp]) / np.linalg.norm(W[nonp]) <= 8 * r * 2.0 ** -53

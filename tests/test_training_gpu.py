@@ -192,6 +192,26 @@ def test_m_path_end_to_end_against_the_oracle():
     check((U_r @ V_r.t()).cpu().numpy(), rU @ rV.T, "U_r V_r^T")
 
 
+@pytest.mark.parametrize("m,n,r,T", [(300, 256, 128, 1000), (700, 1032, 516, 4000)])
+@pytest.mark.parametrize("s", [10, 20])
+def test_m_reconstruct_follows_a_scaling_of_the_channels(m, n, r, T, s):
+    """Input channels scaled by D = 2^-s .. 2^s and V by 1 / D leave V^T (X X^T) V and (Y_t X^T) V as they
+    are, term by term: U_r must stay and V_r become V_r / D, to 1e-11 (both solve well-conditioned
+    systems; powers of two change no rounding of float64 arithmetic)."""
+    _, _, W, XXt, YtXt, V = _accumulated(T, n, m, r, 11)
+    d = np.ldexp(1.0, np.random.default_rng(s).permutation(np.linspace(-s, s, n).astype(int)))
+    D = torch.from_numpy(d).to(DEV)
+    Vd = torch.from_numpy(V).to(DEV)
+    XXt = XXt.triu() + XXt.triu(1).t()
+    U0, V0 = P.pifa_m_reconstruct(XXt, YtXt, Vd)
+    XXd = (D[:, None] * XXt.double() * D[None, :]).float().contiguous()
+    U1, V1 = P.pifa_m_reconstruct(XXd, (YtXt.double() * D).float().contiguous(), Vd / D[:, None])
+    assert P.pifa_device_status() == P.PIFA_OK
+    for got, ref, what in ((U1, U0, "U_r"), (V1 * D[:, None], V0, "V_r")):
+        rel = ((got - ref).norm() / ref.norm()).item()
+        assert rel <= 1e-11, f"{what}: rel {rel:.3e}"
+
+
 def test_m_reconstruct_reports_a_singular_system():
     """Fewer samples than inputs (T < n) leave X X^T singular; without the regulariser
     (alpha = 0) Eq. 7 has no unique solution: PIFA_ERR_RANK_DEFICIENT."""
