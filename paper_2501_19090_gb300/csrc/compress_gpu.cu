@@ -737,7 +737,8 @@ GreedyStep greedy_form(int len, int* threads, size_t* smem) {
 // might come into play; the other rows then take the run's reflectors at once, Z -= W T V^T with
 // W = Z V (the compact WY form of Schreiber and Van Loan, 1989; T^-1 = diag(1 / tau) + the strictly upper
 // part of V^T V), as two products on the tensor cores and a substitution per row, and all norms are
-// recomputed. The pivots, and the order of every comparison that decides one, are those of the
+// recomputed (both products need an error relative to the rows' norms only, as Householder steps have it;
+// see run_scale). The pivots, and the order of every comparison that decides one, are those of the
 // exhaustive steps. 4096 x 4096, r = 2048: the call 86.1 -> 67.8 ms.
 constexpr int kRun = 64;
 // Rows of a run: six for every SM. More make a run longer, fewer a step shorter: 65.3 ms of call at
@@ -747,7 +748,17 @@ constexpr int kRunSlices = 4;  // K-slices of Z V, whose tiles (128 rows each) a
 // Values of Z left (unchosen rows x coordinates) from which on a candidate block pays.
 constexpr int64_t kRunFrom = 2000000;
 
-// V (kRun x len, row-major): row j the reflector of step k0 + j over coordinates k0..r-1, zero rows
+// The power of two by which a run's reflector is scaled, from the pivot's norm |R_kk|: reflectors of norm
+// sqrt(2) to 4, whatever the norms of the run's pivots. In Z -= (W T) V^T the slices' errors are relative
+// to the largest of a row's weights times the largest of a column's reflector entries; a weight is at most
+// tau |v| |z| <= 4 |z|, so that they stay near 2^-58 of |z|, the row's norm, where each step by itself
+// rounds to 2^-53 of it. Unscaled, pivots of falling norms in one run (10^6 to 1) made that 2^-38.
+__device__ __forceinline__ double run_scale(double rkk) {
+  const int ex = (int)(((unsigned long long)__double_as_longlong(rkk) >> 52) & 2047ull);
+  return ex < 1 || ex > 2045 ? 1.0 : __longlong_as_double((long long)(2046 - ex) << 52);
+}
+
+// V (kRun x len, row-major): row j the scaled reflector of step k0 + j over coordinates k0..r-1, zero rows
 // from `steps` on.
 __global__ void run_vectors(Greedy g, int k0, int steps, double* V) {
   const int len = g.r - k0, j = blockIdx.y;
@@ -757,6 +768,7 @@ __global__ void run_vectors(Greedy g, int k0, int steps, double* V) {
   if (j < steps && c >= j) {
     v = g.Z[(int64_t)g.order[k0 + j] * g.r + k0 + c];
     if (c == j) v -= g.rdiag[k0 + j];
+    v *= run_scale(g.rdiag[k0 + j]);
   }
   V[(int64_t)j * len + c] = v;
 }
@@ -786,7 +798,14 @@ __global__ void __launch_bounds__(128) run_substitute(Greedy g, int k0, int step
   __shared__ double s_S[kRun * kRun];
   __shared__ double s_tau[kRun];
   for (int e = threadIdx.x; e < kRun * kRun; e += 128) s_S[e] = e / kRun < e % kRun ? S[e] : 0.0;
-  if (threadIdx.x < kRun) s_tau[threadIdx.x] = (int)threadIdx.x < steps ? g.tau[k0 + threadIdx.x] : 0.0;
+  if (threadIdx.x < kRun) {
+    double t = 0.0;
+    if ((int)threadIdx.x < steps) {
+      const double back = 1.0 / run_scale(g.rdiag[k0 + threadIdx.x]);  // V's reflector is scaled
+      t = g.tau[k0 + threadIdx.x] * back * back;
+    }
+    s_tau[threadIdx.x] = t;
+  }
   __syncthreads();
   const int lane = threadIdx.x & 31, q = lane & 3;
   const int row = blockIdx.x * 32 + (threadIdx.x >> 2);

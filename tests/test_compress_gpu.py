@@ -154,11 +154,12 @@ def test_blocked_cholesky_edges_match_the_greedy_oracle(r):
     _check_eqs(U, V, piv, nonp, Wp, C)
 
 
-@pytest.mark.parametrize("m,n,r", [(7901, 300, 256), (3700, 700, 650), (2500, 1111, 1100)])
+@pytest.mark.parametrize("m,n,r", [(7901, 300, 256), (3700, 700, 650), (2500, 1111, 1100), (2600, 1300, 1000)])
 @pytest.mark.parametrize("kind", ["plain", "twins", "nan"])
 def test_candidate_blocks_match_the_greedy_oracle(m, n, r, kind):
-    """Layers with 2e6 unchosen values of Z and more step over the rows of the largest norms and give
-    the others each block's reflectors at once. Rows that appear twice tie at every step (the first
+    """Layers with 2e6 unchosen values of Z and more, whose workspace holds the block's matrices where G
+    and L were (the last two sizes), step over the rows of the largest norms and give the others each
+    block's reflectors at once; the first two sizes step over every row. Rows that appear twice tie at every step (the first
     copies must be chosen, in the order of the layer without the second ones); a row that holds a NaN
     is never chosen and leaves every other row as it is."""
     U, V, _ = inputs.make_factors(m, n, r, r)
@@ -242,3 +243,17 @@ def test_graded_singular_values_keep_the_residual_of_float64(spread, where):
     assert (np.abs(Wp - U[piv] @ V.T) / bound).max() <= 2.0
     W = U @ V.T
     assert np.linalg.norm(C @ W[piv] - W[nonp]) / np.linalg.norm(W[nonp]) <= 8 * r * 2.0 ** -53
+
+
+@pytest.mark.parametrize("m,n,r,tall", [(2500, 2200, 1100, 1e6), (3700, 1800, 900, 1e6)])
+def test_rows_far_apart_in_one_candidate_block(m, n, r, tall):
+    """24 rows `tall` times the others are chosen first, in one block with ordinary rows; every other
+    row's relation to the pivot rows (Eq. 2) must hold to a small multiple of r 2^-53 of the row itself."""
+    U, V, _ = inputs.make_factors(m, n, r, 3)
+    U, V = U.astype(np.float64), V.astype(np.float64)
+    U[np.random.default_rng(3).permutation(m)[:24]] *= tall
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert P.pifa_device_status() == P.PIFA_OK
+    Wnp = U[nonp] @ V.T
+    err = np.linalg.norm(C @ (U[piv] @ V.T) - Wnp, axis=1) / np.linalg.norm(Wnp, axis=1)
+    assert err.max() <= 8 * r * 2.0 ** -53, err.max()
