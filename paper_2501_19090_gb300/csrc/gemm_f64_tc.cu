@@ -62,6 +62,10 @@ constexpr int DRAIN_WARPS = 8;
 constexpr int THREADS = 64 + 32 * DRAIN_WARPS;
 constexpr size_t SMEM = 1024 + STAGES * STAGE + 256;
 constexpr uint32_t TMEM_COLS = NDIG * SN;  // 512
+// Columns of K per panel: the drain adds up to 2^24 2^24 = 2^48 to a 64-bit sum for every 128 of them
+// (V_4 and V_0 shifted by 24 bits, the others by less).
+constexpr int64_t kMaxPanel = (int64_t)1 << 20;
+static_assert(kMaxPanel / (KBLK * CHUNK) <= ((int64_t)1 << 14), "the drain's sums stay below 2^62");
 // First column of accumulator d: the even ones, then the odd ones (see the MMA issuer).
 __host__ __device__ constexpr uint32_t acc_col(int d) { return (uint32_t)((d & 1) * (NDIG / 2) + (d >> 1)) * SN; }
 
@@ -486,9 +490,9 @@ int gemm_f64_split(const GemmF64& p, void* scratch, int64_t bytes, cudaStream_t 
   bytes -= shift;
   const bool same = with_itself(p), check = checked(p);
   if (check && slices > 1) return pifa_fail(PIFA_ERR_INVALID_ARG, "gemm_f64_split: a checked product in K-slices");
-  int64_t kp = p.K;  // the widest panel of whole 128-column chunks that fits the scratch
-  if (panel_bytes(p, kp) > bytes) {
-    kp = (kp + 127) / 128 * 128;
+  int64_t kp = p.K;  // the widest panel of whole 128-column chunks that fits the scratch and the drain's sums
+  if (kp > kMaxPanel || panel_bytes(p, kp) > bytes) {
+    kp = kp > kMaxPanel ? kMaxPanel : (kp + 127) / 128 * 128;
     while (kp > 128 && panel_bytes(p, kp) > bytes) kp -= 128;
   }
   e = cudaFuncSetAttribute(gemm_f64_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
