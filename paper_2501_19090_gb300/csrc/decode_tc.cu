@@ -306,6 +306,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           }
         }
       }
+      if (dead) linger(100000000ull);
       // nothing may land in shared memory once the CTA has left: the last use of every stage
       for (int j = it > a.stages ? it - a.stages : 0; is_a && j < it; ++j)
         if (!mbar_wait(&full[j % a.stages], (uint32_t)(j / a.stages) & 1u, 100000000ull))

@@ -312,6 +312,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
           }
         }
       }
+      if (dead) linger(100000000ull);
       // nothing may land in shared memory after the CTA has left: the leader waits for both CTAs'
       // copies, and the cluster barrier at the end holds the other CTA until it has
       for (int i = it > STAGES ? it - STAGES : 0; leader && is_a && i < it; ++i)

@@ -73,6 +73,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   return true;
 }
 
+// Stays for `ns` nanoseconds: for a producer that gave up a wait. Where two producers fill a stage under
+// one barrier, the other one may then still issue a copy into a stage that never gets the arrival that
+// announces its bytes, so that no wait covers that copy; the CTA must not leave before it has landed (some
+// microseconds). The other producer issues nothing later than its own wait, of the same limit, allows,
+// and the MMA thread holds the CTA for that limit again, so that this time covers limits below it.
+__device__ __forceinline__ void linger(uint64_t ns) {
+  const uint64_t t0 = globaltimer_ns();
+  while (globaltimer_ns() - t0 < ns) __nanosleep(1000);
+}
+
 // ---- TMA (tensor copies global -> shared, completion on an mbarrier) -----------------------
 __device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* map, int32_t x,
                                             int32_t y, uint64_t* bar) {
