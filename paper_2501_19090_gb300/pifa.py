@@ -209,7 +209,11 @@ def _workspace_size(T, m, n, r, variant, c_dtype) -> int:
 
 def pifa_workspace_size(T: int, m: int, n: int, r: int, variant: int = PIFA_VARIANT_AUTO,
                         c_dtype: int = PIFA_DTYPE_BF16) -> int:
-    return _workspace_size(T, m, n, r, variant, c_dtype)
+    a = (T, m, n, r, variant, c_dtype)
+    # an equal key is the same question only among plain ints: 16.0 is refused although 16 == 16.0, and
+    # an integer tensor's value is not part of its hash
+    f = _workspace_size if all(type(x) is int for x in a) else _workspace_size.__wrapped__
+    return f(*a)
 
 
 def pifa_validate_indices(pivot_idx: np.ndarray, nonpivot_idx: np.ndarray, m: int, r: int) -> int:

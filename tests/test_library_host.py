@@ -267,7 +267,6 @@ def _header_prototypes():
 def test_binding_argtypes_match_the_header(lib):
     """Every declared function's ctypes prototype in the binding matches pifa.h in arity and in
     each argument's width (pointer / int64_t / int): a mismatch would corrupt arguments silently."""
-    import ctypes
     protos = _header_prototypes()
     assert set(P.EXPORTS) <= set(protos), sorted(set(P.EXPORTS) - set(protos))
 
@@ -328,3 +327,19 @@ def test_selector_and_forced_decode_follow_the_documented_rule(lib):
             assert _documented_choice(T, G, m, r) == P.PIFA_VARIANT_PREFILL_SPLIT
             plane = -(-(T * -(-G * r // 8) * 8 * 2) // 256) * 256
             assert lib.pifa_workspace_size_grouped(G, T, m, 4096, r, P.PIFA_DTYPE_BF16) == 256 + 2 * plane
+
+
+def test_workspace_size_answers_each_kind_of_argument_as_the_first_call_would():
+    """The binding keeps the sizes that it has computed; a float that equals a known int is refused all the
+    same, and an integer tensor counts by its value at the call."""
+    import torch
+    small, large = P.pifa_workspace_size(16, 256, 256, 128), P.pifa_workspace_size(64, 256, 256, 128)
+    assert small != large
+    for bad in (16.0, np.float64(16), "16"):
+        with pytest.raises(ctypes.ArgumentError):
+            P.pifa_workspace_size(bad, 256, 256, 128)
+    assert P.pifa_workspace_size(np.int64(16), 256, 256, 128) == small
+    t = torch.tensor(16)
+    assert P.pifa_workspace_size(t, 256, 256, 128) == small
+    t.fill_(64)
+    assert P.pifa_workspace_size(t, 256, 256, 128) == large
