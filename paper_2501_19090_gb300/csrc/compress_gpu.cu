@@ -34,6 +34,7 @@
 #include "pifa.h"
 #include "pifa_internal.h"
 #include "ptx.cuh"
+#include "recip.h"
 
 namespace {
 
@@ -208,22 +209,6 @@ constexpr int CB = 32;    // columns per chol_panel
 constexpr int CP = 128;   // columns per panel
 
 constexpr int CR = 32;    // rows below the diagonal block per CTA of chol_panel
-
-// 1 / d for d > 0: the float32 reciprocal of d's significand, good to 2^-22, and one step of Halley's
-// third-order iteration r (1 + e + e^2), e = 1 - d r: three float64 instructions, of 64 cycles each for
-// a warp alone on its scheduler, where the division takes about ten.
-__device__ __forceinline__ double recip(double d) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-  const int ex = (int)(b >> 52);
-  if (ex < 64 || ex > 1982) return 1.0 / d;  // the scale below would leave the normal range
-  const float m = __uint_as_float(0x3f800000u | (uint32_t)((b >> 29) & 0x7fffffu));  // [1, 2)
-  const uint32_t q = __float_as_uint(__frcp_rn(m));                                   // (0.5, 1]
-  const unsigned long long rb =
-      ((unsigned long long)((int)(q >> 23) - 127 + 1023 - (ex - 1023)) << 52) | ((unsigned long long)(q & 0x7fffffu) << 29);
-  const double r = __longlong_as_double((long long)rb);
-  const double e = fma(-d, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
 
 // Columns [j0, j0 + CB) of L. Every CTA factors the 32 x 32 diagonal block itself (as U D U^T with
 // unit-lower U): the warp that holds column j + 1 finishes it first and takes its reciprocal while the

@@ -6,6 +6,7 @@ layers, LAPACK's pivoted QR on the LLaMA-shaped ones. C is pinned by Eq. 2 (||C 
 fp64 on the host on sampled rows.
 """
 import time
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -141,6 +142,31 @@ def test_float64_products_by_slices_are_exact_on_whole_numbers(m, n, r):
     assert P.pifa_device_status() == P.PIFA_OK
     assert np.array_equal(Wp, U[piv] @ V.T)
     _check_eqs(U, V, piv, nonp, Wp, C)
+
+
+@pytest.mark.parametrize("m,n,r", [(300, 129, 97), (257, 320, 128), (400, 191, 161), (520, 260, 257), (1500, 1500, 257),
+                                   (900, 700, 641)])
+def test_float64_products_by_slices_hold_every_digit(m, n, r):
+    """Operands with all 53 bits, so that all eight digits of every value count (the whole numbers above fill
+    the first three), against exact rational sums on sampled elements of W_p: one rounding to float64 and
+    the slices' truncation, 2^-62.2 sqrt(r) of the largest entries of the row and column in the root mean
+    square; eight times that is allowed. A pair of digits left out costs 2^-56 sqrt(r) at least, digits 7
+    2^-57. Around the 32-column K blocks, the 128-column accumulations and (1500, 1500, 257) two panels."""
+    rng = np.random.default_rng(m + r)
+    U, V = rng.standard_normal((m, r)), rng.standard_normal((n, r))
+    piv, nonp, Wp, C, _ = _device_compress(U, V)
+    assert P.pifa_device_status() == P.PIFA_OK
+    scale = lambda x: 2.0 ** np.frexp(np.abs(x).max())[1]
+    worst = 0.0
+    for _ in range(500):
+        i = int(rng.choice([0, 31, 96, r - 1, int(rng.integers(r))]))
+        j = int(rng.choice([0, 63, 64, n - 1, int(rng.integers(n))]))
+        a, b = U[piv[i]], V[j]
+        exact = sum(Fraction(x) * Fraction(y) for x, y in zip(a.tolist(), b.tolist()))
+        err = abs(Fraction(float(Wp[i, j])) - exact)
+        allowed = 2.0 ** -53 * abs(float(exact)) + 8 * 2.0 ** -62.2 * r ** 0.5 * scale(a) * scale(b)
+        worst = max(worst, float(err) / allowed)
+    assert worst <= 1.0, worst
 
 
 @pytest.mark.parametrize("r", [31, 32, 33, 127, 129, 160, 257, 300])
