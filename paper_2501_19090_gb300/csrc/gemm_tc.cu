@@ -28,6 +28,9 @@
 // on the same persistent grid took 253.6 and 538.1 us.
 // Every wait is bounded (globaltimer); on timeout the CTA latches PIFA_ERR_TIMEOUT, drains what it
 // has in flight and returns.
+#include <map>
+#include <mutex>
+
 #include <cuda_bf16.h>
 
 #include "pifa.h"
@@ -446,28 +449,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
 }
 
-// Pairs of CTAs that run at once: two SMs each, as many as the device's SM groups give.
+// Pairs of CTAs that run at once on the current device: two SMs each, as many as its SM groups give. A query
+// that fails counts as one for this call and is made again by the next.
 int pair_count() {
-  static int n = 0;
-  if (n == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int m = 0;
-    if (cudaOccupancyMaxActiveClusters(&m, gemm_tc_kernel, &cfg) != cudaSuccess || m < 1) {
-      cudaGetLastError();  // leaves no sticky error behind
-      m = 1;
-    }
-    n = m;
+  static std::mutex mu;
+  static std::map<int, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(dev);
+  if (it != known.end()) return it->second;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 2;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int m = 0;
+  if (dev < 0 || cudaOccupancyMaxActiveClusters(&m, gemm_tc_kernel, &cfg) != cudaSuccess || m < 1) {
+    cudaGetLastError();  // leaves no sticky error behind
+    return 1;
   }
-  return n;
+  return known[dev] = m;
 }
 
 int tile_width(const GemmTc& g, int want) {

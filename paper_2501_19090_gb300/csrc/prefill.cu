@@ -37,7 +37,8 @@
 // T = 512 227.2 -> 181.5, 4096 1460.2 -> 1226.3. At T = 2048 on the 7B attention layer each GEMM is one
 // round of 64 pair tiles: what is left is its 34 GFLOP at the tensor rate of 128 of 152 SMs (19 us), its
 // launch and first copies (about 5 us) and its exposed epilogue (about 3 us).
-#include <algorithm>
+#include <map>
+#include <mutex>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -444,35 +445,44 @@ Kern kernel_of(int epi, const GemmShape& sh) {
   return k[epi][sh.pair ? 0 : sh.ks > 1 ? 2 : 1];
 }
 
-// Tiles that run at once on the current device: pairs, single CTAs, clusters of 2 and of 4.
+// Tiles that run at once on the current device: pairs, single CTAs, clusters of 2 and of 4. A query that
+// fails counts as one for this call and is made again by the next.
 struct Slots {
   int pair, one, cl[2];
 };
-const Slots& tile_slots() {
-  static const Slots slots = [] {
-    auto query = [](const GemmShape& sh) {
-      const Kern k = kernel_of(EPI_Y_ONLY, sh);
-      cudaLaunchConfig_t cfg = {};
-      const unsigned c = sh.pair ? 2u : (unsigned)sh.ks;
-      cfg.gridDim = dim3(c);
-      cfg.blockDim = dim3(THREADS);
-      cfg.dynamicSmemBytes = SMEM_BYTES;
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = c;
-      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess ||
-          cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n < 1)
-        n = 1;
-      cudaGetLastError();  // a failed query leaves no sticky error behind
-      return n;
-    };
-    return Slots{query({true, BNMAX, 1}), query({false, BNMAX, 1}), {query({false, BNMAX, 2}), query({false, BNMAX, 4})}};
-  }();
-  return slots;
+Slots tile_slots() {
+  static std::mutex mu;
+  static std::map<int, Slots> known;
+  int dev = 0;
+  bool ok = cudaGetDevice(&dev) == cudaSuccess;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(dev);
+  if (ok && it != known.end()) return it->second;
+  auto query = [&](const GemmShape& sh) {
+    const Kern k = kernel_of(EPI_Y_ONLY, sh);
+    cudaLaunchConfig_t cfg = {};
+    const unsigned c = sh.pair ? 2u : (unsigned)sh.ks;
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = c;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n < 1) {
+      n = 1;
+      ok = false;
+    }
+    cudaGetLastError();  // a failed query leaves no sticky error behind
+    return n;
+  };
+  const Slots s = {query({true, BNMAX, 1}), query({false, BNMAX, 1}), {query({false, BNMAX, 2}), query({false, BNMAX, 4})}};
+  if (ok) known[dev] = s;
+  return s;
 }
 
 // Bytes of one 64-column chunk of a tile in a CTA's ring, and chunks per stage: two where the ring
@@ -485,7 +495,7 @@ int subs_for(bool pair, int bn) { return RING_BYTES / chunk_bytes(pair, bn) >= 6
 // cycles: a chunk's (see the head of this file), an unhidden epilogue's 25 per token of a tile's width,
 // a launch's 9600 (a pair's 10600), a cluster's 12500 and its exchange of partial tiles 20 per token.
 GemmShape pick_shape(int64_t G, int64_t rows, int64_t T, int64_t kchunks) {
-  const Slots& slots = tile_slots();
+  const Slots slots = tile_slots();
   GemmShape best = {true, BNMAX, 1};
   double best_cost = -1.0;
   for (int form = 0; form < 4; ++form) {  // pairs, single CTAs, clusters of 2, of 4
