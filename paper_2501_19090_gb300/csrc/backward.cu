@@ -181,12 +181,10 @@ struct MaccLayout {
   int64_t xmix, xmix_lo, ytt, ytt_lo, total;
 };
 
-// The mixed input's hi and lo planes (T x pad8(n)), Y_t^T's hi and lo planes (m x pad8(T)), all bf16,
-// behind n x pad8(T) values that nothing uses any more: the size that callers are asked for stays.
+// The mixed input's hi and lo planes (T x pad8(n)), Y_t^T's hi and lo planes (m x pad8(T)), all bf16
 MaccLayout macc_layout(int64_t T, int64_t m, int64_t n) {
   MaccLayout L;
   int64_t o = 0;
-  o += a256(n * pad8(T) * 2);
   L.xmix = o;
   o += a256(T * pad8(n) * 2);
   L.xmix_lo = o;

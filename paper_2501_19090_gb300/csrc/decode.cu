@@ -60,7 +60,7 @@ using bf16 = __nv_bfloat16;
 
 // Weight rows per CTA: RG MMA row groups of 16. Taller tiles read less of the broadcast operand
 // per weight byte (RG = 4 reads 4x less than RG = 1) but split K over larger clusters whose
-// partial tiles must be summed; rows_form chooses by the phase's shape and T.
+// partial tiles must be summed; plan_rows chooses by the phase's shape and T.
 template <int RG>
 constexpr int kRowsOf = 16 * RG;
 constexpr int kChunk = 32;          // K elements per warp step (two k16 MMAs)

@@ -117,16 +117,6 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
   asm volatile("mov.u32 %0, %cluster_nctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ uint32_t cluster_id_x() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %clusterid.x;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t nclusters_x() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %nclusterid.x;" : "=r"(r));
-  return r;
-}
 // Hardware cluster barrier, all threads of every CTA in the cluster (used only at kernel start
 // and end, where every CTA is guaranteed to arrive).
 __device__ __forceinline__ void cluster_sync_all() {
@@ -148,12 +138,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void st_dsmem_f32(uint32_t cluster_saddr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_saddr), "f"(v) : "memory");
 }
-// 32-bit load from the shared memory of a CTA of this cluster (shared::cluster address).
-__device__ __forceinline__ float ld_dsmem_f32(uint32_t cluster_saddr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_saddr) : "memory");
-  return v;
-}
+// 128-bit load from the shared memory of a CTA of this cluster (shared::cluster address).
 __device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t cluster_saddr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -208,10 +193,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 // thread has observed complete before its later generic-proxy accesses of the same bytes.
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-// Order this thread's generic-proxy global writes before later async-proxy (TMA) accesses.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
 // Named barrier `id` over `count` threads (a multiple of 32) of this CTA.
