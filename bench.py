@@ -5,7 +5,8 @@ gate/up projection m = 28672, n = 8192, r = 4096 (the largest layer of the workl
 one GPU), decode batch T = 16, bf16. The step runs the whole hot path: the selector, Y_p = X W_p^T,
 Y_np = Y_p C^T and both scatters into Y.
 
-Printed as one JSON line on rank 0:
+Printed as one JSON line of at most 2 KB on rank 0's standard output (the full record, with the texts that
+say how each part was measured and the extras below, goes to standard error, a line per part):
   value      tokens/s, device-timed with CUDA events on the launching stream over exactly --steps
              steps replayed from CUDA graphs; the timed region is repeated until the clock sampler
              has seen it (value = the median repetition); the weights rotate over enough copies
@@ -916,6 +917,31 @@ def _traffic(layer, T):
     return t["bytes"]
 
 
+# The fields that the line on standard output keeps of each of these parts (parts not named here are kept
+# whole, the extras left out): whoever reads a job's output may see no more than its last 2 or 3 KB.
+LINE_PARTS = {
+    "config": ("workload", "m", "n", "r", "tokens_per_step", "c_dtype", "variant", "parallelism", "l2_defeat"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "serial_value"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_source", "algorithmic_bytes_per_launch",
+                 "algorithmic_flops_per_launch"),
+    "comparators": ("us_per_call", "lowrank_us", "dense_us", "speedup_vs_lowrank", "speedup_vs_dense"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+    "clocks": ("sm_mhz", "sm_max_mhz", "reasons", "samples"),
+}
+EXTRAS = ("decode_points", "mlp7b_three_layers", "prefill_points", "rank_sweep", "backward", "m_accumulate")
+
+
+def _line(out):
+    """The record without its extras and longer texts."""
+    line = {}
+    for k, v in out.items():
+        if k in LINE_PARTS and isinstance(v, dict):
+            v = {f: v[f] for f in LINE_PARTS[k] if f in v} or v
+        if k not in EXTRAS:
+            line[k] = v
+    return line
+
+
 # ---------------------------------------------------------------------------------------------
 _DIST = None
 
@@ -1005,7 +1031,9 @@ def main():
         _DIST = dist
     out = run_ours(args, rank, world, local_rank)
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        for k in [k for k in out if k in LINE_PARTS or k in EXTRAS]:
+            print(json.dumps({k: out[k]}), file=sys.stderr, flush=True)
+        print(json.dumps(_line(out)), flush=True)
     if _DIST:
         _DIST.barrier()
         _DIST.destroy_process_group()

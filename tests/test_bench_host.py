@@ -63,3 +63,42 @@ def test_bench_decode_rule_is_the_library_selector(m, n, r):
     from paper_2501_19090_gb300 import pifa as P
     for T in (1, 16, 64, 65, 96, 128, 129, 2048):
         assert (P.pifa_select_variant(T, m, n, r) == P.PIFA_VARIANT_DECODE) == bench.is_decode(T, m, r), T
+
+
+def test_the_printed_line_is_short_and_holds_the_contract():
+    """The line that goes to standard output: every required key, whole numbers' and floats' full digits, no
+    extras, at most 2 KB even with the longest values of each field."""
+    f = 123456.78901234567
+    text = "x" * 700
+    out = {"metric": bench.METRIC, "value": f, "unit": "tokens/s", "n_gpus": 1, "steps": 2000, "warmup": 5,
+           "ms_per_step": f, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
+           "data": "synthetic",
+           "config": {"workload": "llama2_70b_gate_up_28672x8192_r4096 decode T=16", "m": 28672, "n": 8192, "r": 4096,
+                      "tokens_per_step": 16, "c_dtype": "bf16", "variant": "decode", "parallelism": "replicas1",
+                      "operands": text, "l2_defeat": "4 rotating weight copies with their own X and Y (1074 MB > 3x L2)",
+                      "timing": text},
+           "timed_repeats": 4,
+           "e2e": {"value": f, "unit": "tokens/s", "h2d_bytes_per_step": 262144, "d2h_bytes_per_step": 917504,
+                   "mode": text, "serial_value": f, "serial_mode": text},
+           "roofline": {"bound": "hbm", "achieved": f, "peak": 6798.9, "unit": "GB/s", "frac": f, "traffic": 269364992,
+                        "peak_source": "measured hbm_gbs (burst: the call is timed alone)", "kernel": text,
+                        "algorithmic_bytes_per_launch": 269729792},
+           "gpu_launches": 4000, "gpu_launches_per_step": 2, "gpu_launches_all_repeats": 16000,
+           "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 4,
+                      "gpu_temp_c": [35.0, 36.0]},
+           "comparators": {"workload": text, "us_per_call": f, "lowrank_us": f, "dense_us": f, "speedup_vs_lowrank": f,
+                           "speedup_vs_dense": f, "roofline": {"bound": "hbm"}},
+           **{k: [{"workload": text}] * 20 for k in bench.EXTRAS},
+           "cpu_baseline": {"value": f, "unit": "tokens/s", "cores": 16, "kind": "oracle", "sample": text}}
+    line = bench._line(out)
+    assert len(bench.json.dumps(line)) <= 2048
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "gpu_launches"):
+        assert line[k] == out[k]
+    for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"):
+        assert line["e2e"][k] == out["e2e"][k]
+    for k in ("sm_mhz", "sm_max_mhz", "reasons"):
+        assert line["clocks"][k] == out["clocks"][k]
+    assert line["config"]["workload"] == out["config"]["workload"] and line["config"]["l2_defeat"]
+    failed = dict(out, cpu_baseline={"error": "why"})
+    assert bench._line(failed)["cpu_baseline"] == {"error": "why"}
