@@ -817,3 +817,44 @@ def test_binding_refuses_bad_cuda_operands_before_the_library():
     with pytest.raises(ValueError):  # the allocation-free entry point takes bf16 C only
         P.pifa_forward_decode_noalloc(X, Wp, C.half(), piv, nonp, Y=Y)
     assert P.pifa_launch_count() == c0
+
+
+# ---------------------------------------------------------------------------------------------
+# the binding's two operand checks
+# ---------------------------------------------------------------------------------------------
+def test_the_quick_operand_check_accepts_what_the_full_one_accepts(monkeypatch):
+    """_operands_ok answers without messages, _operands' own checks say what is wrong: over well-formed and
+    malformed operands, alone and grouped, both must take the same calls."""
+    T, n, m, r = 4, 64, 48, 16
+    bf = lambda *shape, dtype=torch.bfloat16, device=DEV: torch.zeros(shape, dtype=dtype, device=device)
+    ids = lambda k, dtype=torch.int32, device=DEV: torch.arange(k, dtype=dtype, device=device)
+    changes = [
+        {}, {"Y": None}, {"ws": None}, {"C": bf(m - r, r, dtype=torch.float16)}, {"C": None}, {"nonp": None},
+        {"nonp": None, "C": None, "Y": None}, {"nonp": ids(0), "C": None, "Y": None}, {"nonp": ids(0), "C": bf(0, r), "Y": None},
+        {"X": bf(T, n)[::2]}, {"X": bf(0, n), "Y": bf(0, m)}, {"X": bf(n, T).t()}, {"X": bf(T * n)}, {"X": [1]}, {"X": None},
+        {"X": bf(T, n, dtype=torch.float32)}, {"X": bf(T, n, device="cpu")}, {"X": bf(T, n + 8)}, {"Wp": None}, {"Wp": bf(r, n, 1)},
+        {"Wp": bf(r, n, dtype=torch.float16)}, {"Wp": bf(r, n, device="cpu")}, {"Wp": bf(r + 1, n)}, {"C": bf(m - r, r + 8)},
+        {"C": bf(m - r, r, device="cpu")}, {"C": bf(m - r, r, dtype=torch.float32)}, {"C": [1]}, {"piv": None}, {"piv": ids(r - 1)},
+        {"piv": ids(2 * r)[::2]}, {"piv": ids(r, torch.int64)}, {"piv": ids(r, device="cpu")}, {"piv": ids(r).view(r, 1)},
+        {"nonp": ids(m - r, torch.int64)}, {"nonp": ids(m - r, device="cpu")}, {"nonp": ids(2 * (m - r))[::2]}, {"nonp": [1]},
+        {"nonp": ids(m - r + 1)}, {"nonp": ids(m - r).view(1, -1)}, {"Y": bf(T, m + 8)}, {"Y": bf(T, m, dtype=torch.float32)},
+        {"Y": bf(T, m, device="cpu")}, {"Y": [1]}, {"ws": bf(64, device="cpu")}, {"ws": [1]}]
+    quick = P._operands_ok
+    taken = 0
+    for G in (1, 2):
+        for c16 in (True, False):
+            for ch in changes:
+                a = dict(X=bf(T, n), Wp=bf(G * r, n), C=bf(G * (m - r), r), piv=ids(G * r), nonp=ids(G * (m - r)),
+                         Y=bf(T, G * m), ws=bf(64))
+                a.update(ch)
+                args = (G, a["X"], a["Wp"], a["C"], a["piv"], a["nonp"], a["Y"], a["ws"], c16)
+                got = quick(*args)
+                with monkeypatch.context() as mp:
+                    mp.setattr(P, "_operands_ok", lambda *_: None)
+                    try:
+                        want = P._operands(*args)
+                    except ValueError:
+                        want = None
+                assert got == want, (G, c16, ch)
+                taken += got is not None
+    assert taken >= 12
