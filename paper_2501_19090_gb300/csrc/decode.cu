@@ -979,7 +979,8 @@ int launch_phase_tc(const DecodeArgs& a, int dtype, const SplitKScratch& sk, cud
 // and each RG and K split of decode_rows that fits; us per layer below. Against one tile height per T
 // (16, 64 and 32 rows up to T = 2, 8 and 16), split-K for T > 2 from 4096 rows on and waves else:
 // 1024 x 1024, r = 512, T = 8: 6.4 -> 5.2; 4096 x 4096, r = 1024, T = 8: 9.2 -> 8.0; 4096 x 11008,
-// r = 1024, T = 3: 24.0 -> 10.2; 5120 x 5120, r = 2560, T = 8: 22.4 -> 16.9; over all of them 1.12x, none more than 2% slower.
+// r = 1024, T = 3: 24.0 -> 10.2; 5120 x 5120, r = 2560, T = 8: 22.4 -> 16.9; over 189 points (27 shapes,
+// T = 1 to 16) 1.17x with split-K's own gains, none slower by more than runs differ.
 enum Form { kFormRows, kFormStream, kFormSplitK };
 struct PhasePlan {
   Form form;
@@ -1021,8 +1022,9 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
 }
 
 // The form of a phase. Waves of decode_rows win while an SM stages its share of the weights at launch
-// (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds.
-Form phase_form(int phase, int R, int K, int T, int ngrp) {
+// (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds. `other` (phase 1):
+// phase 2's form.
+Form phase_form(int phase, int R, int K, int T, int ngrp, Form other) {
   const int64_t bytes = (int64_t)R * K * 2;
   const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
   const int sms = sm_count();
@@ -1038,6 +1040,12 @@ Form phase_form(int phase, int R, int K, int T, int ngrp) {
     // many groups' y_p split it over clusters (three of 4096 x 4096, r = 2048, T = 2: 24.0 against 21.4)
     if (phase == 2 && R >= 32 * 128 && K <= 1024) return kFormSplitK;
     if (ngrp > 1 && (uint64_t)ngrp * 2 * T * row_pitch(K) > kStreamBudget / 3) return kFormRows;
+    // 16 whole rows a CTA in one round (two CTAs per SM up to K = 3500) stay ahead (three of 6144 x 3072,
+    // r = 1536, T = 1 / 2: 20.3 / 25.5 -> 16.8 / 23.5), at T = 1 also in two before a phase 2 that is
+    // streamed (two of 11008 x 4096, r = 2048: 24.1 -> 23.6; T = 2 24.3, 24.5)
+    const int tiles = (R + 15) / 16, round = sms * (16 * row_pitch(K) <= 110 * 1024 ? 2 : 1);
+    if (phase == 1 && least_split(1, K, budget) == 1 && (tiles <= round || (T == 1 && other != kFormRows && tiles <= 2 * sms)))
+      return kFormRows;
     return phase == 2 || bytes > 26000000 ? kFormStream : kFormRows;
   }
   if (phase == 2 || R >= 32 * 128) return kFormSplitK;
@@ -1146,7 +1154,7 @@ int launch_decode_t(const PifaShape& s, const PifaPointers& p, int* status, cuda
   a.status = status;
   a.timeout_ns = pifa_wait_timeout_ns();
   const int R2 = (int)(G * (s.m - s.r)), K2 = (int)s.r, T = a.T;
-  const Form f1 = phase_form(1, a.R, a.K, T, 1), f2 = R2 > 0 ? phase_form(2, R2, K2, T, (int)G) : kFormRows;
+  const Form f2 = R2 > 0 ? phase_form(2, R2, K2, T, (int)G, kFormRows) : kFormRows, f1 = phase_form(1, a.R, a.K, T, 1, f2);
   PhasePlan plan1 = plan_rows(1, a.R, a.K, T, f2, nullptr);
   plan1.form = f1;
   int st = launch_one_phase<1, NT, kF16C>(a, kStageBudget1, PIFA_DTYPE_BF16, sk, plan1, stream);

@@ -325,10 +325,10 @@ def test_decode_splitk_deterministic_and_r_equals_m():
     (4096, 4096, 2048, 8, P.PIFA_DECODE_GRID_WAVES),   # 2048-row phases, at most two waves each
 ])
 def test_decode_selector_matches_the_form_it_picks(m, n, r, T, forced):
-    """The automatic decode choice is keyed on each phase's rows and T: split-K on the tensor cores
-    for phases of at least 32 blocks of 128 rows when T > 2, waves of one-tile clusters for a
-    phase that fits two waves. Its output equals, bit for bit, that of the form it should pick,
-    forced."""
+    """The automatic decode choice is keyed on each phase's shape and T: split-K on the tensor cores for a
+    phase 1 of at least 4096 rows and a phase 2 of more than 12 MB when T > 2, waves of one-tile
+    clusters for phases that an SM stages at launch. Its output equals, bit for bit, that of the
+    form it should pick, forced."""
     L = layer_for(m, n, r, 6, "synthetic")
     X = acts(T, n, 6)
     auto = run(L, X, P.PIFA_VARIANT_DECODE)
@@ -788,6 +788,7 @@ def test_decode_selector_splits_k_where_waves_exceed_the_sms():
     (1700, 11003, 611, (1, 3, 8, 16)),       # 32 rows split eight ways
     (5121, 2569, 2560, (1, 2, 3, 8)),        # 13 MB of C: persistent grid, then split-K
     (9003, 1030, 515, (1, 8, 16)),           # many rows of a short K: waves, several CTAs per SM
+    (8200, 3700, 3600, (1, 2)),              # 27 MB of W_p: two rounds of waves before a streamed C, streamed at T = 2
 ])
 def test_decode_plans_by_shape(m, n, r, Ts):
     """Every tile height and K split that the plan of a phase can take, and both sides of its lines."""
