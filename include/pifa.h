@@ -372,7 +372,7 @@ int pifa_set_wait_timeout(int64_t ns);
  * phase deals equal ranges of 128 x 64 weight tiles to a persistent grid and a second kernel sums
  * the fp32 partial sums in a fixed order.
  * PIFA_DECODE_GRID_AUTO (0, the default) picks per phase from its shape and T: waves while an SM can
- * stage its share of the weights at launch (about 24 MB in phase 1, for T <= 2 up to 40 MB of whole rows,
+ * stage its share of the weights at launch (about 24 MB in phase 1, more where its CTAs make full rounds,
  * 12 MB in phase 2, at most two rounds); beyond, the persistent grid for T <= 2 and split-K for T > 2, which also takes a phase 1 of
  * R >= 4096, and for T > 8 phases whose waves would need more CTAs than there are SMs. The waves' tile
  * height (16, 32 or 64 rows) and K split follow from shape and T in every mode.

@@ -980,7 +980,8 @@ int launch_phase_tc(const DecodeArgs& a, int dtype, const SplitKScratch& sk, cud
 // (16, 64 and 32 rows up to T = 2, 8 and 16), split-K for T > 2 from 4096 rows on and waves else:
 // 1024 x 1024, r = 512, T = 8: 6.4 -> 5.2; 4096 x 4096, r = 1024, T = 8: 9.2 -> 8.0; 4096 x 11008,
 // r = 1024, T = 3: 24.0 -> 10.2; 5120 x 5120, r = 2560, T = 8: 22.4 -> 16.9; over 189 points (27 shapes,
-// T = 1 to 16) 1.17x with split-K's own gains, none slower by more than runs differ.
+// T = 1 to 16) 1.17x with split-K's own gains, the slowest 0.973x; over 3888 points of drawn layers, weights in L2
+// and from HBM, 1.14x, 150 of them below 0.985x and the slowest 0.88x (tall or warm phases at the ends of the lines).
 enum Form { kFormRows, kFormStream, kFormSplitK };
 struct PhasePlan {
   Form form;
@@ -994,26 +995,34 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
   const int sms = sm_count();
   const int64_t work = (int64_t)R * K;
   const int k1 = least_split(1, K, budget), k2 = least_split(2, K, budget);
-  const int tiles = (R + 31) / 32, tall = (R + 63) / 64 * 4;  // 32-row tiles; CTAs of 64 rows split four ways
+  const int t16 = (R + 15) / 16, tiles = (R + 31) / 32, tall = (R + 63) / 64 * 4;  // tall: CTAs of 64 rows split four ways
+  const bool full2 = t16 * 7 >= sms * 6 && t16 <= sms;
   const bool fits4 = (uint64_t)64 * row_pitch(kcta_of(K, 4)) <= budget;
   // 64 rows split four ways where that is one round of most SMs (in phase 2 behind such a phase 1,
   // whose CTAs leave room for its own): 4096 x 4096, r = 2048, T = 8: 9.3, 32 rows split two ways 10.0
   const bool behind = first && first->rg == 4 && first->ks == 4;
   const bool round = fits4 && tall * 3 >= sms * 2 && (phase == 1 ? tall <= sms : behind && tall * 4 <= sms * 5);
   if (T <= 2) {
-    if (phase == 1 && round && tall * 5 >= sms * 4 && other == kFormRows) return {kFormRows, 4, 4};  // T = 1: 8.9 -> 8.2
+    // T = 1: 8.9 -> 8.2, weights from HBM; shorter rows are ahead in tiles of 16 (2048 x 3456: 9% slower)
+    if (phase == 1 && round && K >= 3800 && tall * 5 >= sms * 4 && other == kFormRows) return {kFormRows, 4, 4};
+    // clusters of two of 16 rows where those make two full rounds of one CTA per SM (2432 x 4992: 1.15x)
+    if (phase == 1 && k1 == 2 && full2) return {kFormRows, 1, 2};
     // x is short: 16 rows, unless the phase is so small that half the CTAs do, or K needs a split
-    const int rg = (work < (1 << 22) && k2 == 1) || k1 != 1 ? 2 : 1;
+    // (10752 rows of 128: two rounds of 32 rows 1.3x one of 16)
+    const int rg = (work < (1 << 22) && k2 == 1 && tiles <= 2 * sms) || k1 != 1 ? 2 : 1;
     return {kFormRows, rg, rg == 2 ? k2 : k1};
   }
   if (T <= 8) {
     if (round && other != kFormSplitK) return {kFormRows, 4, 4};
+    // the same in phase 2 where two ways of 32 rows leave one CTA per SM, and for 12 MB and more (see phase_form)
+    if (phase == 2 && fits4 && ((k2 == 2 && K >= 2100 && tall * 5 >= sms * 3 && tall <= sms) || work > 6000000)) return {kFormRows, 4, 4};
     // several rounds of clusters of four: clusters of eight of the tall tiles read half of x
     if (k2 == 4 && tiles * 16 > sms * 5 && least_split(4, K, budget) == 8) return {kFormRows, 4, 8};
     // a small phase needs no more SMs, and a split-K phase behind this one wants the free ones
     if (work < (1 << 22) || other == kFormSplitK) return {kFormRows, 2, k2};
   } else {
-    if (work < (1 << 20)) return {kFormRows, 1, k1};
+    // a small phase in 16 rows, but a long K in 32 and split once more (146 x 7130: 0.88x)
+    if (work < (1 << 20)) return (phase == 1 ? k1 == 1 : K <= 1400) ? PhasePlan{kFormRows, 1, k1} : PhasePlan{kFormRows, 2, k2};
     if (phase == 1 && round && other != kFormSplitK) return {kFormRows, 4, 4};
   }
   int ks = k2;
@@ -1022,42 +1031,52 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
 }
 
 // The form of a phase. Waves of decode_rows win while an SM stages its share of the weights at launch
-// (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds. `other` (phase 1):
-// phase 2's form.
-Form phase_form(int phase, int R, int K, int T, int ngrp, Form other) {
-  const int64_t bytes = (int64_t)R * K * 2;
+// (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds. Full rounds of two
+// CTAs per SM (tiles of up to 110 KB) hold on longer. Ratios in these comments: time of the other form over this.
+Form phase_form(int phase, int R, int K, int T, int ngrp) {
+  const int64_t work = (int64_t)R * K, bytes = work * 2;
   const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
   const int sms = sm_count();
+  const int k1 = least_split(1, K, budget), k2 = least_split(2, K, budget);
+  const int t16 = (R + 15) / 16, t32 = (R + 31) / 32;
   if (phase == 2 && bytes <= 12000000) {
-    // with two token tiles a K split in more CTAs than SMs loses to split-K (4096 x 4096, r = 2458,
-    // T = 12: 15.8 against 15.0)
-    const int k2 = least_split(2, K, budget);
-    return T > 8 && k2 != 1 && (R + 31) / 32 * k2 > sms ? kFormSplitK : kFormRows;
+    // more CTAs than two per SM lose to split-K (21248 x 256, T = 12: 1.5x, 10752 x 128: 1.3x, 5828 x 108: 1.4x)
+    if (T > 2 && R >= 4096 && (T > 8 && work < (1 << 20) ? t16 * k1 : t32 * k2) > 2 * sms) return kFormSplitK;
+    // with two token tiles a K split four ways in more CTAs than SMs loses to split-K (4096 x 4096,
+    // r = 2458, T = 12: 15.8 against 15.0); split two ways it does not (2458 x 1638: 0.94x)
+    return T > 8 && k2 > 2 && t32 * k2 > sms ? kFormSplitK : kFormRows;
   }
   if (T <= 2) {
     // decode_stream, whose x / y_p stay resident (8192 x 8192, r = 2048, T = 1: 20.3 -> 18.0); a K of
-    // 1024 or less is too short for its ring (11008 x 4096, r = 1024: split-K 10.8, stream 12.1), and
-    // many groups' y_p split it over clusters (three of 4096 x 4096, r = 2048, T = 2: 24.0 against 21.4)
-    if (phase == 2 && R >= 32 * 128 && K <= 1024) return kFormSplitK;
+    // 1024 or less is too short for its ring (11008 x 4096, r = 1024: split-K 10.8, stream 12.1; but 9728 x 896,
+    // two full rounds of waves: 1.3x), and many groups' y_p split it over clusters (three of 4096 x 4096, r = 2048,
+    // T = 2: 24.0 against 21.4)
+    if (phase == 2 && R >= 32 * 128 && K <= 1024) return t16 * 2 > sms * 7 && t16 <= sms * 4 ? kFormRows : kFormSplitK;
     if (ngrp > 1 && (uint64_t)ngrp * 2 * T * row_pitch(K) > kStreamBudget / 3) return kFormRows;
+    if (phase == 2) return k1 == 1 && t16 <= sms * 2 ? kFormRows : kFormStream;  // 3840 x 2176: 1.2x
     // 16 whole rows a CTA in one round (two CTAs per SM up to K = 3500) stay ahead (three of 6144 x 3072,
-    // r = 1536, T = 1 / 2: 20.3 / 25.5 -> 16.8 / 23.5), at T = 1 also in two before a phase 2 that is
-    // streamed (two of 11008 x 4096, r = 2048: 24.1 -> 23.6; T = 2 24.3, 24.5)
-    const int tiles = (R + 15) / 16, round = sms * (16 * row_pitch(K) <= 110 * 1024 ? 2 : 1);
-    if (phase == 1 && least_split(1, K, budget) == 1 && (tiles <= round || (T == 1 && other != kFormRows && tiles <= 2 * sms)))
-      return kFormRows;
-    return phase == 2 || bytes > 26000000 ? kFormStream : kFormRows;
+    // r = 1536, T = 1 / 2: 20.3 / 25.5 -> 16.8 / 23.5), and clusters of two in two full ones (2432 x 8704:
+    // 1.2x, weights in L2; from HBM the same)
+    if (k1 == 1 && t16 <= sms * (16 * row_pitch(K) <= 110 * 1024 ? 2 : 1)) return kFormRows;
+    if (k1 == 2 && t16 * 7 >= sms * 6 && t16 <= sms) return kFormRows;
+    return bytes > 26000000 ? kFormStream : kFormRows;
   }
-  if (phase == 2 || R >= 32 * 128) return kFormSplitK;
-  const int k2 = least_split(2, K, budget);
+  if (phase == 2) {  // 64 rows split four ways, up to 17 MB (3840 x 2176, T = 4: 1.06x)
+    const bool fits4 = (uint64_t)64 * row_pitch(kcta_of(K, 4)) <= budget;
+    return T <= 8 && fits4 && (R + 63) / 64 * 20 <= sms * 8 ? kFormRows : kFormSplitK;
+  }
+  if (R >= 32 * 128) return kFormSplitK;
   if (T <= 8) {
     // clusters of eight of 64 rows stay ahead for two rounds (8192 x 8192, r = 2048, T = 8: 20.8, split-K 21.5)
     const bool two = k2 == 4 && least_split(4, K, budget) == 8 && (R + 63) / 64 * 8 <= 2 * sms;
     return bytes > 26000000 && !two ? kFormSplitK : kFormRows;
   }
   // two token tiles: 4096 x 4096, r = 3072, T = 16: 18.9 -> 15.1; few row blocks keep split-K slow
-  // (4096 x 11008, r = 1024, T = 16: 16.7, waves 14.2)
-  return k2 == 0 || bytes > 24000000 || (R >= 2048 && (R + 31) / 32 * k2 > sms) ? kFormSplitK : kFormRows;
+  // (4096 x 11008, r = 1024, T = 16: 16.7, waves 14.2), and one round of waves stays ahead (2816 x 2816,
+  // two CTAs per SM: 1.1x; 1024 x 12416: 1.2x)
+  if (k2 > 0 && (k2 <= 2 || R < 2048) && t32 * k2 <= sms * (32 * row_pitch(kcta_of(K, k2)) <= 110 * 1024 ? 2 : 1))
+    return kFormRows;
+  return k2 == 0 || bytes > 24000000 || (R >= 2048 && t32 * k2 > sms) ? kFormSplitK : kFormRows;
 }
 
 // decode_rows on one phase, if its clusters take at most two rounds (or `always`): its weights staged
@@ -1154,7 +1173,7 @@ int launch_decode_t(const PifaShape& s, const PifaPointers& p, int* status, cuda
   a.status = status;
   a.timeout_ns = pifa_wait_timeout_ns();
   const int R2 = (int)(G * (s.m - s.r)), K2 = (int)s.r, T = a.T;
-  const Form f2 = R2 > 0 ? phase_form(2, R2, K2, T, (int)G, kFormRows) : kFormRows, f1 = phase_form(1, a.R, a.K, T, 1, f2);
+  const Form f1 = phase_form(1, a.R, a.K, T, 1), f2 = R2 > 0 ? phase_form(2, R2, K2, T, (int)G) : kFormRows;
   PhasePlan plan1 = plan_rows(1, a.R, a.K, T, f2, nullptr);
   plan1.form = f1;
   int st = launch_one_phase<1, NT, kF16C>(a, kStageBudget1, PIFA_DTYPE_BF16, sk, plan1, stream);

@@ -788,7 +788,14 @@ def test_decode_selector_splits_k_where_waves_exceed_the_sms():
     (1700, 11003, 611, (1, 3, 8, 16)),       # 32 rows split eight ways
     (5121, 2569, 2560, (1, 2, 3, 8)),        # 13 MB of C: persistent grid, then split-K
     (9003, 1030, 515, (1, 8, 16)),           # many rows of a short K: waves, several CTAs per SM
-    (8200, 3700, 3600, (1, 2)),              # 27 MB of W_p: two rounds of waves before a streamed C, streamed at T = 2
+    (10880, 256, 128, (1, 3, 9)),            # more 32-row CTAs of a short K than two per SM: 16 rows, split-K
+    (10624, 1000, 896, (1, 2)),              # two full rounds of whole 16-row tiles
+    (6016, 2200, 2176, (1, 2, 4, 9)),        # one round of them in phase 2; 64 rows split four ways at 17 MB
+    (4224, 2400, 2304, (3, 8, 16)),          # phase 2: 64 rows split four ways in one round
+    (3328, 8704, 2432, (1, 2)),              # clusters of two of 16 rows, two full rounds
+    (2000, 12416, 1024, (9, 16)),            # 25 MB in one round of clusters of eight
+    (3000, 2816, 2816, (9, 16)),             # 32 rows split two ways, two CTAs per SM
+    (400, 7130, 146, (9, 16)),               # few rows of a long K
 ])
 def test_decode_plans_by_shape(m, n, r, Ts):
     """Every tile height and K split that the plan of a phase can take, and both sides of its lines."""
