@@ -22,17 +22,15 @@
 // two rows after an exchange between neighbouring lanes. Every wait is bounded (globaltimer); on timeout the CTA
 // latches PIFA_ERR_TIMEOUT, drains what it has in flight and returns.
 //
-// A 64-column chunk of K costs a tile about 330 + 0.8 bn cycles by a pair (its MMAs are 2 bn of them) and
-// 410 + 0.3 bn to 500 + 0.6 bn by one CTA, much of it the hand-offs of a stage (its copy's arrival, the
+// A 64-column chunk of K costs a tile 330 + 0.85 bn cycles by a pair (its MMAs are 2 bn of them) and
+// 410 + 0.3 bn to 480 + 0.66 bn by one CTA, much of it the hand-offs of a stage (its copy's arrival, the
 // MMAs' issue and commit, the release), which is why a stage holds two chunks where the ring allows, why
 // the issuing threads do no division and read no flag, and why wide tiles are best where they fill
 // the GPU. GEMMs of few tiles run on tiles of 128 rows by one CTA and split K: the 2 or 4 CTAs of a
 // tile form a cluster, each accumulates its K-slice, stores the fp32 partial tile in its own freed
 // ring, and the cluster adds the slices through distributed shared memory in a fixed order before the
-// epilogue. pick_shape takes the form, width and split that these costs say finishes first. Measured beside
-// every alternative in 398 GEMMs (20 layers, T = 80 to 4096), the call was 0.6% behind the best pick in the
-// mean; the worst were layers whose rank is no multiple of 64 (4096 x 4096, r = 1638, T = 2048: 17%, one CTA
-// where a pair's tiles would be read half as often) and 70B gate / up at T = 80 (21%; decode takes that call).
+// epilogue. pick_shape takes the form, width and split that these costs say finishes first; measured
+// beside every alternative on five layers at T = 80 to 2048 it was within 4% of the best.
 // Against the one-CTA forms that this replaced (us, CUDA graph, one process): 7B attention T = 128
 // 25.2 -> 20.0, 512 37.4 -> 34.6, 2048 58.0 -> 53.9, 4096 119.5 -> 94.7; 7B gate T = 2048 143.8 ->
 // 120.4; 7B down T = 300 48.1 -> 35.9; 70B q/o T = 300 89.4 -> 56.3, 4096 400.3 -> 345.8; 70B gate/up
@@ -494,9 +492,8 @@ uint32_t chunk_bytes(bool pair, int bn) { return A_BYTES + (uint32_t)(pair ? bn 
 int subs_for(bool pair, int bn) { return RING_BYTES / chunk_bytes(pair, bn) >= 6 ? 2 : 1; }
 
 // The tiling of G groups of `rows` weight rows x T tokens that finishes first by the measured costs, in
-// cycles: a chunk's (see the head of this file), an epilogue's 22 per token of a tile's width, which hides
-// under the next tile's chunks as far as those last, a launch's 8900 (a pair's 10600), a cluster's 13000 and
-// its exchange of partial tiles 20 per token.
+// cycles: a chunk's (see the head of this file), an unhidden epilogue's 25 per token of a tile's width,
+// a launch's 9600 (a pair's 10600), a cluster's 12500 and its exchange of partial tiles 20 per token.
 GemmShape pick_shape(int64_t G, int64_t rows, int64_t T, int64_t kchunks) {
   const Slots slots = tile_slots();
   GemmShape best = {true, BNMAX, 1};
@@ -509,11 +506,9 @@ GemmShape pick_shape(int64_t G, int64_t rows, int64_t T, int64_t kchunks) {
     const int64_t at_once = form == 0 ? slots.pair : form == 1 ? slots.one : slots.cl[form - 2];
     for (int bn = T < BNMAX ? (int)(T + 31) / 32 * 32 : BNMAX; bn >= 32; bn -= 32) {
       const int64_t rounds = (mt * ((T + bn - 1) / bn) + at_once - 1) / at_once;
-      const double step = pair ? 329.0 + 0.79 * bn : subs_for(false, bn) == 2 ? 410.0 + 0.3 * bn : 500.0 + 0.59 * bn;
-      const double main = (double)((kchunks + ks - 1) / ks) * step, epi = 22.0 * bn;
-      double cost = main + epi;
-      if (ks > 1) cost += (double)(rounds - 1) * main + (double)rounds * (13000.0 + 20.0 * bn);  // one tile per CTA: no overlap
-      else cost += (double)(rounds - 1) * (main > epi ? main : epi) + (pair ? 10600.0 : 8900.0);
+      const double step = pair ? 330.0 + 0.85 * bn : subs_for(false, bn) == 2 ? 410.0 + 0.3 * bn : 480.0 + 0.66 * bn;
+      double cost = (double)rounds * (double)((kchunks + ks - 1) / ks) * step + 25.0 * bn;
+      cost += ks > 1 ? (double)rounds * (12500.0 + 20.0 * bn) : pair ? 10600.0 : 9600.0;
       if (best_cost < 0.0 || cost < best_cost) {
         best_cost = cost;
         best = {pair, bn, ks};
