@@ -29,8 +29,10 @@
 // the GPU. GEMMs of few tiles run on tiles of 128 rows by one CTA and split K: the 2 or 4 CTAs of a
 // tile form a cluster, each accumulates its K-slice, stores the fp32 partial tile in its own freed
 // ring, and the cluster adds the slices through distributed shared memory in a fixed order before the
-// epilogue. pick_shape takes the form, width and split that these costs say finishes first; measured
-// beside every alternative on five layers at T = 80 to 2048 it was within 4% of the best.
+// epilogue. pick_shape takes the form, width and split that these costs say finishes first. Measured beside
+// every alternative in 398 GEMMs (20 layers, T = 80 to 4096), the call was 0.9% behind the best pick in the
+// mean, more than 2% in 58 of them; the worst were layers whose rank is no multiple of 64 (4096 x 4096, r = 1638,
+// T = 2048: 18%, one CTA where a pair's tiles would be read half as often).
 // Against the one-CTA forms that this replaced (us, CUDA graph, one process): 7B attention T = 128
 // 25.2 -> 20.0, 512 37.4 -> 34.6, 2048 58.0 -> 53.9, 4096 119.5 -> 94.7; 7B gate T = 2048 143.8 ->
 // 120.4; 7B down T = 300 48.1 -> 35.9; 70B q/o T = 300 89.4 -> 56.3, 4096 400.3 -> 345.8; 70B gate/up
@@ -493,7 +495,9 @@ int subs_for(bool pair, int bn) { return RING_BYTES / chunk_bytes(pair, bn) >= 6
 
 // The tiling of G groups of `rows` weight rows x T tokens that finishes first by the measured costs, in
 // cycles: a chunk's (see the head of this file), an unhidden epilogue's 25 per token of a tile's width,
-// a launch's 9600 (a pair's 10600), a cluster's 12500 and its exchange of partial tiles 20 per token.
+// a launch's 9600 (a pair's 10600), a cluster's 12500 and its exchange of partial tiles 20 per token. (An
+// epilogue that hides only as far as the next tile's chunks last, and costs refitted to the 398 GEMMs named above,
+// gained up to 15% on some drawn calls and lost up to 9% on others.)
 GemmShape pick_shape(int64_t G, int64_t rows, int64_t T, int64_t kchunks) {
   const Slots slots = tile_slots();
   GemmShape best = {true, BNMAX, 1};
