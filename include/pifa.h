@@ -90,6 +90,9 @@ typedef struct {
  *                nor be used by another call that may run concurrently.
  *   cuda_stream  a cudaStream_t (NULL = legacy default stream).
  *
+ *   X is read after the stream's preceding work has completed. W_p, C and the index sets are taken for
+ *   constants: a kernel that precedes the call in the stream and releases its dependents early
+ *   (programmatic dependent launch) must not be the one that writes them.
  *   Every matrix buffer spans rows x pitch elements: kernels may read a row's padding up to the
  *   next multiple of 8 columns (never write it) and ignore what it holds.
  *   Requirements: 1 <= r <= min(m, n); T >= 0 (T == 0 is a no-op: nothing is read or written and

@@ -427,7 +427,8 @@ def pifa_forward(X, Wp, C, pivot_idx, nonpivot_idx, Y=None, variant: int = PIFA_
         Y = torch.empty((T, m), dtype=torch.bfloat16, device=X.device)
     has_np = m > r
     cdt = c_dtype_of(C if has_np else None)
-    need = pifa_workspace_size(T, m, n, r, variant, cdt)
+    # (the shapes are plain ints)
+    need = (_workspace_size if type(variant) is int else pifa_workspace_size)(T, m, n, r, variant, cdt)
     ws = workspace_tensor
     if need > 0 and ws is None:
         ws = workspace(need, X.device, stream)
