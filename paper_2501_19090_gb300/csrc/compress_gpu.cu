@@ -138,7 +138,9 @@ __global__ void __launch_bounds__(256) gemm_f64_masked(GemmF64 p, const uint32_t
   const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
-    const uint32_t w = i0 + lane < p.M ? mask[(int64_t)(i0 + lane) * words + blockIdx.x] : 0u;
+    // bits beyond N are zero, unless the product that writes the mask gave up a wait and left it as it was
+    const uint32_t in = p.N - j0 < 32 ? (1u << (p.N - j0)) - 1u : 0xffffffffu;
+    const uint32_t w = i0 + lane < p.M ? mask[(int64_t)(i0 + lane) * words + blockIdx.x] & in : 0u;
     s_mask[lane] = w;
     int at = __popc(w);
 #pragma unroll
