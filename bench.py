@@ -63,8 +63,8 @@ NCU_TRAFFIC = {
     # profiles/decode_tc_gateup70b_T16_traffic.md: phase 1 in clusters of 8 CTAs per row block,
     # phase 2 one CTA per row block; two kernels, no partial sums in global memory
     ("llama2_70b_gate_up_28672x8192_r4096", 16): {
-        "sha": {"decode_tc.cu": "60889ab2c50c37f7", "decode.cu": "56fd645c38b82764"},
-        "bytes": 269404160,
+        "sha": {"decode_tc.cu": "793b883af1358eb8", "decode.cu": "f5d86c24bfed89f1"},
+        "bytes": 269429248,
     },
 }
 

@@ -856,16 +856,6 @@ int max_clusters(const void* fn, int ks, size_t smem, int threads = kWarps * 32)
 
 std::atomic<int> g_decode_grid{PIFA_DECODE_GRID_AUTO};  // pifa_set_decode_grid
 
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 1;
-  }
-  return n;
-}
-
 // decode_stream's split of one phase into (ks, kcta, kc, stages, ntiles, ncl) and its shared memory
 // (returned, with 1 KB of alignment slack): the fewest CTAs per cluster giving at least one
 // (tile, K-range) unit per SM (measured: two per SM, through larger clusters, cost more in per-tile
@@ -881,7 +871,7 @@ size_t plan_stream(const void* fn, int kRows, int NT, int NB, DecodeArgs& a, con
   a.bstaged = a.T > 2 ? 1 : 0;
   a.tb = (a.T + 7) / 8 * 8;
   int ks = 1;
-  while (ks < kMaxCluster && ((int64_t)a.ntiles * ks < sm_count() ||
+  while (ks < kMaxCluster && ((int64_t)a.ntiles * ks < pifa_sm_count() ||
                               (!a.bstaged && (size_t)a.ngrp * NB * a.T * row_pitch(kcta_of(a.K, ks)) > kStreamBudget / 3)))
     ks *= 2;
   a.ks = ks;
@@ -992,7 +982,7 @@ struct PhasePlan {
 // phase's form; `first` (phase 2) phase 1's plan.
 PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan* first) {
   const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
-  const int sms = sm_count();
+  const int sms = pifa_sm_count();
   const int64_t work = (int64_t)R * K;
   const int k1 = least_split(1, K, budget), k2 = least_split(2, K, budget);
   const int t16 = (R + 15) / 16, tiles = (R + 31) / 32, tall = (R + 63) / 64 * 4;  // tall: CTAs of 64 rows split four ways
@@ -1036,7 +1026,7 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
 Form phase_form(int phase, int R, int K, int T, int ngrp) {
   const int64_t work = (int64_t)R * K, bytes = work * 2;
   const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
-  const int sms = sm_count();
+  const int sms = pifa_sm_count();
   const int k1 = least_split(1, K, budget), k2 = least_split(2, K, budget);
   const int t16 = (R + 15) / 16, t32 = (R + 31) / 32;
   if (phase == 2 && bytes <= 12000000) {

@@ -633,18 +633,8 @@ __global__ void __launch_bounds__(256) decode_tc_reduce(ReduceArgs a) {
   a.Y[(int64_t)t * a.ldy + col] = __float2bfloat16_rn(sum);
 }
 
-int sm_count_tc() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n = 1;
-  }
-  return n;
-}
-
 int grid_cap() {
-  const int g = CTAS_PER_SM * sm_count_tc();
+  const int g = CTAS_PER_SM * pifa_sm_count();
   return g < GRID_MAX ? g : GRID_MAX;
 }
 

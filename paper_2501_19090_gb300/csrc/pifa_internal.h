@@ -24,6 +24,9 @@ uint64_t pifa_wait_timeout_ns();
 // per successful launch; pifa_launch_count() reads the total.
 void pifa_count_launch();
 
+// SMs of the current device (status.cu); 1 if the query fails, which the next call makes again.
+int pifa_sm_count();
+
 #ifdef __CUDACC__
 #include <utility>
 // cudaLaunchKernelEx, counted.

@@ -43,6 +43,21 @@ int* pifa_status_word(cudaError_t* err) {
   return g_word_addr[dev];
 }
 
+int pifa_sm_count() {
+  static std::atomic<int> known[kMaxDevices];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
+    n = known[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) {
+      known[dev].store(n, std::memory_order_relaxed);
+      return n;
+    }
+  }
+  cudaGetLastError();  // a failed query leaves no sticky error behind
+  return 1;
+}
+
 namespace {
 // Waits, with the library's bound, on an mbarrier that nothing ever arrives on, then latches
 // PIFA_ERR_TIMEOUT: the failure-detection path of every bounded wait, exercised on its own.
