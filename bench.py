@@ -63,7 +63,7 @@ NCU_TRAFFIC = {
     # profiles/decode_tc_gateup70b_T16_traffic.md: phase 1 in clusters of 8 CTAs per row block,
     # phase 2 one CTA per row block; two kernels, no partial sums in global memory
     ("llama2_70b_gate_up_28672x8192_r4096", 16): {
-        "sha": {"decode_tc.cu": "793b883af1358eb8", "decode.cu": "f5d86c24bfed89f1"},
+        "sha": {"decode_tc.cu": "793b883af1358eb8", "decode.cu": "077e3e09eb49a00d"},
         "bytes": 269429248,
     },
 }

@@ -1011,7 +1011,7 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
     // a small phase needs no more SMs, and a split-K phase behind this one wants the free ones
     if (work < (1 << 22) || other == kFormSplitK) return {kFormRows, 2, k2};
   } else {
-    // a small phase in 16 rows, but a long K in 32 and split once more (146 x 7130: 0.88x)
+    // a small phase in 16 rows, but a long K in 32 and split once more (146 x 7130: 16 rows take 1.14x)
     if (work < (1 << 20)) return (phase == 1 ? k1 == 1 : K <= 1400) ? PhasePlan{kFormRows, 1, k1} : PhasePlan{kFormRows, 2, k2};
     if (phase == 1 && round && other != kFormSplitK) return {kFormRows, 4, 4};
   }
@@ -1022,7 +1022,8 @@ PhasePlan plan_rows(int phase, int R, int K, int T, Form other, const PhasePlan*
 
 // The form of a phase. Waves of decode_rows win while an SM stages its share of the weights at launch
 // (about 24 MB in phase 1, 12 MB in phase 2); beyond, their clusters take several rounds. Full rounds of two
-// CTAs per SM (tiles of up to 110 KB) hold on longer. Ratios in these comments: time of the other form over this.
+// CTAs per SM (tiles of up to 110 KB) hold on longer. Ratios in these comments: the other
+// form's time over the taken one's.
 Form phase_form(int phase, int R, int K, int T, int ngrp) {
   const int64_t work = (int64_t)R * K, bytes = work * 2;
   const uint32_t budget = phase == 1 ? kStageBudget1 : kStageBudget2;
@@ -1033,7 +1034,7 @@ Form phase_form(int phase, int R, int K, int T, int ngrp) {
     // more CTAs than two per SM lose to split-K (21248 x 256, T = 12: 1.5x, 10752 x 128: 1.3x, 5828 x 108: 1.4x)
     if (T > 2 && R >= 4096 && (T > 8 && work < (1 << 20) ? t16 * k1 : t32 * k2) > 2 * sms) return kFormSplitK;
     // with two token tiles a K split four ways in more CTAs than SMs loses to split-K (4096 x 4096,
-    // r = 2458, T = 12: 15.8 against 15.0); split two ways it does not (2458 x 1638: 0.94x)
+    // r = 2458, T = 12: 15.8 against 15.0); split two ways it does not (2458 x 1638: 1.07x)
     return T > 8 && k2 > 2 && t32 * k2 > sms ? kFormSplitK : kFormRows;
   }
   if (T <= 2) {
